@@ -10,15 +10,16 @@
 //
 // Kernels:
 //   k_conv3   3x3x3 convolution, zero padding, as an implicit GEMM on the
-//             BF16 tensor cores (mma.sync m16n8k16): rows = cells (16 per
-//             warp), columns = output channels, reduction = 27 taps x input
-//             channels; bias + ReLU fused into the epilogue.  The same kernel
-//             computes the data gradient with flipped, channel-transposed
-//             weights.
-//   k_wgrad   weight gradient per tap, dW_tap = dY^T X_tap, also on the BF16
-//             tensor cores; cells split over blocks, float32 atomics.
-//   the rest  pooling, upsampling, ReLU masks, output layer, the mean-free
-//             mean-square loss and Adam are element-wise kernels.
+//             BF16 tensor cores (mma.sync m16n8k16): rows = cells, columns =
+//             output channels, reduction = 27 taps x input channels, operands
+//             staged in shared memory by halo tiles; bias + ReLU fused.  The
+//             decoder input (upsampled coarse output ++ skip) is gathered
+//             while staging.  The same kernel computes the data gradient with
+//             flipped, channel-transposed weights and the ReLU mask.
+//   k_wgrad   weight gradients, dW_tap = dY^T X_tap of all taps of a tile,
+//             also on the BF16 tensor cores; float32 atomics per block.
+//   the rest  pooling, gradients of pooling / upsampling, output layer, the
+//             mean-free mean-square loss and Adam are element-wise kernels.
 // Layout: activations channel-last ([cell][channel], cells x fastest), every
 // channel count a multiple of 16 (the 4 input channels are zero-padded to 16).
 // Parameters (float32 master copy, BF16 mirror): per convolution c the
@@ -70,240 +71,416 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// cell index of the neighbour of (i, j, k) at tap t, or -1 outside the box
-__device__ __forceinline__ int neighbour(const Dims& d, int i, int j, int k, int t) {
-  const int a = i + t % 3 - 1, b = j + (t / 3) % 3 - 1, c = k + t / 9 - 1;
-  if (a < 0 || a >= d.nx || b < 0 || b >= d.ny || c < 0 || c >= d.nz) return -1;
-  return (c * d.ny + b) * d.nx + a;
+// ------------------------------------------------------------ conv tiles --
+// Both contraction kernels work on spatial tiles of 8 x 4 x 4 cells (level
+// dims are 8, 4, 2, 1 times any integer, so the tiles of level 0 are whole in
+// x and y) staged once, with a one-cell halo, in shared memory as
+// [halo cell][channel] rows.  A row is padded by 16 bytes: with channel counts
+// that are multiples of 16 the row stride is then 16 modulo 32 bytes, so the
+// eight 16-byte rows of an ldmatrix tile fall in different bank groups.
+constexpr int kTX = 8, kTY = 4, kTZ = 4;
+constexpr int kTile = kTX * kTY * kTZ;                              // 128 cells
+constexpr int kHX = kTX + 2, kHY = kTY + 2, kHZ = kTZ + 2;
+constexpr int kHalo = kHX * kHY * kHZ;                              // 360 cells
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+// 16 bytes global -> shared, zeros when !valid (src is not read then)
+__device__ __forceinline__ void cpa16z(void* dst, const void* src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem_u32(dst)), "l"(src),
+               "r"(valid ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cpa_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
 }
 
-// Y[cell][co] = act(bias[co] + sum_{t, ci} X[nb(cell, t)][ci] W[t][co][ci]).
-// X has row stride cin (multiple of 16), Y row stride COUT.  One warp
-// computes 16 cells x COUT channels; rows past the last cell are masked.
-template <int COUT, bool RELU>
-__global__ void __launch_bounds__(128) k_conv3(const bf16* __restrict__ X, int cin,
-                                               const bf16* __restrict__ W,
-                                               const float* __restrict__ bias,
-                                               bf16* __restrict__ Y, Dims d) {
-  const int ncell = d.nx * d.ny * d.nz;
-  const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  const int g = lane >> 2, t4 = lane & 3;
-  const int c0 = warp * 16;
-  if (c0 >= ncell) return;
-  int row[2], ci[2], cj[2], ck[2];
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int c = c0 + g + 8 * h;
-    row[h] = c < ncell ? c : -1;
-    const int cc = c < ncell ? c : 0;
-    ci[h] = cc % d.nx;
-    cj[h] = (cc / d.nx) % d.ny;
-    ck[h] = cc / (d.nx * d.ny);
+// the input of a convolution: X [cell][xc] alone, or (low != null) the decoder
+// input, channels [0, lowc) from the next coarser level (nearest upsampling),
+// the xc others from the skip X
+struct ConvIn {
+  const bf16* X;
+  int xc;
+  const bf16* low;
+  int lowc;
+};
+
+// first cell of spatial tile b of the level
+__device__ __forceinline__ void tile_origin(int b, const Dims& d, int& i, int& j, int& k) {
+  const int tx = (d.nx + kTX - 1) / kTX, ty = (d.ny + kTY - 1) / kTY;
+  i = (b % tx) * kTX;
+  j = (b / tx % ty) * kTY;
+  k = b / (tx * ty) * kTZ;
+}
+
+// channels [c0, c0 + NCH) of the halo of the tile at (i0, j0, k0) -> xs
+// (row pitch NCH + 8 elements); zeros outside the box.  The source of a
+// 16-byte run does not change within it: lowc, xc, c0 are multiples of 8.
+template <int NCH, int NTHR>
+__device__ __forceinline__ void stage_halo(bf16* xs, const ConvIn& in, int c0, int i0, int j0, int k0,
+                                           const Dims& d, int tid) {
+  constexpr int runs = NCH / 8, pitch = NCH + 8;
+#pragma unroll 4
+  for (int e = tid; e < kHalo * runs; e += NTHR) {
+    const int h = e / runs, c = c0 + 8 * (e - h * runs);
+    const int i = i0 + h % kHX - 1, j = j0 + h / kHX % kHY - 1, k = k0 + h / (kHX * kHY) - 1;
+    const bool ok = (unsigned)i < (unsigned)d.nx && (unsigned)j < (unsigned)d.ny && (unsigned)k < (unsigned)d.nz;
+    const bf16* src = in.X;
+    if (ok) {
+      if (c < in.lowc) {
+        const size_t cc = ((size_t)(k >> 1) * (d.ny >> 1) + (j >> 1)) * (d.nx >> 1) + (i >> 1);
+        src = in.low + cc * in.lowc + c;
+      } else {
+        const size_t cc = ((size_t)k * d.ny + j) * d.nx + i;
+        src = in.X + cc * in.xc + (c - in.lowc);
+      }
+    }
+    cpa16z(xs + h * pitch + (c - c0), src, ok);
   }
-  constexpr int NT = COUT / 8;
-  float acc[NT][4];
+}
+
+// Y[cell][co] = act(bias[co] + sum_{t, ci} X[nb(cell, t)][ci] W[t][co][ci]),
+// zero padding; Y has row stride ny_ch.  A block computes 16 output channels
+// (blockIdx.y) of one tile: the halo of X and the 27 x 16 x cin weights are
+// staged once, each of the 4 warps accumulates two 16-cell rows of MMA tiles.
+//   DGRAD: the data gradient with the same kernel: X is the output gradient,
+//   W[t][co][ci] the layer's weights taken as W[26 - t], co the reduction
+//   index; the [co][ci] rows are read transposed by ldmatrix.trans, so no
+//   flipped copy is made.  mask (optional): Y is zeroed where mask <= 0 (the
+//   ReLU of the layer that produced this input).
+// mma.sync rather than tcgen05: the sums must come out in the order (tap,
+// channel chunk) whatever the tiling, because every stored BF16 value (and
+// ReLU decision) downstream flips with the last bit of a float32 sum.
+// Bound by launch latency at the coarse levels (8^3..16^3 cells) and by shared
+// memory at level 0 (3 KB of fragments per 16 KFLOP).  The version that read
+// its fragments from global memory took 111 us for 16 -> 16 at 64^3 and 183 us
+// for 64 -> 64 at 8^3 (8 blocks).
+//   CIN is a template argument so that the staging's index arithmetic and the
+//   channel loop are constants.
+//   MT: 16-cell MMA rows per warp (2: 4 warps; 1: 8 warps, for the levels
+//   whose few blocks leave SMs idle and whose time is one block's chain).
+template <int CIN, bool DGRAD, int MT>
+__global__ void __launch_bounds__(256 / MT) k_conv3(ConvIn in, const bf16* __restrict__ W,
+                                               const float* __restrict__ bias, bf16* __restrict__ Y,
+                                               int cout, const bf16* __restrict__ mask, Dims d) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  constexpr int pitch = CIN + 8, NTHR = 256 / MT;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  bf16* xs = reinterpret_cast<bf16*>(sm);
+  bf16* ws = xs + kHalo * pitch;
+  const int n0 = blockIdx.y * 16;
+  int i0, j0, k0;
+  tile_origin(blockIdx.x, d, i0, j0, k0);
+  stage_halo<CIN, NTHR>(xs, in, 0, i0, j0, k0, d, tid);
+  if (DGRAD) {        // rows (t, reduction index), 16 outputs each, pitch 24
+#pragma unroll 4
+    for (int e = tid; e < 27 * CIN * 2; e += NTHR) {
+      const int r = e >> 1, h = e & 1;
+      cpa16z(ws + r * 24 + 8 * h, W + (size_t)r * cout + n0 + 8 * h, true);
+    }
+  } else {            // rows (t, output), CIN each
+    constexpr int runs = CIN / 8;
+#pragma unroll 4
+    for (int e = tid; e < 27 * 16 * runs; e += NTHR) {
+      const int r = e / runs, q = e - r * runs;
+      cpa16z(ws + r * pitch + 8 * q, W + ((size_t)(r >> 4) * cout + n0 + (r & 15)) * CIN + 8 * q, true);
+    }
+  }
+  cpa_wait_all();
+  __syncthreads();
+  float acc[MT][2][4];
 #pragma unroll
-  for (int n = 0; n < NT; ++n)
+  for (int m = 0; m < MT; ++m)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) acc[n][q] = 0.f;
-  const uint32_t* X32 = reinterpret_cast<const uint32_t*>(X);
-  const uint32_t* W32 = reinterpret_cast<const uint32_t*>(W);
-  for (int t = 0; t < 27; ++t) {
-    int nb[2];
+    for (int n = 0; n < 2; ++n)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) nb[h] = row[h] >= 0 ? neighbour(d, ci[h], cj[h], ck[h], t) : -1;
-    for (int k0 = 0; k0 < cin; k0 += 16) {
-      // A fragment (16 cells x 16 channels): rows g / g+8, columns 2t4.. / 2t4+8..
-      uint32_t a[4];
-      const int col = k0 + 2 * t4;
-      a[0] = nb[0] >= 0 ? X32[((size_t)nb[0] * cin + col) >> 1] : 0u;
-      a[1] = nb[1] >= 0 ? X32[((size_t)nb[1] * cin + col) >> 1] : 0u;
-      a[2] = nb[0] >= 0 ? X32[((size_t)nb[0] * cin + col + 8) >> 1] : 0u;
-      a[3] = nb[1] >= 0 ? X32[((size_t)nb[1] * cin + col + 8) >> 1] : 0u;
+      for (int q = 0; q < 4; ++q) acc[m][n][q] = 0.f;
+  // ldmatrix source rows of this lane: A, cell row (lane & 15), channel half
+  // lane >> 4; B, see below
+  uint32_t abase[MT];
 #pragma unroll
-      for (int n = 0; n < NT; ++n) {
-        // B fragment (16 channels x 8 outputs): W[t][n*8 + g][col], [col + 8]
-        const size_t wb = ((size_t)t * COUT + n * 8 + g) * cin + col;
-        uint32_t b[2];
-        b[0] = __ldg(W32 + (wb >> 1));
-        b[1] = __ldg(W32 + ((wb + 8) >> 1));
-        mma_bf16(acc[n], a, b);
+  for (int m = 0; m < MT; ++m) {
+    const int c = (MT * warp + m) * 16 + (lane & 15);
+    const int x = c % kTX, y = c / kTX % kTY, z = c / (kTX * kTY);
+    abase[m] = smem_u32(xs + ((z * kHY + y) * kHX + x) * pitch + (lane >> 4) * 8);
+  }
+  const uint32_t bbase = DGRAD
+      ? smem_u32(ws + ((lane & 7) + ((lane >> 3) & 1) * 8) * 24 + (lane >> 4) * 8)
+      : smem_u32(ws + ((lane & 7) + (lane >> 4) * 8) * pitch + ((lane >> 3) & 1) * 8);
+  for (int tz = 0; tz < 3; ++tz) {
+#pragma unroll
+    for (int ty = 0; ty < 3; ++ty) {
+#pragma unroll
+      for (int tx = 0; tx < 3; ++tx) {
+        const uint32_t aoff = (uint32_t)(((tz * kHY + ty) * kHX + tx) * pitch) * 2;
+        const int t = 9 * tz + 3 * ty + tx;
+        const uint32_t boff = DGRAD ? (uint32_t)((26 - t) * CIN * 24) * 2 : (uint32_t)(t * 16 * pitch) * 2;
+#pragma unroll
+        for (int kc = 0; kc < CIN; kc += 16) {
+          uint32_t a[MT][4], b[4];
+#pragma unroll
+          for (int m = 0; m < MT; ++m) ldsm4(a[m], abase[m] + aoff + kc * 2);
+          if (DGRAD) ldsm4t(b, bbase + boff + kc * 48);
+          else ldsm4(b, bbase + boff + kc * 2);
+          const uint32_t b0[2] = {b[0], b[1]}, b1[2] = {b[2], b[3]};
+#pragma unroll
+          for (int m = 0; m < MT; ++m) {
+            mma_bf16(acc[m][0], a[m], b0);
+            mma_bf16(acc[m][1], a[m], b1);
+          }
+        }
       }
     }
   }
   // accumulator q: row g + 8 (q >> 1), column 2 t4 + (q & 1)
-#pragma unroll
-  for (int n = 0; n < NT; ++n) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int h = q >> 1;
-      if (row[h] < 0) continue;
-      const int co = n * 8 + 2 * t4 + (q & 1);
-      float v = acc[n][q] + (bias ? bias[co] : 0.f);
-      if (RELU) v = fmaxf(v, 0.f);
-      Y[(size_t)row[h] * COUT + co] = __float2bfloat16(v);
-    }
-  }
-}
-
-// dW[t][co][ci] += sum over the block's cells of dY[cell][co] X[nb(cell, t)][ci].
-// grid: (cell chunks, 27 taps, ceil(items / 4)); one warp per item = (16 co,
-// 16 ci) tile.  A = dY^T (16 co x 16 cells), B = X_t (16 cells x 8 ci).
-__global__ void __launch_bounds__(128) k_wgrad(const bf16* __restrict__ dY, int cout,
-                                               const bf16* __restrict__ X, int cin,
-                                               float* __restrict__ dW, Dims d, int chunk) {
-  const int ncell = d.nx * d.ny * d.nz;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int g = lane >> 2, t4 = lane & 3;
-  const int t = blockIdx.y;
-  const int ci_tiles = cin / 16;
-  const int item = blockIdx.z * 4 + wid;
-  if (item >= (cout / 16) * ci_tiles) return;
-  const int co0 = (item / ci_tiles) * 16, ci0 = (item % ci_tiles) * 16;
-  const int cell_begin = blockIdx.x * chunk;
-  const int cell_end = min(ncell, cell_begin + chunk);
-  float acc[2][4];
 #pragma unroll
-  for (int n = 0; n < 2; ++n)
+  for (int m = 0; m < MT; ++m)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) acc[n][q] = 0.f;
-  const bf16 zero = __float2bfloat16(0.f);
-  for (int c0 = cell_begin; c0 < cell_end; c0 += 16) {
-    const int cell[4] = {c0 + 2 * t4, c0 + 2 * t4 + 1, c0 + 2 * t4 + 8, c0 + 2 * t4 + 9};
-    bf16 lo[4], hi[4];
-    int nb[4];
+    for (int hh = 0; hh < 2; ++hh) {
+      const int c = (MT * warp + m) * 16 + g + 8 * hh;
+      const int i = i0 + c % kTX, j = j0 + c / kTX % kTY, k = k0 + c / (kTX * kTY);
+      if (i >= d.nx || j >= d.ny || k >= d.nz) continue;
+      const size_t o = (((size_t)k * d.ny + j) * d.nx + i) * cout + n0 + 2 * t4;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const bool ok = cell[q] < cell_end;
-      lo[q] = ok ? dY[(size_t)cell[q] * cout + co0 + g] : zero;
-      hi[q] = ok ? dY[(size_t)cell[q] * cout + co0 + g + 8] : zero;
-      const int c = ok ? cell[q] : 0;
-      nb[q] = ok ? neighbour(d, c % d.nx, (c / d.nx) % d.ny, c / (d.nx * d.ny), t) : -1;
+      for (int n = 0; n < 2; ++n) {
+        float v0 = acc[m][n][2 * hh] + (bias ? bias[n0 + n * 8 + 2 * t4] : 0.f);
+        float v1 = acc[m][n][2 * hh + 1] + (bias ? bias[n0 + n * 8 + 2 * t4 + 1] : 0.f);
+        if (!DGRAD) { v0 = fmaxf(v0, 0.f); v1 = fmaxf(v1, 0.f); }   // ReLU
+        if (mask) {
+          const __nv_bfloat162 y = *reinterpret_cast<const __nv_bfloat162*>(mask + o + n * 8);
+          if (!(__bfloat162float(y.x) > 0.f)) v0 = 0.f;
+          if (!(__bfloat162float(y.y) > 0.f)) v1 = 0.f;
+        }
+        *reinterpret_cast<uint32_t*>(Y + o + n * 8) = pack2(__float2bfloat16(v0), __float2bfloat16(v1));
+      }
     }
-    uint32_t a[4];
-    a[0] = pack2(lo[0], lo[1]);   // row g,     cells 2t4, 2t4+1
-    a[1] = pack2(hi[0], hi[1]);   // row g + 8
-    a[2] = pack2(lo[2], lo[3]);   // row g,     cells 2t4+8, 2t4+9
-    a[3] = pack2(hi[2], hi[3]);   // row g + 8
+}
+
+inline size_t conv_smem(int cin, bool dgrad) {
+  return sizeof(bf16) * ((size_t)kHalo * (cin + 8) + (dgrad ? (size_t)27 * cin * 24 : (size_t)27 * 16 * (cin + 8)));
+}
+
+// dW[t][co][ci] += sum over cells dY[cell][co] X[nb(cell, t)][ci], db[co] +=
+// sum dY[cell][co].  blockIdx.y = (16-channel tile of co, 16 NCI channels of
+// ci); the block walks over tiles blockIdx.x, + gridDim.x, ..., stages dY and
+// the halo of X, and each of its 9 warps keeps the accumulators of 3 taps in
+// registers over all of them (M = 16 co, N = 16 NCI ci, K = cells; dY and X
+// are read through ldmatrix.trans), so a weight is added to global memory
+// once per block.  Per 16 cells a warp reads 0.5 KB of dY and 1.5 NCI KB of X
+// for 6 NCI MMAs.  The version with one warp per (tap, 16 x 16) tile gathered
+// 2-byte elements from global memory: 375 us per 16 -> 16 layer at 64^3.
+template <int NCI>
+__global__ void __launch_bounds__(288) k_wgrad(const bf16* __restrict__ dY, int cout, ConvIn in,
+                                               int cin, float* __restrict__ dW,
+                                               float* __restrict__ db, Dims d, int ntile) {
+  constexpr int CI = 16 * NCI, XP = CI + 8, YP = 24;
+  __shared__ __align__(16) bf16 xs[kHalo * XP];
+  __shared__ __align__(16) bf16 ys[kTile * YP];
+  __shared__ float sb[16];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ncc = cin / CI;
+  const int co0 = (blockIdx.y / ncc) * 16, ci0 = (blockIdx.y % ncc) * CI;
+  const bool do_bias = ci0 == 0;
+  float acc[3][2 * NCI][4];
 #pragma unroll
-    for (int n = 0; n < 2; ++n) {
-      const int c = ci0 + n * 8 + g;
-      bf16 x[4];
+  for (int t = 0; t < 3; ++t)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) x[q] = nb[q] >= 0 ? X[(size_t)nb[q] * cin + c] : zero;
-      uint32_t b[2];
-      b[0] = pack2(x[0], x[1]);
-      b[1] = pack2(x[2], x[3]);
-      mma_bf16(acc[n], a, b);
+    for (int n = 0; n < 2 * NCI; ++n)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[t][n][q] = 0.f;
+  float bsum = 0.f;
+  if (tid < 16) sb[tid] = 0.f;
+  // A = dY^T from [cell][co] rows, B = X from [cell][ci] rows, both transposed
+  const uint32_t abase = smem_u32(ys + ((lane & 7) + (lane >> 4) * 8) * YP + ((lane >> 3) & 1) * 8);
+  const int kr = (lane & 7) + ((lane >> 3) & 1) * 8;   // cell row of the 16 this lane addresses for B
+  uint32_t toff[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const int t = 3 * warp + q;
+    toff[q] = (uint32_t)((((t / 9) * kHY + (t / 3) % 3) * kHX + t % 3) * XP) * 2;
+  }
+  for (int b = blockIdx.x; b < ntile; b += gridDim.x) {
+    int i0, j0, k0;
+    tile_origin(b, d, i0, j0, k0);
+    __syncthreads();                          // the previous tile is consumed
+    stage_halo<CI, 288>(xs, in, ci0, i0, j0, k0, d, tid);
+    if (tid < 2 * kTile) {
+      const int c = tid >> 1, h = tid & 1;
+      const int i = i0 + c % kTX, j = j0 + c / kTX % kTY, k = k0 + c / (kTX * kTY);
+      const bool ok = i < d.nx && j < d.ny && k < d.nz;
+      const size_t o = ok ? (((size_t)k * d.ny + j) * d.nx + i) * cout + co0 + 8 * h : 0;
+      cpa16z(ys + c * YP + 8 * h, dY + o, ok);
+    }
+    cpa_wait_all();
+    __syncthreads();
+    if (do_bias && tid < 256) {
+#pragma unroll
+      for (int q = 0; q < kTile / 16; ++q) bsum += __bfloat162float(ys[(q * 16 + (tid >> 4)) * YP + (tid & 15)]);
+    }
+#pragma unroll 2
+    for (int s = 0; s < kTile / 16; ++s) {
+      uint32_t a[4];
+      ldsm4t(a, abase + s * 16 * YP * 2);
+      const int c = s * 16 + kr;
+      const int x = c % kTX, y = c / kTX % kTY, z = c / (kTX * kTY);
+      const uint32_t bb = smem_u32(xs + ((z * kHY + y) * kHX + x) * XP + (lane >> 4) * 8);
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+#pragma unroll
+        for (int n = 0; n < NCI; ++n) {
+          uint32_t r[4];
+          ldsm4t(r, bb + toff[q] + n * 32);
+          const uint32_t b0[2] = {r[0], r[1]}, b1[2] = {r[2], r[3]};
+          mma_bf16(acc[q][2 * n], a, b0);
+          mma_bf16(acc[q][2 * n + 1], a, b1);
+        }
     }
   }
+  const int g = lane >> 2, t4 = lane & 3;
 #pragma unroll
-  for (int n = 0; n < 2; ++n)
+  for (int q = 0; q < 3; ++q)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int co = co0 + g + 8 * (q >> 1);
-      const int c = ci0 + n * 8 + 2 * t4 + (q & 1);
-      atomicAdd(dW + ((size_t)t * cout + co) * cin + c, acc[n][q]);
+    for (int n = 0; n < 2 * NCI; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int co = co0 + g + 8 * (e >> 1);
+        const int c = ci0 + n * 8 + 2 * t4 + (e & 1);
+        atomicAdd(dW + ((size_t)(3 * warp + q) * cout + co) * cin + c, acc[q][n][e]);
+      }
+  if (do_bias) {
+    if (tid < 256) {                          // lanes l and l + 16 hold the same channel
+      bsum += __shfl_xor_sync(0xffffffffu, bsum, 16);
+      if (lane < 16) atomicAdd(&sb[lane], bsum);
     }
-}
-
-// weights of the data-gradient convolution: Wt[26 - t][ci][co] = W[t][co][ci]
-__global__ void k_flip(const bf16* __restrict__ W, bf16* __restrict__ Wt, int cout, int cin) {
-  const int n = 27 * cout * cin;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-    const int t = e / (cout * cin), rem = e % (cout * cin);
-    const int co = rem / cin, c = rem % cin;
-    Wt[((size_t)(26 - t) * cin + c) * cout + co] = W[e];
+    __syncthreads();
+    if (tid < 16) atomicAdd(db + co0 + tid, sb[tid]);
   }
 }
 
-// g[e] = 0 where the ReLU output y[e] is not positive
-__global__ void k_relu_mask(bf16* __restrict__ g, const bf16* __restrict__ y, int64_t n) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-    if (!(__bfloat162float(y[e]) > 0.f)) g[e] = __float2bfloat16(0.f);
+// eight BF16 channels of a 16-byte run
+struct Run8 {
+  float v[8];
+};
+__device__ __forceinline__ Run8 load8(const bf16* p) {
+  const uint4 u = *reinterpret_cast<const uint4*>(p);
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+  Run8 r;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    r.v[2 * q] = __uint_as_float(w[q] << 16);
+    r.v[2 * q + 1] = __uint_as_float(w[q] & 0xffff0000u);
+  }
+  return r;
+}
+__device__ __forceinline__ void store8(bf16* p, const Run8& r) {
+  uint32_t w[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) w[q] = pack2(__float2bfloat16(r.v[2 * q]), __float2bfloat16(r.v[2 * q + 1]));
+  *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+// zero r where the ReLU output at y is not positive
+__device__ __forceinline__ void mask8(Run8& r, const bf16* y) {
+  const Run8 m = load8(y);
+#pragma unroll
+  for (int q = 0; q < 8; ++q)
+    if (!(m.v[q] > 0.f)) r.v[q] = 0.f;
 }
 
-// 2x2x2 mean pooling of X (fine dims d, ch channels) into Y (coarse)
+// 2x2x2 mean pooling of X (fine dims d, ch channels) into Y (coarse); one
+// thread per cell and 8 channels, as in the two kernels below
 __global__ void k_pool(const bf16* __restrict__ X, bf16* __restrict__ Y, int ch, Dims d) {
-  const int cx = d.nx / 2, cy = d.ny / 2, cz = d.nz / 2;
-  const int64_t n = (int64_t)cx * cy * cz * ch;
+  const int cx = d.nx / 2, cy = d.ny / 2, cz = d.nz / 2, runs = ch >> 3;
+  const int64_t n = (int64_t)cx * cy * cz * runs;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(e / ch), k = (int)(e % ch);
+    const int c = (int)(e / runs), k = 8 * (int)(e - (int64_t)c * runs);
     const int i = c % cx, j = (c / cx) % cy, l = c / (cx * cy);
-    float s = 0.f;
+    Run8 s = {};
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const int f = ((2 * l + (q >> 2)) * d.ny + 2 * j + ((q >> 1) & 1)) * d.nx + 2 * i + (q & 1);
-      s += __bfloat162float(X[(size_t)f * ch + k]);
+      const Run8 x = load8(X + (size_t)f * ch + k);
+#pragma unroll
+      for (int o = 0; o < 8; ++o) s.v[o] += x.v[o];
     }
-    Y[e] = __float2bfloat16(0.125f * s);
+#pragma unroll
+    for (int o = 0; o < 8; ++o) s.v[o] *= 0.125f;
+    store8(Y + (size_t)c * ch + k, s);
   }
 }
 
-// adjoint of the pooling, added to dX (fine): dX[f] = dX[f] + dY[coarse(f)] / 8
-__global__ void k_pool_back(const bf16* __restrict__ dY, bf16* __restrict__ dX, int ch, Dims d) {
-  const int64_t n = (int64_t)d.nx * d.ny * d.nz * ch;
-  const int cx = d.nx / 2, cy = d.ny / 2;
+// gradient of an encoder output that feeds the pooling (dY, coarse) and the
+// skip (dS): dX[f] = dS[f] + dY[coarse(f)] / 8, zero where act <= 0
+__global__ void k_pool_back(const bf16* __restrict__ dY, const bf16* __restrict__ dS,
+                            const bf16* __restrict__ act, bf16* __restrict__ dX, int ch, Dims d) {
+  const int cx = d.nx / 2, cy = d.ny / 2, runs = ch >> 3;
+  const int64_t n = (int64_t)d.nx * d.ny * d.nz * runs;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const int f = (int)(e / ch), k = (int)(e % ch);
+    const int f = (int)(e / runs), k = 8 * (int)(e - (int64_t)f * runs);
     const int i = f % d.nx, j = (f / d.nx) % d.ny, l = f / (d.nx * d.ny);
     const int c = ((l / 2) * cy + j / 2) * cx + i / 2;
-    dX[e] = __float2bfloat16(__bfloat162float(dX[e]) + 0.125f * __bfloat162float(dY[(size_t)c * ch + k]));
+    Run8 s = load8(dS + (size_t)f * ch + k);
+    const Run8 y = load8(dY + (size_t)c * ch + k);
+#pragma unroll
+    for (int o = 0; o < 8; ++o) s.v[o] += 0.125f * y.v[o];
+    mask8(s, act + (size_t)f * ch + k);
+    store8(dX + (size_t)f * ch + k, s);
   }
 }
 
-// decoder input: Y[f] = [X_low[coarse(f)] (lowc ch), S[f] (skipc ch)]
-__global__ void k_up_cat(const bf16* __restrict__ Xl, int lowc, const bf16* __restrict__ S,
-                         int skipc, bf16* __restrict__ Y, Dims d) {
-  const int ch = lowc + skipc;
-  const int64_t n = (int64_t)d.nx * d.ny * d.nz * ch;
-  const int cx = d.nx / 2, cy = d.ny / 2;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const int f = (int)(e / ch), k = (int)(e % ch);
-    if (k < lowc) {
-      const int i = f % d.nx, j = (f / d.nx) % d.ny, l = f / (d.nx * d.ny);
-      const int c = ((l / 2) * cy + j / 2) * cx + i / 2;
-      Y[e] = Xl[(size_t)c * lowc + k];
-    } else {
-      Y[e] = S[(size_t)f * skipc + k - lowc];
-    }
-  }
-}
-
-// adjoint of k_up_cat: dXl[c] = sum of the 8 fine gradients (first lowc
-// channels), dS[f] = the remaining channels
+// gradient of a decoder input [low (upsampled, lowc ch), skip]: dXl[c] = sum
+// of the 8 fine gradients, zero where the low output actl <= 0; dS[f] = the
+// remaining channels
 __global__ void k_up_cat_back(const bf16* __restrict__ dY, int lowc, int skipc,
-                              bf16* __restrict__ dXl, bf16* __restrict__ dS, Dims d) {
-  const int ch = lowc + skipc;
+                              const bf16* __restrict__ actl, bf16* __restrict__ dXl,
+                              bf16* __restrict__ dS, Dims d) {
+  const int ch = lowc + skipc, lr = lowc >> 3, sr = skipc >> 3;
   const int cx = d.nx / 2, cy = d.ny / 2, cz = d.nz / 2;
-  const int64_t nc = (int64_t)cx * cy * cz * lowc;
-  const int64_t nf = (int64_t)d.nx * d.ny * d.nz * skipc;
+  const int64_t nc = (int64_t)cx * cy * cz * lr;
+  const int64_t nf = (int64_t)d.nx * d.ny * d.nz * sr;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nc + nf; e += (int64_t)gridDim.x * blockDim.x) {
     if (e < nc) {
-      const int c = (int)(e / lowc), k = (int)(e % lowc);
+      const int c = (int)(e / lr), k = 8 * (int)(e - (int64_t)c * lr);
       const int i = c % cx, j = (c / cx) % cy, l = c / (cx * cy);
-      float s = 0.f;
+      Run8 s = {};
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         const int f = ((2 * l + (q >> 2)) * d.ny + 2 * j + ((q >> 1) & 1)) * d.nx + 2 * i + (q & 1);
-        s += __bfloat162float(dY[(size_t)f * ch + k]);
+        const Run8 y = load8(dY + (size_t)f * ch + k);
+#pragma unroll
+        for (int o = 0; o < 8; ++o) s.v[o] += y.v[o];
       }
-      dXl[e] = __float2bfloat16(s);
+      mask8(s, actl + (size_t)c * lowc + k);
+      store8(dXl + (size_t)c * lowc + k, s);
     } else {
       const int64_t e2 = e - nc;
-      const int f = (int)(e2 / skipc), k = (int)(e2 % skipc);
-      dS[e2] = dY[(size_t)f * ch + lowc + k];
+      const int f = (int)(e2 / sr), k = 8 * (int)(e2 - (int64_t)f * sr);
+      *reinterpret_cast<uint4*>(dS + (size_t)f * skipc + k) =
+          *reinterpret_cast<const uint4*>(dY + (size_t)f * ch + lowc + k);
     }
   }
 }
 
 // raw input planes in[4][ncell] (float32) -> X[ncell][16] (channels 4..15 zero)
 __global__ void k_pack_planes(const float* __restrict__ in, bf16* __restrict__ X, int ncell) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncell; c += gridDim.x * blockDim.x)
+  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncell; c += gridDim.x * blockDim.x) {
+    Run8 r = {};
 #pragma unroll
-    for (int k = 0; k < 16; ++k)
-      X[(size_t)c * 16 + k] = __float2bfloat16(k < 4 ? in[(size_t)k * ncell + c] : 0.f);
+    for (int k = 0; k < 4; ++k) r.v[k] = in[(size_t)k * ncell + c];
+    store8(X + (size_t)c * 16, r);
+    store8(X + (size_t)c * 16 + 8, Run8{});
+  }
 }
 
 // max |r| (non-negative floats order like their bit patterns)
@@ -404,7 +581,9 @@ __global__ void k_err_sum(const float* __restrict__ out, const float* __restrict
 }
 
 // mean-free square loss L = mean (e - mean e)^2, e = out - t.  red[1] += L,
-// dH = dL/dout * w (BF16), dw[k] += sum dL/dout H[k], db += sum dL/dout.
+// dH = dL/dout * w (BF16; zero where the ReLU output H <= 0), dw[k] += sum
+// dL/dout H[k], db += sum dL/dout.  The 17 sums are reduced over the warp
+// before they reach shared memory (one atomic per warp and sum).
 __global__ void k_head_back(const bf16* __restrict__ H, const float* __restrict__ w,
                             const float* __restrict__ out, const float* __restrict__ t, int n,
                             double* red, bf16* __restrict__ dH, float* __restrict__ dw,
@@ -414,38 +593,36 @@ __global__ void k_head_back(const bf16* __restrict__ H, const float* __restrict_
   __syncthreads();
   const double ebar = red[0] / n;
   double l = 0.0;
-  float gw[16], gb = 0.f;
+  float gw[17];
 #pragma unroll
-  for (int k = 0; k < 16; ++k) gw[k] = 0.f;
+  for (int k = 0; k < 17; ++k) gw[k] = 0.f;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
     const double e = (double)out[c] - (double)t[c] - ebar;
     l += e * e / n;
     const float go = (float)(2.0 * e / n);
-    gb += go;
+    gw[16] += go;
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      gw[k] += go * __bfloat162float(H[(size_t)c * 16 + k]);
-      dH[(size_t)c * 16 + k] = __float2bfloat16(go * w[k]);
+    for (int h = 0; h < 2; ++h) {
+      const Run8 x = load8(H + (size_t)c * 16 + 8 * h);
+      Run8 y;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        gw[8 * h + k] += go * x.v[k];
+        y.v[k] = x.v[k] > 0.f ? go * w[8 * h + k] : 0.f;
+      }
+      store8(dH + (size_t)c * 16 + 8 * h, y);
     }
   }
 #pragma unroll
-  for (int k = 0; k < 16; ++k) atomicAdd(&sg[k], gw[k]);
-  atomicAdd(&sg[16], gb);
+  for (int k = 0; k < 17; ++k) {
+    for (int o = 16; o > 0; o >>= 1) gw[k] += __shfl_xor_sync(0xffffffffu, gw[k], o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&sg[k], gw[k]);
+  }
   for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
   if ((threadIdx.x & 31) == 0) atomicAdd(red + 1, l);
   __syncthreads();
   if (threadIdx.x < 16) atomicAdd(dw + threadIdx.x, sg[threadIdx.x]);
   if (threadIdx.x == 16) atomicAdd(db, sg[16]);
-}
-
-// db[co] += sum_cells dY[cell][co]; grid (blocks, cout)
-__global__ void k_bias_grad(const bf16* __restrict__ dY, int cout, int ncell, float* __restrict__ db) {
-  const int co = blockIdx.y;
-  float s = 0.f;
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncell; c += gridDim.x * blockDim.x)
-    s += __bfloat162float(dY[(size_t)c * cout + co]);
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(db + co, s);
 }
 
 // Adam (Kingma & Ba 2015) on the float32 parameters; refreshes the BF16 mirror
@@ -485,7 +662,6 @@ struct fv_unet {
   int head_w = 0, head_b = 0;
   float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;   // params, grads, Adam moments
   fv::unet::bf16* pb = nullptr;   // BF16 mirror of the parameters
-  fv::unet::bf16* wt = nullptr;   // flipped weights of one layer
   int step = 0;
   // activation workspace, sized for cap cells at level 0 (level l: cap / 8^l)
   int64_t cap = 0, gcap = 0;
@@ -494,7 +670,6 @@ struct fv_unet {
   bool have_fwd = false;          // a forward pass at the current dims is in the buffers
   fv::unet::bf16* in16 = nullptr;
   fv::unet::bf16* act[fv::unet::kNConv] = {};
-  fv::unet::bf16* cat[3] = {};    // decoder inputs at levels 2, 1, 0
   fv::unet::bf16* pool[3] = {};   // pooled encoder outputs (inputs of levels 1..3)
   float* out = nullptr;           // network output [cells]
   float* tgt = nullptr;           // normalised target [cells]
@@ -526,7 +701,7 @@ static void dfree(void* p) {
 static void free_ws(fv_unet* u) {
   dfree(u->in16);
   for (auto& a : u->act) { dfree(a); a = nullptr; }
-  for (int q = 0; q < 3; ++q) { dfree(u->cat[q]); dfree(u->pool[q]); u->cat[q] = u->pool[q] = nullptr; }
+  for (auto& p : u->pool) { dfree(p); p = nullptr; }
   dfree(u->out); dfree(u->tgt);
   u->in16 = nullptr; u->out = u->tgt = nullptr;
   u->cap = 0;
@@ -560,10 +735,8 @@ static fv_status ensure_ws(fv_unet* u, int nx, int ny, int nz) {
     A((void**)&u->in16, (size_t)nc * 16 * sizeof(bf16));
     for (int c = 0; c < kNConv; ++c)
       A((void**)&u->act[c], (size_t)(nc >> (3 * kConvs[c].level)) * kConvs[c].cout * sizeof(bf16));
-    for (int q = 0; q < 3; ++q) {
-      A((void**)&u->cat[q], (size_t)(nc >> (3 * (2 - q))) * kConvs[8 + 2 * q].cin * sizeof(bf16));
+    for (int q = 0; q < 3; ++q)
       A((void**)&u->pool[q], (size_t)(nc >> (3 * (q + 1))) * kConvs[2 * q + 1].cout * sizeof(bf16));
-    }
     A((void**)&u->out, (size_t)nc * sizeof(float));
     A((void**)&u->tgt, (size_t)nc * sizeof(float));
     if (s != FV_OK) { free_ws(u); return s; }
@@ -606,28 +779,79 @@ static fv_status ensure_grad(fv_unet* u) {
     FV_CHECK_LAUNCH();     \
   } while (0)
 
-template <int COUT, bool RELU>
-static fv_status conv_t(cudaStream_t st, const bf16* X, int cin, const bf16* W, const float* b,
-                        bf16* Y, const int n[3]) {
+inline int tiles(const int n[3]) {
+  return ((n[0] + kTX - 1) / kTX) * ((n[1] + kTY - 1) / kTY) * ((n[2] + kTZ - 1) / kTZ);
+}
+
+template <int CIN, bool DGRAD>
+static fv_status conv_t(cudaStream_t st, const ConvIn& in, const bf16* W, const float* bias, bf16* Y,
+                        int cout, const bf16* mask, const int n[3]) {
   const Dims d{n[0], n[1], n[2]};
-  const int64_t warps = ((int64_t)n[0] * n[1] * n[2] + 15) / 16;
-  UNET_LAUNCH((k_conv3<COUT, RELU><<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(X, cin, W, b, Y, d)));
+  const dim3 grid(tiles(n), cout / 16);
+  const size_t smem = conv_smem(CIN, DGRAD);
+  // at least one block per SM: throughput counts, two MMA rows share a weight
+  // fragment; fewer: one block's chain of taps counts, half as long with one
+  if ((int64_t)grid.x * grid.y >= 152)
+    UNET_LAUNCH((k_conv3<CIN, DGRAD, 2><<<grid, 128, smem, st>>>(in, W, bias, Y, cout, mask, d)));
+  else
+    UNET_LAUNCH((k_conv3<CIN, DGRAD, 1><<<grid, 256, smem, st>>>(in, W, bias, Y, cout, mask, d)));
   return FV_OK;
 }
 
-template <bool RELU>
-static fv_status conv(cudaStream_t st, const bf16* X, int cin, const bf16* W, const float* b,
-                      bf16* Y, int cout, const int n[3]) {
-  switch (cout) {
-    case 16: return conv_t<16, RELU>(st, X, cin, W, b, Y, n);
-    case 32: return conv_t<32, RELU>(st, X, cin, W, b, Y, n);
-    case 48: return conv_t<48, RELU>(st, X, cin, W, b, Y, n);
-    case 64: return conv_t<64, RELU>(st, X, cin, W, b, Y, n);
-    case 80: return conv_t<80, RELU>(st, X, cin, W, b, Y, n);
-    case 112: return conv_t<112, RELU>(st, X, cin, W, b, Y, n);
-    default: set_error("unet: unsupported channel count"); return FV_EINVAL;
+template <bool DGRAD>
+static fv_status conv_any(cudaStream_t st, const ConvIn& in, int cin, const bf16* W, const float* bias,
+                          bf16* Y, int cout, const bf16* mask, const int n[3]) {
+  switch (cin) {
+    case 16: return conv_t<16, DGRAD>(st, in, W, bias, Y, cout, mask, n);
+    case 32: return conv_t<32, DGRAD>(st, in, W, bias, Y, cout, mask, n);
+    case 48: return conv_t<48, DGRAD>(st, in, W, bias, Y, cout, mask, n);
+    case 64: return conv_t<64, DGRAD>(st, in, W, bias, Y, cout, mask, n);
   }
+  if constexpr (!DGRAD) {
+    if (cin == 80) return conv_t<80, false>(st, in, W, bias, Y, cout, mask, n);
+    if (cin == 112) return conv_t<112, false>(st, in, W, bias, Y, cout, mask, n);
+  }
+  set_error("unet: unsupported channel count");
+  return FV_EINVAL;
 }
+
+template <int CIN, bool DGRAD>
+static fv_status conv_attr() {
+  const int b = (int)conv_smem(CIN, DGRAD);
+  FV_CUDA(cudaFuncSetAttribute(k_conv3<CIN, DGRAD, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, b));
+  FV_CUDA(cudaFuncSetAttribute(k_conv3<CIN, DGRAD, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, b));
+  return FV_OK;
+}
+
+// up to 190 KB of shared memory (112 input channels)
+static fv_status set_conv_attributes() {
+  FV_TRY((conv_attr<16, false>()));
+  FV_TRY((conv_attr<32, false>()));
+  FV_TRY((conv_attr<48, false>()));
+  FV_TRY((conv_attr<64, false>()));
+  FV_TRY((conv_attr<80, false>()));
+  FV_TRY((conv_attr<112, false>()));
+  FV_TRY((conv_attr<16, true>()));
+  FV_TRY((conv_attr<32, true>()));
+  FV_TRY((conv_attr<48, true>()));
+  FV_TRY((conv_attr<64, true>()));
+  return FV_OK;
+}
+
+// activations of layer c from its input
+static fv_status conv(fv_unet* u, int c, const ConvIn& in) {
+  const ConvSpec& s = kConvs[c];
+  return conv_any<false>(u->stream, in, s.cin, u->pb + u->woff[c], u->p + u->boff[c], u->act[c], s.cout,
+                         nullptr, u->n[s.level]);
+}
+
+// input of the first convolution of decoder level q: [up(low), skip]
+static ConvIn decoder_in(const fv_unet* u, int q) {
+  const int l = 2 - q, lowl = q > 0 ? 9 + 2 * (q - 1) : 7;
+  return {u->act[2 * l + 1], kConvs[2 * l + 1].cout, u->act[lowl], kConvs[lowl].cout};
+}
+
+static ConvIn plain_in(const bf16* X, int c) { return {X, kConvs[c].cin, nullptr, 0}; }
 
 // forward pass from u->in16 to u->out
 static fv_status forward(fv_unet* u) {
@@ -635,31 +859,19 @@ static fv_status forward(fv_unet* u) {
   const bf16* X = u->in16;
   for (int l = 0; l < 4; ++l) {
     const int c1 = 2 * l, c2 = 2 * l + 1;
-    FV_TRY(conv<true>(st, X, kConvs[c1].cin, u->pb + u->woff[c1], u->p + u->boff[c1], u->act[c1],
-                      kConvs[c1].cout, u->n[l]));
-    FV_TRY(conv<true>(st, u->act[c1], kConvs[c2].cin, u->pb + u->woff[c2], u->p + u->boff[c2],
-                      u->act[c2], kConvs[c2].cout, u->n[l]));
+    FV_TRY(conv(u, c1, plain_in(X, c1)));
+    FV_TRY(conv(u, c2, plain_in(u->act[c1], c2)));
     if (l < 3) {
       const Dims d{u->n[l][0], u->n[l][1], u->n[l][2]};
-      UNET_LAUNCH((k_pool<<<blocks_for(u->ncell[l + 1] * kConvs[c2].cout), 256, 0, st>>>(
+      UNET_LAUNCH((k_pool<<<blocks_for(u->ncell[l + 1] * kConvs[c2].cout / 8), 256, 0, st>>>(
           u->act[c2], u->pool[l], kConvs[c2].cout, d)));
       X = u->pool[l];
     }
   }
-  const bf16* low = u->act[7];
-  int lowc = kConvs[7].cout;
   for (int q = 0; q < 3; ++q) {
-    const int l = 2 - q, c1 = 8 + 2 * q, c2 = 9 + 2 * q;
-    const int skipc = kConvs[2 * l + 1].cout;
-    const Dims d{u->n[l][0], u->n[l][1], u->n[l][2]};
-    UNET_LAUNCH((k_up_cat<<<blocks_for(u->ncell[l] * (lowc + skipc)), 256, 0, st>>>(
-        low, lowc, u->act[2 * l + 1], skipc, u->cat[q], d)));
-    FV_TRY(conv<true>(st, u->cat[q], kConvs[c1].cin, u->pb + u->woff[c1], u->p + u->boff[c1],
-                      u->act[c1], kConvs[c1].cout, u->n[l]));
-    FV_TRY(conv<true>(st, u->act[c1], kConvs[c2].cin, u->pb + u->woff[c2], u->p + u->boff[c2],
-                      u->act[c2], kConvs[c2].cout, u->n[l]));
-    low = u->act[c2];
-    lowc = kConvs[c2].cout;
+    const int c1 = 8 + 2 * q, c2 = 9 + 2 * q;
+    FV_TRY(conv(u, c1, decoder_in(u, q)));
+    FV_TRY(conv(u, c2, plain_in(u->act[c1], c2)));
   }
   UNET_LAUNCH((k_head<<<blocks_for(u->ncell[0]), 256, 0, st>>>(u->act[13], u->p + u->head_w,
                                                                  u->p + u->head_b, u->out,
@@ -668,37 +880,28 @@ static fv_status forward(fv_unet* u) {
   return FV_OK;
 }
 
-static fv_status relu_back(fv_unet* u, bf16* gy, int c) {
-  const int64_t n = u->ncell[kConvs[c].level] * kConvs[c].cout;
-  UNET_LAUNCH((k_relu_mask<<<blocks_for(n), 256, 0, u->stream>>>(gy, u->act[c], n)));
+// parameter gradients of layer c from its pre-activation gradient gy and its
+// input.  About two blocks per SM over (tiles x channel pairs): fewer blocks
+// leave SMs idle, more only add atomics (27 x 16 x 16 NCI per block).
+static fv_status param_grad(fv_unet* u, int c, const bf16* gy, const ConvIn& in) {
+  const ConvSpec& s = kConvs[c];
+  const int* n = u->n[s.level];
+  const Dims d{n[0], n[1], n[2]};
+  const int nci = s.cin % 48 == 0 ? 3 : s.cin % 32 == 0 ? 2 : 1;
+  const int items = (s.cout / 16) * (s.cin / (16 * nci)), nt = tiles(n);
+  const dim3 grid(std::max(1, std::min(nt, 2 * 152 / items)), items);
+  float *dw = u->g + u->woff[c], *db = u->g + u->boff[c];
+  if (nci == 3) UNET_LAUNCH((k_wgrad<3><<<grid, 288, 0, u->stream>>>(gy, s.cout, in, s.cin, dw, db, d, nt)));
+  else if (nci == 2) UNET_LAUNCH((k_wgrad<2><<<grid, 288, 0, u->stream>>>(gy, s.cout, in, s.cin, dw, db, d, nt)));
+  else UNET_LAUNCH((k_wgrad<1><<<grid, 288, 0, u->stream>>>(gy, s.cout, in, s.cin, dw, db, d, nt)));
   return FV_OK;
 }
 
-// parameter gradients of layer c from its pre-activation gradient gy and input X
-static fv_status param_grad(fv_unet* u, int c, const bf16* gy, const bf16* X) {
+// input gradient of layer c from gy (cin channels), zero where mask <= 0
+static fv_status data_grad(fv_unet* u, int c, const bf16* gy, bf16* dX, const bf16* mask) {
   const ConvSpec& s = kConvs[c];
-  const int64_t nc = u->ncell[s.level];
-  const Dims d{u->n[s.level][0], u->n[s.level][1], u->n[s.level][2]};
-  const int items = (s.cout / 16) * (s.cin / 16);
-  const int zb = (items + 3) / 4;
-  // about 8 blocks per SM over (chunks x 27 taps x zb), chunks of >= 256 cells
-  int64_t chunks = std::max<int64_t>(1, (152 * 8 + 27 * zb - 1) / (27 * zb));
-  chunks = std::min<int64_t>(chunks, std::max<int64_t>(1, nc / 256));
-  const int64_t chunk = ((nc + chunks - 1) / chunks + 15) / 16 * 16;
-  chunks = (nc + chunk - 1) / chunk;
-  UNET_LAUNCH((k_wgrad<<<dim3((unsigned)chunks, 27, zb), 128, 0, u->stream>>>(
-      gy, s.cout, X, s.cin, u->g + u->woff[c], d, (int)chunk)));
-  UNET_LAUNCH((k_bias_grad<<<dim3(std::min<unsigned>(64, blocks_for(nc)), s.cout), 256, 0, u->stream>>>(
-      gy, s.cout, (int)nc, u->g + u->boff[c])));
-  return FV_OK;
-}
-
-// input gradient of layer c: dX = conv(gy, flipped W) (cin channels)
-static fv_status data_grad(fv_unet* u, int c, const bf16* gy, bf16* dX) {
-  const ConvSpec& s = kConvs[c];
-  UNET_LAUNCH((k_flip<<<blocks_for(27 * s.cin * s.cout), 256, 0, u->stream>>>(u->pb + u->woff[c], u->wt,
-                                                                               s.cout, s.cin)));
-  return conv<false>(u->stream, gy, s.cout, u->wt, nullptr, dX, s.cin, u->n[s.level]);
+  return conv_any<true>(u->stream, {gy, s.cout, nullptr, 0}, s.cout, u->pb + u->woff[c], nullptr, dX, s.cin,
+                        mask, u->n[s.level]);
 }
 
 // loss of the last forward pass against u->tgt and all parameter gradients
@@ -713,22 +916,21 @@ static fv_status backward(fv_unet* u, double* loss) {
   UNET_LAUNCH((k_head_back<<<blocks_for(n0), 256, 0, st>>>(u->act[13], u->p + u->head_w, u->out, u->tgt,
                                                            n0, u->red, u->gA, u->g + u->head_w,
                                                            u->g + u->head_b)));
-  bf16* g = u->gA;   // gradient of the current layer's output
+  // g: the pre-activation gradient of the current layer's output (the ReLU
+  // masks are applied by the kernels that write it)
+  bf16* g = u->gA;
   bf16* h = u->gB;
   for (int q = 2; q >= 0; --q) {
     const int l = 2 - q, c1 = 8 + 2 * q, c2 = 9 + 2 * q;
-    const int skipc = kConvs[2 * l + 1].cout;
-    const int lowc = kConvs[c1].cin - skipc;
-    FV_TRY(relu_back(u, g, c2));
-    FV_TRY(param_grad(u, c2, g, u->act[c1]));
-    FV_TRY(data_grad(u, c2, g, h));
+    const ConvIn in = decoder_in(u, q);
+    FV_TRY(param_grad(u, c2, g, plain_in(u->act[c1], c2)));
+    FV_TRY(data_grad(u, c2, g, h, u->act[c1]));
     std::swap(g, h);
-    FV_TRY(relu_back(u, g, c1));
-    FV_TRY(param_grad(u, c1, g, u->cat[q]));
-    FV_TRY(data_grad(u, c1, g, u->gC));
+    FV_TRY(param_grad(u, c1, g, in));
+    FV_TRY(data_grad(u, c1, g, u->gC, nullptr));
     const Dims d{u->n[l][0], u->n[l][1], u->n[l][2]};
-    UNET_LAUNCH((k_up_cat_back<<<blocks_for(u->ncell[l + 1] * lowc + u->ncell[l] * skipc), 256, 0, st>>>(
-        u->gC, lowc, skipc, g, u->gS[l], d)));
+    UNET_LAUNCH((k_up_cat_back<<<blocks_for((u->ncell[l + 1] * in.lowc + u->ncell[l] * in.xc) / 8), 256, 0, st>>>(
+        u->gC, in.lowc, in.xc, in.low, g, u->gS[l], d)));
   }
   for (int l = 3; l >= 0; --l) {
     const int c1 = 2 * l, c2 = 2 * l + 1;
@@ -736,19 +938,17 @@ static fv_status backward(fv_unet* u, double* loss) {
       // act[c2] feeds the pooling (gradient g, coarse) and the skip (gS[l])
       const Dims d{u->n[l][0], u->n[l][1], u->n[l][2]};
       const int ch = kConvs[c2].cout;
-      FV_CUDA(cudaMemcpyAsync(h, u->gS[l], (size_t)u->ncell[l] * ch * sizeof(bf16), cudaMemcpyDeviceToDevice, st));
-      UNET_LAUNCH((k_pool_back<<<blocks_for(u->ncell[l] * ch), 256, 0, st>>>(g, h, ch, d)));
+      UNET_LAUNCH((k_pool_back<<<blocks_for(u->ncell[l] * ch / 8), 256, 0, st>>>(g, u->gS[l], u->act[c2], h,
+                                                                                ch, d)));
       std::swap(g, h);
     }
     const bf16* X = l == 0 ? u->in16 : u->pool[l - 1];
-    FV_TRY(relu_back(u, g, c2));
-    FV_TRY(param_grad(u, c2, g, u->act[c1]));
-    FV_TRY(data_grad(u, c2, g, h));
+    FV_TRY(param_grad(u, c2, g, plain_in(u->act[c1], c2)));
+    FV_TRY(data_grad(u, c2, g, h, u->act[c1]));
     std::swap(g, h);
-    FV_TRY(relu_back(u, g, c1));
-    FV_TRY(param_grad(u, c1, g, X));
+    FV_TRY(param_grad(u, c1, g, plain_in(X, c1)));
     if (l > 0) {
-      FV_TRY(data_grad(u, c1, g, h));
+      FV_TRY(data_grad(u, c1, g, h, nullptr));
       std::swap(g, h);
     }
   }
@@ -847,7 +1047,7 @@ void fv_unet_destroy(fv_unet* u) {
   if (!u) return;
   free_ws(u);
   free_grad(u);
-  dfree(u->p); dfree(u->g); dfree(u->m); dfree(u->v); dfree(u->pb); dfree(u->wt);
+  dfree(u->p); dfree(u->g); dfree(u->m); dfree(u->v); dfree(u->pb);
   dfree(u->red); dfree(u->scale);
   delete u;
 }
@@ -857,6 +1057,7 @@ fv_status fv_unet_create(uint64_t seed, void* cuda_stream, fv_unet** out) {
   *out = nullptr;
   fv_unet* u = new fv_unet();
   u->stream = (cudaStream_t)cuda_stream;
+  if (set_conv_attributes() != FV_OK) { delete u; return FV_ECUDA; }
   int off = 0;
   for (int c = 0; c < kNConv; ++c) {
     u->woff[c] = off;
@@ -869,8 +1070,6 @@ fv_status fv_unet_create(uint64_t seed, void* cuda_stream, fv_unet** out) {
   u->head_b = off;
   off += 1;
   u->nparam = off;
-  int wmax = 0;
-  for (const ConvSpec& s : kConvs) wmax = std::max(wmax, 27 * s.cin * s.cout);
   fv_status s = FV_OK;
   auto A = [&](void** p, size_t b) { if (s == FV_OK) s = dalloc(p, b); };
   A((void**)&u->p, off * sizeof(float));
@@ -878,7 +1077,6 @@ fv_status fv_unet_create(uint64_t seed, void* cuda_stream, fv_unet** out) {
   A((void**)&u->m, off * sizeof(float));
   A((void**)&u->v, off * sizeof(float));
   A((void**)&u->pb, off * sizeof(bf16));
-  A((void**)&u->wt, wmax * sizeof(bf16));
   A((void**)&u->red, 4 * sizeof(double));
   A((void**)&u->scale, sizeof(float));
   if (s != FV_OK) { fv_unet_destroy(u); return s; }
