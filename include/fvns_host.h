@@ -40,6 +40,11 @@ int fv_host_ff_dot(int64_t n, const double* a, const double* b, double* out);
 /* Float-float arithmetic check: out = (a + b) * c, operands as (hi, lo) pairs. */
 int fv_host_ff_arith(int64_t n, const float* a, const float* b, const float* c, float* out);
 
+/* The 1-D Neumann eigenbasis of an axis with n cells and stretching map, as
+ * the pressure solves use it: E and Einv (n x n row-major), lam (n), the index
+ * of the null eigenvalue.  Returns 0, FV_EINVAL or 4 (no convergence). */
+int fv_host_axis_basis(int n, int map, double* E, double* Einv, double* lam, int* null_index);
+
 /* The 1-D multigrid hierarchy of fv_pressure_solve_mg along one axis with n
  * cells and stretching map: the axis at coarsening level `level` (n_out
  * cells; faces[n_out + 1] its faces, every other face of the level above and

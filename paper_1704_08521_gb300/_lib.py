@@ -65,6 +65,7 @@ _SIGS = {
     "fv_pressure_solve": (_I, [_P, _P, _P, _I]),
     "fv_pressure_solve_noalloc": (_I, [_I, _I, _I, _I, _P, _P, _P]),
     "fv_pressure_solve_mg": (_I, [_P, _P, _P, _P, _P, _P]),
+    "fv_host_axis_basis": (_I, [_I, _I, _P, _P, _P, _P]),
     "fv_host_mg_axis": (_I, [_I, _I, _I, _P, _P, _P, _P]),
     "fv_host_mg_levels": (_I, [_I, _I, _I]),
     "fv_profile_enable": (_I, [_P, _I]),

@@ -95,6 +95,14 @@ struct TcMats {
   const float* az[2] = {nullptr, nullptr};
 };
 
+// Operands of the float64 transforms on the tensor cores (fv_oz.cu), per axis
+// with n <= 128: digits and row exponents of Einv (0) and E (1)
+struct OzMats {
+  const void* mat[3][2] = {};
+  const int* rexp[3][2] = {};
+  double* inv = nullptr;   // 1 / (lam_x + lam_y + lam_z) per mode, when every axis is covered
+};
+
 // device-side state of one SIMPLE loop (graph path)
 struct LoopState {
   float phi1, phi_prev, phi_last, div_last;
@@ -141,6 +149,8 @@ struct fv_grid {
   fv::TpfDev<float> tpf_f;
   void* d_tc = nullptr;      // tensor-core operands of the fused pressure solve
   fv::TcMats tc;
+  void* d_oz = nullptr;      // digits of the float64 transforms
+  fv::OzMats oz;
 
   // workspace
   double* vel_buf[3] = {nullptr, nullptr, nullptr};   // n_vel each
@@ -291,9 +301,14 @@ void destroy_graph_cache(GraphCache& c);
 // tensor-product pressure solve: phi = (D G)^+ r ; phi is float or double
 fv_status tpf_solve(const fv_grid* g, const double* r, void* phi, int prec);
 fv_status tpf_solve_f32(const fv_grid* g, const float* r, float* phi);
-// one float64 1-D transform along `axis` with the matrix M (n x n, row-major)
-fv_status transform_axis_f64(const fv_grid* g, int axis, const double* M, const double* in,
-                             double* out);
+// one float64 1-D transform along `axis`: by Einv (inverse = 0) or E (1)
+fv_status transform_axis_f64(const fv_grid* g, int axis, int inverse, const double* in, double* out);
+// the float64 transforms on the tensor cores (fv_oz.cu): operands (with the
+// grid), whether `axis` has them, one transform; scale: times 1 / (lam_x +
+// lam_y + lam_z) (z axis, every axis covered)
+fv_status build_oz(fv_grid* g);
+bool oz_ok(const fv_grid* g, int axis);
+fv_status oz_transform(const fv_grid* g, int axis, int inverse, bool scale, const double* in, double* out);
 // the unfused float32 transforms with the tables and eigenvalues of tp
 // (scaling by 1 / (lam_z + lam_y + lam_x); null_index -1: no null mode)
 fv_status tpf_run_f32(const fv_grid* g, const TpfDev<float>& tp, const float* r, float* phi);

@@ -826,7 +826,13 @@ static fv_status simple_loop(const fv_grid* g, double* cur, double* spare, doubl
     res->passes = pass;
     const double ph = h[S_PHI_MAX];
     res->div_max = h[S_DIV_MAX];
-    if (h[S_NAN] != 0.0) { set_error("SIMPLE loop: NaN/Inf in the correction"); return FV_ENAN; }
+    if (h[S_NAN] != 0.0) {
+      bool timed_out = false;
+      if (!mg) FV_TRY(take_fault(g, &timed_out));   // a transform's wait gave up
+      if (timed_out) return status_error(4);
+      set_error("SIMPLE loop: NaN/Inf in the correction");
+      return FV_ENAN;
+    }
     if (pass == 1) phi1 = ph;
     res->phi_first = phi1;
     const double prev = res->phi_last;

@@ -748,33 +748,13 @@ fv_status set_tc_attributes() {
   return FV_OK;
 }
 
-// Launch with programmatic stream serialization: the kernel's constant
-// set-up (tensor-memory allocation, eigenbasis staging) overlaps the tail of
-// the kernel before it; its pdl_wait() orders every use of that kernel's
-// output.  Captured into the evaluation graphs as a programmatic edge.
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                              cudaStream_t s, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
-}
-
 // dir 0: forward (Einv) transforms, 1: inverse (E)
 fv_status launch_slab(const fv_grid* g, const float* in, float* out, int dir) {
   // dir 0: forward x-y transforms, dir 1: inverse
   const int nx = g->n[0], ny = g->n[1], nz = g->n[2];
   const int N = g->tc.slab_n;
   LaunchScope ls_(g, dir == 0 ? FV_K_TPF_X : FV_K_TPF_XINV);
-  FV_CUDA(launch_pdl(k_slab_umma, dim3(nz, g->tc.slab_nsplit), dim3(kUmmaThreads),
+  FV_CUDA(tc5::launch_pdl(k_slab_umma, dim3(nz, g->tc.slab_nsplit), dim3(kUmmaThreads),
                      slab_smem(nx, ny, N), g->stream, in, out, (const float*)g->tc.bx[dir],
                      (const float*)g->tc.ay[dir], nx, ny, N,
                      tmem_cols(up16(ny) > N ? up16(ny) : N),
@@ -786,7 +766,7 @@ fv_status launch_col(const fv_grid* g, const float* in, float* out) {
   const int N = g->tc.col_n;
   const int64_t Q = (int64_t)g->n[0] * g->n[1];
   LaunchScope ls_(g, FV_K_TPF_YZ);
-  FV_CUDA(launch_pdl(k_col_umma, dim3((unsigned)((Q + N - 1) / N)), dim3(kUmmaThreads),
+  FV_CUDA(tc5::launch_pdl(k_col_umma, dim3((unsigned)((Q + N - 1) / N)), dim3(kUmmaThreads),
                      col_smem(g->n[2], N), g->stream, in, out, g->tpf_f,
                      (const float*)g->tc.az[0], (const float*)g->tc.az[1], N, tmem_cols(N),
                      (Q % 4 == 0 && N % 4 == 0) ? 1 : 0, g->d_fault));
@@ -905,12 +885,26 @@ fv_status build_tc_mats(fv_grid* g) {
   return FV_OK;
 }
 
-// One float64 1-D transform out = M applied along `axis` (0 x, 1 y, 2 z) of
-// the nz x ny x nx array `in` (the unfused kernels of the pressure solve)
-fv_status transform_axis_f64(const fv_grid* g, int axis, const double* M, const double* in,
-                             double* out) {
+// One float64 1-D transform along `axis` (0 x, 1 y, 2 z) of the nz x ny x nx
+// array `in`, by Einv or (inverse) E
+fv_status transform_axis_f64(const fv_grid* g, int axis, int inverse, const double* in, double* out) {
+  if (oz_ok(g, axis)) return oz_transform(g, axis, inverse, false, in, out);
+  const double* M = inverse ? g->tpf_d.E[axis] : g->tpf_d.Einv[axis];
   if (axis == 0) return run_right<double, double, double>(g, M, in, out);
   return run_left<double, double, double, false>(g, axis, M, in, out, g->tpf_d);
+}
+
+// The float64 solve: transforms on the tensor cores for the axes they cover
+static fv_status tpf_run_f64(const fv_grid* g, const double* r, double* phi) {
+  double* a = (double*)g->tpf_buf[0];
+  double* b = (double*)g->tpf_buf[1];
+  FV_TRY(transform_axis_f64(g, 0, 0, r, a));
+  FV_TRY(transform_axis_f64(g, 1, 0, a, b));
+  if (g->oz.inv) FV_TRY(oz_transform(g, 2, 0, true, b, a));
+  else FV_TRY((run_left<double, double, double, true>(g, 2, g->tpf_d.Einv[2], b, a, g->tpf_d)));
+  FV_TRY(transform_axis_f64(g, 2, 1, a, b));
+  FV_TRY(transform_axis_f64(g, 1, 1, b, a));
+  return transform_axis_f64(g, 0, 1, a, phi);
 }
 
 // The unfused float32 tensor-product solve with the tables of tp (the
@@ -921,7 +915,7 @@ fv_status tpf_run_f32(const fv_grid* g, const TpfDev<float>& tp, const float* r,
 
 fv_status tpf_solve(const fv_grid* g, const double* r, void* phi, int prec) {
   if (prec == FV_MIXED) return tpf_run<float, double, float>(g, g->tpf_f, r, (float*)phi);
-  return tpf_run<double, double, double>(g, g->tpf_d, r, (double*)phi);
+  return tpf_run_f64(g, r, (double*)phi);
 }
 
 fv_status tpf_solve_f32(const fv_grid* g, const float* r, float* phi) {

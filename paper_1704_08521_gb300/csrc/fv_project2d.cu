@@ -130,15 +130,15 @@ fv_status plane_projection(const fv_grid* g, const double* v, int plane, double*
     k_div2d<<<blocks_for(g->ncell), 256, 0, g->stream>>>(g->met_d, v, a, c, r);
   }
   FV_CHECK_LAUNCH();
-  FV_TRY(transform_axis_f64(g, a, g->tpf_d.Einv[a], r, t0));
-  FV_TRY(transform_axis_f64(g, c, g->tpf_d.Einv[c], t0, t1));
+  FV_TRY(transform_axis_f64(g, a, 0, r, t0));
+  FV_TRY(transform_axis_f64(g, c, 0, t0, t1));
   {
     LaunchScope ls_(g, FV_K_VECTOR);
     k_scale2d<<<blocks_for(g->ncell), 256, 0, g->stream>>>(g->tpf_d, a, c, t1, g->ncell);
   }
   FV_CHECK_LAUNCH();
-  FV_TRY(transform_axis_f64(g, c, g->tpf_d.E[c], t1, t0));
-  FV_TRY(transform_axis_f64(g, a, g->tpf_d.E[a], t0, r));   // r = phi
+  FV_TRY(transform_axis_f64(g, c, 1, t1, t0));
+  FV_TRY(transform_axis_f64(g, a, 1, t0, r));   // r = phi
   {
     LaunchScope ls_(g, FV_K_CORRECT);
     k_correct2d<<<blocks_for(g->ncell), 256, 0, g->stream>>>(g->met_d, v, r, a, c, vp);
