@@ -284,7 +284,7 @@ static fv_status build_graph(fv_grid* g, double sigma, GraphCache& gc, int prec 
     if ((st = launch_div_ff(g, g->vff[1], g->r32)) != FV_OK) return fail(st);
     if (cudaMemsetAsync(g->pff, 0, g->ncell * sizeof(float2), cs) != cudaSuccess)
       return fail(cuda_fail(cudaGetLastError(), "cudaMemsetAsync", __FILE__, __LINE__));
-    if ((st = tpf_solve_f32(g, g->r32, g->phi32)) != FV_OK) return fail(st);
+    if ((st = tpf_solve_f32(g, g->r32, g->phi32, prec)) != FV_OK) return fail(st);
     k_correct_g<false, true><<<cg, bx, 0, cs>>>(g->met_ff, g->w32, g->vff[0], g->vff[1], g->phi32,
                                                 g->pff, g->r32, dcb, gc.d_loop, part);
   } else {
@@ -292,7 +292,7 @@ static fv_status build_graph(fv_grid* g, double sigma, GraphCache& gc, int prec 
     k_base_from_call<false><<<grid1d(g->nvel), 256, 0, cs>>>(dcb, g->U32, g->Uff, g->nvel);
     if ((st = launch_jv_f32(g, nullptr, nullptr, g->w32, sigma, dcb)) != FV_OK) return fail(st);
     if ((st = launch_div_f32(g, g->w32, g->r32)) != FV_OK) return fail(st);
-    if ((st = tpf_solve_f32(g, g->r32, g->phi32)) != FV_OK) return fail(st);
+    if ((st = tpf_solve_f32(g, g->r32, g->phi32, prec)) != FV_OK) return fail(st);
     k_correct_g<true><<<cg, bx, 0, cs>>>(g->met_ff, g->w32, g->vff[0], g->vff[1], g->phi32, g->pff,
                                          g->r32, dcb, gc.d_loop, part);
   }
@@ -327,7 +327,7 @@ static fv_status build_graph(fv_grid* g, double sigma, GraphCache& gc, int prec 
       return fail(cuda_fail(cudaGetLastError(), "cudaStreamBeginCaptureToGraph", __FILE__, __LINE__));
     }
     g->stream = bs;
-    fv_status s2 = tpf_solve_f32(g, g->r32, g->phi32);
+    fv_status s2 = tpf_solve_f32(g, g->r32, g->phi32, prec);
     if (s2 == FV_OK) {
       if (prec == FV_FF)
         k_correct_g<false, true><<<cg, bx, 0, bs>>>(g->met_ff, g->w32, g->vff[0], g->vff[1],
@@ -743,7 +743,7 @@ static fv_status batch_build_graph(BatchImpl& b) {
     const CallBlock* dcb = b.d_call + i;
     LoopState* dls = b.d_loop + i;
     BTRY(launch_div_f32(g, g->w32, g->r32));
-    BTRY(tpf_solve_f32(g, g->r32, g->phi32));
+    BTRY(tpf_solve_f32(g, g->r32, g->phi32, FV_MIXED));
     k_correct_g<true><<<cg, bx, 0, s>>>(g->met_ff, g->w32, g->vff[0], g->vff[1], g->phi32, g->pff,
                                         g->r32, dcb, dls, part);
     BCHK(cudaGetLastError());
@@ -768,7 +768,7 @@ static fv_status batch_build_graph(BatchImpl& b) {
     BCHK(cudaStreamBeginCaptureToGraph(bs[i], body, nullptr, nullptr, 0,
                                        cudaStreamCaptureModeThreadLocal));
     g->stream = bs[i];
-    fv_status s2 = tpf_solve_f32(g, g->r32, g->phi32);
+    fv_status s2 = tpf_solve_f32(g, g->r32, g->phi32, FV_MIXED);
     if (s2 == FV_OK) {
       k_correct_g<false><<<cg, bx, 0, bs[i]>>>(g->met_ff, g->w32, g->vff[0], g->vff[1], g->phi32,
                                                g->pff, g->r32, dcb, dls, part);

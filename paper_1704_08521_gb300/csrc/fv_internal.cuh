@@ -151,6 +151,8 @@ struct fv_grid {
   fv::TcMats tc;
   void* d_oz = nullptr;      // digits of the float64 transforms
   fv::OzMats oz;
+  void* d_xf = nullptr;      // BF16 parts of the eigenbases (grids without fused kernels)
+  const unsigned char* xf[3][2] = {};   // per axis: Einv, E
 
   // workspace
   double* vel_buf[3] = {nullptr, nullptr, nullptr};   // n_vel each
@@ -300,7 +302,13 @@ void destroy_graph_cache(GraphCache& c);
 
 // tensor-product pressure solve: phi = (D G)^+ r ; phi is float or double
 fv_status tpf_solve(const fv_grid* g, const double* r, void* phi, int prec);
-fv_status tpf_solve_f32(const fv_grid* g, const float* r, float* phi);
+// float32 solve of one SIMPLE pass of the form prec (FV_MIXED or FV_FF)
+fv_status tpf_solve_f32(const fv_grid* g, const float* r, float* phi, int prec);
+// the float32 transforms of long axes on the tensor cores (fv_xf.cu): operands
+// (with the grid), whether the grid has them, the solve
+fv_status build_xf(fv_grid* g);
+bool xf_ok(const fv_grid* g);
+fv_status xf_solve(const fv_grid* g, const float* r, float* phi);
 // one float64 1-D transform along `axis`: by Einv (inverse = 0) or E (1)
 fv_status transform_axis_f64(const fv_grid* g, int axis, int inverse, const double* in, double* out);
 // the float64 transforms on the tensor cores (fv_oz.cu): operands (with the

@@ -879,7 +879,7 @@ static fv_status simple_loop_ff(const fv_grid* g, double* out, double* p_out, co
   for (int pass = 1; pass <= max_pass; ++pass) {
     const float* phi = g->phi32;
     if (pass == 1 && phi_guess) phi = phi_guess;
-    else FV_TRY(tpf_solve_f32(g, g->r32, g->phi32));
+    else FV_TRY(tpf_solve_f32(g, g->r32, g->phi32, ff_start ? FV_FF : FV_MIXED));
     FV_TRY(reset_scalars(g));
     FV_TRY(launch_correct_ff(g, pass == 1 && !ff_start, cur, g->vff[nxt], phi, g->pff, g->r32,
                              omega, ff_start));

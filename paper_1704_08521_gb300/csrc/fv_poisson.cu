@@ -918,8 +918,15 @@ fv_status tpf_solve(const fv_grid* g, const double* r, void* phi, int prec) {
   return tpf_run_f64(g, r, (double*)phi);
 }
 
-fv_status tpf_solve_f32(const fv_grid* g, const float* r, float* phi) {
+// Grids too large for the fused kernels: the float-float form takes the
+// tensor-core transforms of fv_xf.cu.  Its result does not depend on how the
+// inner solve rounds (velocity and gradient are float-float, the loop removes
+// the rest).  The mixed form's does: v = w - fl32(G phi) keeps the float32
+// rounding of the first correction (~5e-8 of v), so its solve stays the one
+// whose vectors users have stored and compare bases with.
+fv_status tpf_solve_f32(const fv_grid* g, const float* r, float* phi, int prec) {
   if (fused_ok(g)) return tpf_fused_f32(g, r, phi);
+  if (prec == FV_FF && xf_ok(g)) return xf_solve(g, r, phi);
   return tpf_run<float, float, float>(g, g->tpf_f, r, phi);
 }
 
@@ -946,7 +953,7 @@ extern "C" fv_status fv_pressure_solve(const fv_grid* g, const double* r, double
   if (prec == FV_FP64) return tpf_solve(g, r, phi, FV_FP64);
   // mixed: float32 solve, widened into phi
   FV_TRY(launch_round_f32(g, r, g->r32, g->ncell));
-  FV_TRY(tpf_solve_f32(g, g->r32, g->phi32));
+  FV_TRY(tpf_solve_f32(g, g->r32, g->phi32, FV_MIXED));
   return launch_widen_f32(g, g->phi32, phi, g->ncell);
 }
 

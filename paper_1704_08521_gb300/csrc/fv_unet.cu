@@ -163,9 +163,9 @@ __device__ __forceinline__ void stage_halo(bf16* xs, const ConvIn& in, int c0, i
 // channel chunk) whatever the tiling, because every stored BF16 value (and
 // ReLU decision) downstream flips with the last bit of a float32 sum.
 // Bound by launch latency at the coarse levels (8^3..16^3 cells) and by shared
-// memory at level 0 (3 KB of fragments per 16 KFLOP).  The version that read
-// its fragments from global memory took 111 us for 16 -> 16 at 64^3 and 183 us
-// for 64 -> 64 at 8^3 (8 blocks).
+// memory at level 0 (3 KB of fragments per 16 KFLOP).  Measured 33 us for
+// 16 -> 16 at 64^3 and 10 us for 64 -> 64 at 8^3; the version that read its
+// fragments from global memory took 111 us and 183 us (8 blocks).
 //   CIN is a template argument so that the staging's index arithmetic and the
 //   channel loop are constants.
 //   MT: 16-cell MMA rows per warp (2: 4 warps; 1: 8 warps, for the levels
@@ -280,7 +280,7 @@ inline size_t conv_smem(int cin, bool dgrad) {
 // are read through ldmatrix.trans), so a weight is added to global memory
 // once per block.  Per 16 cells a warp reads 0.5 KB of dY and 1.5 NCI KB of X
 // for 6 NCI MMAs.  The version with one warp per (tap, 16 x 16) tile gathered
-// 2-byte elements from global memory: 375 us per 16 -> 16 layer at 64^3.
+// 2-byte elements from global memory: 375 us per 16 -> 16 layer at 64^3, 28 us here.
 template <int NCI>
 __global__ void __launch_bounds__(288) k_wgrad(const bf16* __restrict__ dY, int cout, ConvIn in,
                                                int cin, float* __restrict__ dW,
