@@ -32,7 +32,7 @@ def sources():
 
 
 # float-float arithmetic must see each rounding exactly as written
-EXTRA = {"fv_mixed.cu": ["-fmad=false"]}
+EXTRA = {"fv_mixed.cu": ["-fmad=false"], "fv_pass.cu": ["-fmad=false"]}
 
 
 def _compile(src, verbose=False):

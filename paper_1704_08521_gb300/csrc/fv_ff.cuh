@@ -128,10 +128,32 @@ FF_HD float pow2f(int k) {
   return from_bits32((uint32_t)(k + 127) << 23);
 }
 
+// nearest int of |f| < 2^30 (ties to even)
+FF_HD int rint_i(float f) {
+#ifdef __CUDA_ARCH__
+  return __float2int_rn(f);
+#else
+  return (int)__builtin_rintf(f);
+#endif
+}
+
+// Values whose rests are normal floats take a short path: the lower 29 bits of
+// the significand (less 2^29 where hi was rounded up) times a power of two.
 FF_HD ff f64_split(double d) {
   const uint64_t b = bits64(d);
   const int e = (int)((b >> 52) & 0x7ff);
   ff r;
+  if ((unsigned)(e - 952) < 1149u - 952u) {
+    const uint32_t hw = (uint32_t)(b >> 32), lw = (uint32_t)b;
+    const uint32_t sign = hw & 0x80000000u;
+    const uint32_t down = sign | (((hw & 0x7fffffffu) - 0x38000000u) << 3) | (lw >> 29);
+    const uint32_t rem = lw & 0x1fffffffu;
+    const uint32_t up = (rem > 0x10000000u) | ((rem == 0x10000000u) & (down & 1u));
+    r.hi = from_bits32(down + up);
+    const float rest = (float)((int)rem - (int)(up << 29));
+    r.lo = rest * from_bits32(((uint32_t)(e - 948) << 23) | sign);   // 2^(e - 1075), signed
+    return r;
+  }
   r.hi = f64_round_f32(d);
   r.lo = 0.0f;
   const int ef = e - 1023 + 127;
@@ -152,10 +174,21 @@ FF_HD ff f64_split(double d) {
   return r;
 }
 
-// hi + lo as a float64, integer operations only.
+// hi + lo as a float64, integer operations only.  A normalised pair (lo at
+// most half an ulp of hi, hi neither tiny nor a power of two that lo takes
+// down into the next lower binade) takes a short path: lo in units of the
+// float64 ulp of hi, rounded to an integer, is added to the significand.
 FF_HD double ff_join(float hi, float lo) {
   const uint32_t hb = bits32(hi), lb = bits32(lo);
   const int eh = (int)((hb >> 23) & 0xff), el = (int)((lb >> 23) & 0xff);
+  if ((unsigned)(eh - 54) < 200u && eh - el >= 24 &&
+      ((hb & 0x7fffffu) != 0u || (int32_t)(hb ^ lb) >= 0)) {
+    const float t = lo * from_bits32(((uint32_t)(306 - eh) << 23) | (hb & 0x80000000u));   // +- 2^(179 - eh)
+    const int q = rint_i(t);                                 // |q| < 2^29
+    const uint64_t top = (uint64_t)((((hb & 0x7fffffffu) >> 3) + 0x38000000u) | (hb & 0x80000000u)) << 32 |
+                         (uint32_t)(hb << 29);
+    return from_bits64(top + (uint64_t)(int64_t)q);
+  }
   if (eh == 255) return f32_to_f64(hi);                    // inf / nan
   if (el == 0) return f32_to_f64(hi);
   if (eh == 0) return f32_to_f64(lo);

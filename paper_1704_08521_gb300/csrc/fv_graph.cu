@@ -2,16 +2,15 @@
 // loop) in the mixed precision of fv_mixed.cu, captured once per grid as a
 // CUDA graph whose pass loop is a device-side WHILE conditional node:
 //
-//   init(call) -> base(U, if given) -> J.v -> D w -> [TPF -> correct -> decide]
-//   -> while (decide says go on) { TPF -> correct -> decide } -> join
+//   init(call) -> base(U, if given) -> J.v -> D w -> [TPF -> pass] x 3
+//   -> while (the last pass says go on) { TPF -> pass } -> join
 //
 // The stop test of the loop (||phi_k|| <= eps ||phi_1||, round-off floor,
-// pass cap) is taken on the device by the one-block `decide` kernel, so a
-// whole evaluation is one graph launch with no host round trip.  Per-call
+// pass cap) is taken on the device by the last block of each pass (fv_pass.cu),
+// so a whole evaluation is one graph launch with no host round trip.  Per-call
 // arguments (pointers, eps, omega) are kernel arguments of the first node,
 // updated in the executable graph before each launch; the loop reads them
-// from a small device block.  The velocity state alternates between two
-// float-float buffers by pass parity, read from the loop state.
+// from a small device block.
 #include <algorithm>
 #include <cstddef>
 #include <cstring>
@@ -24,20 +23,6 @@
 namespace fv {
 
 namespace {
-
-// the first two members are read by the J.v kernels as their U and x
-// pointers (U null: the grid's registered base flow)
-struct CallBlock {
-  const double* U;
-  const double* x;
-  double* out;
-  double* p;
-  float sigma, eps, omega;
-  int max_pass;
-};
-
-__device__ __forceinline__ float2 to2(ff a) { return make_float2(a.hi, a.lo); }
-__device__ __forceinline__ ff of2(float2 a) { return {a.x, a.y}; }
 
 __global__ void k_call_init(CallBlock cb, CallBlock* dcb, LoopState* ls) {
   *dcb = cb;
@@ -78,164 +63,54 @@ __global__ void k_round2(const CallBlock* __restrict__ cb, float* __restrict__ U
   }
 }
 
-__device__ __forceinline__ float block_maxf(float v) {
-  __shared__ float red[32];
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nw = (blockDim.x + 31) >> 5;
-  __syncthreads();
-  if (lane == 0) red[wid] = v;
-  __syncthreads();
-  if (wid == 0) {
-    v = (lane < nw) ? red[lane] : 0.f;
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  }
-  return v;
-}
-
-// One SIMPLE pass on the float-float state (see k_correct_ff in
-// fv_mixed.cu); buffers chosen by the number of completed passes.  Block
-// maxima of |phi| and |D v| go to per-block partials (no atomics).
-template <bool FIRST, bool FFG = false>
-__global__ void __launch_bounds__(256) k_correct_g(MetFF m, const float* __restrict__ w32,
-                                                   float2* vff0, float2* vff1,
-                                                   const float* __restrict__ phi,
-                                                   float2* __restrict__ p, float* __restrict__ r,
-                                                   const CallBlock* __restrict__ cb,
-                                                   const LoopState* __restrict__ ls,
-                                                   float* __restrict__ part) {
-  tc5::pdl_trigger();   // the pressure transform that follows may start its set-up
-  const int done = FIRST ? 0 : ls->pass;
-  // result of pass `done` is in vff[(done-1)&1]; the two buffers never overlap
-  const float2* __restrict__ vin = (done & 1) ? vff0 : vff1;
-  float2* __restrict__ vout = (done & 1) ? vff1 : vff0;
-  const float omega = cb->omega;
-  const int plane_ = m.n[0] * m.n[1];
-  const int t_ = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool act_ = t_ < plane_;
-  const int i = act_ ? t_ % m.n[0] : 0;
-  const int j = act_ ? t_ / m.n[0] : 0;
-  float aphi = 0.f, adiv = 0.f;
-#pragma unroll
-  for (int kk = 0; kk < kCellKz; ++kk) {
-    const int k = blockIdx.y * kCellKz + kk;
-    if (!act_ || k >= m.n[2]) continue;
-    const int pos[3] = {i, j, k};
-    const int st[3] = {1, m.n[0], m.n[0] * m.n[1]};
-    const int nc = (int)m.ncell;
-    const int base = (k * m.n[1] + j) * m.n[0] + i;
-    auto load = [&](int e) -> ff {
-      if (FIRST) return {__ldg(w32 + e), 0.f};
-      return of2(vin[e]);
-    };
-    const float f0 = __ldg(phi + base);
-    ff dv = {0.f, 0.f};
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const int q = pos[c];
-      ff lo = {0.f, 0.f}, hi = {0.f, 0.f};
-      if (q > 0) {
-        if (FFG) {   // gradient of the float32 phi evaluated in float-float
-          const ff gr = ff_mul(two_sum(f0, -__ldg(phi + base - st[c])), of2(m.idcf[c][q]));
-          lo = ff_sub(load(c * nc + base), ff_mul_f(gr, omega));
-        } else {
-          const float g = (f0 - __ldg(phi + base - st[c])) * m.idc[c][q];
-          lo = ff_add_f(load(c * nc + base), -omega * g);
-        }
-      }
-      vout[c * nc + base] = to2(lo);
-      if (q + 1 < m.n[c]) {
-        if (FFG) {
-          const ff gr = ff_mul(two_sum(__ldg(phi + base + st[c]), -f0), of2(m.idcf[c][q + 1]));
-          hi = ff_sub(load(c * nc + base + st[c]), ff_mul_f(gr, omega));
-        } else {
-          const float g = (__ldg(phi + base + st[c]) - f0) * m.idc[c][q + 1];
-          hi = ff_add_f(load(c * nc + base + st[c]), -omega * g);
-        }
-      }
-      dv = ff_add(dv, ff_mul(ff_sub(hi, lo), of2(m.idx[c][q])));
-    }
-    r[base] = dv.hi;
-    if (FIRST) p[base] = make_float2(omega * f0, 0.f);
-    else p[base] = to2(ff_add_f(of2(p[base]), omega * f0));
-    float a1 = fabsf(f0), a2 = fabsf(dv.hi);
-    if (!(a1 <= 3e38f) || !(a2 <= 3e38f)) a1 = a2 = __int_as_float(0x7f800000);
-    aphi = fmaxf(aphi, a1);
-    adiv = fmaxf(adiv, a2);
-  }
-  aphi = block_maxf(aphi);
-  adiv = block_maxf(adiv);
-  if (threadIdx.x == 0) {
-    const int64_t b = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    const int64_t nb = (int64_t)gridDim.x * gridDim.y * gridDim.z;
-    part[b] = aphi;
-    part[nb + b] = adiv;
-  }
-}
-
-// Stop test of the SIMPLE loop (Section 3: until ||phi|| < eps, read as
-// ||phi_k||_inf <= eps ||phi_1||_inf; plus the round-off floor and the pass
-// cap).  Sets the WHILE condition of the graph.
-__global__ void __launch_bounds__(1024) k_decide(const float* __restrict__ part, int64_t nb,
-                                                 LoopState* ls, const CallBlock* __restrict__ cb,
-                                                 cudaGraphConditionalHandle h, int set_handle,
-                                                 const unsigned* __restrict__ fault) {
-  float a = 0.f, d = 0.f;
-  for (int64_t b = threadIdx.x; b < nb; b += blockDim.x) {
-    a = fmaxf(a, part[b]);
-    d = fmaxf(d, part[nb + b]);
-  }
-  a = block_maxf(a);
-  d = block_maxf(d);
-  if (threadIdx.x == 0) {
-    const int pass = ls->pass + 1;
-    ls->pass = pass;
-    if (pass == 1) ls->phi1 = a;
-    const float prev = ls->phi_last;
-    ls->phi_prev = prev;
-    ls->phi_last = a;
-    ls->div_last = d;
-    const float phi1 = ls->phi1;
-    int go = 1;
-    if (*fault) { ls->status = 4; go = 0; }   // a pressure transform's wait gave up
-    else if (isinf(a) || isinf(d) || isnan(a) || isnan(d)) { ls->nan = 1; ls->status = 3; go = 0; }
-    else if (a == 0.f || a <= cb->eps * phi1) { ls->status = 1; go = 0; }
-    else if (pass >= 3 && a > 0.25f * prev && a <= 1e-9f * phi1) { ls->status = 1; go = 0; }
-    else if (pass >= cb->max_pass) { ls->status = 2; go = 0; }
-    if (set_handle) cudaGraphSetConditional(h, go ? 1u : 0u);
-  }
-}
-
-__global__ void k_join_g(const float2* __restrict__ vff0, const float2* __restrict__ vff1,
-                         const float2* __restrict__ pff, LoopState* __restrict__ ls,
-                         const CallBlock* __restrict__ cb, int64_t nvel, int64_t ncell) {
-  const float2* v = ((ls->pass - 1) & 1) ? vff1 : vff0;
-  if (blockIdx.x == 0 && threadIdx.x == 0 && ls->status > ls->worst) ls->worst = ls->status;
-  const double* x = cb->x;
-  double* out = cb->out;
-  double* p = cb->p;
-  const float sigma = cb->sigma;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nvel;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    ff a = of2(v[e]);
-    if (sigma != 0.f) a = ff_sub(a, ff_mul_f(f64_split(__ldg(x + e)), sigma));
-    out[e] = ff_join(a.hi, a.lo);
-    if (p && e < ncell) {
-      const ff q = of2(pff[e]);
-      p[e] = ff_join(q.hi, q.lo);
-    }
-  }
-}
-
 inline unsigned grid1d(int64_t n) {
   int64_t b = (n + 255) / 256;
   if (b > 152 * 16) b = 152 * 16;
   return (unsigned)(b < 1 ? 1 : b);
 }
 
-inline int block_x(const fv_grid*) { return kCellThreads; }
-
 }  // namespace
+
+// The passes of one evaluation, captured on the stream cs: three passes in a
+// row (three is the usual number; a loop that ends earlier makes the rest
+// return at once), then a WHILE node for what may follow, then the join.  bs:
+// a stream for the body's capture.  On an error the capture on cs is left to
+// the caller.
+static fv_status capture_passes(fv_grid* g, int prec, cudaStream_t cs, cudaStream_t bs, const CallBlock* cb,
+                                LoopState* ls) {
+  cudaStreamCaptureStatus cst;
+  cudaGraph_t cap_graph;
+  const cudaGraphNode_t* deps = nullptr;
+  size_t ndeps = 0;
+  FV_CUDA(cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cap_graph, &deps, nullptr, &ndeps));
+  cudaGraphConditionalHandle h;
+  FV_CUDA(cudaGraphConditionalHandleCreate(&h, cap_graph, 0, cudaGraphCondAssignDefault));
+  g->stream = cs;
+  for (int q = 0; q < 3; ++q) {
+    FV_TRY(tpf_solve_f32(g, g->r32, g->phis[q], prec, q > 0 ? &ls->status : nullptr));
+    FV_TRY(launch_pass(g, prec, q, cb, ls, &h, true));
+  }
+  FV_CUDA(cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cap_graph, &deps, nullptr, &ndeps));
+  cudaGraphNodeParams cp = {};
+  cp.type = cudaGraphNodeTypeConditional;
+  cp.conditional.handle = h;
+  cp.conditional.type = cudaGraphCondTypeWhile;
+  cp.conditional.size = 1;
+  cudaGraphNode_t cnode;
+  FV_CUDA(cudaGraphAddNode(&cnode, cap_graph, deps, nullptr, ndeps, &cp));
+  cudaGraph_t body = cp.conditional.phGraph_out[0];
+  FV_CUDA(cudaStreamBeginCaptureToGraph(bs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+  g->stream = bs;
+  fv_status s2 = tpf_solve_f32(g, g->r32, g->phis[3], prec);
+  if (s2 == FV_OK) s2 = launch_pass(g, prec, 3, cb, ls, &h, true);
+  cudaGraph_t bg = body;
+  const cudaError_t e2 = cudaStreamEndCapture(bs, &bg);
+  g->stream = cs;
+  FV_TRY(s2);
+  FV_CUDA(e2);
+  FV_CUDA(cudaStreamUpdateCaptureDependencies(cs, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies));
+  return launch_join(g, prec, cb, ls);
+}
 
 // Build (once per grid and shift) the executable graph of a mixed-precision
 // Krylov-vector evaluation.
@@ -245,115 +120,50 @@ static fv_status build_graph(fv_grid* g, double sigma, GraphCache& gc, int prec 
   FV_CUDA(cudaMalloc(&gc.d_call, sizeof(CallBlock)));
   FV_CUDA(cudaMalloc((void**)&gc.d_loop, sizeof(LoopState)));
   FV_CUDA(cudaMemset(gc.d_loop, 0, sizeof(LoopState)));
-  cudaStream_t cs;
+  cudaStream_t cs, bs;
   FV_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
+  if (cudaStreamCreateWithFlags(&bs, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaStreamDestroy(cs);
+    return cuda_fail(cudaGetLastError(), "cudaStreamCreate", __FILE__, __LINE__);
+  }
   const cudaStream_t saved = g->stream;
   g->stream = cs;                     // the launch helpers enqueue on g->stream
   const bool prof = g->prof_on;
   g->prof_on = false;
   g->capturing = true;
-  fv_status st = FV_OK;
   cudaGraph_t graph = nullptr;
-  auto fail = [&](fv_status s) {
-    cudaStreamEndCapture(cs, &graph);
-    if (graph) cudaGraphDestroy(graph);
-    (void)cudaGetLastError();
-    g->stream = saved;
-    g->prof_on = prof;
-    g->capturing = false;
-    cudaStreamDestroy(cs);
-    return s;
-  };
-  if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
-    return fail(cuda_fail(cudaGetLastError(), "cudaStreamBeginCapture", __FILE__, __LINE__));
-  const int bx = block_x(g);
-  const dim3 cg = cell_launch_grid(g->n);
-  const int64_t nb = (int64_t)cg.x * cg.y * cg.z;
-  float* part = (float*)g->d_part;
   const CallBlock* dcb = (const CallBlock*)gc.d_call;
-  {
+  auto capture = [&]() -> fv_status {
+    FV_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     CallBlock cb0 = {};
     k_call_init<<<1, 1, 0, cs>>>(cb0, (CallBlock*)gc.d_call, gc.d_loop);
-  }
-  if (prec == FV_FF) {
-    // float-float J.v straight from the float64 operands (or the registered
-    // base flow); the predictor lands in vff[1], which the first
-    // (non-initialising) pass reads, with p starting from zero
-    k_base_from_call<true><<<grid1d(g->nvel), 256, 0, cs>>>(dcb, g->U32, g->Uff, g->nvel);
-    if ((st = launch_jv_ff(g, nullptr, nullptr, g->vff[1], sigma, dcb)) != FV_OK) return fail(st);
-    if ((st = launch_div_ff(g, g->vff[1], g->r32)) != FV_OK) return fail(st);
-    if (cudaMemsetAsync(g->pff, 0, g->ncell * sizeof(float2), cs) != cudaSuccess)
-      return fail(cuda_fail(cudaGetLastError(), "cudaMemsetAsync", __FILE__, __LINE__));
-    if ((st = tpf_solve_f32(g, g->r32, g->phi32, prec)) != FV_OK) return fail(st);
-    k_correct_g<false, true><<<cg, bx, 0, cs>>>(g->met_ff, g->w32, g->vff[0], g->vff[1], g->phi32,
-                                                g->pff, g->r32, dcb, gc.d_loop, part);
-  } else {
-    // float32 J.v straight from the float64 operands (or the registered base)
-    k_base_from_call<false><<<grid1d(g->nvel), 256, 0, cs>>>(dcb, g->U32, g->Uff, g->nvel);
-    if ((st = launch_jv_f32(g, nullptr, nullptr, g->w32, sigma, dcb)) != FV_OK) return fail(st);
-    if ((st = launch_div_f32(g, g->w32, g->r32)) != FV_OK) return fail(st);
-    if ((st = tpf_solve_f32(g, g->r32, g->phi32, prec)) != FV_OK) return fail(st);
-    k_correct_g<true><<<cg, bx, 0, cs>>>(g->met_ff, g->w32, g->vff[0], g->vff[1], g->phi32, g->pff,
-                                         g->r32, dcb, gc.d_loop, part);
-  }
-  // the conditional handle belongs to the graph being captured
-  cudaStreamCaptureStatus cst;
-  cudaGraph_t cap_graph;
-  const cudaGraphNode_t* deps = nullptr;
-  size_t ndeps = 0;
-  if (cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cap_graph, &deps, nullptr, &ndeps) != cudaSuccess)
-    return fail(cuda_fail(cudaGetLastError(), "cudaStreamGetCaptureInfo", __FILE__, __LINE__));
-  cudaGraphConditionalHandle h;
-  if (cudaGraphConditionalHandleCreate(&h, cap_graph, 1, cudaGraphCondAssignDefault) != cudaSuccess)
-    return fail(cuda_fail(cudaGetLastError(), "cudaGraphConditionalHandleCreate", __FILE__, __LINE__));
-  k_decide<<<1, 1024, 0, cs>>>(part, nb, gc.d_loop, dcb, h, 1, g->d_fault);
-  if (cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cap_graph, &deps, nullptr, &ndeps) != cudaSuccess)
-    return fail(cuda_fail(cudaGetLastError(), "cudaStreamGetCaptureInfo", __FILE__, __LINE__));
-  cudaGraphNodeParams cp = {};
-  cp.type = cudaGraphNodeTypeConditional;
-  cp.conditional.handle = h;
-  cp.conditional.type = cudaGraphCondTypeWhile;
-  cp.conditional.size = 1;
-  cudaGraphNode_t cnode;
-  if (cudaGraphAddNode(&cnode, cap_graph, deps, nullptr, ndeps, &cp) != cudaSuccess)
-    return fail(cuda_fail(cudaGetLastError(), "cudaGraphAddNode(conditional)", __FILE__, __LINE__));
-  cudaGraph_t body = cp.conditional.phGraph_out[0];
-  {
-    cudaStream_t bs;
-    if (cudaStreamCreateWithFlags(&bs, cudaStreamNonBlocking) != cudaSuccess)
-      return fail(cuda_fail(cudaGetLastError(), "cudaStreamCreate", __FILE__, __LINE__));
-    if (cudaStreamBeginCaptureToGraph(bs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-      cudaStreamDestroy(bs);
-      return fail(cuda_fail(cudaGetLastError(), "cudaStreamBeginCaptureToGraph", __FILE__, __LINE__));
+    if (prec == FV_FF) {
+      // float-float J.v straight from the float64 operands (or the registered
+      // base flow); the predictor lands in vff[1]
+      k_base_from_call<true><<<grid1d(g->nvel), 256, 0, cs>>>(dcb, g->U32, g->Uff, g->nvel);
+      FV_TRY(launch_jv_ff(g, nullptr, nullptr, g->vff[1], sigma, dcb));
+      FV_TRY(launch_div_ff(g, g->vff[1], g->r32));
+    } else {
+      // float32 J.v straight from the float64 operands (or the registered base)
+      k_base_from_call<false><<<grid1d(g->nvel), 256, 0, cs>>>(dcb, g->U32, g->Uff, g->nvel);
+      FV_TRY(launch_jv_f32(g, nullptr, nullptr, g->w32, sigma, dcb));
+      FV_TRY(launch_div_f32(g, g->w32, g->r32));
     }
-    g->stream = bs;
-    fv_status s2 = tpf_solve_f32(g, g->r32, g->phi32, prec);
-    if (s2 == FV_OK) {
-      if (prec == FV_FF)
-        k_correct_g<false, true><<<cg, bx, 0, bs>>>(g->met_ff, g->w32, g->vff[0], g->vff[1],
-                                                    g->phi32, g->pff, g->r32, dcb, gc.d_loop, part);
-      else
-        k_correct_g<false><<<cg, bx, 0, bs>>>(g->met_ff, g->w32, g->vff[0], g->vff[1], g->phi32,
-                                              g->pff, g->r32, dcb, gc.d_loop, part);
-      k_decide<<<1, 1024, 0, bs>>>(part, nb, gc.d_loop, dcb, h, 1, g->d_fault);
-    }
-    cudaGraph_t bg = body;
-    cudaError_t e2 = cudaStreamEndCapture(bs, &bg);
-    cudaStreamDestroy(bs);
-    g->stream = cs;
-    if (s2 != FV_OK) return fail(s2);
-    if (e2 != cudaSuccess) return fail(cuda_fail(e2, "cudaStreamEndCapture(body)", __FILE__, __LINE__));
-  }
-  if (cudaStreamUpdateCaptureDependencies(cs, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies) != cudaSuccess)
-    return fail(cuda_fail(cudaGetLastError(), "cudaStreamUpdateCaptureDependencies", __FILE__, __LINE__));
-  k_join_g<<<grid1d(g->nvel), 256, 0, cs>>>(g->vff[0], g->vff[1], g->pff, gc.d_loop, dcb, g->nvel,
-                                            g->ncell);
-  if (cudaStreamEndCapture(cs, &graph) != cudaSuccess)
-    return fail(cuda_fail(cudaGetLastError(), "cudaStreamEndCapture", __FILE__, __LINE__));
+    return capture_passes(g, prec, cs, bs, dcb, gc.d_loop);
+  };
+  fv_status st = capture();
+  const cudaError_t ec = cudaStreamEndCapture(cs, &graph);
   g->stream = saved;
   g->prof_on = prof;
   g->capturing = false;
   cudaStreamDestroy(cs);
+  cudaStreamDestroy(bs);
+  if (st == FV_OK && ec != cudaSuccess) st = cuda_fail(ec, "cudaStreamEndCapture", __FILE__, __LINE__);
+  if (st != FV_OK) {
+    if (graph) cudaGraphDestroy(graph);
+    (void)cudaGetLastError();
+    return st;
+  }
   // the first node (k_call_init) carries the per-call arguments
   size_t nroot = 0;
   FV_CUDA(cudaGraphGetRootNodes(graph, nullptr, &nroot));
@@ -471,9 +281,6 @@ fv_status bench_kernel(fv_grid* g, int kind, int reps, double* ms) {
     FV_CUDA(cudaMemsetAsync(gc->d_call, 0, sizeof(CallBlock), g->stream));
     FV_CUDA(cudaMemsetAsync(gc->d_loop, 0, sizeof(LoopState), g->stream));
   }
-  const int bx = block_x(g);
-  const dim3 cg = cell_launch_grid(g->n);
-  float* part = (float*)g->d_part;
   cudaEvent_t e0, e1;
   FV_CUDA(cudaEventCreate(&e0));
   FV_CUDA(cudaEventCreate(&e1));
@@ -482,12 +289,8 @@ fv_status bench_kernel(fv_grid* g, int kind, int reps, double* ms) {
       case FV_K_MOMENTUM: return launch_jv_f32(g, nullptr, g->vel_buf[1], g->w32, 0.0);
       case FV_K_DIVERGENCE: return launch_div_f32(g, g->w32, g->r32);
       case FV_K_CORRECT:
-        count_launch();
-        k_correct_g<false><<<cg, bx, 0, g->stream>>>(g->met_ff, g->w32, g->vff[0], g->vff[1],
-                                                     g->phi32, g->pff, g->r32,
-                                                     (const CallBlock*)gc->d_call, gc->d_loop, part);
-        FV_CHECK_LAUNCH();
-        return FV_OK;
+        // the second pass: the predictor and two corrections
+        return launch_pass(g, FV_MIXED, 1, (const CallBlock*)gc->d_call, gc->d_loop, nullptr, false);
       case FV_K_TPF_X: return tpf_one_transform_f32(g, 0);
       case FV_K_TPF_XINV: return tpf_one_transform_f32(g, 1);
       case FV_K_TPF_YZ: return tpf_one_transform_f32(g, 2);
@@ -736,53 +539,8 @@ static fv_status batch_build_graph(BatchImpl& b) {
     cudaStream_t s = ss[i];
     BCHK(cudaStreamWaitEvent(s, ev[b.n], 0));
     g->stream = s;
-    const int bx = kCellThreads;
-    const dim3 cg = cell_launch_grid(g->n);
-    const int64_t nb = (int64_t)cg.x * cg.y * cg.z;
-    float* part = (float*)g->d_part;
-    const CallBlock* dcb = b.d_call + i;
-    LoopState* dls = b.d_loop + i;
     BTRY(launch_div_f32(g, g->w32, g->r32));
-    BTRY(tpf_solve_f32(g, g->r32, g->phi32, FV_MIXED));
-    k_correct_g<true><<<cg, bx, 0, s>>>(g->met_ff, g->w32, g->vff[0], g->vff[1], g->phi32, g->pff,
-                                        g->r32, dcb, dls, part);
-    BCHK(cudaGetLastError());
-    cudaStreamCaptureStatus cst;
-    cudaGraph_t cap;
-    const cudaGraphNode_t* deps = nullptr;
-    size_t nd = 0;
-    BCHK(cudaStreamGetCaptureInfo(s, &cst, nullptr, &cap, &deps, nullptr, &nd));
-    cudaGraphConditionalHandle h;
-    BCHK(cudaGraphConditionalHandleCreate(&h, cap, 1, cudaGraphCondAssignDefault));
-    k_decide<<<1, 1024, 0, s>>>(part, nb, dls, dcb, h, 1, g->d_fault);
-    BCHK(cudaGetLastError());
-    BCHK(cudaStreamGetCaptureInfo(s, &cst, nullptr, &cap, &deps, nullptr, &nd));
-    cudaGraphNodeParams cp = {};
-    cp.type = cudaGraphNodeTypeConditional;
-    cp.conditional.handle = h;
-    cp.conditional.type = cudaGraphCondTypeWhile;
-    cp.conditional.size = 1;
-    cudaGraphNode_t cnode;
-    BCHK(cudaGraphAddNode(&cnode, cap, deps, nullptr, nd, &cp));
-    cudaGraph_t body = cp.conditional.phGraph_out[0];
-    BCHK(cudaStreamBeginCaptureToGraph(bs[i], body, nullptr, nullptr, 0,
-                                       cudaStreamCaptureModeThreadLocal));
-    g->stream = bs[i];
-    fv_status s2 = tpf_solve_f32(g, g->r32, g->phi32, FV_MIXED);
-    if (s2 == FV_OK) {
-      k_correct_g<false><<<cg, bx, 0, bs[i]>>>(g->met_ff, g->w32, g->vff[0], g->vff[1], g->phi32,
-                                               g->pff, g->r32, dcb, dls, part);
-      k_decide<<<1, 1024, 0, bs[i]>>>(part, nb, dls, dcb, h, 1, g->d_fault);
-    }
-    cudaGraph_t bg = body;
-    cudaError_t e2 = cudaStreamEndCapture(bs[i], &bg);
-    g->stream = s;
-    BTRY(s2);
-    BCHK(e2);
-    BCHK(cudaStreamUpdateCaptureDependencies(s, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies));
-    k_join_g<<<grid1d(g->nvel), 256, 0, s>>>(g->vff[0], g->vff[1], g->pff, dls, dcb, g->nvel,
-                                             g->ncell);
-    BCHK(cudaGetLastError());
+    BTRY(capture_passes(g, FV_MIXED, s, bs[i], b.d_call + i, b.d_loop + i));
     BCHK(cudaEventRecord(ev[i], s));
     BCHK(cudaStreamWaitEvent(cs, ev[i], 0));
   }
@@ -836,6 +594,7 @@ fv_status fv_batch_create(int n, fv_grid* const* grids, void* cuda_stream, fv_ba
   if (e == cudaSuccess) e = cudaMalloc((void**)&B.d_loop, kBatchMax * sizeof(LoopState));
   if (e == cudaSuccess) e = cudaMalloc((void**)&B.d_desc, kBatchMax * sizeof(InstDesc));
   if (e == cudaSuccess) e = cudaMalloc((void**)&B.d_counter, sizeof(unsigned));
+  if (e == cudaSuccess) e = cudaMemset(B.d_loop, 0, kBatchMax * sizeof(LoopState));
   if (e != cudaSuccess) {
     cuda_fail(e, "cudaMalloc", __FILE__, __LINE__);
     fv_batch_destroy(b);

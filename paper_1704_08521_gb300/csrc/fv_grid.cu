@@ -298,7 +298,8 @@ static fv_status build(fv_grid* g) {
   for (int i = 0; i < 2; ++i) FV_TRY(alloc(g, (void**)&g->vff[i], g->nvel * sizeof(float2)));
   FV_TRY(alloc(g, (void**)&g->pff, g->ncell * sizeof(float2)));
   FV_TRY(alloc(g, (void**)&g->r32, g->ncell * sizeof(float)));
-  FV_TRY(alloc(g, (void**)&g->phi32, g->ncell * sizeof(float)));
+  for (auto& q : g->phis) FV_TRY(alloc(g, (void**)&q, g->ncell * sizeof(float)));
+  g->phi32 = g->phis[0];
   {
     size_t tot = 0;
     for (int d = 0; d < 3; ++d) tot += g->n[d];
@@ -499,7 +500,7 @@ void fv_grid_destroy(fv_grid* g) {
   void* ptrs[] = {g->d_met_d, g->d_met_f, g->d_tpf_d, g->d_tpf_f, g->vel_buf[0], g->vel_buf[1],
                   g->vel_buf[2], g->cell_buf[0], g->cell_buf[1], g->cell_buf[2], g->tpf_buf[0],
                   g->tpf_buf[1], g->d_scal, g->d_part, g->kry, g->kry_small, g->U32, g->x32,
-                  g->w32, g->vff[0], g->vff[1], g->pff, g->r32, g->phi32, g->d_met_ff,
+                  g->w32, g->vff[0], g->vff[1], g->pff, g->r32, g->phis[0], g->phis[1], g->phis[2], g->phis[3], g->d_met_ff,
                   g->d_met_fn, g->Uff, g->xff, g->d_tc, g->d_oz, g->d_xf, g->wts, g->wts_ff, g->d_fault};
   for (void* p : ptrs)
     if (p) cudaFree(p);

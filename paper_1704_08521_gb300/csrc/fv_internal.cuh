@@ -111,6 +111,19 @@ struct LoopState {
   int worst;                    // largest status of the evaluations since graph_take_status
                                 // (kept across evaluations: lets drivers launch them
                                 // asynchronously and check once per cycle)
+  unsigned ticket;              // blocks of the running pass that are done (0 between passes)
+};
+
+// per-call arguments of an evaluation graph; the first two members are read by
+// the J.v kernels as their U and x pointers (U null: the grid's registered
+// base flow)
+struct CallBlock {
+  const double* U;
+  const double* x;
+  double* out;
+  double* p;
+  float sigma, eps, omega;
+  int max_pass;
 };
 
 // one captured, instantiated evaluation graph (per grid and shift sigma)
@@ -175,6 +188,7 @@ struct fv_grid {
   float2* pff = nullptr;         // n_cell
   float* r32 = nullptr;          // n_cell
   float* phi32 = nullptr;        // n_cell
+  float* phis[4] = {};           // corrections of the passes of an evaluation ([0] = phi32)
   void* d_met_ff = nullptr;      // float-float 1/dx per axis
   fv::MetFF met_ff;
   // float-float metrics and operands of the FV_FF J.v
@@ -299,16 +313,23 @@ fv_status mixed_krylov_graph(const fv_grid* g, const double* U, const double* x,
                              bool sync, int* passes, double* phi1, double* phil, double* divl,
                              int* status, int prec = FV_MIXED);
 void destroy_graph_cache(GraphCache& c);
+// the passes and the end of an evaluation (fv_pass.cu): pass idx = 0, 1, 2 of
+// the loop, or any later one (3), from the solution in g->phis[idx]; decide:
+// count it, take the stop decision and (h) set the WHILE condition
+fv_status launch_pass(const fv_grid* g, int prec, int idx, const CallBlock* cb, LoopState* ls,
+                      const cudaGraphConditionalHandle* h, bool decide);
+fv_status launch_join(const fv_grid* g, int prec, const CallBlock* cb, LoopState* ls);
 
 // tensor-product pressure solve: phi = (D G)^+ r ; phi is float or double
 fv_status tpf_solve(const fv_grid* g, const double* r, void* phi, int prec);
-// float32 solve of one SIMPLE pass of the form prec (FV_MIXED or FV_FF)
-fv_status tpf_solve_f32(const fv_grid* g, const float* r, float* phi, int prec);
+// float32 solve of one SIMPLE pass of the form prec (FV_MIXED or FV_FF); skip
+// (device, optional): nothing to do once it is nonzero (phi is then undefined)
+fv_status tpf_solve_f32(const fv_grid* g, const float* r, float* phi, int prec, const int* skip = nullptr);
 // the float32 transforms of long axes on the tensor cores (fv_xf.cu): operands
 // (with the grid), whether the grid has them, the solve
 fv_status build_xf(fv_grid* g);
 bool xf_ok(const fv_grid* g);
-fv_status xf_solve(const fv_grid* g, const float* r, float* phi);
+fv_status xf_solve(const fv_grid* g, const float* r, float* phi, const int* skip);
 // one float64 1-D transform along `axis`: by Einv (inverse = 0) or E (1)
 fv_status transform_axis_f64(const fv_grid* g, int axis, int inverse, const double* in, double* out);
 // the float64 transforms on the tensor cores (fv_oz.cu): operands (with the

@@ -340,30 +340,37 @@ __global__ void __launch_bounds__(kOzThreads) k_oz(OzArgs A) {
 }
 
 // digits of the n x n row-major matrix M in the order the kernel streams them
+// (out starts as zeros)
 void lay_out(const std::vector<double>& M, int n, bf16b* out, int* rexp) {
-  const int K = up16(n);
-  float w[kDig];
-  for (int i = 0; i < kDig; ++i) w[i] = std::ldexp(1.f, -8 * i);
-  std::memset(out, 0, (size_t)(K / 16) * kChunkBytes);
+  struct Table {                         // BF16 bits of (byte - 128) 2^(-8 i)
+    bf16b v[kDig][256];
+    Table() {
+      for (int i = 0; i < kDig; ++i)
+        for (int b = 0; b < 256; ++b) {
+          const float f = std::ldexp((float)(b - 128), -8 * i);
+          uint32_t u;
+          std::memcpy(&u, &f, 4);
+          v[i][b] = (bf16b)(u >> 16);
+        }
+    }
+  };
+  static const Table tab;
   for (int p = 0; p < n; ++p) {
+    const double* row = &M[(size_t)p * n];
     int b = 1;
     for (int k = 0; k < n; ++k) {
       uint64_t u;
-      std::memcpy(&u, &M[(size_t)p * n + k], 8);
+      std::memcpy(&u, row + k, 8);
       b = std::max(b, (int)((u >> 52) & 0x7ff));
     }
     rexp[p] = b;
-    for (int k = 0; k < n; ++k) {
-      uint64_t u;
-      std::memcpy(&u, &M[(size_t)p * n + k], 8);
-      const uint64_t bytes = digit_bytes(to_fixed(u, b));
-      for (int i = 0; i < kDig; ++i) {
-        const int byte = (int)((bytes >> (56 - 8 * i)) & 0xff);
-        const float f = (float)(byte - 128) * w[i];
-        uint32_t fb;
-        std::memcpy(&fb, &f, 4);
-        out[((size_t)(k >> 4) * kChunkBytes + (size_t)i * 128 * 32 + tc5::canon_offset16(p, k & 15, 16)) / 2] =
-            (bf16b)(fb >> 16);
+    for (int k0 = 0; k0 < n; k0 += 8) {  // one 16-byte run per digit
+      bf16b* dst = out + ((size_t)(k0 >> 4) * kChunkBytes + tc5::canon_offset16(p, k0 & 15, 16)) / 2;
+      for (int q = 0; q < 8 && k0 + q < n; ++q) {
+        uint64_t u;
+        std::memcpy(&u, row + k0 + q, 8);
+        const uint64_t bytes = digit_bytes(to_fixed(u, b));
+        for (int i = 0; i < kDig; ++i) dst[i * 128 * 16 + q] = tab.v[i][(bytes >> (56 - 8 * i)) & 0xff];
       }
     }
   }

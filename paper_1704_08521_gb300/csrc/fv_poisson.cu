@@ -167,7 +167,9 @@ template <typename TA, typename TB, typename TO, bool QN, bool SCALE>
 __global__ void __launch_bounds__(GT) k_gemm32(const TA* __restrict__ A, int64_t abs, int64_t lda,
                                                const TB* __restrict__ B, int64_t bbs, int64_t ldb,
                                                TO* __restrict__ C, int64_t cbs, int64_t ldc,
-                                               int P, int64_t Q, int K, TpfDev<float> tp) {
+                                               int P, int64_t Q, int K, TpfDev<float> tp,
+                                               const int* skip) {
+  if (skip && *skip != 0) return;
   __shared__ __align__(16) float As[GK][GP + 4];
   __shared__ __align__(16) float Bs[GK][GQ + 4];
   const int tid = threadIdx.x;
@@ -254,7 +256,7 @@ __global__ void __launch_bounds__(GT) k_gemm32(const TA* __restrict__ A, int64_t
 }
 
 template <typename T, typename TI, typename TO>
-fv_status run_right(const fv_grid* g, const T* M, const TI* in, TO* out) {
+fv_status run_right(const fv_grid* g, const T* M, const TI* in, TO* out, const int* skip = nullptr) {
   if constexpr (sizeof(T) == 4) {
     // out[row][a] = sum_i in[row][i] M[a][i]: p = row, q = a, k = i
     const int n = g->n[0];
@@ -263,7 +265,7 @@ fv_status run_right(const fv_grid* g, const T* M, const TI* in, TO* out) {
     {
       LaunchScope ls_(g, FV_K_TPF_X);
       k_gemm32<TI, float, TO, false, false><<<grid, GT, 0, g->stream>>>(
-          in, 0, n, M, 0, n, out, 0, n, (int)R, n, n, g->tpf_f);
+          in, 0, n, M, 0, n, out, 0, n, (int)R, n, n, g->tpf_f, skip);
     }
     FV_CHECK_LAUNCH();
     return FV_OK;
@@ -281,7 +283,7 @@ fv_status run_right(const fv_grid* g, const T* M, const TI* in, TO* out) {
 
 template <typename T, typename TI, typename TO, bool SCALE>
 fv_status run_left(const fv_grid* g, int axis, const T* M, const TI* in, TO* out,
-                   const TpfDev<T>& tp) {
+                   const TpfDev<T>& tp, const int* skip = nullptr) {
   if constexpr (sizeof(T) == 4) {
     // out[b][p][q] = sum_m M[p][m] in[b][m][q]
     const int n = g->n[axis];
@@ -293,7 +295,7 @@ fv_status run_left(const fv_grid* g, int axis, const T* M, const TI* in, TO* out
     {
       LaunchScope ls_(g, FV_K_TPF_YZ);
       k_gemm32<float, TI, TO, true, SCALE><<<grid, GT, 0, g->stream>>>(
-          M, 0, n, in, (int64_t)n * Q, Q, out, (int64_t)n * Q, Q, n, Q, n, tp);
+          M, 0, n, in, (int64_t)n * Q, Q, out, (int64_t)n * Q, Q, n, Q, n, tp, skip);
     }
     FV_CHECK_LAUNCH();
     return FV_OK;
@@ -414,7 +416,8 @@ __global__ void __launch_bounds__(kUmmaThreads) k_slab_umma(const float* __restr
                                                             const float* __restrict__ bx,
                                                             const float* __restrict__ ay, int nx, int ny,
                                                             int Na, uint32_t tcols, int vec,
-                                                            unsigned* __restrict__ fault) {
+                                                            unsigned* __restrict__ fault,
+                                                            const int* skip) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ uint64_t bar;
   __shared__ uint32_t tslot;
@@ -433,6 +436,12 @@ __global__ void __launch_bounds__(kUmmaThreads) k_slab_umma(const float* __restr
   stage_pair(bx + (size_t)blockIdx.y * 2 * 128 * K1, Ah, Al, 128 * K1, tid, kUmmaThreads);
   // everything above uses constants only; the field is the predecessor's output
   tc5::pdl_wait();
+  if (skip && *skip != 0) {      // the loop ended before this pass
+    tc5::cp_async_wait_all();
+    __syncthreads();
+    if (warp == 0) tc5::tmem_dealloc(tslot, tcols);
+    return;
+  }
   // the plane (N1 x K1: rows j, columns i) -> Bl in canonical order; a warp
   // pass covers 8 rows x 4 runs (lane: row 8 rb + lane % 8, run 4 kq + lane / 8)
   const float* ink = in + (size_t)k * nx * ny;
@@ -555,7 +564,8 @@ __global__ void __launch_bounds__(kUmmaThreads) k_col_umma(const float* __restri
                                                            const float* __restrict__ azi,
                                                            const float* __restrict__ aze, int N,
                                                            uint32_t tcols, int vec,
-                                                           unsigned* __restrict__ fault) {
+                                                           unsigned* __restrict__ fault,
+                                                           const int* skip) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ uint64_t bar;
   __shared__ uint32_t tslot;
@@ -577,6 +587,12 @@ __global__ void __launch_bounds__(kUmmaThreads) k_col_umma(const float* __restri
   stage_pair(azi, Ah, Al, 128 * Kz, tid, kUmmaThreads);
   // everything above uses constants only; the field is the predecessor's output
   tc5::pdl_wait();
+  if (skip && *skip != 0) {      // the loop ended before this pass
+    tc5::cp_async_wait_all();
+    __syncthreads();
+    if (warp == 0) tc5::tmem_dealloc(tslot, tcols);
+    return;
+  }
   // the tile in[kk][q0 .. q0 + N) -> R in 16-byte runs (rows kk >= nz and
   // columns beyond Q zero-filled)
   {
@@ -749,7 +765,7 @@ fv_status set_tc_attributes() {
 }
 
 // dir 0: forward (Einv) transforms, 1: inverse (E)
-fv_status launch_slab(const fv_grid* g, const float* in, float* out, int dir) {
+fv_status launch_slab(const fv_grid* g, const float* in, float* out, int dir, const int* skip = nullptr) {
   // dir 0: forward x-y transforms, dir 1: inverse
   const int nx = g->n[0], ny = g->n[1], nz = g->n[2];
   const int N = g->tc.slab_n;
@@ -758,28 +774,28 @@ fv_status launch_slab(const fv_grid* g, const float* in, float* out, int dir) {
                      slab_smem(nx, ny, N), g->stream, in, out, (const float*)g->tc.bx[dir],
                      (const float*)g->tc.ay[dir], nx, ny, N,
                      tmem_cols(up16(ny) > N ? up16(ny) : N),
-                     (nx % 4 == 0 && N % 4 == 0) ? 1 : 0, g->d_fault));
+                     (nx % 4 == 0 && N % 4 == 0) ? 1 : 0, g->d_fault, skip));
   return FV_OK;
 }
 
-fv_status launch_col(const fv_grid* g, const float* in, float* out) {
+fv_status launch_col(const fv_grid* g, const float* in, float* out, const int* skip = nullptr) {
   const int N = g->tc.col_n;
   const int64_t Q = (int64_t)g->n[0] * g->n[1];
   LaunchScope ls_(g, FV_K_TPF_YZ);
   FV_CUDA(tc5::launch_pdl(k_col_umma, dim3((unsigned)((Q + N - 1) / N)), dim3(kUmmaThreads),
                      col_smem(g->n[2], N), g->stream, in, out, g->tpf_f,
                      (const float*)g->tc.az[0], (const float*)g->tc.az[1], N, tmem_cols(N),
-                     (Q % 4 == 0 && N % 4 == 0) ? 1 : 0, g->d_fault));
+                     (Q % 4 == 0 && N % 4 == 0) ? 1 : 0, g->d_fault, skip));
   return FV_OK;
 }
 
-fv_status tpf_fused_f32(const fv_grid* g, const float* r, float* phi) {
+fv_status tpf_fused_f32(const fv_grid* g, const float* r, float* phi, const int* skip) {
   FV_TRY(set_tc_attributes());
   float* a = (float*)g->tpf_buf[0];
   float* b = (float*)g->tpf_buf[1];
-  FV_TRY(launch_slab(g, r, a, 0));
-  FV_TRY(launch_col(g, a, b));
-  FV_TRY(launch_slab(g, b, phi, 1));
+  FV_TRY(launch_slab(g, r, a, 0, skip));
+  FV_TRY(launch_col(g, a, b, skip));
+  FV_TRY(launch_slab(g, b, phi, 1, skip));
   return FV_OK;
 }
 
@@ -788,15 +804,15 @@ inline bool fused_ok(const fv_grid* g) {
 }
 
 template <typename T, typename TI, typename TO>
-fv_status tpf_run(const fv_grid* g, const TpfDev<T>& tp, const TI* r, TO* phi) {
+fv_status tpf_run(const fv_grid* g, const TpfDev<T>& tp, const TI* r, TO* phi, const int* skip = nullptr) {
   T* a = (T*)g->tpf_buf[0];
   T* b = (T*)g->tpf_buf[1];
-  FV_TRY((run_right<T, TI, T>(g, tp.Einv[0], r, a)));                  // x forward
-  FV_TRY((run_left<T, T, T, false>(g, 1, tp.Einv[1], a, b, tp)));      // y forward
-  FV_TRY((run_left<T, T, T, true>(g, 2, tp.Einv[2], b, a, tp)));       // z forward + scale
-  FV_TRY((run_left<T, T, T, false>(g, 2, tp.E[2], a, b, tp)));         // z inverse
-  FV_TRY((run_left<T, T, T, false>(g, 1, tp.E[1], b, a, tp)));         // y inverse
-  FV_TRY((run_right<T, T, TO>(g, tp.E[0], a, phi)));                   // x inverse
+  FV_TRY((run_right<T, TI, T>(g, tp.Einv[0], r, a, skip)));                  // x forward
+  FV_TRY((run_left<T, T, T, false>(g, 1, tp.Einv[1], a, b, tp, skip)));      // y forward
+  FV_TRY((run_left<T, T, T, true>(g, 2, tp.Einv[2], b, a, tp, skip)));       // z forward + scale
+  FV_TRY((run_left<T, T, T, false>(g, 2, tp.E[2], a, b, tp, skip)));         // z inverse
+  FV_TRY((run_left<T, T, T, false>(g, 1, tp.E[1], b, a, tp, skip)));         // y inverse
+  FV_TRY((run_right<T, T, TO>(g, tp.E[0], a, phi, skip)));                   // x inverse
   return FV_OK;
 }
 
@@ -924,10 +940,10 @@ fv_status tpf_solve(const fv_grid* g, const double* r, void* phi, int prec) {
 // the rest).  The mixed form's does: v = w - fl32(G phi) keeps the float32
 // rounding of the first correction (~5e-8 of v), so its solve stays the one
 // whose vectors users have stored and compare bases with.
-fv_status tpf_solve_f32(const fv_grid* g, const float* r, float* phi, int prec) {
-  if (fused_ok(g)) return tpf_fused_f32(g, r, phi);
-  if (prec == FV_FF && xf_ok(g)) return xf_solve(g, r, phi);
-  return tpf_run<float, float, float>(g, g->tpf_f, r, phi);
+fv_status tpf_solve_f32(const fv_grid* g, const float* r, float* phi, int prec, const int* skip) {
+  if (fused_ok(g)) return tpf_fused_f32(g, r, phi, skip);
+  if (prec == FV_FF && xf_ok(g)) return xf_solve(g, r, phi, skip);
+  return tpf_run<float, float, float>(g, g->tpf_f, r, phi, skip);
 }
 
 // one float32 transform along `axis` (0: x, 1: y, 2: z) between the two

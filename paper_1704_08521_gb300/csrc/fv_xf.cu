@@ -56,6 +56,7 @@ struct XfArgs {
   int64_t nvec, Q;            // vectors; entry k of vector v is at (v / Q) n Q + k Q + v % Q
   uint32_t tcols;
   unsigned* fault;
+  const int* skip;            // nothing to do once nonzero
 };
 
 // two floats -> BF16 pair (lo in the lower half); the floats become the rests
@@ -95,6 +96,11 @@ __global__ void __launch_bounds__(kXThreads, 2) k_xf(XfArgs A) {
   // after that, so that no block waits for columns held by a kernel that waits
   // for this one.
   tc5::pdl_wait();
+  if (A.skip && *A.skip != 0) {          // the loop ended before this pass
+    if (tid == 0)                        // no copy may outlive the block
+      for (int c = 0; c < kXStages && c < nk; ++c) tc5::mbar_wait(&full[c], 0, kXLimit);
+    return;
+  }
   if (warp == 0) tc5::tmem_alloc(&tslot, A.tcols);
   tc5::fence_before_sync();
   __syncthreads();
@@ -307,7 +313,8 @@ fv_status build_xf(fv_grid* g) {
   return FV_OK;
 }
 
-static fv_status xf_transform(const fv_grid* g, int axis, int inverse, bool scale, const float* in, float* out) {
+static fv_status xf_transform(const fv_grid* g, int axis, int inverse, bool scale, const float* in, float* out,
+                              const int* skip) {
   XfArgs A;
   A.in = in;
   A.out = out;
@@ -325,6 +332,7 @@ static fv_status xf_transform(const fv_grid* g, int axis, int inverse, bool scal
   A.tcols = 32;
   while ((int)A.tcols < chunk_rows(A.n)) A.tcols <<= 1;
   A.fault = g->d_fault;
+  A.skip = skip;
   const dim3 grid((unsigned)((A.nvec + 127) / 128), (unsigned)chunks_of(A.n));
   const size_t smem = xf_smem(A.n);
   LaunchScope ls_(g, axis == 0 ? FV_K_TPF_X : FV_K_TPF_YZ);
@@ -336,15 +344,15 @@ static fv_status xf_transform(const fv_grid* g, int axis, int inverse, bool scal
 
 bool xf_ok(const fv_grid* g) { return g->d_xf != nullptr; }
 
-fv_status xf_solve(const fv_grid* g, const float* r, float* phi) {
+fv_status xf_solve(const fv_grid* g, const float* r, float* phi, const int* skip) {
   float* a = (float*)g->tpf_buf[0];
   float* b = (float*)g->tpf_buf[1];
-  FV_TRY(xf_transform(g, 0, 0, false, r, a));
-  FV_TRY(xf_transform(g, 1, 0, false, a, b));
-  FV_TRY(xf_transform(g, 2, 0, true, b, a));
-  FV_TRY(xf_transform(g, 2, 1, false, a, b));
-  FV_TRY(xf_transform(g, 1, 1, false, b, a));
-  return xf_transform(g, 0, 1, false, a, phi);
+  FV_TRY(xf_transform(g, 0, 0, false, r, a, skip));
+  FV_TRY(xf_transform(g, 1, 0, false, a, b, skip));
+  FV_TRY(xf_transform(g, 2, 0, true, b, a, skip));
+  FV_TRY(xf_transform(g, 2, 1, false, a, b, skip));
+  FV_TRY(xf_transform(g, 1, 1, false, b, a, skip));
+  return xf_transform(g, 0, 1, false, a, phi, skip);
 }
 
 }  // namespace fv
