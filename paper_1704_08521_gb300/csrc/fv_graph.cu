@@ -2,15 +2,15 @@
 // loop) in the mixed precision of fv_mixed.cu, captured once per grid as a
 // CUDA graph whose pass loop is a device-side WHILE conditional node:
 //
-//   init(call) -> base(U, if given) -> J.v -> D w -> [TPF -> pass] x 3
+//   [base(U, if given)] -> J.v -> D w -> [TPF -> pass] x 3
 //   -> while (the last pass says go on) { TPF -> pass } -> join
 //
 // The stop test of the loop (||phi_k|| <= eps ||phi_1||, round-off floor,
 // pass cap) is taken on the device by the last block of each pass (fv_pass.cu),
 // so a whole evaluation is one graph launch with no host round trip.  Per-call
-// arguments (pointers, eps, omega) are kernel arguments of the first node,
-// updated in the executable graph before each launch; the loop reads them
-// from a small device block.
+// arguments (pointers, eps, omega) are arguments of the J.v node (and, for U,
+// of the base node), updated in the executable graph before each launch; J.v
+// hands them on to the other kernels through a small device block.
 #include <algorithm>
 #include <cstddef>
 #include <cstring>
@@ -24,22 +24,11 @@ namespace fv {
 
 namespace {
 
-__global__ void k_call_init(CallBlock cb, CallBlock* dcb, LoopState* ls) {
-  *dcb = cb;
-  ls->phi1 = ls->phi_prev = ls->phi_last = ls->div_last = 0.f;
-  ls->pass = 0;
-  ls->nan = 0;
-  ls->status = 0;
-}
-
-// The evaluation's base flow when the call passes one (U non-null): rounded
-// (FV_MIXED) or split (FV_FF) into the grid's stored copy that the J.v kernel
-// reads; with U null the registered base flow is already there.
+// The evaluation's base flow when the call passes one: rounded (FV_MIXED) or
+// split (FV_FF) into the grid's stored copy that the J.v kernel reads.
 template <bool FF>
-__global__ void k_base_from_call(const CallBlock* __restrict__ cb, float* __restrict__ U32,
+__global__ void k_base_from_call(const double* __restrict__ U, float* __restrict__ U32,
                                  float2* __restrict__ Uff, int64_t n) {
-  const double* U = cb->U;
-  if (!U) return;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
        e += (int64_t)gridDim.x * blockDim.x) {
     const double d = __ldg(U + e);
@@ -112,69 +101,114 @@ static fv_status capture_passes(fv_grid* g, int prec, cudaStream_t cs, cudaStrea
   return launch_join(g, prec, cb, ls);
 }
 
-// Build (once per grid and shift) the executable graph of a mixed-precision
-// Krylov-vector evaluation.
-static_assert(offsetof(CallBlock, U) == 0 && offsetof(CallBlock, x) == sizeof(void*),
-              "the J.v kernels read U and x from the head of the call block");
-static fv_status build_graph(fv_grid* g, double sigma, GraphCache& gc, int prec = FV_MIXED) {
-  FV_CUDA(cudaMalloc(&gc.d_call, sizeof(CallBlock)));
-  FV_CUDA(cudaMalloc((void**)&gc.d_loop, sizeof(LoopState)));
-  FV_CUDA(cudaMemset(gc.d_loop, 0, sizeof(LoopState)));
-  cudaStream_t cs, bs;
-  FV_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-  if (cudaStreamCreateWithFlags(&bs, cudaStreamNonBlocking) != cudaSuccess) {
-    cudaStreamDestroy(cs);
-    return cuda_fail(cudaGetLastError(), "cudaStreamCreate", __FILE__, __LINE__);
+// The two streams that graphs are captured on, kept by each host thread for
+// the device it last captured on (creating and destroying them costs more than
+// the capture) and given back with the thread.
+namespace {
+struct CaptureStreams {
+  int dev = -1;
+  cudaStream_t s[2] = {nullptr, nullptr};
+  void drop() {
+    for (auto& q : s) {
+      if (q) cudaStreamDestroy(q);
+      q = nullptr;
+    }
+    dev = -1;
   }
+  ~CaptureStreams() { drop(); }
+};
+thread_local CaptureStreams t_capture;
+
+fv_status capture_streams(cudaStream_t* cs, cudaStream_t* bs) {
+  int dev = 0;
+  FV_CUDA(cudaGetDevice(&dev));
+  if (t_capture.dev != dev) {
+    t_capture.drop();
+    for (auto& q : t_capture.s) FV_CUDA(cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking));
+    t_capture.dev = dev;
+  }
+  *cs = t_capture.s[0];
+  *bs = t_capture.s[1];
+  return FV_OK;
+}
+
+// the node captured last on s
+fv_status last_node(cudaStream_t s, cudaGraphNode_t* node) {
+  cudaStreamCaptureStatus cst;
+  cudaGraph_t graph;
+  const cudaGraphNode_t* deps = nullptr;
+  size_t nd = 0;
+  FV_CUDA(cudaStreamGetCaptureInfo(s, &cst, nullptr, &graph, &deps, nullptr, &nd));
+  if (nd != 1) { set_error("graph: unexpected capture state"); return FV_ECUDA; }
+  *node = deps[0];
+  return FV_OK;
+}
+}  // namespace
+
+// Build (once per grid, shift, form and kind of base flow) the executable
+// graph of a Krylov-vector evaluation.
+static fv_status build_graph(fv_grid* g, double sigma, GraphCache& gc, int prec, bool has_u) {
+  const size_t slot = &gc - g->graphs;
+  gc.d_call = (CallBlock*)(g->d_eval + slot * 256);
+  gc.d_loop = (LoopState*)(g->d_eval + slot * 256 + 128);
+  static_assert(sizeof(CallBlock) <= 128 && sizeof(LoopState) <= 128, "evaluation slots");
+  cudaStream_t cs, bs;
+  FV_TRY(capture_streams(&cs, &bs));
   const cudaStream_t saved = g->stream;
+  FV_CUDA(cudaMemsetAsync(gc.d_call, 0, 256, saved));
   g->stream = cs;                     // the launch helpers enqueue on g->stream
   const bool prof = g->prof_on;
   g->prof_on = false;
   g->capturing = true;
   cudaGraph_t graph = nullptr;
-  const CallBlock* dcb = (const CallBlock*)gc.d_call;
+  bool begun = false;
   auto capture = [&]() -> fv_status {
     FV_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    CallBlock cb0 = {};
-    k_call_init<<<1, 1, 0, cs>>>(cb0, (CallBlock*)gc.d_call, gc.d_loop);
-    if (prec == FV_FF) {
-      // float-float J.v straight from the float64 operands (or the registered
-      // base flow); the predictor lands in vff[1]
-      k_base_from_call<true><<<grid1d(g->nvel), 256, 0, cs>>>(dcb, g->U32, g->Uff, g->nvel);
-      FV_TRY(launch_jv_ff(g, nullptr, nullptr, g->vff[1], sigma, dcb));
-      FV_TRY(launch_div_ff(g, g->vff[1], g->r32));
-    } else {
-      // float32 J.v straight from the float64 operands (or the registered base)
-      k_base_from_call<false><<<grid1d(g->nvel), 256, 0, cs>>>(dcb, g->U32, g->Uff, g->nvel);
-      FV_TRY(launch_jv_f32(g, nullptr, nullptr, g->w32, sigma, dcb));
-      FV_TRY(launch_div_f32(g, g->w32, g->r32));
+    begun = true;
+    const bool ff = prec == FV_FF;
+    if (has_u) {
+      if (ff) k_base_from_call<true><<<grid1d(g->nvel), 256, 0, cs>>>(nullptr, g->U32, g->Uff, g->nvel);
+      else k_base_from_call<false><<<grid1d(g->nvel), 256, 0, cs>>>(nullptr, g->U32, g->Uff, g->nvel);
+      FV_CHECK_LAUNCH();
+      FV_TRY(last_node(cs, &gc.base_node));
     }
-    return capture_passes(g, prec, cs, bs, dcb, gc.d_loop);
+    // J.v straight from the float64 vector; the float-float predictor lands in
+    // vff[1], the float32 one in w32
+    if (ff) FV_TRY(launch_jv_ff(g, nullptr, nullptr, g->vff[1], sigma, gc.d_call, gc.d_loop));
+    else FV_TRY(launch_jv_f32(g, nullptr, nullptr, g->w32, sigma, gc.d_call, gc.d_loop));
+    FV_TRY(last_node(cs, &gc.jv_node));
+    if (ff) FV_TRY(launch_div_ff(g, g->vff[1], g->r32));
+    else FV_TRY(launch_div_f32(g, g->w32, g->r32));
+    return capture_passes(g, prec, cs, bs, gc.d_call, gc.d_loop);
   };
   fv_status st = capture();
-  const cudaError_t ec = cudaStreamEndCapture(cs, &graph);
+  const cudaError_t ec = begun ? cudaStreamEndCapture(cs, &graph) : cudaSuccess;
   g->stream = saved;
   g->prof_on = prof;
   g->capturing = false;
-  cudaStreamDestroy(cs);
-  cudaStreamDestroy(bs);
   if (st == FV_OK && ec != cudaSuccess) st = cuda_fail(ec, "cudaStreamEndCapture", __FILE__, __LINE__);
+  auto finish = [&]() -> fv_status {
+    // the arguments that change from call to call: U of the base node, x and
+    // the call block of the J.v node
+    FV_CUDA(cudaGraphKernelNodeGetParams(gc.jv_node, &gc.jv_kp));
+    gc.patch = prec == FV_FF ? jv_patch_ff() : jv_patch_f32();
+    const unsigned char* a = (const unsigned char*)gc.jv_kp.kernelParams[0];
+    gc.jv_args.assign(a, a + gc.patch.size);
+    if (has_u) FV_CUDA(cudaGraphKernelNodeGetParams(gc.base_node, &gc.base_kp));
+    FV_CUDA(cudaGraphInstantiate(&gc.exec, graph, 0));
+    return FV_OK;
+  };
+  if (st == FV_OK) st = finish();
   if (st != FV_OK) {
     if (graph) cudaGraphDestroy(graph);
+    t_capture.drop();                 // a stream may still be capturing
     (void)cudaGetLastError();
     return st;
   }
-  // the first node (k_call_init) carries the per-call arguments
-  size_t nroot = 0;
-  FV_CUDA(cudaGraphGetRootNodes(graph, nullptr, &nroot));
-  std::vector<cudaGraphNode_t> roots(nroot);
-  FV_CUDA(cudaGraphGetRootNodes(graph, roots.data(), &nroot));
-  if (nroot != 1) { cudaGraphDestroy(graph); set_error("graph: unexpected root count"); return FV_ECUDA; }
-  gc.init_node = roots[0];
-  FV_CUDA(cudaGraphInstantiate(&gc.exec, graph, 0));
   gc.graph = graph;
   gc.sigma = sigma;
   gc.prec = prec;
+  gc.has_u = has_u;
   gc.ready = true;
   return FV_OK;
 }
@@ -186,18 +220,18 @@ fv_status mixed_krylov_graph(const fv_grid* gcst, const double* U, const double*
   fv_grid* g = const_cast<fv_grid*>(gcst);
   GraphCache* gc = nullptr;
   for (auto& c : g->graphs)
-    if (c.ready && c.sigma == sigma && c.prec == prec) gc = &c;
+    if (c.ready && c.sigma == sigma && c.prec == prec && c.has_u == (U != nullptr)) gc = &c;
   if (!gc) {
     GraphCache* slot = nullptr;
     for (auto& c : g->graphs)
       if (!c.ready) { slot = &c; break; }
     if (!slot) slot = &g->graphs[0];
     destroy_graph_cache(*slot);
-    FV_TRY(build_graph(g, sigma, *slot, prec));
+    FV_TRY(build_graph(g, sigma, *slot, prec, U != nullptr));
     gc = slot;
   }
   CallBlock cb;
-  cb.U = U;
+  cb.U = nullptr;
   cb.x = x;
   if (U) g->base_ptr = nullptr;   // the graph overwrites the stored base copy
   cb.out = out;
@@ -206,16 +240,21 @@ fv_status mixed_krylov_graph(const fv_grid* gcst, const double* U, const double*
   cb.eps = (float)eps;
   cb.omega = (float)omega;
   cb.max_pass = max_pass;
-  void* dcb = gc->d_call;
   LoopState* dls = gc->d_loop;
-  void* args[3] = {&cb, &dcb, &dls};
-  cudaKernelNodeParams kp = {};
-  kp.func = (void*)k_call_init;
-  kp.gridDim = dim3(1);
-  kp.blockDim = dim3(1);
-  kp.sharedMemBytes = 0;
-  kp.kernelParams = args;
-  FV_CUDA(cudaGraphExecKernelNodeSetParams(gc->exec, gc->init_node, &kp));
+  if (U) {
+    void* args[4] = {&U, &g->U32, &g->Uff, &g->nvel};
+    cudaKernelNodeParams kp = gc->base_kp;
+    kp.kernelParams = args;
+    FV_CUDA(cudaGraphExecKernelNodeSetParams(gc->exec, gc->base_node, &kp));
+  }
+  {
+    std::memcpy(gc->jv_args.data() + gc->patch.x, &x, sizeof x);
+    std::memcpy(gc->jv_args.data() + gc->patch.cb, &cb, sizeof cb);
+    void* args[1] = {gc->jv_args.data()};
+    cudaKernelNodeParams kp = gc->jv_kp;
+    kp.kernelParams = args;
+    FV_CUDA(cudaGraphExecKernelNodeSetParams(gc->exec, gc->jv_node, &kp));
+  }
   count_launch();                     // one graph launch
   FV_CUDA(cudaGraphLaunch(gc->exec, g->stream));
   if (!sync) return FV_OK;
@@ -277,7 +316,7 @@ fv_status bench_kernel(fv_grid* g, int kind, int reps, double* ms) {
   if (!gc) {
     // host-driven grids have no graph yet: capture one for its device blocks
     gc = &g->graphs[0];
-    FV_TRY(build_graph(g, 0.0, *gc));
+    FV_TRY(build_graph(g, 0.0, *gc, FV_MIXED, false));
     FV_CUDA(cudaMemsetAsync(gc->d_call, 0, sizeof(CallBlock), g->stream));
     FV_CUDA(cudaMemsetAsync(gc->d_loop, 0, sizeof(LoopState), g->stream));
   }
@@ -313,8 +352,6 @@ fv_status bench_kernel(fv_grid* g, int kind, int reps, double* ms) {
 void destroy_graph_cache(GraphCache& c) {
   if (c.exec) cudaGraphExecDestroy(c.exec);
   if (c.graph) cudaGraphDestroy(c.graph);
-  if (c.d_call) cudaFree(c.d_call);
-  if (c.d_loop) cudaFree(c.d_loop);
   c = GraphCache();
 }
 
@@ -474,80 +511,57 @@ static void batch_release_graph(BatchImpl& b) {
 static fv_status batch_build_graph(BatchImpl& b) {
   batch_release_graph(b);
   FV_TRY(batch_descriptors(b));
-  cudaStream_t cs;
-  FV_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-  std::vector<cudaStream_t> ss(b.n), bs(b.n);
-  std::vector<cudaEvent_t> ev(b.n + 1);
-  for (int i = 0; i < b.n; ++i) {
-    FV_CUDA(cudaStreamCreateWithFlags(&ss[i], cudaStreamNonBlocking));
-    FV_CUDA(cudaStreamCreateWithFlags(&bs[i], cudaStreamNonBlocking));
-  }
-  for (auto& e : ev) FV_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  cudaStream_t cs, bs;
+  FV_TRY(capture_streams(&cs, &bs));
   std::vector<cudaStream_t> saved(b.n);
   for (int i = 0; i < b.n; ++i) {
     saved[i] = b.grids[i]->stream;
     b.grids[i]->capturing = true;
   }
-  fv_status st = FV_OK;
   cudaGraph_t graph = nullptr;
-  auto cleanup = [&]() {
+  bool begun = false;
+  auto capture = [&]() -> fv_status {
+    FV_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+    begun = true;
+    BatchCall bc = {};
+    k_batch_init<<<1, kBatchMax, 0, cs>>>(bc, b.d_call, b.d_loop);
+    FV_CHECK_LAUNCH();
     for (int i = 0; i < b.n; ++i) {
-      b.grids[i]->stream = saved[i];
-      b.grids[i]->capturing = false;
-      cudaStreamDestroy(ss[i]);
-      cudaStreamDestroy(bs[i]);
+      fv_grid* g = b.grids[i];
+      k_round2<<<grid1d(g->nvel), 256, 0, cs>>>(b.d_call + i, g->U32, g->x32, g->nvel);
+      FV_CHECK_LAUNCH();
     }
-    for (auto& e : ev) cudaEventDestroy(e);
-    cudaStreamDestroy(cs);
+    FV_TRY(launch_batch_jv(b, cs));
+    // one stream captures every branch: each starts from the J.v node, and the
+    // capture ends where they all have
+    cudaGraphNode_t jv;
+    FV_TRY(last_node(cs, &jv));
+    std::vector<cudaGraphNode_t> ends(b.n);
+    for (int i = 0; i < b.n; ++i) {
+      fv_grid* g = b.grids[i];
+      g->stream = cs;
+      FV_CUDA(cudaStreamUpdateCaptureDependencies(cs, &jv, nullptr, 1, cudaStreamSetCaptureDependencies));
+      FV_TRY(launch_div_f32(g, g->w32, g->r32));
+      FV_TRY(capture_passes(g, FV_MIXED, cs, bs, b.d_call + i, b.d_loop + i));
+      FV_TRY(last_node(cs, &ends[i]));
+    }
+    FV_CUDA(cudaStreamUpdateCaptureDependencies(cs, ends.data(), nullptr, ends.size(),
+                                                cudaStreamSetCaptureDependencies));
+    return FV_OK;
   };
-#define BCHK(call)                                      \
-  do {                                                  \
-    cudaError_t e_ = (call);                            \
-    if (e_ != cudaSuccess) {                            \
-      st = cuda_fail(e_, #call, __FILE__, __LINE__);    \
-      cudaStreamEndCapture(cs, &graph);                 \
-      if (graph) cudaGraphDestroy(graph);               \
-      (void)cudaGetLastError();                         \
-      cleanup();                                        \
-      return st;                                        \
-    }                                                   \
-  } while (0)
-#define BTRY(call)                                      \
-  do {                                                  \
-    fv_status s_ = (call);                              \
-    if (s_ != FV_OK) {                                  \
-      cudaStreamEndCapture(cs, &graph);                 \
-      if (graph) cudaGraphDestroy(graph);               \
-      (void)cudaGetLastError();                         \
-      cleanup();                                        \
-      return s_;                                        \
-    }                                                   \
-  } while (0)
-  BCHK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-  BatchCall bc = {};
-  k_batch_init<<<1, kBatchMax, 0, cs>>>(bc, b.d_call, b.d_loop);
-  BCHK(cudaGetLastError());
+  fv_status st = capture();
+  const cudaError_t ec = begun ? cudaStreamEndCapture(cs, &graph) : cudaSuccess;
   for (int i = 0; i < b.n; ++i) {
-    fv_grid* g = b.grids[i];
-    k_round2<<<grid1d(g->nvel), 256, 0, cs>>>(b.d_call + i, g->U32, g->x32, g->nvel);
-    BCHK(cudaGetLastError());
+    b.grids[i]->stream = saved[i];
+    b.grids[i]->capturing = false;
   }
-  BTRY(launch_batch_jv(b, cs));
-  BCHK(cudaEventRecord(ev[b.n], cs));
-  for (int i = 0; i < b.n; ++i) {
-    fv_grid* g = b.grids[i];
-    cudaStream_t s = ss[i];
-    BCHK(cudaStreamWaitEvent(s, ev[b.n], 0));
-    g->stream = s;
-    BTRY(launch_div_f32(g, g->w32, g->r32));
-    BTRY(capture_passes(g, FV_MIXED, s, bs[i], b.d_call + i, b.d_loop + i));
-    BCHK(cudaEventRecord(ev[i], s));
-    BCHK(cudaStreamWaitEvent(cs, ev[i], 0));
+  if (st == FV_OK && ec != cudaSuccess) st = cuda_fail(ec, "cudaStreamEndCapture", __FILE__, __LINE__);
+  if (st != FV_OK) {
+    if (graph) cudaGraphDestroy(graph);
+    t_capture.drop();                 // a stream may still be capturing
+    (void)cudaGetLastError();
+    return st;
   }
-  BCHK(cudaStreamEndCapture(cs, &graph));
-#undef BCHK
-#undef BTRY
-  cleanup();
   size_t nroot = 0;
   FV_CUDA(cudaGraphGetRootNodes(graph, nullptr, &nroot));
   std::vector<cudaGraphNode_t> roots(nroot);

@@ -252,15 +252,61 @@ static fv_status upload_tpf(fv_grid* g, void** dst, TpfDev<T>& t) {
   return FV_OK;
 }
 
-static fv_status alloc(fv_grid* g, void** p, size_t bytes) {
-  cudaError_t e = cudaMalloc(p, bytes);
+// All workspace of a grid in one allocation (two dozen separate ones cost
+// more than the rest of a small grid's creation): requests first, then the
+// memory, every array on a 256-byte boundary.
+struct Arena {
+  struct Req {
+    void** p;
+    size_t off;
+  };
+  std::vector<Req> req;
+  size_t total = 0;
+  template <typename T>
+  void want(T*& p, size_t bytes) {
+    req.push_back({(void**)&p, total});
+    total += (bytes + 255) / 256 * 256;
+  }
+};
+
+static fv_status alloc_workspace(fv_grid* g) {
+  Arena A;
+  const size_t nv = g->nvel, nc = g->ncell;
+  for (auto& p : g->vel_buf) A.want(p, nv * sizeof(double));
+  for (auto& p : g->cell_buf) A.want(p, nc * sizeof(double));
+  for (auto& p : g->tpf_buf) A.want(p, nc * sizeof(double));
+  // mixed-precision workspace
+  A.want(g->U32, nv * sizeof(float));
+  A.want(g->x32, nv * sizeof(float));
+  A.want(g->w32, nv * sizeof(float));
+  for (auto& p : g->vff) A.want(p, nv * sizeof(float2));
+  A.want(g->pff, nc * sizeof(float2));
+  A.want(g->r32, nc * sizeof(float));
+  for (auto& p : g->phis) A.want(p, nc * sizeof(float));
+  A.want(g->Uff, nv * sizeof(float2));
+  A.want(g->xff, nv * sizeof(float2));
+  size_t cells = 0;
+  for (int d = 0; d < 3; ++d) cells += g->n[d] + 1;
+  A.want(g->d_met_ff, cells * sizeof(float2));
+  A.want(g->d_met_fn, 5 * cells * sizeof(float2));
+  A.want(g->d_scal, kScalars * sizeof(double));
+  A.want(g->d_fault, 256);
+  A.want(g->d_eval, kGraphSlots * 256);
+  g->part_len = 4096 * 130;
+  A.want(g->d_part, g->part_len * sizeof(double));
+  A.want(g->wts, nv * sizeof(double));
+  A.want(g->wts_ff, nv * sizeof(float2));
+  const cudaError_t e = cudaMalloc(&g->d_work, A.total);
   if (e != cudaSuccess) {
-    set_error(std::string("cudaMalloc of ") + std::to_string(bytes) + " bytes failed: " +
+    set_error(std::string("cudaMalloc of ") + std::to_string(A.total) + " bytes failed: " +
               cudaGetErrorString(e));
     (void)cudaGetLastError();
+    g->d_work = nullptr;
     return FV_ENOMEM;
   }
-  g->ws_bytes += (int64_t)bytes;
+  for (auto& r : A.req) *r.p = (char*)g->d_work + r.off;
+  g->ws_bytes += (int64_t)A.total;
+  g->phi32 = g->phis[0];
   return FV_OK;
 }
 
@@ -288,18 +334,7 @@ static fv_status build(fv_grid* g) {
   FV_TRY(build_tc_mats(g));
   FV_TRY(build_oz(g));
   FV_TRY(build_xf(g));
-  for (int i = 0; i < 3; ++i) FV_TRY(alloc(g, (void**)&g->vel_buf[i], g->nvel * sizeof(double)));
-  for (int i = 0; i < 3; ++i) FV_TRY(alloc(g, (void**)&g->cell_buf[i], g->ncell * sizeof(double)));
-  for (int i = 0; i < 2; ++i) FV_TRY(alloc(g, &g->tpf_buf[i], g->ncell * sizeof(double)));
-  // mixed-precision workspace
-  FV_TRY(alloc(g, (void**)&g->U32, g->nvel * sizeof(float)));
-  FV_TRY(alloc(g, (void**)&g->x32, g->nvel * sizeof(float)));
-  FV_TRY(alloc(g, (void**)&g->w32, g->nvel * sizeof(float)));
-  for (int i = 0; i < 2; ++i) FV_TRY(alloc(g, (void**)&g->vff[i], g->nvel * sizeof(float2)));
-  FV_TRY(alloc(g, (void**)&g->pff, g->ncell * sizeof(float2)));
-  FV_TRY(alloc(g, (void**)&g->r32, g->ncell * sizeof(float)));
-  for (auto& q : g->phis) FV_TRY(alloc(g, (void**)&q, g->ncell * sizeof(float)));
-  g->phi32 = g->phis[0];
+  FV_TRY(alloc_workspace(g));
   {
     size_t tot = 0;
     for (int d = 0; d < 3; ++d) tot += g->n[d];
@@ -313,7 +348,6 @@ static fv_status build(fv_grid* g) {
       }
       o += g->n[d];
     }
-    FV_TRY(alloc(g, &g->d_met_ff, tot * sizeof(float2)));
     FV_CUDA(cudaMemcpy(g->d_met_ff, h.data(), tot * sizeof(float2), cudaMemcpyHostToDevice));
     for (int d = 0; d < 3; ++d) {
       g->met_ff.n[d] = g->n[d];
@@ -341,7 +375,6 @@ static fv_status build(fv_grid* g) {
       for (int f = 0; f <= n; ++f) q[4 * (n + 1) + f] = put(g->h_dc[d][f]);
       o += 5 * (size_t)(n + 1);
     }
-    FV_TRY(alloc(g, &g->d_met_fn, total * sizeof(float2)));
     FV_CUDA(cudaMemcpy(g->d_met_fn, h.data(), total * sizeof(float2), cudaMemcpyHostToDevice));
     const ffn* base = (const ffn*)g->d_met_fn;
     for (int d = 0; d < 3; ++d) {
@@ -356,15 +389,7 @@ static fv_status build(fv_grid* g) {
     g->met_fn.ncell = g->ncell;
     for (int d = 0; d < 3; ++d) g->met_ff.idcf[d] = (const float2*)g->met_fn.idc[d];
   }
-  FV_TRY(alloc(g, (void**)&g->Uff, g->nvel * sizeof(float2)));
-  FV_TRY(alloc(g, (void**)&g->xff, g->nvel * sizeof(float2)));
-  FV_TRY(alloc(g, (void**)&g->d_scal, kScalars * sizeof(double)));
-  FV_TRY(alloc(g, (void**)&g->d_fault, 256));
   FV_CUDA(cudaMemset(g->d_fault, 0, 256));
-  g->part_len = 4096 * 130;
-  FV_TRY(alloc(g, (void**)&g->d_part, g->part_len * sizeof(double)));
-  FV_TRY(alloc(g, (void**)&g->wts, g->nvel * sizeof(double)));
-  FV_TRY(alloc(g, (void**)&g->wts_ff, g->nvel * sizeof(float2)));
   FV_TRY(fill_face_weights(g));
   FV_CUDA(cudaMallocHost((void**)&g->h_scal, kScalars * sizeof(double)));
   FV_CUDA(cudaMemset(g->d_scal, 0, kScalars * sizeof(double)));
@@ -497,11 +522,8 @@ void fv_grid_destroy(fv_grid* g) {
   destroy_mg(g);
   if (g->d_arn) cudaFree(g->d_arn);
   for (cudaEvent_t e : g->ev_pool) cudaEventDestroy(e);
-  void* ptrs[] = {g->d_met_d, g->d_met_f, g->d_tpf_d, g->d_tpf_f, g->vel_buf[0], g->vel_buf[1],
-                  g->vel_buf[2], g->cell_buf[0], g->cell_buf[1], g->cell_buf[2], g->tpf_buf[0],
-                  g->tpf_buf[1], g->d_scal, g->d_part, g->kry, g->kry_small, g->U32, g->x32,
-                  g->w32, g->vff[0], g->vff[1], g->pff, g->r32, g->phis[0], g->phis[1], g->phis[2], g->phis[3], g->d_met_ff,
-                  g->d_met_fn, g->Uff, g->xff, g->d_tc, g->d_oz, g->d_xf, g->wts, g->wts_ff, g->d_fault};
+  void* ptrs[] = {g->d_met_d, g->d_met_f, g->d_tpf_d, g->d_tpf_f, g->d_tc, g->d_oz, g->d_xf, g->d_work,
+                  g->kry, g->kry_small};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (g->h_scal) cudaFreeHost(g->h_scal);

@@ -114,11 +114,9 @@ struct LoopState {
   unsigned ticket;              // blocks of the running pass that are done (0 between passes)
 };
 
-// per-call arguments of an evaluation graph; the first two members are read by
-// the J.v kernels as their U and x pointers (U null: the grid's registered
-// base flow)
+// per-call arguments of an evaluation (x, out: velocity vectors; p: optional)
 struct CallBlock {
-  const double* U;
+  const double* U;             // batched evaluations
   const double* x;
   double* out;
   double* p;
@@ -126,17 +124,28 @@ struct CallBlock {
   int max_pass;
 };
 
-// one captured, instantiated evaluation graph (per grid and shift sigma)
+// size of the J.v kernel's argument block, offsets of its x and CallBlock
+struct JvPatch {
+  size_t size = 0, x = 0, cb = 0;
+};
+
+// one captured, instantiated evaluation graph (per grid, shift sigma, form and
+// whether the call passes a base flow)
 struct GraphCache {
   bool ready = false;
   double sigma = 0.0;
   int prec = FV_MIXED;
+  bool has_u = false;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
-  cudaGraphNode_t init_node = nullptr;
-  void* d_call = nullptr;
+  cudaGraphNode_t base_node = nullptr, jv_node = nullptr;
+  cudaKernelNodeParams base_kp = {}, jv_kp = {};
+  std::vector<unsigned char> jv_args;
+  JvPatch patch;
+  CallBlock* d_call = nullptr;   // in the grid's workspace
   LoopState* d_loop = nullptr;
 };
+constexpr int kGraphSlots = 8;
 
 }  // namespace fv
 
@@ -167,7 +176,8 @@ struct fv_grid {
   void* d_xf = nullptr;      // BF16 parts of the eigenbases (grids without fused kernels)
   const unsigned char* xf[3][2] = {};   // per axis: Einv, E
 
-  // workspace
+  // workspace: one allocation, the arrays below in it
+  void* d_work = nullptr;
   double* vel_buf[3] = {nullptr, nullptr, nullptr};   // n_vel each
   double* cell_buf[3] = {nullptr, nullptr, nullptr};  // n_cell each
   void* tpf_buf[2] = {nullptr, nullptr};              // n_cell doubles each (float use half)
@@ -201,7 +211,8 @@ struct fv_grid {
   const double* base_ptr = nullptr;
 
   // captured evaluation graphs of the mixed path (built on first use)
-  fv::GraphCache graphs[4];
+  fv::GraphCache graphs[fv::kGraphSlots];
+  unsigned char* d_eval = nullptr;   // call blocks and loop states of the slots
   mutable bool capturing = false;
   bool use_graph = true;          // FVNS_NO_GRAPH=1 selects the host-driven loop
 
@@ -279,14 +290,16 @@ fv_status launch_zero_walls(const fv_grid* g, double* v);
 
 // mixed-precision path (fv_mixed.cu)
 // J.v tiled kernels (fv_jv.cuh): U from Ud (float64) or, when null, the
-// grid's registered base flow (U32 / Uff); x float64; call (graph launches):
-// a device block whose first two members are the U and x pointers
+// grid's registered base flow (U32 / Uff); x float64; dcb, ls (graphs): see
+// jv::Args
 fv_status launch_jv_f32(const fv_grid* g, const double* Ud, const double* x, float* out,
-                        double shift, const void* call = nullptr);
+                        double shift, CallBlock* dcb = nullptr, LoopState* ls = nullptr);
+JvPatch jv_patch_f32();
+JvPatch jv_patch_ff();
 fv_status launch_jv_f32_out64(const fv_grid* g, const double* Ud, const double* x, double* out,
                               double shift);
 fv_status launch_jv_ff(const fv_grid* g, const double* Ud, const double* x, float2* out,
-                       double shift, const void* call = nullptr);
+                       double shift, CallBlock* dcb = nullptr, LoopState* ls = nullptr);
 fv_status launch_jv_ff_out64(const fv_grid* g, const double* Ud, const double* x, double* out,
                              double shift);
 fv_status launch_round_f32(const fv_grid* g, const double* in, float* out, int64_t n);

@@ -43,6 +43,8 @@
 // converted.
 #pragma once
 
+#include <cstddef>
+
 #include "fv_ff.cuh"
 #include "fv_internal.cuh"
 
@@ -71,23 +73,21 @@ template <> __device__ __forceinline__ double to_store<double, double>(double v)
 template <> __device__ __forceinline__ float2 to_store<ffn, float2>(ffn v) { return make_float2(v.hi, v.lo); }
 template <> __device__ __forceinline__ double to_store<ffn, double>(ffn v) { return ff_join(v.hi, v.lo); }
 
-// Pointers of one launch: Ur the base flow in its stored form (float32
-// rounding, float-float split or float64), x the float64 perturbation; when
-// `call` is given (graph launches) x is read from it.
-struct CallPtrs {
-  const double* U;
-  const double* x;
-};
-
+// One launch: Ur the base flow in its stored form (float32 rounding,
+// float-float split or float64), x the float64 perturbation.  dcb (evaluation
+// graphs): the kernel, the first of the evaluation to depend on the call,
+// stores the call's arguments there and resets the loop state.
 template <typename T, typename TU, typename TO>
 struct Args {
   Met<T> m;
   const TU* Ur;
   const double* x;
   TO* out;
-  const CallPtrs* call;
   T inv_re, shift;
   Tile t;
+  CallBlock cb;
+  CallBlock* dcb;
+  LoopState* ls;
 };
 
 // six fields in a plane slot: U_u, U_v, U_w, Q_u, Q_v, Q_w
@@ -159,8 +159,13 @@ __global__ void __launch_bounds__(kJvMaxThreads, MinBlocks<T>::value) k_jv_tile(
   T* gys = gxs + 3 * nthr;                                   // [3][nthr]
 
   const double* X = a.x;
-  if (a.call) X = a.call->x;
   const TU* Ur = a.Ur;
+  if (a.dcb && tid == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {
+    *a.dcb = a.cb;
+    LoopState* ls = a.ls;
+    ls->phi1 = ls->phi_prev = ls->phi_last = ls->div_last = 0.f;
+    ls->pass = ls->nan = ls->status = 0;
+  }
 
   // this thread's tile cell in the plane
   const int ci = i0 - 1 + li, cj = j0 - 1 + lj;
@@ -388,6 +393,13 @@ inline size_t tile_smem(const Tile& t) {
   const size_t lxy = (size_t)(t.txo + 2) * (t.tyo + 2);
   const size_t ring = kRing * (3 * lxy * sizeof(double) + ((3 * lxy * sizeof(TU) + 15) & ~(size_t)15));
   return ring + sizeof(T) * (2 * 6 * lxy + 6 * (size_t)tile_threads(t));
+}
+
+// where an evaluation graph's launch patches the arguments of its J.v node
+template <typename T, typename TU, typename TO>
+inline JvPatch patch_of() {
+  typedef Args<T, TU, TO> A;
+  return {sizeof(A), offsetof(A, x), offsetof(A, cb)};
 }
 
 // Launch with the z-chunks sized by the kernel's measured residency.

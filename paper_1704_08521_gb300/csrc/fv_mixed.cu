@@ -272,7 +272,7 @@ fv_status launch_split_ff(const fv_grid* g, const double* in, float2* out, int64
 // float-float result (this file is compiled without FMA contraction, so
 // every TwoSum and TwoProd keeps its rounding)
 fv_status launch_jv_ff(const fv_grid* g, const double* Ud, const double* x, float2* out,
-                       double shift, const void* call) {
+                       double shift, CallBlock* dcb, LoopState* ls) {
   if (Ud) {
     FV_TRY(launch_split_ff(g, Ud, g->Uff, g->nvel));
     const_cast<fv_grid*>(g)->base_ptr = nullptr;
@@ -282,7 +282,9 @@ fv_status launch_jv_ff(const fv_grid* g, const double* Ud, const double* x, floa
   a.Ur = g->Uff;
   a.x = x;
   a.out = out;
-  a.call = (const jv::CallPtrs*)call;
+  a.cb = CallBlock();
+  a.dcb = dcb;
+  a.ls = ls;
   a.inv_re = ffn(f64_split(1.0 / g->re));
   a.shift = ffn(f64_split(shift));
   {
@@ -291,6 +293,8 @@ fv_status launch_jv_ff(const fv_grid* g, const double* Ud, const double* x, floa
   }
   return FV_OK;
 }
+
+JvPatch jv_patch_ff() { return jv::patch_of<ffn, float2, float2>(); }
 
 fv_status launch_jv_ff_out64(const fv_grid* g, const double* Ud, const double* x, double* out,
                              double shift) {
@@ -303,7 +307,9 @@ fv_status launch_jv_ff_out64(const fv_grid* g, const double* Ud, const double* x
   a.Ur = g->Uff;
   a.x = x;
   a.out = out;
-  a.call = nullptr;
+  a.cb = CallBlock();
+  a.dcb = nullptr;
+  a.ls = nullptr;
   a.inv_re = ffn(f64_split(1.0 / g->re));
   a.shift = ffn(f64_split(shift));
   {

@@ -210,7 +210,9 @@ fv_status launch_momentum_jac(const fv_grid* g, const double* U, const double* v
   a.Ur = U;
   a.x = v;
   a.out = out;
-  a.call = nullptr;
+  a.cb = CallBlock();
+  a.dcb = nullptr;
+  a.ls = nullptr;
   a.inv_re = 1.0 / g->re;
   a.shift = shift;
   {
@@ -226,7 +228,7 @@ fv_status launch_momentum_jac(const fv_grid* g, const double* U, const double* v
 // staged; float32 result.  call: graph launches read x from the evaluation's
 // device call block (whose U the graph has already rounded into g->U32).
 fv_status launch_jv_f32(const fv_grid* g, const double* Ud, const double* x, float* out,
-                        double shift, const void* call) {
+                        double shift, CallBlock* dcb, LoopState* ls) {
   if (Ud) {
     FV_TRY(launch_round_f32(g, Ud, g->U32, g->nvel));
     const_cast<fv_grid*>(g)->base_ptr = nullptr;
@@ -236,7 +238,9 @@ fv_status launch_jv_f32(const fv_grid* g, const double* Ud, const double* x, flo
   a.Ur = g->U32;
   a.x = x;
   a.out = out;
-  a.call = (const jv::CallPtrs*)call;
+  a.cb = CallBlock();
+  a.dcb = dcb;
+  a.ls = ls;
   a.inv_re = float(1.0 / g->re);
   a.shift = float(shift);
   {
@@ -245,6 +249,8 @@ fv_status launch_jv_f32(const fv_grid* g, const double* Ud, const double* x, flo
   }
   return FV_OK;
 }
+
+JvPatch jv_patch_f32() { return jv::patch_of<float, float, float>(); }
 
 fv_status launch_jv_f32_out64(const fv_grid* g, const double* Ud, const double* x, double* out,
                               double shift) {
@@ -257,7 +263,9 @@ fv_status launch_jv_f32_out64(const fv_grid* g, const double* Ud, const double* 
   a.Ur = g->U32;
   a.x = x;
   a.out = out;
-  a.call = nullptr;
+  a.cb = CallBlock();
+  a.dcb = nullptr;
+  a.ls = nullptr;
   a.inv_re = float(1.0 / g->re);
   a.shift = float(shift);
   {
