@@ -7,6 +7,7 @@
 // register-tiled shared-memory kernel (64 x 64 outputs per block, 4 x 4 per
 // thread); the eigenvalue scaling is fused into the epilogue of the third
 // forward transform.  float32 in the mixed mode, float64 otherwise.
+#include <algorithm>
 #include <atomic>
 #include <cstring>
 #include <map>
@@ -389,7 +390,22 @@ __device__ __forceinline__ void cp_async4(float* dst, const float* src, bool val
                : "memory");
 }
 
-constexpr int kUmmaThreads = 256;   // 8 warps: warps w and w + 4 share accumulator lanes 32 (w % 4) ..
+// Warps w, w + 4, ... of a block share the accumulator lanes 32 (w % 4) ...
+// 16 warps: the copies, splits and epilogues between the two GEMMs are chains
+// of latencies (at 100^3 the column kernel takes 13.1 us with 16 warps and 15.4
+// with 8, the slab kernel 11.0 and 11.7).  Blocks whose phases are a few
+// passes over 8 warps anyway keep 8 (16^3: 3.35 us against 3.5).
+constexpr int kUmmaThreads = 512;
+constexpr int kUmmaMaxWarps = kUmmaThreads / 32;
+inline int umma_threads(int n) { return n <= 32 ? 256 : kUmmaThreads; }
+
+// this warp's share [begin, end) of N accumulator columns, in eighths
+__device__ __forceinline__ void column_share(int warp, int nwarp, int N, int& begin, int& end) {
+  const int parts = nwarp >> 2;
+  const int per = (N / 8 + parts - 1) / parts * 8;
+  begin = min(N, (warp >> 2) * per);
+  end = min(N, begin + per);
+}
 
 __device__ __forceinline__ float4 split4(float4& v) {   // v -> lo parts, returns hi parts
   float4 h;
@@ -409,8 +425,8 @@ __device__ __forceinline__ float4 split4(float4& v) {   // v -> lo parts, return
 // The plane is copied with cp.async straight into its canonical positions
 // (16-byte runs of 4 columns; vec: nx % 4 == 0 so that every full run is
 // 16-byte aligned in global memory) and split in place by the thread that
-// copied it.  256 threads; warps w and w + 4 own accumulator rows
-// 32 (w % 4) .. + 31, the first and second half of the columns.
+// copied it.  The warps w % 4 own accumulator rows 32 (w % 4) .. + 31, a
+// quarter of the columns each.
 __global__ void __launch_bounds__(kUmmaThreads) k_slab_umma(const float* __restrict__ in,
                                                             float* __restrict__ out,
                                                             const float* __restrict__ bx,
@@ -428,12 +444,13 @@ __global__ void __launch_bounds__(kUmmaThreads) k_slab_umma(const float* __restr
   float* Bh = Al + 128 * Km;
   float* Bl = Bh + Nb * Km;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nthr = blockDim.x, nwarp = nthr >> 5;
   const int k = blockIdx.x, a0 = blockIdx.y * Na;
   tc5::pdl_trigger();
   if (warp == 0) tc5::tmem_alloc(&tslot, tcols);
   if (tid == 0) tc5::mbar_init(&bar, 1);
   // M1 chunk [hi | lo] (128 x K1) -> region A
-  stage_pair(bx + (size_t)blockIdx.y * 2 * 128 * K1, Ah, Al, 128 * K1, tid, kUmmaThreads);
+  stage_pair(bx + (size_t)blockIdx.y * 2 * 128 * K1, Ah, Al, 128 * K1, tid, nthr);
   // everything above uses constants only; the field is the predecessor's output
   tc5::pdl_wait();
   if (skip && *skip != 0) {      // the loop ended before this pass
@@ -447,7 +464,7 @@ __global__ void __launch_bounds__(kUmmaThreads) k_slab_umma(const float* __restr
   const float* ink = in + (size_t)k * nx * ny;
   const int kb4 = K1 >> 2, kq4 = (kb4 + 3) >> 2;
   const int sbo1 = kb4 * 32;   // floats per 8-row block
-  for (int t = warp; t < (N1 >> 3) * kq4; t += 8) {
+  for (int t = warp; t < (N1 >> 3) * kq4; t += nwarp) {
     const int rb = t / kq4, kq = t - rb * kq4;
     const int j = 8 * rb + (lane & 7), kb = 4 * kq + (lane >> 3);
     if (kb < kb4) {
@@ -465,7 +482,7 @@ __global__ void __launch_bounds__(kUmmaThreads) k_slab_umma(const float* __restr
     }
   }
   tc5::cp_async_wait_all();
-  for (int t = warp; t < (N1 >> 3) * kq4; t += 8) {
+  for (int t = warp; t < (N1 >> 3) * kq4; t += nwarp) {
     const int rb = t / kq4, kq = t - rb * kq4;
     const int kb = 4 * kq + (lane >> 3);
     if (kb < kb4) {
@@ -489,12 +506,12 @@ __global__ void __launch_bounds__(kUmmaThreads) k_slab_umma(const float* __restr
   __syncwarp();   // tcgen05.ld is warp-collective
   tc5::fence_after_sync();
   // region A is free: stage M2 while T^T moves from tensor memory to region B
-  stage_pair(ay, Ah, Al, 128 * K2, tid, kUmmaThreads);
+  stage_pair(ay, Ah, Al, 128 * K2, tid, nthr);
   const int row = 32 * (warp & 3) + lane;
   const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
   {
-    const int half = ((N1 >> 3) + 1) >> 1;   // 8-column chunks of the first half
-    const int c_begin = warp < 4 ? 0 : 8 * half, c_end = warp < 4 ? 8 * half : N1;
+    int c_begin, c_end;
+    column_share(warp, nwarp, N1, c_begin, c_end);
     for (int c = c_begin; c < c_end; c += 8) {
       float v[8];
       tc5::ld8(trow + (uint32_t)c, v);
@@ -525,8 +542,8 @@ __global__ void __launch_bounds__(kUmmaThreads) k_slab_umma(const float* __restr
   if (tid == 0 && !(ok1 && ok2)) atomicOr(fault, 1u);   // reported as FV_ETIMEOUT
   {
     float* outr = out + (size_t)k * nx * ny + (size_t)row * nx;
-    const int half = ((Na >> 3) + 1) >> 1;
-    const int c_begin = warp < 4 ? 0 : 8 * half, c_end = warp < 4 ? 8 * half : Na;
+    int c_begin, c_end;
+    column_share(warp, nwarp, Na, c_begin, c_end);
     for (int c = c_begin; c < c_end; c += 8) {
       float v[8];
       tc5::ld8(trow + (uint32_t)c, v);
@@ -553,7 +570,7 @@ __global__ void __launch_bounds__(kUmmaThreads) k_slab_umma(const float* __restr
 // columns q0 + [0, N), q = j nx + i:
 //   t[c][q] = sum_k Ez^-1[c][k] in[k][q] / (lam_z[c] + lam_y[j] + lam_x[i])  (null mode -> 0)
 //   out[m][q] = sum_c Ez[m][c] t[c][q]
-// GEMM 1: A = Ez^-1, B = in^T; GEMM 2: A = Ez, B = t^T.  256 threads (as above).
+// GEMM 1: A = Ez^-1, B = in^T; GEMM 2: A = Ez, B = t^T.
 // The input tile is copied in its own order (16-byte runs along q) into a
 // padded row-major tile R and transposed + split from there into the
 // canonical operand; the scaled intermediate goes through a per-warp 32 x 9
@@ -581,10 +598,11 @@ __global__ void __launch_bounds__(kUmmaThreads) k_col_umma(const float* __restri
   const int ldR = N + 4;
   float* R = reinterpret_cast<float*>(nullq + N);   // Kz x ldR raw tile, later transpose scratch
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nthr = blockDim.x, nwarp = nthr >> 5;
   tc5::pdl_trigger();
   if (warp == 0) tc5::tmem_alloc(&tslot, tcols);
   if (tid == 0) tc5::mbar_init(&bar, 1);
-  stage_pair(azi, Ah, Al, 128 * Kz, tid, kUmmaThreads);
+  stage_pair(azi, Ah, Al, 128 * Kz, tid, nthr);
   // everything above uses constants only; the field is the predecessor's output
   tc5::pdl_wait();
   if (skip && *skip != 0) {      // the loop ended before this pass
@@ -597,7 +615,7 @@ __global__ void __launch_bounds__(kUmmaThreads) k_col_umma(const float* __restri
   // columns beyond Q zero-filled)
   {
     const int n4 = N >> 2;
-    for (int e = tid; e < Kz * n4; e += kUmmaThreads) {
+    for (int e = tid; e < Kz * n4; e += nthr) {
       const int kk = e / n4, j4 = e - kk * n4;
       float* dst = R + kk * ldR + 4 * j4;
       const int64_t qq = q0 + 4 * j4;
@@ -612,7 +630,7 @@ __global__ void __launch_bounds__(kUmmaThreads) k_col_umma(const float* __restri
       }
     }
   }
-  for (int q = tid; q < N; q += kUmmaThreads) {
+  for (int q = tid; q < N; q += nthr) {
     const int64_t qq = q0 + q;
     float lq = 1.f;
     int nl = 0;
@@ -630,7 +648,7 @@ __global__ void __launch_bounds__(kUmmaThreads) k_col_umma(const float* __restri
   // a warp covers 8 consecutive q x 4 consecutive kb (512 contiguous bytes)
   {
     const int kb4 = Kz >> 2;
-    for (int e = tid; e < N * kb4; e += kUmmaThreads) {
+    for (int e = tid; e < N * kb4; e += nthr) {
       const int ql = e & 7, rest = e >> 3;
       const int qh = rest / kb4, kb = rest - qh * kb4;
       const int q = 8 * qh + ql;
@@ -654,11 +672,11 @@ __global__ void __launch_bounds__(kUmmaThreads) k_col_umma(const float* __restri
   const bool ok1 = tc5::mbar_wait(&bar, 0, kMbarLimit);
   __syncwarp();   // tcgen05.ld is warp-collective
   tc5::fence_after_sync();
-  stage_pair(aze, Ah, Al, 128 * Kz, tid, kUmmaThreads);
+  stage_pair(aze, Ah, Al, 128 * Kz, tid, nthr);
   const int row = 32 * (warp & 3) + lane;   // c of GEMM 1, m of GEMM 2
   const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
-  const int half = ((N >> 3) + 1) >> 1;
-  const int c_begin = warp < 4 ? 0 : 8 * half, c_end = warp < 4 ? 8 * half : N;
+  int c_begin, c_end;
+  column_share(warp, nwarp, N, c_begin, c_end);
   {
     const float lz = row < nz ? tp.lam[2][row] : 1.f;
     const bool nullrow = row == tp.null_index[2];
@@ -734,8 +752,8 @@ inline size_t slab_smem(int nx, int ny, int Na) {
 }
 
 inline size_t col_smem(int nz, int N) {
-  // eigenbasis hi / lo, operand hi / lo, lam / null per column, raw tile R (>= 8 x 32 x 9 scratch)
-  const size_t R = (size_t)up8(nz) * (N + 4) > 8 * 32 * 9 ? (size_t)up8(nz) * (N + 4) : 8 * 32 * 9;
+  // eigenbasis hi / lo, operand hi / lo, lam / null per column, raw tile R (also 32 x 9 scratch per warp)
+  const size_t R = std::max<size_t>((size_t)up8(nz) * (N + 4), kUmmaMaxWarps * 32 * 9);
   return sizeof(float) * ((size_t)(2 * 128 + 2 * N) * up8(nz) + 2 * (size_t)N + R);
 }
 
@@ -770,7 +788,7 @@ fv_status launch_slab(const fv_grid* g, const float* in, float* out, int dir, co
   const int nx = g->n[0], ny = g->n[1], nz = g->n[2];
   const int N = g->tc.slab_n;
   LaunchScope ls_(g, dir == 0 ? FV_K_TPF_X : FV_K_TPF_XINV);
-  FV_CUDA(tc5::launch_pdl(k_slab_umma, dim3(nz, g->tc.slab_nsplit), dim3(kUmmaThreads),
+  FV_CUDA(tc5::launch_pdl(k_slab_umma, dim3(nz, g->tc.slab_nsplit), dim3(umma_threads(nx > ny ? nx : ny)),
                      slab_smem(nx, ny, N), g->stream, in, out, (const float*)g->tc.bx[dir],
                      (const float*)g->tc.ay[dir], nx, ny, N,
                      tmem_cols(up16(ny) > N ? up16(ny) : N),
@@ -782,7 +800,7 @@ fv_status launch_col(const fv_grid* g, const float* in, float* out, const int* s
   const int N = g->tc.col_n;
   const int64_t Q = (int64_t)g->n[0] * g->n[1];
   LaunchScope ls_(g, FV_K_TPF_YZ);
-  FV_CUDA(tc5::launch_pdl(k_col_umma, dim3((unsigned)((Q + N - 1) / N)), dim3(kUmmaThreads),
+  FV_CUDA(tc5::launch_pdl(k_col_umma, dim3((unsigned)((Q + N - 1) / N)), dim3(umma_threads(g->n[2])),
                      col_smem(g->n[2], N), g->stream, in, out, g->tpf_f,
                      (const float*)g->tc.az[0], (const float*)g->tc.az[1], N, tmem_cols(N),
                      (Q % 4 == 0 && N % 4 == 0) ? 1 : 0, g->d_fault, skip));
