@@ -422,13 +422,15 @@ fv_status fv_pressure_solve(const fv_grid* g, const double* r, double* phi, int 
  * than 4 cells, alternating-direction zebra line Gauss-Seidel smoothing (one
  * tridiagonal solve per grid line), linear interpolation between coarse
  * centres and its transpose, rediscretised coarse operators, an exact
- * separable solve on the coarsest grid.  guess (device, optional, may equal
+ * separable solve on the first grid with at most 32 cells per axis (in place of
+ * the coarser ones).  guess (device, optional, may equal
  * phi) is the initial phi, zero if NULL.  Stops at ||b - A phi||_2 <=
  * rtol ||b||_2; FV_ENOCONV (stats filled) after max_iter iterations.  The
- * hierarchy and its workspace (~6 float32 and 5 float64 cell arrays) are
- * built on the first call and kept with the grid.  Runs on the grid's
- * stream; returns after the last convergence check (the final mean removal
- * is queued). */
+ * hierarchy and its workspace (~8 float32 and 3 float64 cell arrays) are
+ * built on the first call and kept with the grid, with the iteration captured
+ * as a CUDA graph whose stop test runs on the device (make the call outside
+ * any stream capture).  Runs on the grid's stream and synchronises it once, at
+ * the end. */
 typedef struct {
   double rtol;     /* relative residual target                        [1e-10] */
   int max_iter;    /* conjugate-gradient iteration cap                  [100] */

@@ -118,6 +118,9 @@ struct CaptureStreams {
   ~CaptureStreams() { drop(); }
 };
 thread_local CaptureStreams t_capture;
+}  // namespace
+
+void drop_capture_streams() { t_capture.drop(); }
 
 fv_status capture_streams(cudaStream_t* cs, cudaStream_t* bs) {
   int dev = 0;
@@ -132,6 +135,7 @@ fv_status capture_streams(cudaStream_t* cs, cudaStream_t* bs) {
   return FV_OK;
 }
 
+namespace {
 // the node captured last on s
 fv_status last_node(cudaStream_t s, cudaGraphNode_t* node) {
   cudaStreamCaptureStatus cst;
@@ -201,7 +205,7 @@ static fv_status build_graph(fv_grid* g, double sigma, GraphCache& gc, int prec,
   if (st == FV_OK) st = finish();
   if (st != FV_OK) {
     if (graph) cudaGraphDestroy(graph);
-    t_capture.drop();                 // a stream may still be capturing
+    drop_capture_streams();           // a stream may still be capturing
     (void)cudaGetLastError();
     return st;
   }
@@ -558,7 +562,7 @@ static fv_status batch_build_graph(BatchImpl& b) {
   if (st == FV_OK && ec != cudaSuccess) st = cuda_fail(ec, "cudaStreamEndCapture", __FILE__, __LINE__);
   if (st != FV_OK) {
     if (graph) cudaGraphDestroy(graph);
-    t_capture.drop();                 // a stream may still be capturing
+    drop_capture_streams();           // a stream may still be capturing
     (void)cudaGetLastError();
     return st;
   }

@@ -326,6 +326,10 @@ fv_status mixed_krylov_graph(const fv_grid* g, const double* U, const double* x,
                              bool sync, int* passes, double* phi1, double* phil, double* divl,
                              int* status, int prec = FV_MIXED);
 void destroy_graph_cache(GraphCache& c);
+// this thread's two streams for graph capture (a graph and a conditional
+// body); dropped after a failed capture
+fv_status capture_streams(cudaStream_t* cs, cudaStream_t* bs);
+void drop_capture_streams();
 // the passes and the end of an evaluation (fv_pass.cu): pass idx = 0, 1, 2 of
 // the loop, or any later one (3), from the solution in g->phis[idx]; decide:
 // count it, take the stop decision and (h) set the WHILE condition

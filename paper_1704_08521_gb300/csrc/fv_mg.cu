@@ -27,21 +27,23 @@
 // cosine-stretched grids have cells with aspect ratios of tens, for which
 // point smoothers fail and line smoothers do not.  Each half-sweep solves
 // every line of one colour (lines coloured like a checkerboard of their two
-// transverse indices, so neighbour lines differ in colour) exactly, in
-// place: lines of up to kPartMaxLine cells are split over up to 8 warps (the
-// partition method, k_line_part), longer ones take one thread each (the
-// Thomas recurrence, k_line).  Pre-smoothing x, y, z (colours 0, 1) and
-// post-smoothing in the exact reverse order, so the V-cycle is a symmetric
-// preconditioner.  Coarsest
-// level (at most 4 cells per axis): exact solve by the separable eigenbases
-// of the coarse operator (A = sum over axes of K_d (x) W_others, K_d E_d =
-// W_d E_d Lambda_d), null mode dropped.
+// transverse indices, so neighbour lines differ in colour) exactly, in place
+// (k_line).  Pre-smoothing x, y, z (colours 0, 1) and post-smoothing in the
+// exact reverse order, so the V-cycle is a symmetric preconditioner.  The first
+// level with at most 32 cells per axis is solved exactly by the separable
+// eigenbases of its operator (A = sum over axes of K_d (x) W_others, K_d E_d =
+// W_d E_d Lambda_d), null mode dropped, in place of the levels below it.
+//
+// The whole iteration, its stop test included, is one CUDA graph whose WHILE
+// node runs the conjugate-gradient steps on the device; the host waits once.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
 
+#include "fv_ff.cuh"
 #include "fv_internal.cuh"
+#include "fv_tc5.cuh"
 #include "fvns_host.h"
 
 namespace fv {
@@ -49,9 +51,9 @@ namespace fv {
 namespace {
 
 constexpr int kMgMaxLevels = 16;
-constexpr int kCoarseMax = 4;       // coarsest level: at most this many cells per axis
+constexpr int kCoarseMax = 4;       // the hierarchy ends with at most this many cells per axis
 constexpr int kRedThreads = 256;
-constexpr int kRedBlocks = 592;     // 4 x 148: fixed, so the reductions are deterministic
+constexpr int kRedBlocks = 608;     // 4 x 152: fixed, so the reductions are deterministic
 
 // ------------------------------------------------------------ host tables --
 struct Axis1D {
@@ -144,6 +146,7 @@ struct LevDev {
   int64_t ncell;
   const float* w[3];
   const float* t[3];
+  const float* ip[3];    // per direction: inverse pivots of the line solves, per cell
   // transfer between this level and the next coarser one
   const int* pc0[3];     // per index of this level
   const float* pw1[3];
@@ -164,424 +167,391 @@ struct CoarseDev {
   const float* lam[3];
 };
 
-__device__ __forceinline__ void cell_ijk(int64_t c, const int n[3], int& i, int& j, int& k) {
-  i = (int)(c % n[0]);
-  const int64_t r = c / n[0];
-  j = (int)(r % n[1]);
-  k = (int)(r / n[1]);
+// (3 n_cell < 2^31: 32-bit arithmetic)
+__device__ __forceinline__ void cell_ijk(unsigned c, const int n[3], int& i, int& j, int& k) {
+  const unsigned r = c / (unsigned)n[0];
+  i = (int)(c - r * (unsigned)n[0]);
+  k = (int)(r / (unsigned)n[1]);
+  j = (int)(r - (unsigned)k * (unsigned)n[1]);
 }
 
-// A x at cell (i, j, k) and the diagonal of A there
+// A x at cell (i, j, k), as the sum of the fluxes to its neighbours (t is 0 at
+// the walls, where the clamped neighbour is the cell itself)
 template <typename T, typename Lv>
-__device__ __forceinline__ T apply_at(const Lv& L, const T* __restrict__ x, int i, int j, int k,
-                                      int64_t c, T* diag) {
-  const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
-  const int64_t sy = nx, sz = (int64_t)nx * ny;
+__device__ __forceinline__ T apply_at(const Lv& L, const T* __restrict__ x, int i, int j, int k, int c) {
+  const int nx = L.n[0], ny = L.n[1], nz = L.n[2], sy = nx, sz = nx * ny;
   const T wx = L.w[0][i], wy = L.w[1][j], wz = L.w[2][k];
-  const T ax0 = wy * wz * L.t[0][i], ax1 = wy * wz * L.t[0][i + 1];
-  const T ay0 = wx * wz * L.t[1][j], ay1 = wx * wz * L.t[1][j + 1];
-  const T az0 = wx * wy * L.t[2][k], az1 = wx * wy * L.t[2][k + 1];
   const T xp = x[c];
-  T s = (ax0 + ax1 + ay0 + ay1 + az0 + az1) * xp;
-  if (i > 0) s -= ax0 * x[c - 1];
-  if (i + 1 < nx) s -= ax1 * x[c + 1];
-  if (j > 0) s -= ay0 * x[c - sy];
-  if (j + 1 < ny) s -= ay1 * x[c + sy];
-  if (k > 0) s -= az0 * x[c - sz];
-  if (k + 1 < nz) s -= az1 * x[c + sz];
-  if (diag) *diag = ax0 + ax1 + ay0 + ay1 + az0 + az1;
-  return s;
+  const T fx = L.t[0][i] * (xp - x[i > 0 ? c - 1 : c]) + L.t[0][i + 1] * (xp - x[i + 1 < nx ? c + 1 : c]);
+  const T fy = L.t[1][j] * (xp - x[j > 0 ? c - sy : c]) + L.t[1][j + 1] * (xp - x[j + 1 < ny ? c + sy : c]);
+  const T fz = L.t[2][k] * (xp - x[k > 0 ? c - sz : c]) + L.t[2][k + 1] * (xp - x[k + 1 < nz ? c + sz : c]);
+  return wy * wz * fx + wx * (wz * fy + wy * fz);
 }
 
 // --------------------------------------------------------- V-cycle kernels --
+// the thread's cell of line (a, b) along D at row m, as strides
+template <int D>
+__device__ __forceinline__ void line_cell(const LevDev& L, int a, int b, int& i0, int& j0, int& k0, int& c00,
+                                          int& stride) {
+  if (D == 0) { i0 = 0; j0 = a; k0 = b; stride = 1; }
+  else if (D == 1) { i0 = a; j0 = 0; k0 = b; stride = L.n[0]; }
+  else { i0 = a; j0 = b; k0 = 0; stride = L.n[0] * L.n[1]; }
+  c00 = (k0 * L.n[1] + j0) * L.n[0] + i0;
+}
+
+// rows of a line eliminated from its low end; the others from its high end
+__host__ __device__ inline int low_rows(int nl) { return (nl + 1) / 2; }
+
+// Inverse pivots of the tridiagonal matrices of all lines along D, eliminated
+// from both ends towards the middle: 1 / (diag_m - lo_m^2 ip_{m-1}) below it,
+// 1 / (diag_m - up_m^2 ip_{m+1}) above, one thread per line; once per hierarchy.
+template <int D>
+__global__ void k_pivots(LevDev L, float* __restrict__ ip) {
+  const int na = D == 0 ? L.n[1] : L.n[0], nb = D == 2 ? L.n[1] : L.n[2];
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= na * nb) return;
+  int i0, j0, k0, c00, stride;
+  line_cell<D>(L, t % na, t / na, i0, j0, k0, c00, stride);
+  const float wa = D == 0 ? L.w[1][j0] : L.w[0][i0], wb = D == 2 ? L.w[1][j0] : L.w[2][k0];
+  const float cross = wa * wb;
+  const int nl = L.n[D], h = low_rows(nl);
+  float q = 0.f;
+  for (int s = 0; s < nl; ++s) {
+    if (s == h) q = 0.f;
+    const int m = s < h ? s : nl - 1 - (s - h);
+    const int i = D == 0 ? m : i0, j = D == 1 ? m : j0, k = D == 2 ? m : k0;
+    const float wx = L.w[0][i], wy = L.w[1][j], wz = L.w[2][k];
+    const float dg = wy * wz * L.t[0][i] + wy * wz * L.t[0][i + 1] + wx * wz * L.t[1][j] +
+                     wx * wz * L.t[1][j + 1] + wx * wy * L.t[2][k] + wx * wy * L.t[2][k + 1];
+    const float o = cross * L.t[D][s < h ? m : m + 1];
+    q = 1.f / (dg - o * o * q);
+    ip[c00 + m * stride] = q;
+  }
+}
+
+// The recurrences of the lines of a block, by one warp: lanes l and l + 16 own
+// line l, eliminate it from its low and its high end, solve the two rows where
+// they meet together and substitute back outwards, so a chain is nl and not
+// 2 nl multiply-adds long.  S (residual times inverse pivot, entry m at
+// m pitch) becomes the solution; Q the inverse pivots, cross the product of
+// the two widths across the line (off-diagonals -cross t).
+__device__ __forceinline__ void solve_line(float* S, const float* Q, int pitch, int nl, float cross,
+                                           const float* __restrict__ t, bool high) {
+  const int h = low_rows(nl), count = high ? nl - h : h;
+  const int m0 = high ? nl - 1 : 0, dm = high ? -1 : 1;
+  const float* ti = t + (high ? 1 : 0);          // coupling towards the end the row is eliminated from
+  const float* to = t + (high ? 0 : 1);          // and towards the middle
+  float d = 0.f;
+#pragma unroll 8
+  for (int q = 0; q < count; ++q) {
+    const int m = m0 + dm * q;
+    d = fmaf(cross * __ldg(ti + m) * Q[m * pitch], d, S[m * pitch]);
+    S[m * pitch] = d;
+  }
+  const int ml = m0 + dm * (count - 1);
+  const float al = cross * __ldg(t + h) * Q[ml * pitch];
+  const float d2 = __shfl_xor_sync(0xffffffffu, d, 16), al2 = __shfl_xor_sync(0xffffffffu, al, 16);
+  float e = (d + al * d2) / (1.f - al * al2);
+  S[ml * pitch] = e;
+#pragma unroll 8
+  for (int q = count - 2; q >= 0; --q) {
+    const int m = m0 + dm * q;
+    e = fmaf(cross * __ldg(to + m) * Q[m * pitch], e, S[m * pitch]);
+    S[m * pitch] = e;
+  }
+}
+
 // One half-sweep of zebra line Gauss-Seidel along axis D: every line along
 // D of colour `color` (the parity of its two transverse indices' sum) is
 // solved exactly for the current values of its neighbour lines, which all
 // have the other colour and are not written by this launch:
 //   x_line += omega * D_line^-1 (b - A x)_line,
-// D_line the tridiagonal part of A along the line.  In place.  One thread per
-// line; the Thomas recurrence keeps its c' and d' in cb / db (same indexing
-// as the cells).  Transverse indices: a (the faster one: i for y- and
-// z-lines, j for x-lines) and b (k for x- and y-lines, j for z-lines); the
-// thread's line has a = 2 t_a + ((b + color) & 1).
-template <int D>
-__global__ void __launch_bounds__(128) k_line(LevDev L, float* __restrict__ x,
-                                              const float* __restrict__ b, float* __restrict__ cb,
-                                              float* __restrict__ db, float omega, int color) {
-  const int nx = L.n[0], ny = L.n[1];
-  const int nl = L.n[D];
-  const int na = D == 0 ? ny : nx;
-  const int nb = D == 2 ? ny : L.n[2];
-  const int ha = (na + 1) >> 1;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)ha * nb) return;
-  const int tb = (int)(t / ha);
-  const int ta = 2 * (int)(t - (int64_t)tb * ha) + ((tb + color) & 1);
-  if (ta >= na) return;
-  // first cell of the line and the stride along it
-  int i0, j0, k0;
-  int64_t stride;
-  if (D == 0) {
-    i0 = 0; j0 = ta; k0 = tb; stride = 1;
-  } else if (D == 1) {
-    i0 = ta; j0 = 0; k0 = tb; stride = nx;
-  } else {
-    i0 = ta; j0 = tb; k0 = 0; stride = (int64_t)nx * ny;
-  }
-  const int64_t c00 = ((int64_t)k0 * ny + j0) * nx + i0;
-  const float* tD = L.t[D];
-  // the two widths across the line
-  const float wa = D == 0 ? L.w[1][j0] : L.w[0][i0];
-  const float wb = D == 2 ? L.w[1][j0] : L.w[2][k0];
-  const float cross = wa * wb;
-  constexpr int U = 4;
-  float cp = 0.f, dp = 0.f;
-  for (int m0 = 0; m0 < nl; m0 += U) {
-    float res[U], dg[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int m = m0 + u;
-      if (m < nl) {
-        const int i = D == 0 ? m : i0, j = D == 1 ? m : j0, k = D == 2 ? m : k0;
-        const int64_t c = c00 + (int64_t)m * stride;
-        float diag;
-        const float ax = apply_at<float>(L, x, i, j, k, c, &diag);
-        res[u] = b[c] - ax;
-        dg[u] = diag;
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int m = m0 + u;
-      if (m < nl) {
-        const int64_t c = c00 + (int64_t)m * stride;
-        const float lo = -cross * tD[m], up = -cross * tD[m + 1];
-        const float inv = 1.f / (dg[u] - lo * cp);
-        const float cc = up * inv;
-        const float dd = (res[u] - lo * dp) * inv;
-        cb[c] = cc;
-        db[c] = dd;
-        cp = cc;
-        dp = dd;
-      }
-    }
-  }
-  float dn = 0.f;
-  for (int m1 = nl - 1; m1 >= 0; m1 -= U) {
-    float cc[U], dd[U], xi[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int m = m1 - u;
-      if (m >= 0) {
-        const int64_t c = c00 + (int64_t)m * stride;
-        cc[u] = cb[c];
-        dd[u] = db[c];
-        xi[u] = x[c];
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int m = m1 - u;
-      if (m >= 0) {
-        const int64_t c = c00 + (int64_t)m * stride;
-        const float del = dd[u] - cc[u] * dn;
-        x[c] = xi[u] + omega * del;
-        dn = del;
-      }
-    }
-  }
-}
+// D_line the tridiagonal part of A along the line.  In place.  Transverse
+// indices: a (the faster one: i for y- and z-lines, j for x-lines) and b (k
+// for x- and y-lines, j for z-lines); line t has a = 2 (t mod half) + ((b +
+// color) & 1).
+//
+// A block owns 16 lines.  All its threads form the residuals of their cells,
+// coalesced, times the inverse pivots, and keep both in shared memory; one
+// warp then runs the recurrences (solve_line), one multiply-add of latency per
+// row because the pivots do not depend on x and are stored with the hierarchy;
+// all threads add the result to x.
+// Measured at 100^3 (cold caches): 14-15 us a half-sweep in each direction.  The
+// partition method it replaces (each line split over 8 warps, a division per
+// row in every chain) took 26-28 us for y- and z-lines and 75 us for x-lines,
+// whose threads read whole lines apart; 32 lines and 256 threads per block 23-25
+// us (12 % of the warps active).  Three blocks per SM need at most 42 registers:
+// at two the 313 blocks of 100^3 take a second wave (20 us).
+constexpr int kLineThreads = 512, kLines = 16;
 
-// The same half-sweep with each line split over P warps (the partition
-// method for tridiagonal systems): a block owns 32 lines of the colour (one
-// per lane) and P segments of each (one per warp).  Segment p of a line has
-// rows [s, e) and couples to the rows s - 1 and e of its neighbours only
-// through its first row's lower and its last row's upper coefficient.
-//  1. forward over the segment: residuals r_m (kept in shared memory), the
-//     inverse pivots 1/den_m of the segment's own tridiagonal matrix T (kept),
-//     and the last rows of y = T^-1 r, v = T^-1 e_first, w = T^-1 e_last;
-//  2. the same elimination from the bottom: the first rows of y, v, w;
-//  3. warp 0 solves, per line, the 2P boundary unknowns (first and last row
-//     of each segment): a block-tridiagonal system with 2 x 2 blocks;
-//  4. each segment solves T x = r - (coupling to the neighbours' boundary
-//     values) with the kept pivots and adds omega x to the line.
-// Shared memory: r and the pivots as [row][lane] (conflict-free), the
-// boundary values [P][8][lane].
 template <int D>
-__global__ void __launch_bounds__(256) k_line_part(LevDev L, float* __restrict__ x,
-                                                   const float* __restrict__ b, float omega,
-                                                   int color, int P) {
-  extern __shared__ float ps[];
-  const int nx = L.n[0], ny = L.n[1];
+__global__ void __launch_bounds__(kLineThreads, 3) k_line(LevDev L, float* __restrict__ x,
+                                              const float* __restrict__ b, float omega, int color,
+                                              int b_early) {
+  extern __shared__ float sm[];
+  tc5::pdl_trigger();
+  constexpr int NL = kLines, LP = NL + 1;    // pitch: rows and lines both conflict-free
+  const int nx = L.n[0], ny = L.n[1], nz = L.n[2], sy = nx, sz = nx * ny;
   const int nl = L.n[D];
-  const int na = D == 0 ? ny : nx;
-  const int nb = D == 2 ? ny : L.n[2];
+  const int na = D == 0 ? ny : nx, nb = D == 2 ? ny : nz;
   const int ha = (na + 1) >> 1;
-  const int lane = threadIdx.x & 31, p = threadIdx.x >> 5;
-  float* R = ps;                    // [nl][32]
-  float* Q = ps + nl * 32;          // [nl][32] inverse pivots
-  float* S = Q + nl * 32;           // [P][8][32]
-  const int64_t t = (int64_t)blockIdx.x * 32 + lane;
-  bool valid = t < (int64_t)ha * nb;
-  int ta = 0, tb = 0;
-  if (valid) {
-    tb = (int)(t / ha);
-    ta = 2 * (int)(t - (int64_t)tb * ha) + ((tb + color) & 1);
-    valid = ta < na;
+  float* S = sm;                             // [nl][LP] residual times inverse pivot, then the solution
+  float* Q = sm + nl * LP;                   // [nl][LP] inverse pivots
+  __shared__ int sa[NL], sb[NL];             // the block's lines (sa < 0: none)
+  const int tid = threadIdx.x;
+  if (tid < NL) {
+    const int t = blockIdx.x * NL + tid;
+    int ta = -1, tb = 0;
+    if (t < ha * nb) {
+      tb = t / ha;
+      ta = 2 * (t - tb * ha) + ((tb + color) & 1);
+      if (ta >= na) ta = -1;
+    }
+    sa[tid] = ta;
+    sb[tid] = tb;
   }
-  int i0, j0, k0;
-  int64_t stride;
-  if (D == 0) {
-    i0 = 0; j0 = ta; k0 = tb; stride = 1;
-  } else if (D == 1) {
-    i0 = ta; j0 = 0; k0 = tb; stride = nx;
-  } else {
-    i0 = ta; j0 = tb; k0 = 0; stride = (int64_t)nx * ny;
-  }
-  const int64_t c00 = ((int64_t)k0 * ny + j0) * nx + i0;
-  const float* tD = L.t[D];
-  const float wa = valid ? (D == 0 ? L.w[1][j0] : L.w[0][i0]) : 0.f;
-  const float wb = valid ? (D == 2 ? L.w[1][j0] : L.w[2][k0]) : 0.f;
-  const float cross = wa * wb;
-  const int s0 = (int)(((int64_t)p * nl) / P), e0 = (int)(((int64_t)(p + 1) * nl) / P);
-  // coefficient of row m: lower -cross t[m], upper -cross t[m + 1]; the
-  // diagonal is A's (all six faces)
-  auto diag_at = [&](int m) {       // the expression apply_at evaluates
-    const int i = D == 0 ? m : i0, j = D == 1 ? m : j0, k = D == 2 ? m : k0;
-    const float wx = L.w[0][i], wy = L.w[1][j], wz = L.w[2][k];
-    const float ax0 = wy * wz * L.t[0][i], ax1 = wy * wz * L.t[0][i + 1];
-    const float ay0 = wx * wz * L.t[1][j], ay1 = wx * wz * L.t[1][j + 1];
-    const float az0 = wx * wy * L.t[2][k], az1 = wx * wy * L.t[2][k + 1];
-    return ax0 + ax1 + ay0 + ay1 + az0 + az1;
+  __syncthreads();
+  // cells in an order that is coalesced for D: x-lines row by row of one line,
+  // the others line by line of one row.  Missing lines load line (0, 0), whose
+  // values go nowhere, so that no branch keeps the loads of several cells apart.
+  const int total = nl * NL;
+  auto cell_of = [&](int e0, int& l, int& m, int& i, int& j, int& k) {
+    const int e = min(e0 + tid, total - 1);  // (the last cell possibly by several threads)
+    l = D == 0 ? e / nl : e % NL;
+    m = D == 0 ? e - l * nl : e / NL;
+    int c00, stride;
+    line_cell<D>(L, max(sa[l], 0), sb[l], i, j, k, c00, stride);
+    if (D == 0) i = m; else if (D == 1) j = m; else k = m;
+    return c00 + m * stride;
   };
-  float yl = 0.f, vl = 0.f, wl = 0.f, yf = 0.f, vf = 0.f, wf = 0.f;
-  const float lext = -cross * tD[s0], uext = -cross * tD[e0];
-  if (valid) {
-    // 1. forward
-    float dy = 0.f, dv = 0.f, dw = 0.f, cprev = 0.f;
-    constexpr int U = 4;
-    for (int m0 = s0; m0 < e0; m0 += U) {
-      float res[U], dg[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int m = m0 + u;
-        if (m < e0) {
-          const int i = D == 0 ? m : i0, j = D == 1 ? m : j0, k = D == 2 ? m : k0;
-          const int64_t c = c00 + (int64_t)m * stride;
-          float dgv;
-          const float ax = apply_at<float>(L, x, i, j, k, c, &dgv);
-          res[u] = b[c] - ax;
-          dg[u] = dgv;
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int m = m0 + u;
-        if (m < e0) {
-          const float lo = m > s0 ? -cross * tD[m] : 0.f;
-          const float up = m < e0 - 1 ? -cross * tD[m + 1] : 0.f;
-          const float inv = 1.f / (dg[u] - lo * cprev);
-          dy = (res[u] - lo * dy) * inv;
-          dv = ((m == s0 ? 1.f : 0.f) - lo * dv) * inv;
-          dw = ((m == e0 - 1 ? 1.f : 0.f) - lo * dw) * inv;
-          cprev = up * inv;
-          R[m * 32 + lane] = res[u];
-          Q[m * 32 + lane] = inv;
-        }
-      }
-    }
-    yl = dy; vl = dv; wl = dw;
-    // 2. the same elimination from the bottom row up
-    float ry = 0.f, rv = 0.f, rw = 0.f, gprev = 0.f;
-    for (int m = e0 - 1; m >= s0; --m) {
-      const float lo = m > s0 ? -cross * tD[m] : 0.f;
-      const float up = m < e0 - 1 ? -cross * tD[m + 1] : 0.f;
-      const float inv = 1.f / (diag_at(m) - up * gprev);
-      const float r = R[m * 32 + lane];
-      ry = (r - up * ry) * inv;
-      rv = ((m == s0 ? 1.f : 0.f) - up * rv) * inv;
-      rw = ((m == e0 - 1 ? 1.f : 0.f) - up * rw) * inv;
-      gprev = lo * inv;
-    }
-    yf = ry; vf = rv; wf = rw;
+  // what the previous kernels do not write is fetched while they finish: the
+  // pivots, and b unless the predecessor is the kernel that made it
+#pragma unroll 4
+  for (int e0 = 0; e0 < total; e0 += kLineThreads) {
+    int l, m, i, j, k;
+    const int c = cell_of(e0, l, m, i, j, k);
+    Q[m * LP + l] = __ldg(L.ip[D] + c);
+    if (b_early) S[m * LP + l] = b[c];
   }
-  float* Sp = S + (p * 8) * 32 + lane;
-  Sp[0 * 32] = yf; Sp[1 * 32] = yl; Sp[2 * 32] = vf; Sp[3 * 32] = vl;
-  Sp[4 * 32] = wf; Sp[5 * 32] = wl; Sp[6 * 32] = lext; Sp[7 * 32] = uext;
-  __syncthreads();
-  // 3. boundary unknowns X_q = (a_q, b_q) (first, last row of segment q):
-  //    A_q X_{q-1} + X_q + C_q X_{q+1} = Y_q, A_q = lext_q [0 v_f; 0 v_l],
-  //    C_q = uext_q [w_f 0; w_l 0]; block elimination, then back-substitution
-  if (p == 0 && valid) {
-    float Ch[8][4], Yh[8][2];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      if (q < P) {
-        const float* Sq = S + (q * 8) * 32 + lane;
-        const float qyf = Sq[0], qyl = Sq[32], qvf = Sq[64], qvl = Sq[96];
-        const float qwf = Sq[128], qwl = Sq[160], ql = Sq[192], qu = Sq[224];
-        // B = I - A_q Ch_{q-1}; A_q has only a second column (lext v_f, lext v_l)
-        float b00 = 1.f, b01 = 0.f, b10 = 0.f, b11 = 1.f, y0 = qyf, y1 = qyl;
-        if (q > 0) {
-          const float a0 = ql * qvf, a1 = ql * qvl;        // A_q = [0 a0; 0 a1]
-          // A_q Ch = [a0 Ch[1][:]; a1 Ch[1][:]] (row 1 of Ch: entries 2, 3)
-          b00 -= a0 * Ch[q - 1][2]; b01 -= a0 * Ch[q - 1][3];
-          b10 -= a1 * Ch[q - 1][2]; b11 -= a1 * Ch[q - 1][3];
-          y0 -= a0 * Yh[q - 1][1];
-          y1 -= a1 * Yh[q - 1][1];
-        }
-        const float det = b00 * b11 - b01 * b10;
-        const float i00 = b11 / det, i01 = -b01 / det, i10 = -b10 / det, i11 = b00 / det;
-        // C_q = [c0 0; c1 0] with c0 = uext w_f, c1 = uext w_l
-        const float c0 = qu * qwf, c1 = qu * qwl;
-        Ch[q][0] = i00 * c0 + i01 * c1; Ch[q][1] = 0.f;
-        Ch[q][2] = i10 * c0 + i11 * c1; Ch[q][3] = 0.f;
-        Yh[q][0] = i00 * y0 + i01 * y1;
-        Yh[q][1] = i10 * y0 + i11 * y1;
-      }
+  tc5::pdl_wait();
+  if (!b_early) {
+#pragma unroll 4
+    for (int e0 = 0; e0 < total; e0 += kLineThreads) {
+      int l, m, i, j, k;
+      const int c = cell_of(e0, l, m, i, j, k);
+      S[m * LP + l] = b[c];
     }
-    float xa = 0.f;                  // a_{q+1}
-#pragma unroll
-    for (int q = 7; q >= 0; --q) {
-      if (q < P) {
-        const float a = Yh[q][0] - Ch[q][0] * xa;
-        const float bq = Yh[q][1] - Ch[q][2] * xa;
-        S[(q * 8 + 0) * 32 + lane] = a;     // first row of segment q
-        S[(q * 8 + 1) * 32 + lane] = bq;    // last row of segment q
-        xa = a;
-      }
-    }
+  }
+  __syncthreads();     // the last cell's entry is shared
+#pragma unroll 4
+  for (int e0 = 0; e0 < total; e0 += kLineThreads) {
+    if (e0 + tid >= total) break;
+    int l, m, i, j, k;
+    const int c = cell_of(e0, l, m, i, j, k);
+    const float wx = __ldg(L.w[0] + i), wy = __ldg(L.w[1] + j), wz = __ldg(L.w[2] + k);
+    const float xp = x[c];
+    // fluxes towards the six neighbours (t is 0 at the walls, where the
+    // clamped neighbour is the cell itself)
+    const float fx = __ldg(L.t[0] + i) * (xp - x[i > 0 ? c - 1 : c]) +
+                     __ldg(L.t[0] + i + 1) * (xp - x[i + 1 < nx ? c + 1 : c]);
+    const float fy = __ldg(L.t[1] + j) * (xp - x[j > 0 ? c - sy : c]) +
+                     __ldg(L.t[1] + j + 1) * (xp - x[j + 1 < ny ? c + sy : c]);
+    const float fz = __ldg(L.t[2] + k) * (xp - x[k > 0 ? c - sz : c]) +
+                     __ldg(L.t[2] + k + 1) * (xp - x[k + 1 < nz ? c + sz : c]);
+    const int o = m * LP + l;
+    S[o] = (S[o] - (wy * wz * fx + wx * wz * fy + wx * wy * fz)) * Q[o];
   }
   __syncthreads();
-  if (!valid) return;
-  // 4. the segment's rows from its modified right-hand side
-  const float xprev = p > 0 ? S[((p - 1) * 8 + 1) * 32 + lane] : 0.f;
-  const float xnext = p < P - 1 ? S[((p + 1) * 8 + 0) * 32 + lane] : 0.f;
-  float d = 0.f;
-  for (int m = s0; m < e0; ++m) {
-    const float lo = m > s0 ? -cross * tD[m] : 0.f;
-    float rhs = R[m * 32 + lane];
-    if (m == s0) rhs -= lext * xprev;
-    if (m == e0 - 1) rhs -= uext * xnext;
-    d = (rhs - lo * d) * Q[m * 32 + lane];
-    R[m * 32 + lane] = d;
+  if (tid < 32) {          // (missing lines hold line (0, 0)'s values)
+    const int l = tid & 15;
+    int i, j, k, c00, stride;
+    line_cell<D>(L, max(sa[l], 0), sb[l], i, j, k, c00, stride);
+    const float wa = D == 0 ? L.w[1][j] : L.w[0][i], wb = D == 2 ? L.w[1][j] : L.w[2][k];
+    solve_line(S + l, Q + l, LP, nl, wa * wb, L.t[D], tid >= 16);
   }
-  float dn = 0.f;
-  for (int m = e0 - 1; m >= s0; --m) {
-    const float up = m < e0 - 1 ? -cross * tD[m + 1] : 0.f;
-    const float del = R[m * 32 + lane] - up * Q[m * 32 + lane] * dn;
-    const int64_t c = c00 + (int64_t)m * stride;
-    x[c] += omega * del;
-    dn = del;
+  __syncthreads();
+#pragma unroll 4
+  for (int e = tid; e < total; e += kLineThreads) {
+    const int l = D == 0 ? e / nl : e % NL, m = D == 0 ? e - l * nl : e / NL;
+    const int ta = sa[l], tb = sb[l];
+    if (ta < 0) continue;
+    int i, j, k, c00, stride;
+    line_cell<D>(L, ta, tb, i, j, k, c00, stride);
+    const int c = c00 + m * stride;
+    x[c] += omega * S[m * LP + l];
   }
 }
 
 __global__ void k_resid32(LevDev L, const float* __restrict__ x, const float* __restrict__ b,
                           float* __restrict__ res) {
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < L.ncell;
-       c += (int64_t)gridDim.x * blockDim.x) {
+  for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < (unsigned)L.ncell; c += gridDim.x * blockDim.x) {
     int i, j, k;
     cell_ijk(c, L.n, i, j, k);
-    res[c] = b[c] - apply_at<float>(L, x, i, j, k, c, nullptr);
+    res[c] = b[c] - apply_at<float>(L, x, i, j, k, c);
   }
 }
 
-// bc = R res (R = P^T), per coarse cell
-__global__ void k_restrict(LevDev L, int nc0, int nc1, int nc2, const float* __restrict__ res,
-                           float* __restrict__ bc) {
-  const int64_t ncc = (int64_t)nc0 * nc1 * nc2;
+// (R res) at a coarse cell, R = P^T: four slots per axis (unused ones have
+// weight 0 and index 0), all 64 loads at once
+__device__ __forceinline__ float restricted(const LevDev& L, const float* res, int I, int J, int K) {
   const int nx = L.n[0], ny = L.n[1];
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < ncc;
-       c += (int64_t)gridDim.x * blockDim.x) {
-    const int I = (int)(c % nc0);
-    const int J = (int)((c / nc0) % nc1);
-    const int K = (int)(c / ((int64_t)nc0 * nc1));
-    float s = 0.f;
+  const int4 fx = __ldg(reinterpret_cast<const int4*>(L.rf[0]) + I);
+  const int4 fy = __ldg(reinterpret_cast<const int4*>(L.rf[1]) + J);
+  const int4 fz = __ldg(reinterpret_cast<const int4*>(L.rf[2]) + K);
+  const float4 wx = __ldg(reinterpret_cast<const float4*>(L.rw[0]) + I);
+  const float4 wy = __ldg(reinterpret_cast<const float4*>(L.rw[1]) + J);
+  const float4 wz = __ldg(reinterpret_cast<const float4*>(L.rw[2]) + K);
+  const int ky[4] = {fy.x, fy.y, fy.z, fy.w}, kz[4] = {fz.x, fz.y, fz.z, fz.w};
+  const float vy[4] = {wy.x, wy.y, wy.z, wy.w}, vz[4] = {wz.x, wz.y, wz.z, wz.w};
+  float s = 0.f;
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const float wz = L.rw[2][K * 4 + r];
-      if (wz == 0.f) continue;
-      const int k = L.rf[2][K * 4 + r];
+  for (int r = 0; r < 4; ++r)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float wy = L.rw[1][J * 4 + q];
-        if (wy == 0.f) continue;
-        const int j = L.rf[1][J * 4 + q];
-        const float* row = res + ((int64_t)k * ny + j) * nx;
-        float sx = 0.f;
-#pragma unroll
-        for (int p = 0; p < 4; ++p) sx += L.rw[0][I * 4 + p] * row[L.rf[0][I * 4 + p]];
-        s += wz * wy * sx;
-      }
+    for (int q = 0; q < 4; ++q) {
+      const float* row = res + (kz[r] * ny + ky[q]) * nx;
+      s += vz[r] * vy[q] * (wx.x * row[fx.x] + wx.y * row[fx.y] + wx.z * row[fx.z] + wx.w * row[fx.w]);
     }
+  return s;
+}
+
+// bc = R res, per coarse cell; the coarse iterate starts at zero
+__global__ void k_restrict(LevDev L, int nc0, int nc1, int nc2, const float* __restrict__ res,
+                           float* __restrict__ bc, float* __restrict__ xc) {
+  const int nc[3] = {nc0, nc1, nc2};
+  for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < (unsigned)(nc0 * nc1 * nc2);
+       c += gridDim.x * blockDim.x) {
+    int I, J, K;
+    cell_ijk(c, nc, I, J, K);
+    const float s = restricted(L, res, I, J, K);
     bc[c] = s;
+    xc[c] = 0.f;
   }
+}
+
+// (P xc) at a fine cell
+__device__ __forceinline__ float prolonged(const LevDev& L, int nc0, int nc1, const float* xc, int i, int j,
+                                           int k) {
+  const int I = __ldg(L.pc0[0] + i), J = __ldg(L.pc0[1] + j), K = __ldg(L.pc0[2] + k);
+  const float a = __ldg(L.pw1[0] + i), b = __ldg(L.pw1[1] + j), g = __ldg(L.pw1[2] + k);
+  const int I1 = a != 0.f ? I + 1 : I, J1 = b != 0.f ? J + 1 : J, K1 = g != 0.f ? K + 1 : K;
+  auto at = [&](int kk, int jj, int ii) { return xc[(kk * nc1 + jj) * nc0 + ii]; };
+  const float v00 = (1.f - a) * at(K, J, I) + a * at(K, J, I1);
+  const float v01 = (1.f - a) * at(K, J1, I) + a * at(K, J1, I1);
+  const float v10 = (1.f - a) * at(K1, J, I) + a * at(K1, J, I1);
+  const float v11 = (1.f - a) * at(K1, J1, I) + a * at(K1, J1, I1);
+  return (1.f - g) * ((1.f - b) * v00 + b * v01) + g * ((1.f - b) * v10 + b * v11);
 }
 
 // x += P xc, per fine cell
 __global__ void k_prolong_add(LevDev L, int nc0, int nc1, const float* __restrict__ xc,
                               float* __restrict__ x) {
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < L.ncell;
-       c += (int64_t)gridDim.x * blockDim.x) {
+  for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < (unsigned)L.ncell; c += gridDim.x * blockDim.x) {
     int i, j, k;
     cell_ijk(c, L.n, i, j, k);
-    const int I = L.pc0[0][i], J = L.pc0[1][j], K = L.pc0[2][k];
-    const float a = L.pw1[0][i], bq = L.pw1[1][j], g = L.pw1[2][k];
-    const int I1 = a != 0.f ? I + 1 : I, J1 = bq != 0.f ? J + 1 : J, K1 = g != 0.f ? K + 1 : K;
-    auto at = [&](int kk, int jj, int ii) { return xc[((int64_t)kk * nc1 + jj) * nc0 + ii]; };
-    const float v00 = (1.f - a) * at(K, J, I) + a * at(K, J, I1);
-    const float v01 = (1.f - a) * at(K, J1, I) + a * at(K, J1, I1);
-    const float v10 = (1.f - a) * at(K1, J, I) + a * at(K1, J, I1);
-    const float v11 = (1.f - a) * at(K1, J1, I) + a * at(K1, J1, I1);
-    x[c] += (1.f - g) * ((1.f - bq) * v00 + bq * v01) + g * ((1.f - bq) * v10 + bq * v11);
+    x[c] += prolonged(L, nc0, nc1, xc, i, j, k);
   }
 }
 
-// exact coarsest solve x = E Lambda^+ E^T b (3-D Kronecker), one block
-__global__ void k_coarse(CoarseDev C, const float* __restrict__ b, float* __restrict__ x) {
-  __shared__ float bh[kCoarseMax * kCoarseMax * kCoarseMax];
-  const int nx = C.n[0], ny = C.n[1], nz = C.n[2];
-  const int nc = nx * ny * nz;
-  const int t = threadIdx.x;
-  if (t < nc) {              // bh[c,b,a] = sum E_x[i][a] E_y[j][b] E_z[k][c] b[k][j][i] / lam
-    const int a = t % nx, bb = (t / nx) % ny, cc = t / (nx * ny);
-    float s = 0.f;
-    for (int k = 0; k < nz; ++k)
-      for (int j = 0; j < ny; ++j)
-        for (int i = 0; i < nx; ++i)
-          s += C.E[0][i * nx + a] * C.E[1][j * ny + bb] * C.E[2][k * nz + cc] *
-               b[(k * ny + j) * nx + i];
-    const float lam = C.lam[0][a] + C.lam[1][bb] + C.lam[2][cc];
-    bh[t] = lam > 0.f ? s / lam : 0.f;
+// Exact solve x = E Lambda^+ E^T b (3-D Kronecker) of the first level whose
+// axes have at most 32 cells, in one block and in place in shared memory: six
+// passes of dense transforms along the axes, one line per thread, its results
+// in registers, the rows of the eigenbasis broadcast four at a time.  It stands
+// in for the rest of the hierarchy below that level: as launches, a V-cycle
+// over 25^3, 13^3, 7^3 and 4^3 cells took 230 us of launch and chain latency
+// (97 us as one block from 13^3 down, with barriers for launches); this takes
+// 42 us for 25^3 (cold caches; one SM's multiply-adds alone 11 us) and saves a
+// quarter of the iterations (39 -> 29 at 100^3 to 1e-12).
+constexpr int kExactMax = 32;          // cells per axis
+constexpr int kExactThreads = 1024;
+
+template <int NM>
+__global__ void __launch_bounds__(kExactThreads) k_exact(CoarseDev C, const float* __restrict__ b,
+                                                         float* __restrict__ x) {
+  extern __shared__ __align__(16) float sm[];
+  const int tid = threadIdx.x;
+  tc5::pdl_trigger();
+  const int n[3] = {C.n[0], C.n[1], C.n[2]};
+  const int px = n[0] | 1;             // odd pitch: x-lines of a warp fall in different banks
+  float* E = sm;                       // [axis][forward, inverse][in][out], NM x NM each
+  float* a = sm + 6 * NM * NM;
+  for (int e = tid; e < 6 * NM * NM; e += kExactThreads) {
+    const int ax = e / (2 * NM * NM), inv = e / (NM * NM) & 1, i = e / NM % NM, o = e % NM, m = n[ax];
+    E[e] = i < m && o < m ? __ldg(C.E[ax] + (inv ? o * m + i : i * m + o)) : 0.f;
+  }
+  tc5::pdl_wait();
+  const int nc = n[0] * n[1] * n[2];
+  for (int c = tid; c < nc; c += kExactThreads) {
+    int i, j, k;
+    cell_ijk(c, C.n, i, j, k);
+    a[(k * n[1] + j) * px + i] = b[c];
   }
   __syncthreads();
-  if (t < nc) {
-    const int i = t % nx, j = (t / nx) % ny, k = t / (nx * ny);
-    float s = 0.f;
-    for (int cc = 0; cc < nz; ++cc)
-      for (int bb = 0; bb < ny; ++bb)
-        for (int a = 0; a < nx; ++a)
-          s += C.E[0][i * nx + a] * C.E[1][j * ny + bb] * C.E[2][k * nz + cc] *
-               bh[(cc * ny + bb) * nx + a];
-    x[t] = s;
+#pragma unroll 1
+  for (int s = 0; s < 6; ++s) {        // x, y, z forward; z, y, x back
+    const int ax = s < 3 ? s : 5 - s;
+    const int m = n[ax], la = ax == 0 ? n[1] : n[0], lb = ax == 2 ? n[1] : n[2];
+    const float* Es = E + (2 * ax + (s >= 3)) * NM * NM;
+    if (tid < la * lb) {
+      const int q = tid / la, p = tid - q * la;
+      const int stride = ax == 0 ? 1 : ax == 1 ? px : n[1] * px;
+      float* line = a + (ax == 0 ? tid * px : ax == 1 ? q * n[1] * px + p : q * px + p);
+      float acc[NM];
+#pragma unroll
+      for (int o = 0; o < NM; ++o) acc[o] = 0.f;
+#pragma unroll 2
+      for (int i = 0; i < m; ++i) {
+        const float v = line[i * stride];
+#pragma unroll
+        for (int o = 0; o < NM; o += 4) {
+          const float4 w = *reinterpret_cast<const float4*>(Es + i * NM + o);
+          acc[o] = fmaf(v, w.x, acc[o]);
+          acc[o + 1] = fmaf(v, w.y, acc[o + 1]);
+          acc[o + 2] = fmaf(v, w.z, acc[o + 2]);
+          acc[o + 3] = fmaf(v, w.w, acc[o + 3]);
+        }
+      }
+      if (s == 2) {                    // z forward: p = mode along x, q along y
+        const float l2 = __ldg(C.lam[0] + p) + __ldg(C.lam[1] + q);
+#pragma unroll
+        for (int o = 0; o < NM; ++o) {
+          const float l = o < m ? l2 + __ldg(C.lam[2] + o) : 0.f;
+          acc[o] = l > 0.f ? acc[o] / l : 0.f;
+        }
+      }
+#pragma unroll
+      for (int o = 0; o < NM; ++o)
+        if (o < m) line[o * stride] = acc[o];
+    }
+    __syncthreads();
+  }
+  for (int c = tid; c < nc; c += kExactThreads) {
+    int i, j, k;
+    cell_ijk(c, C.n, i, j, k);
+    x[c] = a[(k * n[1] + j) * px + i];
   }
 }
 
-__global__ void k_round_cells(int64_t n, const double* __restrict__ in, float* __restrict__ out) {
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-       c += (int64_t)gridDim.x * blockDim.x)
-    out[c] = (float)in[c];
-}
-
-__global__ void k_widen_cells(int64_t n, const float* __restrict__ in, double* __restrict__ out) {
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-       c += (int64_t)gridDim.x * blockDim.x)
-    out[c] = (double)in[c];
+inline size_t exact_smem(const int n[3], int NM) {
+  return sizeof(float) * ((size_t)6 * NM * NM + (size_t)(n[0] | 1) * n[1] * n[2]);
 }
 
 // ---------------------------------------------------------- float64 CG part --
 // scalar slots of the CG recurrences (device)
-enum { S_RHO = 0, S_PQ, S_ALPHA, S_RR, S_RZ, S_RZO, S_BETA, S_VR, S_BB, S_VPHI, S_N };
+enum { S_RHO = 0, S_PQ, S_ALPHA, S_RR, S_RZ, S_RZO, S_BETA, S_VR, S_BB, S_VPHI, S_IT, S_N };
+
+// one solve's arguments, read by the kernels of the iteration graph
+struct MgCall {
+  double* phi;
+  double rtol;
+  int max_iter;
+};
+
+// partial sums of a reduction and the count of blocks that have delivered
+struct Reduce {
+  double* part;
+  unsigned* ticket;
+  double* s;
+};
 
 __device__ __forceinline__ double block_sum(double v, double* sh) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -595,168 +565,205 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return s;   // valid in thread 0
 }
 
-__device__ __forceinline__ double vol(const Fine64& F, int64_t c) {
+// Sums a (and b) over the grid: every block delivers its partial sums, the
+// last one adds them in a fixed order and returns true in its thread 0 with
+// the totals in a, b.
+template <int NV>
+__device__ __forceinline__ bool grid_sum(const Reduce& R, double& a, double& b, double* sh) {
+  __shared__ unsigned last;
+  const int nb = gridDim.x * gridDim.y, bid = blockIdx.y * gridDim.x + blockIdx.x;
+  a = block_sum(a, sh);
+  if (NV > 1) b = block_sum(b, sh);
+  if (threadIdx.x == 0) {
+    __stcg(R.part + NV * bid, a);
+    if (NV > 1) __stcg(R.part + NV * bid + 1, b);
+    __threadfence();
+    last = atomicAdd(R.ticket, 1u);
+  }
+  __syncthreads();
+  if (last != (unsigned)nb - 1) return false;
+  __threadfence();
+  a = b = 0.0;
+  for (int q = threadIdx.x; q < nb; q += blockDim.x) {
+    a += __ldcg(R.part + NV * q);
+    if (NV > 1) b += __ldcg(R.part + NV * q + 1);
+  }
+  a = block_sum(a, sh);
+  if (NV > 1) b = block_sum(b, sh);
+  if (threadIdx.x != 0) return false;
+  *R.ticket = 0;
+  return true;
+}
+
+__device__ __forceinline__ double vol(const Fine64& F, unsigned c) {
   int i, j, k;
   cell_ijk(c, F.n, i, j, k);
   return F.w[0][i] * F.w[1][j] * F.w[2][k];
 }
 
-// part[block] = sum V r
-__global__ void k_sum_vr(Fine64 F, const double* __restrict__ r, double* __restrict__ part) {
+// s[dst] = sum V r
+__global__ void k_sum_vr(Fine64 F, const double* __restrict__ r, Reduce R, int dst) {
   __shared__ double sh[32];
-  double s = 0.0;
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < F.ncell;
-       c += (int64_t)gridDim.x * blockDim.x)
+  double s = 0.0, u = 0.0;
+  for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < (unsigned)F.ncell; c += gridDim.x * blockDim.x)
     s += vol(F, c) * r[c];
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
+  if (grid_sum<1>(R, s, u, sh)) R.s[dst] = s;
 }
 
-// b = -V (r - c), c = S_VR / vtot; rcg = b (phi = 0) or b - A phi (guess);
-// part[block] = sum b^2
-__global__ void k_rhs(Fine64 F, const double* __restrict__ r, const double* __restrict__ s,
-                      double vtot, const double* __restrict__ phi, double* __restrict__ rcg,
-                      double* __restrict__ part) {
+// b = -V (r - c), c = S_VR / vtot; rcg = b (phi = 0) or b - A phi (guess), its
+// float32 copy for the first V-cycle, whose iterate and the previous
+// preconditioned residual start at zero; |b|^2 and |rcg|^2
+__global__ void k_rhs(Fine64 F, const double* __restrict__ r, double vtot, const double* __restrict__ phi,
+                      double* __restrict__ rcg, float* __restrict__ b32, float* __restrict__ x32,
+                      float* __restrict__ zo32, Reduce R) {
   __shared__ double sh[32];
-  const double cm = s[S_VR] / vtot;
-  double acc = 0.0;
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < F.ncell;
-       c += (int64_t)gridDim.x * blockDim.x) {
+  const double cm = R.s[S_VR] / vtot;
+  double bb = 0.0, rr = 0.0;
+  for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < (unsigned)F.ncell; c += gridDim.x * blockDim.x) {
     const double b = -vol(F, c) * (r[c] - cm);
-    acc += b * b;
+    bb += b * b;
     double v = b;
     if (phi) {
       int i, j, k;
       cell_ijk(c, F.n, i, j, k);
-      v -= apply_at<double>(F, phi, i, j, k, c, nullptr);
+      v -= apply_at<double>(F, phi, i, j, k, (int)c);
     }
+    rr += v * v;
     rcg[c] = v;
+    b32[c] = f64_round_f32(v);
+    x32[c] = 0.f;
+    zo32[c] = 0.f;
   }
-  acc = block_sum(acc, sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = acc;
+  if (grid_sum<2>(R, bb, rr, sh)) {
+    R.s[S_BB] = bb;
+    R.s[S_RR] = rr;
+    R.s[S_RHO] = 0.0;
+    R.s[S_IT] = 0.0;
+  }
 }
 
-// part2[block] = (sum r z, sum r zo)
-__global__ void k_dots2(int64_t n, const double* __restrict__ r, const double* __restrict__ z,
-                        const double* __restrict__ zo, double* __restrict__ part) {
+// whether another iteration is wanted: ||r|| > rtol ||b||, below the cap, finite
+__device__ __forceinline__ bool go_on(const double* s, const MgCall* call) {
+  const double rn = sqrt(fmax(s[S_RR], 0.0)), bn = sqrt(s[S_BB]);
+  return bn > 0.0 && isfinite(s[S_RR]) && rn > call->rtol * bn && s[S_IT] < call->max_iter;
+}
+
+__global__ void k_begin(const double* s, const MgCall* call, cudaGraphConditionalHandle h) {
+  cudaGraphSetConditional(h, go_on(s, call) ? 1u : 0u);
+}
+
+// r . z and r . z_old of the V-cycle's z = x32, then z_old = z and x32 = 0 (the
+// next cycle's start); beta = (r.z - r.z_old) / rho (0 in the first
+// iteration), rho = r . z
+__global__ void k_dots2(unsigned n, const double* __restrict__ r, float* __restrict__ x32,
+                        float* __restrict__ zo32, Reduce R) {
   __shared__ double sh[32];
   double a = 0.0, b = 0.0;
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-       c += (int64_t)gridDim.x * blockDim.x) {
+  for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
     const double rc = r[c];
-    a += rc * z[c];
-    b += rc * zo[c];
+    const float z = x32[c];
+    a += rc * f32_to_f64(z);                 // (integer conversions: the FP64 pipe converts at its own slow rate)
+    b += rc * f32_to_f64(zo32[c]);
+    zo32[c] = z;
+    x32[c] = 0.f;
   }
-  a = block_sum(a, sh);
-  b = block_sum(b, sh);
-  if (threadIdx.x == 0) {
-    part[2 * blockIdx.x] = a;
-    part[2 * blockIdx.x + 1] = b;
+  if (grid_sum<2>(R, a, b, sh)) {
+    double* s = R.s;
+    s[S_RZ] = a;
+    s[S_RZO] = b;
+    s[S_BETA] = s[S_RHO] == 0.0 ? 0.0 : (a - b) / s[S_RHO];
+    s[S_RHO] = a;
   }
-}
-
-// q = A p, part[block] = sum p q
-__global__ void k_apply64(Fine64 F, const double* __restrict__ p, double* __restrict__ q,
-                          double* __restrict__ part) {
-  __shared__ double sh[32];
-  double acc = 0.0;
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < F.ncell;
-       c += (int64_t)gridDim.x * blockDim.x) {
-    int i, j, k;
-    cell_ijk(c, F.n, i, j, k);
-    const double v = apply_at<double>(F, p, i, j, k, c, nullptr);
-    q[c] = v;
-    acc += p[c] * v;
-  }
-  acc = block_sum(acc, sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = acc;
-}
-
-// phi += alpha p, r -= alpha q, part[block] = sum r^2
-__global__ void k_cg_step(int64_t n, const double* __restrict__ s, const double* __restrict__ p,
-                          const double* __restrict__ q, double* __restrict__ phi,
-                          double* __restrict__ r, double* __restrict__ part) {
-  __shared__ double sh[32];
-  const double al = s[S_ALPHA];
-  double acc = 0.0;
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-       c += (int64_t)gridDim.x * blockDim.x) {
-    phi[c] += al * p[c];
-    const double rv = r[c] - al * q[c];
-    r[c] = rv;
-    acc += rv * rv;
-  }
-  acc = block_sum(acc, sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
 // p = z + beta p
-__global__ void k_cg_dir(int64_t n, const double* __restrict__ s, const double* __restrict__ z,
+__global__ void k_cg_dir(unsigned n, const double* __restrict__ s, const float* __restrict__ z,
                          double* __restrict__ p) {
   const double be = s[S_BETA];
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-       c += (int64_t)gridDim.x * blockDim.x)
-    p[c] = z[c] + be * p[c];
+  for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x)
+    p[c] = be == 0.0 ? f32_to_f64(z[c]) : f32_to_f64(z[c]) + be * p[c];
+}
+
+// q = A p; alpha = rho / p . q (0 unless positive).  Bound by the FP64 pipe
+// (~1 TFLOP/s): a thread marches up a chunk of planes of its column and keeps
+// the z-flux of the face above, 16 float64 instructions per cell: 41 us at 100^3
+// with cold caches, 47 us for the cell-wise form (28 us are the pipe's).
+__global__ void k_apply64(Fine64 F, const double* __restrict__ p, double* __restrict__ q, int kz, Reduce R) {
+  __shared__ double sh[32];
+  const int nx = F.n[0], ny = F.n[1], nz = F.n[2], nxy = nx * ny;
+  const int k0 = blockIdx.y * kz, k1 = min(k0 + kz, nz);
+  double acc = 0.0, u = 0.0;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nxy; t += gridDim.x * blockDim.x) {
+    const int i = t % nx, j = t / nx;
+    const double wx = F.w[0][i], wy = F.w[1][j], wxy = wx * wy;
+    const double tx0 = F.t[0][i], tx1 = F.t[0][i + 1], ty0 = F.t[1][j], ty1 = F.t[1][j + 1];
+    const int dxm = i > 0 ? 1 : 0, dxp = i + 1 < nx ? 1 : 0, dym = j > 0 ? nx : 0, dyp = j + 1 < ny ? nx : 0;
+    int c = k0 * nxy + t;
+    double pc = p[c];
+    double below = k0 > 0 ? F.t[2][k0] * (p[c - nxy] - pc) : 0.0;   // flux out of the plane below, upwards
+#pragma unroll 4
+    for (int k = k0; k < k1; ++k, c += nxy) {
+      const double pn = p[k + 1 < nz ? c + nxy : c];
+      const double wz = F.w[2][k];
+      const double fx = tx0 * (pc - p[c - dxm]) + tx1 * (pc - p[c + dxp]);
+      const double fy = ty0 * (pc - p[c - dym]) + ty1 * (pc - p[c + dyp]);
+      const double up = F.t[2][k + 1] * (pc - pn);
+      const double v = wz * (wy * fx + wx * fy) + wxy * (up - below);
+      q[c] = v;
+      acc += pc * v;
+      below = up;
+      pc = pn;
+    }
+  }
+  if (grid_sum<1>(R, acc, u, sh)) {
+    R.s[S_PQ] = acc;
+    R.s[S_ALPHA] = acc > 0.0 ? R.s[S_RHO] / acc : 0.0;
+  }
+}
+
+// phi += alpha p, r -= alpha q (and its float32 copy), |r|^2, the stop test
+__global__ void k_cg_step(unsigned n, const double* __restrict__ p, const double* __restrict__ q,
+                          const MgCall* __restrict__ call, double* __restrict__ r, float* __restrict__ b32,
+                          Reduce R, cudaGraphConditionalHandle h, int set_handle) {
+  __shared__ double sh[32];
+  const double al = R.s[S_ALPHA];
+  double* phi = call->phi;
+  double acc = 0.0, u = 0.0;
+  for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
+    phi[c] += al * p[c];
+    const double rv = r[c] - al * q[c];
+    r[c] = rv;
+    b32[c] = f64_round_f32(rv);
+    acc += rv * rv;
+  }
+  if (grid_sum<1>(R, acc, u, sh)) {
+    R.s[S_RR] = acc;
+    R.s[S_IT] += 1.0;
+    if (set_handle) cudaGraphSetConditional(h, go_on(R.s, call) ? 1u : 0u);
+  }
 }
 
 // phi -= S_VPHI / vtot
-__global__ void k_sub_mean(int64_t n, const double* __restrict__ s, double vtot,
-                           double* __restrict__ phi) {
+__global__ void k_sub_mean(unsigned n, const double* __restrict__ s, double vtot, double* __restrict__ phi) {
   const double m = s[S_VPHI] / vtot;
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-       c += (int64_t)gridDim.x * blockDim.x)
-    phi[c] -= m;
-}
-
-// one block: reduce the partials in a fixed order and run the scalar step
-//   op 0: s[dst] = sum
-//   op 1: (r z, r zo) pairs; beta = first ? 0 : (rz - rzo) / rho; rho = rz
-//   op 2: s[S_PQ] = sum; alpha = rho / pq (0 if pq <= 0)
-enum { OP_STORE = 0, OP_BETA = 1, OP_ALPHA = 2 };
-__global__ void k_finalize(const double* __restrict__ part, int nblk, int op, int dst, int first,
-                           double* __restrict__ s) {
-  __shared__ double sh[32];
-  double a = 0.0, b = 0.0;
-  for (int q = threadIdx.x; q < nblk; q += blockDim.x) {
-    if (op == OP_BETA) {
-      a += part[2 * q];
-      b += part[2 * q + 1];
-    } else {
-      a += part[q];
-    }
-  }
-  a = block_sum(a, sh);
-  if (op == OP_BETA) b = block_sum(b, sh);
-  if (threadIdx.x != 0) return;
-  if (op == OP_STORE) {
-    s[dst] = a;
-  } else if (op == OP_BETA) {
-    s[S_RZ] = a;
-    s[S_RZO] = b;
-    s[S_BETA] = first || s[S_RHO] == 0.0 ? 0.0 : (a - b) / s[S_RHO];
-    s[S_RHO] = a;
-  } else {
-    s[S_PQ] = a;
-    s[S_ALPHA] = a > 0.0 ? s[S_RHO] / a : 0.0;
-  }
+  for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) phi[c] -= m;
 }
 
 // ------------------------------------------------------------- the state --
 struct MgLevelHost {
   Axis1D ax[3];
   LevDev dev;
-  float* x[2] = {nullptr, nullptr};
+  float* x = nullptr;
   float* b = nullptr;
   float* res = nullptr;
-  float* cb = nullptr;
-  float* db = nullptr;
-  int cur = 0;      // which x holds the level's iterate
+  float* ip[3] = {nullptr, nullptr, nullptr};
 };
 
 }  // namespace
 
 struct MgState {
   int nlev = 0;
+  int exact = 0;              // the level that k_exact solves
   MgLevelHost lev[kMgMaxLevels];
   Fine64 fine;
   CoarseDev coarse;
@@ -764,15 +771,25 @@ struct MgState {
   void* d_tab = nullptr;      // 1-D tables of all levels (floats, ints, doubles)
   void* d_work = nullptr;     // level arrays
   double* r = nullptr;        // CG vectors (float64, n_cell each)
-  double* z[2] = {nullptr, nullptr};
   double* p = nullptr;
   double* q = nullptr;
-  double* part = nullptr;     // 2 x kRedBlocks
-  double* s = nullptr;        // S_N scalars
-  double* h_s = nullptr;      // pinned mirror
+  float* zo = nullptr;        // the previous preconditioned residual
+  Reduce red = {};            // 2 x kRedBlocks partials, S_N scalars
+  MgCall* call = nullptr;     // device copy of the running solve's arguments
+  struct Host {               // pinned
+    double s[S_N];
+    MgCall call;
+  }* h = nullptr;
+  // the captured iteration for (nu, omega)
+  int nu = 0;
+  float omega = 0.f;
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
 };
 
 namespace {
+
+constexpr size_t kLineSmemMax = 200 * 1024;
 
 int blocks_for(int64_t n, int t = 256) {
   int64_t b = (n + t - 1) / t;
@@ -810,12 +827,14 @@ fv_status build_mg(fv_grid* g) {
         restriction(c0, w1, c.n, rf, rw);
         o.pw1 = tf.size();
         for (double v : w1) tf.push_back((float)v);
+        while (tf.size() % 4) tf.push_back(0.f);   // four slots per coarse cell: one 16-byte load
+        while (ti.size() % 4) ti.push_back(0);
         o.rw = tf.size();
         for (double v : rw) tf.push_back((float)v);
-        o.pc0 = ti.size();
-        ti.insert(ti.end(), c0.begin(), c0.end());
         o.rf = ti.size();
         ti.insert(ti.end(), rf.begin(), rf.end());
+        o.pc0 = ti.size();
+        ti.insert(ti.end(), c0.begin(), c0.end());
       } else {
         o.pw1 = o.rw = o.pc0 = o.rf = 0;
       }
@@ -828,9 +847,13 @@ fv_status build_mg(fv_grid* g) {
     t64[d] = td.size();
     td.insert(td.end(), M->lev[0].ax[d].t.begin(), M->lev[0].ax[d].t.end());
   }
-  // coarsest level: W-orthonormal eigenvectors of K_d E = W_d E Lambda
+  // the exactly solved level: W-orthonormal eigenvectors of K_d E = W_d E Lambda
   size_t cE[3], cL[3];
-  const int lc = M->nlev - 1;
+  M->exact = 0;
+  while (std::max(M->lev[M->exact].ax[0].n, std::max(M->lev[M->exact].ax[1].n, M->lev[M->exact].ax[2].n)) >
+         kExactMax)
+    ++M->exact;
+  const int lc = M->exact;
   for (int d = 0; d < 3; ++d) {
     const Axis1D& a = M->lev[lc].ax[d];
     const int n = a.n;
@@ -866,7 +889,7 @@ fv_status build_mg(fv_grid* g) {
   const float* F = (const float*)base;
   const int* I = (const int*)(base + oi);
   const double* Dd = (const double*)(base + od);
-  // level arrays: x0, x1, b, res, cb, db per level
+  // level arrays: x, b, res and the pivots of three directions per level
   size_t cells = 0;
   for (int l = 0; l < M->nlev; ++l) {
     int64_t nc = 1;
@@ -892,12 +915,14 @@ fv_status build_mg(fv_grid* g) {
     }
     v.ncell = nc;
     const size_t stride = (size_t)(nc + 63) / 64 * 64;
-    H.x[0] = wp; wp += stride;
-    H.x[1] = wp; wp += stride;
+    H.x = wp; wp += stride;
     H.b = wp; wp += stride;
     H.res = wp; wp += stride;
-    H.cb = wp; wp += stride;
-    H.db = wp; wp += stride;
+    for (int d = 0; d < 3; ++d) {
+      H.ip[d] = wp;
+      v.ip[d] = wp;
+      wp += stride;
+    }
   }
   for (int d = 0; d < 3; ++d) {
     M->fine.n[d] = g->n[d];
@@ -911,33 +936,46 @@ fv_status build_mg(fv_grid* g) {
   M->vtot = 1.0;
   for (int d = 0; d < 3; ++d) M->vtot *= g->h_x[d].back() - g->h_x[d].front();
   const size_t nb = (size_t)g->ncell * sizeof(double);
-  double* cg = nullptr;
-  FV_CUDA(cudaMalloc((void**)&cg, 5 * nb + (2 * kRedBlocks + S_N) * sizeof(double)));
-  M->r = cg;
-  M->z[0] = cg + g->ncell;
-  M->z[1] = cg + 2 * g->ncell;
-  M->p = cg + 3 * g->ncell;
-  M->q = cg + 4 * g->ncell;
-  M->part = cg + 5 * g->ncell;
-  M->s = M->part + 2 * kRedBlocks;
-  FV_CUDA(cudaMallocHost((void**)&M->h_s, S_N * sizeof(double)));
+  const size_t tail = (2 * kRedBlocks + S_N) * sizeof(double) + 256 + sizeof(MgCall);
+  char* cg = nullptr;
+  FV_CUDA(cudaMalloc((void**)&cg, 3 * nb + tail + (size_t)g->ncell * sizeof(float)));
+  M->r = (double*)cg;
+  M->p = M->r + g->ncell;
+  M->q = M->p + g->ncell;
+  M->red.part = M->q + g->ncell;
+  M->red.s = M->red.part + 2 * kRedBlocks;
+  M->call = (MgCall*)(M->red.s + S_N);
+  M->red.ticket = (unsigned*)((char*)M->call + sizeof(MgCall));
+  M->zo = (float*)(cg + 3 * nb + tail);
+  FV_CUDA(cudaMemset(M->red.part, 0, tail));
+  FV_CUDA(cudaMallocHost((void**)&M->h, sizeof(*M->h)));
+  for (int l = 0; l < M->exact; ++l) {
+    const MgLevelHost& H = M->lev[l];
+    const LevDev& v = H.dev;
+    auto blocks = [](int lines) { return (lines + 127) / 128; };
+    k_pivots<0><<<blocks(v.n[1] * v.n[2]), 128, 0, g->stream>>>(v, H.ip[0]);
+    k_pivots<1><<<blocks(v.n[0] * v.n[2]), 128, 0, g->stream>>>(v, H.ip[1]);
+    k_pivots<2><<<blocks(v.n[0] * v.n[1]), 128, 0, g->stream>>>(v, H.ip[2]);
+    FV_CHECK_LAUNCH();
+  }
   FV_CUDA(cudaDeviceSynchronize());
   return FV_OK;
 }
 
-// lines of at most this many cells take the partitioned kernel (its shared
-// memory grows with the line)
-constexpr int kPartMaxLine = 640;
+// shared memory of a line kernel for lines of nl cells
+size_t line_smem(int nl) { return sizeof(float) * (size_t)2 * nl * (kLines + 1); }
 
-size_t part_smem(int nl, int P) { return sizeof(float) * ((size_t)2 * nl * 32 + (size_t)P * 8 * 32); }
-
-fv_status set_part_attributes() {
+fv_status set_line_attributes() {
   static bool done = false;
   if (!done) {
-    const int bytes = (int)part_smem(kPartMaxLine, 8);
-    FV_CUDA(cudaFuncSetAttribute(k_line_part<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    FV_CUDA(cudaFuncSetAttribute(k_line_part<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    FV_CUDA(cudaFuncSetAttribute(k_line_part<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    const void* k[3] = {(const void*)k_line<0>, (const void*)k_line<1>, (const void*)k_line<2>};
+    for (const void* f : k)
+      FV_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLineSmemMax));
+    const int n32[3] = {32, 32, 32};
+    const void* e[5] = {(const void*)k_exact<16>, (const void*)k_exact<20>, (const void*)k_exact<24>,
+                        (const void*)k_exact<28>, (const void*)k_exact<32>};
+    for (const void* f : e)
+      FV_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)exact_smem(n32, 32)));
     done = true;
   }
   return FV_OK;
@@ -951,64 +989,149 @@ fv_status set_part_attributes() {
     FV_CHECK_LAUNCH();                \
   } while (0)
 
-// one V-cycle on level l: lev[l].b -> lev[l].x[cur] (zero start)
+fv_status line_sweep(const fv_grid* g, const MgLevelHost& H, int D, int color, float omega, bool b_early,
+                     cudaStream_t st) {
+  const LevDev& L = H.dev;
+  const int na = D == 0 ? L.n[1] : L.n[0], nb = D == 2 ? L.n[1] : L.n[2];
+  const int nblk = ((na + 1) / 2 * nb + kLines - 1) / kLines;
+  const size_t sm = line_smem(L.n[D]);
+  void (*kern)(LevDev, float*, const float*, float, int, int) =
+      D == 0 ? k_line<0> : D == 1 ? k_line<1> : k_line<2>;
+  LaunchScope ls_(g, FV_K_MG_SMOOTH);
+  FV_CUDA(tc5::launch_pdl(kern, dim3(nblk), dim3(kLineThreads), sm, st, L, H.x, (const float*)H.b, omega, color,
+                          b_early ? 1 : 0));
+  return FV_OK;
+}
+
+// one V-cycle on level l: lev[l].b -> lev[l].x (which starts at zero)
 fv_status vcycle(const fv_grid* g, MgState* M, int l, int nu, float omega, cudaStream_t st) {
   MgLevelHost& H = M->lev[l];
   const LevDev& L = H.dev;
-  if (l == M->nlev - 1) {
-    MG_LAUNCH(FV_K_MG_OTHER, k_coarse<<<1, 64, 0, st>>>(M->coarse, H.b, H.x[0]));
-    H.cur = 0;
+  if (l == M->exact) {
+    const int m = std::max(L.n[0], std::max(L.n[1], L.n[2]));
+    LaunchScope ls_(g, FV_K_MG_OTHER);
+    auto run = [&](void (*kern)(CoarseDev, const float*, float*), int NM) {
+      return tc5::launch_pdl(kern, dim3(1), dim3(kExactThreads), exact_smem(L.n, NM), st, M->coarse,
+                             (const float*)H.b, H.x);
+    };
+    FV_CUDA(m <= 16 ? run(k_exact<16>, 16) : m <= 20 ? run(k_exact<20>, 20) : m <= 24 ? run(k_exact<24>, 24)
+            : m <= 28 ? run(k_exact<28>, 28) : run(k_exact<32>, 32));
     return FV_OK;
   }
-  FV_CUDA(cudaMemsetAsync(H.x[0], 0, L.ncell * sizeof(float), st));
-  float* x = H.x[0];
-  auto sweep = [&](int D, int color) -> fv_status {
-    const int na = D == 0 ? L.n[1] : L.n[0];
-    const int nb = D == 2 ? L.n[1] : L.n[2];
-    const int64_t nlines = (int64_t)((na + 1) / 2) * nb;
-    const int nl = L.n[D];
-    if (nl <= kPartMaxLine) {     // lines split over P warps, 32 lines per block
-      // segments of >= 4 rows: short chains on the coarse levels too
-      const int P = std::max(1, std::min(8, nl / 4));
-      const int nblk = (int)((nlines + 31) / 32);
-      const size_t sm = part_smem(nl, P);
-      if (D == 0) MG_LAUNCH(FV_K_MG_SMOOTH, k_line_part<0><<<nblk, 32 * P, sm, st>>>(L, x, H.b, omega, color, P));
-      else if (D == 1) MG_LAUNCH(FV_K_MG_SMOOTH, k_line_part<1><<<nblk, 32 * P, sm, st>>>(L, x, H.b, omega, color, P));
-      else MG_LAUNCH(FV_K_MG_SMOOTH, k_line_part<2><<<nblk, 32 * P, sm, st>>>(L, x, H.b, omega, color, P));
-      return FV_OK;
-    }
-    const int nblk = (int)((nlines + 127) / 128);
-    if (D == 0) MG_LAUNCH(FV_K_MG_SMOOTH, k_line<0><<<nblk, 128, 0, st>>>(L, x, H.b, H.cb, H.db, omega, color));
-    else if (D == 1) MG_LAUNCH(FV_K_MG_SMOOTH, k_line<1><<<nblk, 128, 0, st>>>(L, x, H.b, H.cb, H.db, omega, color));
-    else MG_LAUNCH(FV_K_MG_SMOOTH, k_line<2><<<nblk, 128, 0, st>>>(L, x, H.b, H.cb, H.db, omega, color));
-    return FV_OK;
+  // 16 lines per block: at 100^3 two blocks per SM (1024 cells per line still
+  // fit one block's shared memory)
+  bool b_early = false;      // the first sweep follows the kernel that wrote b
+  auto sweep = [&](int D, int color) {
+    const fv_status r = line_sweep(g, H, D, color, omega, b_early, st);
+    b_early = true;
+    return r;
   };
   // symmetric Gauss-Seidel: x, y, z (colours 0, 1) before, the exact reverse after
   for (int s = 0; s < nu; ++s)
     for (int D = 0; D < 3; ++D)
       for (int c = 0; c < 2; ++c) FV_TRY(sweep(D, c));
   const MgLevelHost& C = M->lev[l + 1];
-  MG_LAUNCH(FV_K_MG_OTHER, k_resid32<<<blocks_for(L.ncell), 256, 0, st>>>(L, x, H.b, H.res));
-  MG_LAUNCH(FV_K_MG_OTHER, k_restrict<<<blocks_for(C.dev.ncell), 256, 0, st>>>(L, C.dev.n[0], C.dev.n[1], C.dev.n[2], H.res,
-                                                    C.b));
+  MG_LAUNCH(FV_K_MG_OTHER, k_resid32<<<blocks_for(L.ncell), 256, 0, st>>>(L, H.x, H.b, H.res));
+  MG_LAUNCH(FV_K_MG_OTHER, k_restrict<<<blocks_for(C.dev.ncell), 256, 0, st>>>(L, C.dev.n[0], C.dev.n[1], C.dev.n[2],
+                                                                             H.res, C.b, C.x));
   FV_TRY(vcycle(g, M, l + 1, nu, omega, st));
-  MG_LAUNCH(FV_K_MG_OTHER, k_prolong_add<<<blocks_for(L.ncell), 256, 0, st>>>(L, C.dev.n[0], C.dev.n[1], C.x[C.cur],
-                                                     x));
+  MG_LAUNCH(FV_K_MG_OTHER, k_prolong_add<<<blocks_for(L.ncell), 256, 0, st>>>(L, C.dev.n[0], C.dev.n[1], C.x, H.x));
   for (int s = 0; s < nu; ++s)
     for (int D = 2; D >= 0; --D)
       for (int c = 1; c >= 0; --c) FV_TRY(sweep(D, c));
-  H.cur = 0;
   return FV_OK;
 }
 
-// z = M^-1 r: round r into level 0, one V-cycle, widen
-fv_status precondition(fv_grid* g, MgState* M, const double* r, double* z, int nu, float omega) {
-  cudaStream_t st = g->stream;
-  FV_TRY(set_part_attributes());
+// one conjugate-gradient iteration on the stream st; h: the WHILE node's
+// handle when captured
+fv_status iteration(const fv_grid* g, MgState* M, int nu, float omega, cudaStream_t st,
+                    const cudaGraphConditionalHandle* h) {
+  const unsigned n = (unsigned)g->ncell;
   MgLevelHost& H = M->lev[0];
-  MG_LAUNCH(FV_K_MG_OTHER, k_round_cells<<<blocks_for(g->ncell), 256, 0, st>>>(g->ncell, r, H.b));
   FV_TRY(vcycle(g, M, 0, nu, omega, st));
-  MG_LAUNCH(FV_K_MG_OTHER, k_widen_cells<<<blocks_for(g->ncell), 256, 0, st>>>(g->ncell, H.x[H.cur], z));
+  MG_LAUNCH(FV_K_MG_OTHER, k_dots2<<<kRedBlocks, kRedThreads, 0, st>>>(n, M->r, H.x, M->zo, M->red));
+  MG_LAUNCH(FV_K_MG_OTHER, k_cg_dir<<<blocks_for(n), 256, 0, st>>>(n, M->red.s, M->zo, M->p));
+  {
+    // about kRedBlocks blocks over plane tiles x chunks of planes
+    const int tiles = std::min(kRedBlocks, (g->n[0] * g->n[1] + kRedThreads - 1) / kRedThreads);
+    const int chunks = std::min(g->n[2], std::max(1, kRedBlocks / tiles));
+    const int kz = (g->n[2] + chunks - 1) / chunks;
+    MG_LAUNCH(FV_K_MG_OTHER, k_apply64<<<dim3(tiles, (g->n[2] + kz - 1) / kz), kRedThreads, 0, st>>>(
+                                 M->fine, M->p, M->q, kz, M->red));
+  }
+  cudaGraphConditionalHandle hh = {};
+  if (h) hh = *h;
+  MG_LAUNCH(FV_K_MG_OTHER, k_cg_step<<<kRedBlocks, kRedThreads, 0, st>>>(n, M->p, M->q, M->call, M->r, H.b,
+                                                                       M->red, hh, h ? 1 : 0));
+  return FV_OK;
+}
+
+void drop_mg_graph(MgState* M) {
+  if (M->exec) cudaGraphExecDestroy(M->exec);
+  if (M->graph) cudaGraphDestroy(M->graph);
+  M->exec = nullptr;
+  M->graph = nullptr;
+}
+
+// The iterations as a graph: k_begin -> WHILE { iteration }
+fv_status build_mg_graph(fv_grid* g, MgState* M, int nu, float omega) {
+  drop_mg_graph(M);
+  cudaStream_t cs, bs;
+  FV_TRY(capture_streams(&cs, &bs));
+  const bool prof = g->prof_on;
+  g->prof_on = false;
+  g->capturing = true;
+  cudaGraph_t graph = nullptr;
+  bool begun = false;
+  auto capture = [&]() -> fv_status {
+    FV_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+    begun = true;
+    cudaStreamCaptureStatus cst;
+    cudaGraph_t cap;
+    const cudaGraphNode_t* deps = nullptr;
+    size_t nd = 0;
+    FV_CUDA(cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cap, &deps, nullptr, &nd));
+    cudaGraphConditionalHandle h;
+    FV_CUDA(cudaGraphConditionalHandleCreate(&h, cap, 0, cudaGraphCondAssignDefault));
+    k_begin<<<1, 1, 0, cs>>>(M->red.s, M->call, h);
+    FV_CHECK_LAUNCH();
+    FV_CUDA(cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cap, &deps, nullptr, &nd));
+    cudaGraphNodeParams cp = {};
+    cp.type = cudaGraphNodeTypeConditional;
+    cp.conditional.handle = h;
+    cp.conditional.type = cudaGraphCondTypeWhile;
+    cp.conditional.size = 1;
+    cudaGraphNode_t cnode;
+    FV_CUDA(cudaGraphAddNode(&cnode, cap, deps, nullptr, nd, &cp));
+    cudaGraph_t body = cp.conditional.phGraph_out[0];
+    FV_CUDA(cudaStreamBeginCaptureToGraph(bs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+    const fv_status s2 = iteration(g, M, nu, omega, bs, &h);
+    cudaGraph_t bg = body;
+    const cudaError_t e2 = cudaStreamEndCapture(bs, &bg);
+    FV_TRY(s2);
+    FV_CUDA(e2);
+    FV_CUDA(cudaStreamUpdateCaptureDependencies(cs, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies));
+    return FV_OK;
+  };
+  fv_status s = capture();
+  const cudaError_t ec = begun ? cudaStreamEndCapture(cs, &graph) : cudaSuccess;
+  g->prof_on = prof;
+  g->capturing = false;
+  if (s == FV_OK && ec != cudaSuccess) s = cuda_fail(ec, "cudaStreamEndCapture", __FILE__, __LINE__);
+  if (s == FV_OK) {
+    const cudaError_t ei = cudaGraphInstantiate(&M->exec, graph, 0);
+    if (ei != cudaSuccess) s = cuda_fail(ei, "cudaGraphInstantiate", __FILE__, __LINE__);
+  }
+  if (s != FV_OK) {
+    if (graph) cudaGraphDestroy(graph);
+    M->exec = nullptr;
+    drop_capture_streams();
+    (void)cudaGetLastError();
+    return s;
+  }
+  M->graph = graph;
+  M->nu = nu;
+  M->omega = omega;
   return FV_OK;
 }
 
@@ -1020,7 +1143,8 @@ void destroy_mg(fv_grid* g) {
   if (M->d_tab) cudaFree(M->d_tab);
   if (M->d_work) cudaFree(M->d_work);
   if (M->r) cudaFree(M->r);
-  if (M->h_s) cudaFreeHost(M->h_s);
+  if (M->h) cudaFreeHost(M->h);
+  drop_mg_graph(M);
   delete M;
   g->mg = nullptr;
 }
@@ -1035,62 +1159,56 @@ fv_status mg_solve(fv_grid* g, const double* r, double* phi, const double* guess
     }
   }
   MgState* M = (MgState*)g->mg;
+  FV_TRY(set_line_attributes());
   cudaStream_t st = g->stream;
-  const int64_t n = g->ncell;
+  const unsigned n = (unsigned)g->ncell;
   const int nb = kRedBlocks;
-  fv_mg_stats sv = {};
-  sv.levels = M->nlev;
+  const float omega = (float)o.omega;
+  MgLevelHost& H = M->lev[0];
   // compatible right-hand side and the initial residual
-  MG_LAUNCH(FV_K_MG_OTHER, k_sum_vr<<<nb, kRedThreads, 0, st>>>(M->fine, r, M->part));
-  MG_LAUNCH(FV_K_MG_OTHER, k_finalize<<<1, kRedThreads, 0, st>>>(M->part, nb, OP_STORE, S_VR, 0, M->s));
+  M->h->call = {phi, o.rtol, o.max_iter};
+  FV_CUDA(cudaMemcpyAsync(M->call, &M->h->call, sizeof(MgCall), cudaMemcpyHostToDevice, st));
+  MG_LAUNCH(FV_K_MG_OTHER, k_sum_vr<<<nb, kRedThreads, 0, st>>>(M->fine, r, M->red, S_VR));
   if (guess && guess != phi)
     FV_CUDA(cudaMemcpyAsync(phi, guess, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
   if (!guess) FV_CUDA(cudaMemsetAsync(phi, 0, n * sizeof(double), st));
-  MG_LAUNCH(FV_K_MG_OTHER, k_rhs<<<nb, kRedThreads, 0, st>>>(M->fine, r, M->s, M->vtot, guess ? phi : nullptr, M->r,
-                                     M->part));
-  MG_LAUNCH(FV_K_MG_OTHER, k_finalize<<<1, kRedThreads, 0, st>>>(M->part, nb, OP_STORE, S_BB, 0, M->s));
-  // the initial residual norm (guess given) for the convergence test
-  MG_LAUNCH(FV_K_MG_OTHER, k_dots2<<<nb, kRedThreads, 0, st>>>(n, M->r, M->r, M->r, M->part));
-  MG_LAUNCH(FV_K_MG_OTHER, k_finalize<<<1, kRedThreads, 0, st>>>(M->part, nb, OP_BETA, 0, 1, M->s));
-  FV_CUDA(cudaMemcpyAsync(M->h_s, M->s, S_N * sizeof(double), cudaMemcpyDeviceToHost, st));
-  FV_CUDA(cudaStreamSynchronize(st));
-  const double bnorm = std::sqrt(M->h_s[S_BB]);
-  double rnorm = std::sqrt(std::max(M->h_s[S_RZ], 0.0));
-  const float omega = (float)o.omega;
-  int it = 0, zc = 0;
-  if (bnorm > 0.0 && std::isfinite(rnorm)) {
-    while (rnorm > o.rtol * bnorm && it < o.max_iter) {
-      double* z = M->z[zc];
-      double* zo = M->z[zc ^ 1];
-      FV_TRY(precondition(g, M, M->r, z, o.nu, omega));
-      if (it == 0) FV_CUDA(cudaMemsetAsync(zo, 0, n * sizeof(double), st));
-      MG_LAUNCH(FV_K_MG_OTHER, k_dots2<<<nb, kRedThreads, 0, st>>>(n, M->r, z, zo, M->part));
-      MG_LAUNCH(FV_K_MG_OTHER, k_finalize<<<1, kRedThreads, 0, st>>>(M->part, nb, OP_BETA, 0, it == 0, M->s));
-      MG_LAUNCH(FV_K_MG_OTHER, k_cg_dir<<<blocks_for(n), 256, 0, st>>>(n, M->s, z, M->p));
-      MG_LAUNCH(FV_K_MG_OTHER, k_apply64<<<nb, kRedThreads, 0, st>>>(M->fine, M->p, M->q, M->part));
-      MG_LAUNCH(FV_K_MG_OTHER, k_finalize<<<1, kRedThreads, 0, st>>>(M->part, nb, OP_ALPHA, 0, 0, M->s));
-      MG_LAUNCH(FV_K_MG_OTHER, k_cg_step<<<nb, kRedThreads, 0, st>>>(n, M->s, M->p, M->q, phi, M->r, M->part));
-      MG_LAUNCH(FV_K_MG_OTHER, k_finalize<<<1, kRedThreads, 0, st>>>(M->part, nb, OP_STORE, S_RR, 0, M->s));
-      FV_CUDA(cudaMemcpyAsync(M->h_s, M->s, S_N * sizeof(double), cudaMemcpyDeviceToHost, st));
-      FV_CUDA(cudaStreamSynchronize(st));
-      ++it;
-      zc ^= 1;
-      rnorm = std::sqrt(std::max(M->h_s[S_RR], 0.0));
-      if (!std::isfinite(rnorm)) break;
+  MG_LAUNCH(FV_K_MG_OTHER, k_rhs<<<nb, kRedThreads, 0, st>>>(M->fine, r, M->vtot, guess ? phi : nullptr, M->r, H.b,
+                                                            H.x, M->zo, M->red));
+  auto fetch = [&]() -> fv_status {
+    FV_CUDA(cudaMemcpyAsync(M->h->s, M->red.s, S_N * sizeof(double), cudaMemcpyDeviceToHost, st));
+    FV_CUDA(cudaStreamSynchronize(st));
+    return FV_OK;
+  };
+  const double* hs = M->h->s;
+  auto rnorm = [&]() { return std::sqrt(std::max(hs[S_RR], 0.0)); };
+  if (g->use_graph && !g->prof_on) {
+    if (!M->exec || M->nu != o.nu || M->omega != omega) FV_TRY(build_mg_graph(g, M, o.nu, omega));
+    count_launch();
+    FV_CUDA(cudaGraphLaunch(M->exec, st));
+  } else {                 // launch by launch (per-kernel timing)
+    FV_TRY(fetch());
+    while (std::isfinite(hs[S_RR]) && hs[S_BB] > 0.0 && rnorm() > o.rtol * std::sqrt(hs[S_BB]) &&
+           hs[S_IT] < o.max_iter) {
+      FV_TRY(iteration(g, M, o.nu, omega, st, nullptr));
+      FV_TRY(fetch());
     }
   }
   // zero volume-weighted mean
-  MG_LAUNCH(FV_K_MG_OTHER, k_sum_vr<<<nb, kRedThreads, 0, st>>>(M->fine, phi, M->part));
-  MG_LAUNCH(FV_K_MG_OTHER, k_finalize<<<1, kRedThreads, 0, st>>>(M->part, nb, OP_STORE, S_VPHI, 0, M->s));
-  MG_LAUNCH(FV_K_MG_OTHER, k_sub_mean<<<blocks_for(n), 256, 0, st>>>(n, M->s, M->vtot, phi));
-  sv.iterations = it;
-  sv.rel_res = bnorm > 0.0 ? rnorm / bnorm : 0.0;
+  MG_LAUNCH(FV_K_MG_OTHER, k_sum_vr<<<nb, kRedThreads, 0, st>>>(M->fine, phi, M->red, S_VPHI));
+  MG_LAUNCH(FV_K_MG_OTHER, k_sub_mean<<<blocks_for(n), 256, 0, st>>>(n, M->red.s, M->vtot, phi));
+  FV_TRY(fetch());
+  const double bnorm = std::sqrt(hs[S_BB]);
+  fv_mg_stats sv = {};
+  sv.levels = M->nlev;
+  sv.iterations = (int)hs[S_IT];
+  sv.rel_res = bnorm > 0.0 ? rnorm() / bnorm : 0.0;
   if (stats) *stats = sv;
-  if (!std::isfinite(rnorm)) {
+  // (a NaN right-hand side gives a NaN norm; max() above would hide it)
+  if (!std::isfinite(hs[S_RR]) || !std::isfinite(bnorm)) {
     set_error("fv_pressure_solve_mg: NaN in the residual");
     return FV_ENAN;
   }
-  if (bnorm > 0.0 && rnorm > o.rtol * bnorm) {
+  if (bnorm > 0.0 && rnorm() > o.rtol * bnorm) {
     set_error("fv_pressure_solve_mg: no convergence within max_iter");
     return FV_ENOCONV;
   }
