@@ -32,7 +32,7 @@ def sources():
 
 
 # float-float arithmetic must see each rounding exactly as written
-EXTRA = {"fv_mixed.cu": ["-fmad=false"], "fv_pass.cu": ["-fmad=false"]}
+EXTRA = {f: ["-fmad=false"] for f in ("fv_gs.cu", "fv_mixed.cu", "fv_pass.cu")}
 
 
 def _compile(src, verbose=False):

@@ -288,7 +288,7 @@ fv_status status_error(int status) {
     case 2: set_error("SIMPLE loop reached max_pass"); return FV_ENOCONV;
     case 3: set_error("SIMPLE loop: NaN/Inf in the correction"); return FV_ENAN;
     case 4:
-      set_error("pressure transform: a bounded wait on the tensor cores gave up (device timeout)");
+      set_error("a bounded wait of a pressure transform or a Gram-Schmidt step gave up (device timeout)");
       return FV_ETIMEOUT;
     default: return FV_OK;
   }

@@ -527,6 +527,7 @@ void fv_grid_destroy(fv_grid* g) {
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (g->h_scal) cudaFreeHost(g->h_scal);
+  if (g->h_kry) cudaFreeHost(g->h_kry);
   delete g;
 }
 

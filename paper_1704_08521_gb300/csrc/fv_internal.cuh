@@ -232,6 +232,8 @@ struct fv_grid {
   double* kry = nullptr;
   int kry_cols = 0;
   double* kry_small = nullptr;   // device small-matrix area
+  unsigned long long* kry_bar = nullptr;   // barrier counter of the fused Gram-Schmidt step (in kry_small)
+  double* h_kry = nullptr;       // pinned: its coefficients and norm
   void* d_arn = nullptr;         // device Arnoldi area: the cycle's Hessenberg H, a scale
 
   // multigrid pressure solve: hierarchy, level arrays, CG vectors (first use)
@@ -373,6 +375,16 @@ fv_status unet_guess_f32(fv_unet* u, const fv_grid* g, const float* r, float* ph
 // max |x[0..n)| of a float32 array to the host (synchronises g's stream)
 fv_status absmax_f32_host(const fv_grid* g, const float* x, int64_t n, double* out);
 fv_status tpf_one_transform_f32(const fv_grid* g, int axis);
+
+// A Gram-Schmidt step as one kernel, float-float arithmetic: w against the j1
+// columns of V (float-float pairs or doubles, ldv apart), twice; coefficients
+// and norm into hcol (entries ldh apart; norm_only: the norm alone), 1 / norm
+// into *scale, w / norm into the column colf or (scale_w) into w.  h2: device
+// scratch of 260 doubles; bar: a counter zeroed once.
+bool gs_fused_ok(const fv_grid* g, int j1);
+fv_status gs_fused(const fv_grid* g, const void* V, bool pairs, int64_t ldv, int j1, double* w, double* h2,
+                   unsigned long long* bar, double* hcol, int64_t ldh, double* scale, float2* colf,
+                   bool scale_w, bool norm_only);
 
 // the largest status (1 converged, 2 pass cap, 3 NaN, 4 timeout; 0 none) of
 // the graph evaluations on g since the last call, then reset (synchronises

@@ -983,15 +983,28 @@ static fv_status ensure_krylov(fv_grid* g, int cols) {
     set_error("Krylov basis allocation failed");
     return FV_ENOMEM;
   }
-  FV_CUDA(cudaMalloc((void**)&g->kry_small, (size_t)(kMaxVec + 2) * (kMaxVec + 2) * sizeof(double)));
+  // the small-matrix area, and behind it the barrier counter of gs_fused
+  const size_t small = (size_t)(kMaxVec + 2) * (kMaxVec + 2) * sizeof(double);
+  FV_CUDA(cudaMalloc((void**)&g->kry_small, small + 256));
+  g->kry_bar = (unsigned long long*)((char*)g->kry_small + small);
+  FV_CUDA(cudaMemsetAsync(g->kry_bar, 0, 256, g->stream));
+  if (!g->h_kry) FV_CUDA(cudaMallocHost((void**)&g->h_kry, (kMaxVec + 2) * sizeof(double)));
   g->kry_cols = cols;
   return FV_OK;
 }
 
 // CGS2 of w against V[0..j] in the W-inner product; returns h (j+1) and
-// ||w||_W on the host.
+// ||w||_W on the host and leaves w / ||w||_W (w itself if that is zero).
 static fv_status cgs2(const fv_grid* g, const double* V, int j1, double* w, double* h_host,
                       double* wnorm, bool ff_arith) {
+  if (ff_arith && gs_fused_ok(g, j1)) {      // the coefficients straight into pinned memory
+    FV_TRY(gs_fused(g, V, false, g->nvel, j1, w, g->kry_small, g->kry_bar, g->h_kry, 1, nullptr, nullptr,
+                    true, false));
+    FV_CUDA(cudaStreamSynchronize(g->stream));
+    std::memcpy(h_host, g->h_kry, j1 * sizeof(double));
+    *wnorm = g->h_kry[j1];
+    return FV_OK;
+  }
   double* dh1 = g->kry_small;
   double* dh2 = g->kry_small + kMaxVec;
   double* dnn = g->kry_small + 2 * kMaxVec;
@@ -1006,35 +1019,19 @@ static fv_status cgs2(const fv_grid* g, const double* V, int j1, double* w, doub
   FV_CUDA(cudaStreamSynchronize(g->stream));
   for (int i = 0; i < j1; ++i) h_host[i] = tmp[i] + tmp[kMaxVec + i];
   *wnorm = std::sqrt(std::max(tmp[2 * kMaxVec], 0.0));
-  return FV_OK;
-}
-
-// cgs2 against a float-float basis (w stays a double vector)
-static fv_status cgs2_ffb(const fv_grid* g, const float2* Vf, int j1, double* w, double* h_host,
-                          double* wnorm) {
-  double* dh1 = g->kry_small;
-  double* dh2 = g->kry_small + kMaxVec;
-  double* dnn = g->kry_small + 2 * kMaxVec;
-  FV_TRY(ffb_dots(g, Vf, j1, w, dh1));
-  FV_TRY(ffb_update(g, w, Vf, j1, dh1, -1.0));
-  FV_TRY(ffb_dots(g, Vf, j1, w, dh2));
-  FV_TRY(ffb_update(g, w, Vf, j1, dh2, -1.0));
-  FV_TRY(vec_dots(g, w, g->nvel, 1, w, dnn, true));
-  std::vector<double> tmp(2 * kMaxVec + 1);
-  FV_CUDA(cudaMemcpyAsync(tmp.data(), g->kry_small, (2 * kMaxVec + 1) * sizeof(double),
-                          cudaMemcpyDeviceToHost, g->stream));
-  FV_CUDA(cudaStreamSynchronize(g->stream));
-  for (int i = 0; i < j1; ++i) h_host[i] = tmp[i] + tmp[kMaxVec + i];
-  *wnorm = std::sqrt(std::max(tmp[2 * kMaxVec], 0.0));
+  if (*wnorm > 0) FV_TRY(vec_axpby(g, g->nvel, 1.0 / *wnorm, w, 0.0, nullptr, w));
   return FV_OK;
 }
 
 // CGS2 of w against the first j1 basis vectors (float-float basis Vf, or the
 // FP64 basis V), the coefficients and the norm written into column `Hcol` of
-// the device Hessenberg (leading dimension ld) by k_gs_finish, *dscale =
-// 1 / norm: nothing returns to the host
-static fv_status cgs2_dev(const fv_grid* g, const float2* Vf, const double* V, int j1, double* w,
+// the device Hessenberg (leading dimension ld), w / norm stored as basis
+// column j1: nothing returns to the host.  *dscale = 1 / norm.
+static fv_status cgs2_dev(const fv_grid* g, float2* Vf, double* V, int j1, double* w,
                           double* Hcol, int ld, double* dscale, bool sub_only) {
+  if (Vf && gs_fused_ok(g, j1))
+    return gs_fused(g, Vf, true, g->nvel, j1, w, g->kry_small, g->kry_bar, Hcol, ld, dscale,
+                    Vf + (int64_t)j1 * g->nvel, false, sub_only);
   double* dh1 = g->kry_small;
   double* dh2 = g->kry_small + kMaxVec;
   double* dnn = g->kry_small + 2 * kMaxVec;
@@ -1056,18 +1053,12 @@ static fv_status cgs2_dev(const fv_grid* g, const float2* Vf, const double* V, i
     k_gs_finish<<<1, 128, 0, g->stream>>>(dh1, dh2, dnn, j1, Hcol, ld, dscale, sub_only ? 1 : 0);
   }
   FV_CHECK_LAUNCH();
-  return FV_OK;
-}
-
-// store w / norm (device scale) as basis column `col`
-static fv_status store_scaled(const fv_grid* g, const double* w, const double* dscale, float2* colf,
-                              double* cold) {
   {
     LaunchScope ls_(g, FV_K_VECTOR);
-    if (colf)
-      k_store_ff_dev<<<grid1d(g->nvel), 256, 0, g->stream>>>(g->nvel, w, dscale, colf);
+    if (Vf)
+      k_store_ff_dev<<<grid1d(g->nvel), 256, 0, g->stream>>>(g->nvel, w, dscale, Vf + (int64_t)j1 * g->nvel);
     else
-      k_scale_dev<<<grid1d(g->nvel), 256, 0, g->stream>>>(g->nvel, w, dscale, 1, cold);
+      k_scale_dev<<<grid1d(g->nvel), 256, 0, g->stream>>>(g->nvel, w, dscale, 1, V + (int64_t)j1 * g->nvel);
   }
   FV_CHECK_LAUNCH();
   return FV_OK;
@@ -1533,7 +1524,6 @@ fv_status newton_steady(fv_grid* g, double* U, double* P, const fv_newton_opts* 
         if (o.tau != 0.0) NT_TRY(vec_axpby(g, nv, 1.0, w, -o.tau, vj, w));
         double hn;
         NT_TRY(cgs2(g, V, j + 1, w, hcol.data(), &hn, cur_prec != FV_FP64));
-        if (hn > 0) NT_TRY(vec_axpby(g, nv, 1.0 / hn, w, 0.0, nullptr, w));
         for (int i = 0; i <= j; ++i) H[(size_t)i * m + j] = hcol[i];
         H[(size_t)(j + 1) * m + j] = hn;
         for (int i = 0; i < j; ++i) {
@@ -1697,7 +1687,6 @@ fv_status arnoldi_leading(const fv_grid* gc, const double* U, const double* v0, 
       FV_TRY(krylov_apply(g, nullptr, xj, w, nullptr, o.sigma, o.prec, o.simple_eps, 200, 1.0, nullptr));
       ++matvecs;
       FV_TRY(cgs2_dev(g, gs_ff ? Vf : nullptr, V, j + 1, w, dH + j, m, dsc, false));
-      FV_TRY(store_scaled(g, w, dsc, gs_ff ? Vf + (int64_t)(j + 1) * nv : nullptr, w));
     }
     FV_TRY(check_products(g, o.prec));
     FV_CUDA(cudaMemcpyAsync(H.data(), dH, (size_t)(m + 1) * m * sizeof(double), cudaMemcpyDeviceToHost,
@@ -1817,7 +1806,6 @@ fv_status arnoldi_leading(const fv_grid* gc, const double* U, const double* v0, 
                             g->stream));
     double* f = gs_ff ? ws : V + (int64_t)k * nv;
     FV_TRY(cgs2_dev(g, gs_ff ? Vf : nullptr, V, k, f, dH + (k - 1), m, dsc, true));
-    FV_TRY(store_scaled(g, f, dsc, gs_ff ? Vf + (int64_t)k * nv : nullptr, f));
   }
   set_error("arnoldi_leading: max_restarts reached");
   return FV_ENOCONV;
