@@ -352,11 +352,16 @@ fv_status xf_solve(const fv_grid* g, const float* r, float* phi, const int* skip
 // one float64 1-D transform along `axis`: by Einv (inverse = 0) or E (1)
 fv_status transform_axis_f64(const fv_grid* g, int axis, int inverse, const double* in, double* out);
 // the float64 transforms on the tensor cores (fv_oz.cu): operands (with the
-// grid), whether `axis` has them, one transform; scale: times 1 / (lam_x +
-// lam_y + lam_z) (z axis, every axis covered)
+// grid), whether `axis` has them, one transform, its results times factors
+// (y or z axis; vectors are at most 2^30 / n)
 fv_status build_oz(fv_grid* g);
 bool oz_ok(const fv_grid* g, int axis);
-fv_status oz_transform(const fv_grid* g, int axis, int inverse, bool scale, const double* in, double* out);
+struct OzScale {
+  const double* inv = nullptr;   // factors, or none
+  int da = 0, na = 0;            // na = 0: one per cell; else of entry p and index i along another axis
+                                 // (of na entries, da vectors apart) inv[i n + p]
+};
+fv_status oz_transform(const fv_grid* g, int axis, int inverse, OzScale scale, const double* in, double* out);
 // the unfused float32 transforms with the tables and eigenvalues of tp
 // (scaling by 1 / (lam_z + lam_y + lam_x); null_index -1: no null mode)
 fv_status tpf_run_f32(const fv_grid* g, const TpfDev<float>& tp, const float* r, float* phi);

@@ -142,13 +142,14 @@ struct OzArgs {
   double* out;
   const bf16b* mat;        // [K / 16][digit][128 x 16 canonical]
   const int* rexp;         // biased exponent of each row's largest entry
-  const double* inv;       // SCALE: 1 / (lam_x + lam_y + lam_z) per cell, 0 at the null mode
+  OzScale sc;              // SCALE: factors of the results
   int n;                   // rows of M = entries of a vector
   int64_t nvec, Q;         // vectors; entry k of vector v is at (v / Q) n Q + k Q + v % Q
   unsigned* fault;
 };
 
-template <bool RIGHT, bool SCALE>
+// SCALE: 0 none, 1 a factor per cell, 2 one per entry and index along another axis
+template <bool RIGHT, int SCALE>
 __global__ void __launch_bounds__(kOzThreads) k_oz(OzArgs A) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ uint64_t full[2], empty[2], ready[kOzMax / 16], done;
@@ -312,11 +313,23 @@ __global__ void __launch_bounds__(kOzThreads) k_oz(OzArgs A) {
           o[q] = join96(s1, s0, ea + eb - 2108);
           if (eb == 2047 || failed) o[q] = __longlong_as_double(0x7ff8000000000000ll);
         }
+        if (SCALE == 2) {
+          const unsigned t = (unsigned)v / (unsigned)A.sc.da;   // index along the other axis: t % na
+          int r = (int)((unsigned)v - t * A.sc.da), i = (int)(t % (unsigned)A.sc.na);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            o[q] *= __ldg(A.sc.inv + i * n + p);
+            if (++r == A.sc.da) {
+              r = 0;
+              if (++i == A.sc.na) i = 0;
+            }
+          }
+        }
         const int64_t e = RIGHT ? v * n + p : (v / A.Q) * n * A.Q + (int64_t)p * A.Q + v % A.Q;
         if (!RIGHT && (A.Q & 3) == 0) {      // four vectors of one row: two 16-byte stores
-          if (SCALE) {
-            const double2 i0 = __ldg(reinterpret_cast<const double2*>(A.inv + e));
-            const double2 i1 = __ldg(reinterpret_cast<const double2*>(A.inv + e) + 1);
+          if (SCALE == 1) {
+            const double2 i0 = __ldg(reinterpret_cast<const double2*>(A.sc.inv + e));
+            const double2 i1 = __ldg(reinterpret_cast<const double2*>(A.sc.inv + e) + 1);
             o[0] *= i0.x; o[1] *= i0.y; o[2] *= i1.x; o[3] *= i1.y;
           }
           *reinterpret_cast<double2*>(A.out + e) = make_double2(o[0], o[1]);
@@ -327,7 +340,7 @@ __global__ void __launch_bounds__(kOzThreads) k_oz(OzArgs A) {
             const int64_t w = v + q;
             if (w < A.nvec) {
               const int64_t f = RIGHT ? w * n + p : (w / A.Q) * n * A.Q + (int64_t)p * A.Q + w % A.Q;
-              A.out[f] = SCALE ? o[q] * __ldg(A.inv + f) : o[q];
+              A.out[f] = SCALE == 1 ? o[q] * __ldg(A.sc.inv + f) : o[q];
             }
           }
         }
@@ -438,19 +451,20 @@ fv_status build_oz(fv_grid* g) {
     FV_CHECK_LAUNCH();
   }
   const int cap = (int)std::max(oz_smem(112), oz_smem(kOzMax));
-  FV_CUDA(cudaFuncSetAttribute(k_oz<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-  FV_CUDA(cudaFuncSetAttribute(k_oz<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-  FV_CUDA(cudaFuncSetAttribute(k_oz<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+  FV_CUDA(cudaFuncSetAttribute(k_oz<true, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+  FV_CUDA(cudaFuncSetAttribute(k_oz<false, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+  FV_CUDA(cudaFuncSetAttribute(k_oz<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+  FV_CUDA(cudaFuncSetAttribute(k_oz<false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   return FV_OK;
 }
 
-fv_status oz_transform(const fv_grid* g, int axis, int inverse, bool scale, const double* in, double* out) {
+fv_status oz_transform(const fv_grid* g, int axis, int inverse, OzScale scale, const double* in, double* out) {
   OzArgs A;
   A.in = in;
   A.out = out;
   A.mat = (const bf16b*)g->oz.mat[axis][inverse];
   A.rexp = g->oz.rexp[axis][inverse];
-  A.inv = scale ? g->oz.inv : nullptr;
+  A.sc = scale;
   A.n = g->n[axis];
   A.nvec = g->ncell / A.n;
   A.Q = axis == 0 ? 1 : axis == 1 ? g->n[0] : (int64_t)g->n[0] * g->n[1];
@@ -458,9 +472,8 @@ fv_status oz_transform(const fv_grid* g, int axis, int inverse, bool scale, cons
   const int N = tile_n(A.n);
   const dim3 grid((unsigned)((A.nvec + N - 1) / N));
   LaunchScope ls_(g, axis == 0 ? FV_K_TPF_X : FV_K_TPF_YZ);
-  if (axis == 0) FV_CUDA(tc5::launch_pdl(k_oz<true, false>, grid, dim3(kOzThreads), oz_smem(A.n), g->stream, A));
-  else if (scale) FV_CUDA(tc5::launch_pdl(k_oz<false, true>, grid, dim3(kOzThreads), oz_smem(A.n), g->stream, A));
-  else FV_CUDA(tc5::launch_pdl(k_oz<false, false>, grid, dim3(kOzThreads), oz_smem(A.n), g->stream, A));
+  auto* kern = axis == 0 ? k_oz<true, 0> : !scale.inv ? k_oz<false, 0> : scale.na ? k_oz<false, 2> : k_oz<false, 1>;
+  FV_CUDA(tc5::launch_pdl(kern, grid, dim3(kOzThreads), oz_smem(A.n), g->stream, A));
   return FV_OK;
 }
 

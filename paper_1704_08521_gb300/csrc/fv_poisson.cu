@@ -922,7 +922,7 @@ fv_status build_tc_mats(fv_grid* g) {
 // One float64 1-D transform along `axis` (0 x, 1 y, 2 z) of the nz x ny x nx
 // array `in`, by Einv or (inverse) E
 fv_status transform_axis_f64(const fv_grid* g, int axis, int inverse, const double* in, double* out) {
-  if (oz_ok(g, axis)) return oz_transform(g, axis, inverse, false, in, out);
+  if (oz_ok(g, axis)) return oz_transform(g, axis, inverse, OzScale{}, in, out);
   const double* M = inverse ? g->tpf_d.E[axis] : g->tpf_d.Einv[axis];
   if (axis == 0) return run_right<double, double, double>(g, M, in, out);
   return run_left<double, double, double, false>(g, axis, M, in, out, g->tpf_d);
@@ -934,7 +934,7 @@ static fv_status tpf_run_f64(const fv_grid* g, const double* r, double* phi) {
   double* b = (double*)g->tpf_buf[1];
   FV_TRY(transform_axis_f64(g, 0, 0, r, a));
   FV_TRY(transform_axis_f64(g, 1, 0, a, b));
-  if (g->oz.inv) FV_TRY(oz_transform(g, 2, 0, true, b, a));
+  if (g->oz.inv) FV_TRY(oz_transform(g, 2, 0, OzScale{g->oz.inv, 0, 0}, b, a));
   else FV_TRY((run_left<double, double, double, true>(g, 2, g->tpf_d.Einv[2], b, a, g->tpf_d)));
   FV_TRY(transform_axis_f64(g, 2, 1, a, b));
   FV_TRY(transform_axis_f64(g, 1, 1, b, a));

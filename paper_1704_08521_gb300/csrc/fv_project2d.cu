@@ -24,91 +24,137 @@ namespace {
 
 constexpr int kPlaneA[3] = {0, 1, 0}, kPlaneC[3] = {2, 2, 1}, kPlaneB[3] = {1, 0, 2};
 
-__device__ __forceinline__ void cell_of(int64_t e, const int n[3], int (&p)[3]) {
-  p[0] = (int)(e % n[0]);
-  p[1] = (int)((e / n[0]) % n[1]);
-  p[2] = (int)(e / ((int64_t)n[0] * n[1]));
+// at most 1024 cells per axis: a cell number fits in 32 bits
+__device__ __forceinline__ void cell_of(unsigned e, const int n[3], int (&p)[3]) {
+  const unsigned r = e / (unsigned)n[0];
+  p[0] = (int)(e - r * n[0]);
+  p[2] = (int)(r / (unsigned)n[1]);
+  p[1] = (int)(r - (unsigned)p[2] * n[1]);
 }
 
-// r = D_ac q (the in-plane divergence; wall faces read as zero)
-__global__ void k_div2d(Met<double> m, const double* __restrict__ q, int a, int c, double* __restrict__ r) {
-  const int64_t nc = m.ncell;
-  const int64_t st[3] = {1, m.n[0], (int64_t)m.n[0] * m.n[1]};
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nc;
-       e += (int64_t)gridDim.x * blockDim.x) {
+__device__ __forceinline__ double factor(const TpfDev<double>& tp, int a, int c, int i, int k) {
+  return i == tp.null_index[a] && k == tp.null_index[c] ? 0.0 : 1.0 / (tp.lam[a][i] + tp.lam[c][k]);
+}
+
+// r = D_ac q (the in-plane divergence; wall faces read as zero), and the plane's
+// n_a n_c factors 1 / (lam_a + lam_c) (0 at the constant mode) for the transform
+// along c: a division per cell is 21 us at 100^3, GB300's float64 rate being
+// what it is.  What is left, 14 -> 12 us, is mostly four float64 operations per cell.
+__global__ void k_div2d(Met<double> m, TpfDev<double> tp, const double* __restrict__ q, int a, int c,
+                        double* __restrict__ r, double* __restrict__ inv) {
+  const unsigned nc = (unsigned)m.ncell, stride = gridDim.x * blockDim.x;
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned st[3] = {1, (unsigned)m.n[0], (unsigned)m.n[0] * m.n[1]};
+  const double *qa = q + a * m.ncell, *qc = q + c * m.ncell;
+  for (unsigned e = t; e < (unsigned)m.n[a] * m.n[c]; e += stride)
+    inv[e] = factor(tp, a, c, (int)(e / (unsigned)m.n[c]), (int)(e % (unsigned)m.n[c]));
+  for (unsigned e = t; e < nc; e += stride) {
     int p[3];
     cell_of(e, m.n, p);
-    double s = 0.0;
-    const int ds[2] = {a, c};
-    for (int t = 0; t < 2; ++t) {
-      const int d = ds[t];
-      const double lo = p[d] > 0 ? q[d * nc + e] : 0.0;
-      const double hi = p[d] + 1 < m.n[d] ? q[d * nc + e + st[d]] : 0.0;
-      s += (hi - lo) * m.idx[d][p[d]];
-    }
-    r[e] = s;
+    const double la = p[a] > 0 ? qa[e] : 0.0, ha = p[a] + 1 < m.n[a] ? qa[e + st[a]] : 0.0;
+    const double lc = p[c] > 0 ? qc[e] : 0.0, hc = p[c] + 1 < m.n[c] ? qc[e + st[c]] : 0.0;
+    r[e] = (ha - la) * m.idx[a][p[a]] + (hc - lc) * m.idx[c][p[c]];
   }
 }
 
-// hat /= lam_a + lam_c; the constant mode of each plane -> 0
-__global__ void k_scale2d(TpfDev<double> tp, int a, int c, double* __restrict__ h, int64_t ncell) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ncell;
-       e += (int64_t)gridDim.x * blockDim.x) {
+// hat *= 1 / (lam_a + lam_c) where the transform does not cover axis c
+__global__ void k_scale2d(Met<double> m, const double* __restrict__ inv, int a, int c, double* __restrict__ h) {
+  for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < (unsigned)m.ncell; e += gridDim.x * blockDim.x) {
     int p[3];
-    cell_of(e, tp.n, p);
-    if (p[a] == tp.null_index[a] && p[c] == tp.null_index[c]) h[e] = 0.0;
-    else h[e] = h[e] / (tp.lam[a][p[a]] + tp.lam[c][p[c]]);
+    cell_of(e, m.n, p);
+    h[e] *= inv[p[a] * m.n[c] + p[c]];
   }
 }
 
 // vp = q - G_ac phi on the in-plane components (walls zero), vp_b = 0
 __global__ void k_correct2d(Met<double> m, const double* __restrict__ q, const double* __restrict__ phi,
-                            int a, int c, double* __restrict__ vp) {
-  const int64_t nc = m.ncell;
-  const int64_t st[3] = {1, m.n[0], (int64_t)m.n[0] * m.n[1]};
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nc;
-       e += (int64_t)gridDim.x * blockDim.x) {
+                            int a, int c, int b, double* __restrict__ vp) {
+  const unsigned nc = (unsigned)m.ncell;
+  const unsigned st[3] = {1, (unsigned)m.n[0], (unsigned)m.n[0] * m.n[1]};
+  const double *qa = q + a * m.ncell, *qc = q + c * m.ncell;
+  double *va = vp + a * m.ncell, *vc = vp + c * m.ncell, *vb = vp + b * m.ncell;
+  for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < nc; e += gridDim.x * blockDim.x) {
     int p[3];
     cell_of(e, m.n, p);
-    for (int d = 0; d < 3; ++d) {
-      double v = 0.0;
-      if ((d == a || d == c) && p[d] > 0)
-        v = q[d * nc + e] - (phi[e] - phi[e - st[d]]) * m.idc[d][p[d]];
-      vp[d * nc + e] = v;
-    }
+    const double f = phi[e];
+    va[e] = p[a] > 0 ? qa[e] - (f - phi[e - st[a]]) * m.idc[a][p[a]] : 0.0;
+    vc[e] = p[c] > 0 ? qc[e] - (f - phi[e - st[c]]) * m.idc[c][p[c]] : 0.0;
+    vb[e] = 0.0;
   }
 }
 
-// Psi on the corners: one thread per line along a (index b, c-corner k)
-__global__ void k_potential(Met<double> m, const double* __restrict__ vp, int a, int c, int b, double sgn,
-                            double* __restrict__ psi) {
-  const int nb = m.n[b], ncp = m.n[c] + 1, nap = m.n[a] + 1;
-  const int64_t lines = (int64_t)nb * ncp;
-  const int64_t nc = m.ncell;
-  const int64_t st[3] = {1, m.n[0], (int64_t)m.n[0] * m.n[1]};
-  // strides of the corner array: [z][y][x] with n + 1 along a and c
-  int64_t cs[3];
-  {
-    int64_t dims[3] = {m.n[0], m.n[1], m.n[2]};
-    dims[a] += 1;
-    dims[c] += 1;
-    cs[0] = 1;
-    cs[1] = dims[0];
-    cs[2] = dims[0] * dims[1];
+// Psi on the corners, the running integral along a.  Corner array: [z][y][x]
+// with n + 1 along a and c.
+//
+// a = x: a block takes 32 lines; runs of kRun cells pass through shared memory,
+// so that memory is read and written along x, and 32 threads add up one line
+// each.  One thread per line straight from memory took 44 us at 100^3 (32 lines
+// per request); this takes 18, of which the dependent float64 additions are most.
+constexpr int kLines = 32, kRun = 128;
+
+__global__ void __launch_bounds__(256) k_potential_x(Met<double> m, const double* __restrict__ vc, int c, int b,
+                                                     double sgn, double* __restrict__ psi) {
+  __shared__ double tile[kLines][kRun + 1];
+  __shared__ int64_t src[kLines], dst[kLines];
+  const int nx = m.n[0], nb = m.n[b], nc1 = m.n[c] + 1;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const unsigned l0 = blockIdx.x * kLines, lines = (unsigned)nb * nc1;
+  if (tid < kLines) {
+    const unsigned l = l0 + tid;
+    // y and z of the line, y fastest in memory
+    const unsigned ny1 = c == 1 ? nc1 : nb;
+    const int y = (int)(l % ny1), z = (int)(l / ny1);
+    const bool wall = (c == 1 ? y : z) == m.n[c];        // the last face: a wall
+    src[tid] = l >= lines || wall ? -1 : ((int64_t)z * m.n[1] + y) * nx;
+    dst[tid] = l >= lines ? -1 : (int64_t)l * (nx + 1);
+    if (l < lines) psi[dst[tid]] = 0.0;
   }
-  for (int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; l < lines;
-       l += (int64_t)gridDim.x * blockDim.x) {
-    const int jb = (int)(l % nb), kc = (int)(l / nb);
-    double s = 0.0;
-    int64_t o = jb * cs[b] + kc * cs[c];
-    psi[o] = 0.0;
-    for (int ia = 0; ia < nap - 1; ++ia) {
-      // component c on c-face kc (face n_c is the wall: zero), centre ia
-      double comp = 0.0;
-      if (kc < m.n[c]) comp = vp[c * nc + (int64_t)ia * st[a] + (int64_t)jb * st[b] + (int64_t)kc * st[c]];
-      s += sgn * comp * m.dx[a][ia];
-      psi[o + (int64_t)(ia + 1) * cs[a]] = kc < m.n[c] ? s : 0.0;
-    }
+  __syncthreads();
+  double s = 0.0;
+  for (int x0 = 0; x0 < nx; x0 += kRun) {
+    const int cnt = min(kRun, nx - x0);
+    for (int l = warp; l < kLines; l += 8)
+      for (int i = lane; i < kRun; i += 32)
+        tile[l][i] = i < cnt && src[l] >= 0 ? vc[src[l] + x0 + i] * (sgn * m.dx[0][x0 + i]) : 0.0;
+    __syncthreads();
+    if (tid < kLines)
+      for (int i = 0; i < cnt; i += 8) {     // the loads first: a store could alias the next one
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = tile[tid][i + q];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) tile[tid][i + q] = s += v[q];
+      }
+    __syncthreads();
+    for (int l = warp; l < kLines; l += 8)
+      if (dst[l] >= 0)
+        for (int i = lane; i < cnt; i += 32) psi[dst[l] + x0 + i + 1] = tile[l][i];
+    __syncthreads();
+  }
+}
+
+// a = y (b = x, c = z): one thread per line, lines along x, eight loads ahead
+__global__ void __launch_bounds__(64) k_potential_y(Met<double> m, const double* __restrict__ vc, double sgn,
+                                                    double* __restrict__ psi) {
+  const int nx = m.n[0], ny = m.n[1];
+  const unsigned l = blockIdx.x * 64 + threadIdx.x;
+  const int z = (int)(l / (unsigned)nx), x = (int)(l - (unsigned)z * nx);
+  if (z > m.n[2]) return;
+  const bool wall = z == m.n[2];
+  const double* p = vc + (int64_t)z * nx * ny + x;
+  double* o = psi + (int64_t)z * nx * (ny + 1) + x;
+  double s = 0.0;
+  *o = 0.0;
+  for (int y0 = 0; y0 < ny; y0 += 8) {
+    double v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = !wall && y0 + q < ny ? p[(int64_t)(y0 + q) * nx] : 0.0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (y0 + q < ny) {
+        s += v[q] * (sgn * m.dx[1][y0 + q]);
+        o[(int64_t)(y0 + q + 1) * nx] = s;
+      }
   }
 }
 
@@ -123,32 +169,39 @@ inline unsigned blocks_for(int64_t n) {
 fv_status plane_projection(const fv_grid* g, const double* v, int plane, double* vp, double* psi) {
   const int a = kPlaneA[plane], c = kPlaneC[plane], b = kPlaneB[plane];
   double* r = g->cell_buf[0];
+  double* inv = g->cell_buf[1];              // n_a n_c factors
   double* t0 = (double*)g->tpf_buf[0];
   double* t1 = (double*)g->tpf_buf[1];
   {
     LaunchScope ls_(g, FV_K_DIVERGENCE);
-    k_div2d<<<blocks_for(g->ncell), 256, 0, g->stream>>>(g->met_d, v, a, c, r);
+    k_div2d<<<blocks_for(g->ncell), 256, 0, g->stream>>>(g->met_d, g->tpf_d, v, a, c, r, inv);
   }
   FV_CHECK_LAUNCH();
   FV_TRY(transform_axis_f64(g, a, 0, r, t0));
-  FV_TRY(transform_axis_f64(g, c, 0, t0, t1));
-  {
+  if (oz_ok(g, c)) {
+    FV_TRY(oz_transform(g, c, 0, OzScale{inv, a == 0 ? 1 : g->n[0], g->n[a]}, t0, t1));
+  } else {
+    FV_TRY(transform_axis_f64(g, c, 0, t0, t1));
     LaunchScope ls_(g, FV_K_VECTOR);
-    k_scale2d<<<blocks_for(g->ncell), 256, 0, g->stream>>>(g->tpf_d, a, c, t1, g->ncell);
+    k_scale2d<<<blocks_for(g->ncell), 256, 0, g->stream>>>(g->met_d, inv, a, c, t1);
   }
   FV_CHECK_LAUNCH();
   FV_TRY(transform_axis_f64(g, c, 1, t1, t0));
   FV_TRY(transform_axis_f64(g, a, 1, t0, r));   // r = phi
   {
     LaunchScope ls_(g, FV_K_CORRECT);
-    k_correct2d<<<blocks_for(g->ncell), 256, 0, g->stream>>>(g->met_d, v, r, a, c, vp);
+    k_correct2d<<<blocks_for(g->ncell), 256, 0, g->stream>>>(g->met_d, v, r, a, c, b, vp);
   }
   FV_CHECK_LAUNCH();
   if (psi) {
     const double sgn = plane == 0 ? 1.0 : -1.0;
-    const int64_t lines = (int64_t)g->n[b] * (g->n[c] + 1);
+    const double* vc = vp + c * g->ncell;
+    const unsigned lines = (unsigned)g->n[b] * (g->n[c] + 1);
     LaunchScope ls_(g, FV_K_VECTOR);
-    k_potential<<<blocks_for(lines), 256, 0, g->stream>>>(g->met_d, vp, a, c, b, sgn, psi);
+    if (a == 0)
+      k_potential_x<<<(lines + kLines - 1) / kLines, 256, 0, g->stream>>>(g->met_d, vc, c, b, sgn, psi);
+    else
+      k_potential_y<<<(lines + 63) / 64, 64, 0, g->stream>>>(g->met_d, vc, sgn, psi);
   }
   FV_CHECK_LAUNCH();
   return FV_OK;
