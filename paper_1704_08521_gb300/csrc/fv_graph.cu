@@ -520,7 +520,7 @@ static fv_status batch_build_graph(BatchImpl& b) {
   std::vector<cudaStream_t> saved(b.n);
   for (int i = 0; i < b.n; ++i) {
     saved[i] = b.grids[i]->stream;
-    b.grids[i]->capturing = true;
+    b.grids[i]->capturing = b.grids[i]->in_batch = true;
   }
   cudaGraph_t graph = nullptr;
   bool begun = false;
@@ -557,7 +557,7 @@ static fv_status batch_build_graph(BatchImpl& b) {
   const cudaError_t ec = begun ? cudaStreamEndCapture(cs, &graph) : cudaSuccess;
   for (int i = 0; i < b.n; ++i) {
     b.grids[i]->stream = saved[i];
-    b.grids[i]->capturing = false;
+    b.grids[i]->capturing = b.grids[i]->in_batch = false;
   }
   if (st == FV_OK && ec != cudaSuccess) st = cuda_fail(ec, "cudaStreamEndCapture", __FILE__, __LINE__);
   if (st != FV_OK) {

@@ -214,6 +214,7 @@ struct fv_grid {
   fv::GraphCache graphs[fv::kGraphSlots];
   unsigned char* d_eval = nullptr;   // call blocks and loop states of the slots
   mutable bool capturing = false;
+  mutable bool in_batch = false;  // captured beside other grids' evaluations
   bool use_graph = true;          // FVNS_NO_GRAPH=1 selects the host-driven loop
 
   // optional per-kernel-class event timing
@@ -274,6 +275,21 @@ inline dim3 cell_launch_grid(const int n[3]) {
   const int64_t plane = (int64_t)n[0] * n[1];
   return dim3((unsigned)((plane + kCellThreads - 1) / kCellThreads),
               (unsigned)((n[2] + kCellKz - 1) / kCellKz), 1);
+}
+
+// The graph's cell kernels (D w and the join) below kFewCells: one plane per
+// thread and half the threads per block, since four planes per thread leave a
+// 16^3 grid on four SMs.  An evaluation with four planes / one: 16^3 84.5 / 80.4 us,
+// 48^3 105.4 / 101.3, 64^3 127.9 / 125.8, 80^3 151.2 / 151.0, 100^3 216.6 / 216.5, and float-float at
+// 150^3 914 / 918, 256^3 3619 / 3640 (join alone).  Not in a batch, whose grids
+// fill the GPU together: 48^3 .. 96^3 1155 us with four planes, 1190 with one.
+constexpr int64_t kFewCells = 1 << 19;
+inline bool few_cells(const fv_grid* g) { return !g->in_batch && g->ncell < kFewCells; }
+inline int cell_threads(const fv_grid* g) { return few_cells(g) ? kCellThreads / 2 : kCellThreads; }
+inline int cell_planes(const fv_grid* g) { return few_cells(g) ? 1 : kCellKz; }
+inline dim3 cell_grid_fit(const fv_grid* g) {
+  const int thr = cell_threads(g), kz = cell_planes(g);
+  return dim3((unsigned)(((int64_t)g->n[0] * g->n[1] + thr - 1) / thr), (unsigned)((g->n[2] + kz - 1) / kz), 1);
 }
 
 // ------------------------------------------------------------- kernels ---

@@ -50,6 +50,7 @@ __global__ void k_widen_f32(const float* __restrict__ in, double* __restrict__ o
 }
 
 // D w in float32 (first residual of the loop; w holds float32 values).
+template <int KZ>
 __global__ void __launch_bounds__(256) k_div_f32(MetFF m, const float* __restrict__ w,
                                                  float* __restrict__ r) {
   tc5::pdl_trigger();   // the pressure transform that follows may start its set-up
@@ -59,8 +60,8 @@ __global__ void __launch_bounds__(256) k_div_f32(MetFF m, const float* __restric
   const int i = act_ ? t_ % m.n[0] : 0;
   const int j = act_ ? t_ / m.n[0] : 0;
   if (!act_) return;
-  for (int kk = 0; kk < kCellKz; ++kk) {
-  const int k = blockIdx.y * kCellKz + kk;
+  for (int kk = 0; kk < KZ; ++kk) {
+  const int k = blockIdx.y * KZ + kk;
   if (k >= m.n[2]) return;
   const int64_t nx = m.n[0], nxy = nx * m.n[1], nc = m.ncell;
   const int64_t base = ((int64_t)k * m.n[1] + j) * nx + i;
@@ -163,6 +164,7 @@ __global__ void k_split_ff(const double* __restrict__ in, float2* __restrict__ o
 }
 
 // D w of a float-float field, rounded to float32 (first pressure rhs of FV_FF)
+template <int KZ>
 __global__ void __launch_bounds__(256) k_div_ff(MetFF m, const float2* __restrict__ w,
                                                 float* __restrict__ r) {
   tc5::pdl_trigger();   // the pressure transform that follows may start its set-up
@@ -172,8 +174,8 @@ __global__ void __launch_bounds__(256) k_div_ff(MetFF m, const float2* __restric
   const int i = t_ % m.n[0], j = t_ / m.n[0];
   const int nx = m.n[0], ny = m.n[1], nz = m.n[2];
   const int nc = (int)m.ncell;
-  for (int kk = 0; kk < kCellKz; ++kk) {
-    const int k = blockIdx.y * kCellKz + kk;
+  for (int kk = 0; kk < KZ; ++kk) {
+    const int k = blockIdx.y * KZ + kk;
     if (k >= nz) return;
     const int base = k * plane_ + t_;
     const ff z = {0.f, 0.f};
@@ -219,10 +221,10 @@ fv_status launch_widen_f32(const fv_grid* g, const float* in, double* out, int64
 }
 
 fv_status launch_div_f32(const fv_grid* g, const float* w32, float* r32) {
-  const int bx = block_x(g);
   {
     LaunchScope ls_(g, FV_K_DIVERGENCE);
-    k_div_f32<<<cell_grid(g, bx), bx, 0, g->stream>>>(g->met_ff, w32, r32);
+    auto* kern = few_cells(g) ? k_div_f32<1> : k_div_f32<kCellKz>;
+    kern<<<cell_grid_fit(g), cell_threads(g), 0, g->stream>>>(g->met_ff, w32, r32);
   }
   FV_CHECK_LAUNCH();
   return FV_OK;
@@ -322,7 +324,8 @@ fv_status launch_jv_ff_out64(const fv_grid* g, const double* Ud, const double* x
 fv_status launch_div_ff(const fv_grid* g, const float2* w, float* r32) {
   {
     LaunchScope ls_(g, FV_K_DIVERGENCE);
-    k_div_ff<<<cell_grid(g, 0), kCellThreads, 0, g->stream>>>(g->met_ff, w, r32);
+    auto* kern = few_cells(g) ? k_div_ff<1> : k_div_ff<kCellKz>;
+    kern<<<cell_grid_fit(g), cell_threads(g), 0, g->stream>>>(g->met_ff, w, r32);
   }
   FV_CHECK_LAUNCH();
   return FV_OK;

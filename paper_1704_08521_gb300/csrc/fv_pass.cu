@@ -425,6 +425,7 @@ struct JoinArgs {
   const float2* p;
   const CallBlock* cb;
   LoopState* ls;
+  int kz;                  // planes per thread
 };
 
 // out = v - sigma x, p_out = p (float64): v and p from the terms that hold them
@@ -443,9 +444,7 @@ __device__ __forceinline__ void join_body(const JoinArgs& A) {
   const int pass = A.ls->pass;
   const float2* v = A.vff[pass & 1];          // NS == 0: the last fold
 #pragma unroll 1
-  for (int kk = 0; kk < kCellKz; ++kk) {
-    const int k = blockIdx.y * kCellKz + kk;
-    if (k >= nz) break;
+  for (int k = blockIdx.y * A.kz; k < min(nz, (int)(blockIdx.y + 1) * A.kz); ++k) {
     const int e = k * nxy + t;
     float f[NS > 0 ? NS : 1];
 #pragma unroll
@@ -583,9 +582,11 @@ fv_status launch_join(const fv_grid* g, int prec, const CallBlock* cb, LoopState
   A.p = g->pff;
   A.cb = cb;
   A.ls = ls;
+  A.kz = cell_planes(g);
+  const int thr = cell_threads(g);
   LaunchScope ls_(g, FV_K_VECTOR);
-  if (prec == FV_FF) k_join<true><<<cell_launch_grid(g->n), kCellThreads, 0, g->stream>>>(A);
-  else k_join<false><<<cell_launch_grid(g->n), kCellThreads, 0, g->stream>>>(A);
+  if (prec == FV_FF) k_join<true><<<cell_grid_fit(g), thr, 0, g->stream>>>(A);
+  else k_join<false><<<cell_grid_fit(g), thr, 0, g->stream>>>(A);
   FV_CHECK_LAUNCH();
   return FV_OK;
 }
