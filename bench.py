@@ -126,7 +126,7 @@ def algorithmic(kind, n, prec):
     else:
         f = 4
         table = {"momentum": 36,                 # read U, v (3 x 4 B each), write w (3 x 4 B)
-                 "correct": 24 + 4 + 16 + 24 + 4,  # read v (ff), phi, r/w p (ff), write v (ff), r
+                 "correct": 12 + 2 * 4 + 4,       # second pass: read w (3 x 4 B), two corrections, write r
                  "divergence": 16}               # read w (3 x 4 B), write r
     if kind in ("tpf_x", "tpf_xinv", "tpf_yz"):
         # fused tensor-core kernels (n <= 112) apply two 1-D transforms per
@@ -213,11 +213,11 @@ def run_ours(args):
         dist.all_reduce(t, op=dist.ReduceOp.MAX)
     ms_max = float(t.item())
     value = ws * args.steps / (ms_max / 1e3)
-    # kernels per evaluation: graph = init, round, J.v, D w, pressure solve,
-    # correct, decide (first pass) + solve, correct, decide per further pass
-    # + join; the pressure solve is 3 fused kernels for n <= 128, else 6
+    # kernels per evaluation: J.v, D w, at least three passes (the graph runs
+    # three in a row) of a pressure solve and a correction, join; the pressure
+    # solve is 3 fused kernels for n <= 112, else 6
     tpf_k = 3 if n <= 112 else 6
-    kernels_per_solve = (7 + tpf_k + (tpf_k + 2) * (passes - 1)) if mixed else None
+    kernels_per_solve = (3 + (tpf_k + 1) * max(passes, 3)) if mixed else None
     gpu_launches = kernels_per_solve * args.steps if mixed else host_launches
 
     # same workload in the plain FP64 form, a few steps (context for the
@@ -387,12 +387,13 @@ def run_ours(args):
     # writes w in float32; each pass moves the float64 state and the float32
     # pressure right-hand side and correction), over the time per solve; beside
     # it the bytes this implementation moves by design (float64 x read by J.v,
-    # D w, three transform launches and the fused correction per pass, join of
-    # v and p to float64)
+    # D w, per pass m three transform launches and a pass over w and m
+    # corrections, join of v and p to float64)
     solve_roof = None
     if mixed:
         bpc = 36 + 80 * passes
-        impl = 48 + 16 + passes * (3 * 8 + 72) + 64
+        k = min(passes, 3)   # passes beyond the third store the float-float state (72 B)
+        impl = 48 + 16 + sum(3 * 8 + 16 + 4 * m for m in range(1, k + 1)) + (passes - k) * (3 * 8 + 72) + 12 + 4 * k + 32
         bytes_solve = bpc * n ** 3
         ach = bytes_solve * value / ws / 1e9
         pk_hbm = pk.get("hbm_gbs", 6800.0)
@@ -457,7 +458,7 @@ def mg_measure(fv, torch, g, U, v, n, stream, barrier, reps=5):
     """Multigrid pressure solve at rtol 1e-8: CG iterations, ms per solve and
     per V-cycle, and the line-smoothing sweeps' bandwidth on their
     algorithmic bytes (x in, b in, x out: 12 B per cell per sweep; six sweeps
-    per level above the coarsest)."""
+    per level of more than 32 cells per axis; the next one is solved exactly)."""
     w = torch.empty(g.n_vel, dtype=torch.float64, device=v.device)
     fv.ns_jacvec(g, U, v, w, prec="fp64")
     r = torch.empty(g.n_cell, dtype=torch.float64, device=v.device)
@@ -465,20 +466,23 @@ def mg_measure(fv, torch, g, U, v, n, stream, barrier, reps=5):
     phi = torch.empty_like(r)
     st = fv.fv_pressure_solve_mg(g, r, phi, rtol=1e-8)
     barrier()
-    fv.fv_profile_enable(g, True)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     e0.record(stream)
     for _ in range(reps):
         fv.fv_pressure_solve_mg(g, r, phi, rtol=1e-8)
     e1.record(stream)
     barrier()
+    ms = e0.elapsed_time(e1) / reps
+    fv.fv_profile_enable(g, True)   # the same iterations from the host, each sweep timed
+    for _ in range(reps):
+        fv.fv_pressure_solve_mg(g, r, phi, rtol=1e-8)
+    barrier()
     prof = fv.fv_profile_read(g)
     fv.fv_profile_enable(g, False)
-    ms = e0.elapsed_time(e1) / reps
     its = st["iterations"]
     sm_ms, sm_n = prof["mg_smooth"]
     lv = mg_levels(n)
-    alg_bytes = 6 * 12 * sum(lv[:-1]) * its * reps
+    alg_bytes = 6 * 12 * sum(c for c in lv if c > 32 ** 3) * its * reps
     peak = peaks().get("hbm_gbs", 6800.0)
     sm_gbs = alg_bytes / (sm_ms / 1e3) / 1e9 if sm_ms > 0 else None
     # the FP64 Krylov vector with multigrid pressure passes
@@ -493,7 +497,7 @@ def mg_measure(fv, torch, g, U, v, n, stream, barrier, reps=5):
     return {"rtol": 1e-8, "levels": st["levels"], "cg_iterations": its, "ms_per_solve": ms,
             "ms_per_vcycle_iteration": ms / max(its, 1),
             "smooth_ms_per_solve": sm_ms / reps, "smooth_launches_per_solve": sm_n / reps,
-            "smooth_share": sm_ms / reps / ms,
+            "smooth_share": sm_ms / reps / ms,   # sweeps timed one by one over the graph's time
             "smooth_roofline": {"bound": "hbm", "achieved": sm_gbs, "peak": peak, "unit": "GB/s",
                                 "frac": sm_gbs / peak if sm_gbs else None,
                                 "bytes_per_cell_per_sweep": 12},
