@@ -41,17 +41,6 @@ __global__ void k_base_from_call(const double* __restrict__ U, float* __restrict
   }
 }
 
-__global__ void k_round2(const CallBlock* __restrict__ cb, float* __restrict__ U32,
-                         float* __restrict__ x32, int64_t n) {
-  const double* U = cb->U;
-  const double* x = cb->x;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    U32[e] = f64_round_f32(__ldg(U + e));
-    x32[e] = f64_round_f32(__ldg(x + e));
-  }
-}
-
 inline unsigned grid1d(int64_t n) {
   int64_t b = (n + 255) / 256;
   if (b > 152 * 16) b = 152 * 16;
@@ -372,6 +361,7 @@ namespace {
 
 constexpr int kBatchMax = 32;
 constexpr int kBatchBlocks = 152 * 4;
+constexpr int kBand = 1024;      // cells of a plane in one work item at most
 
 struct BatchCall {
   const double* U[kBatchMax];
@@ -383,11 +373,12 @@ struct BatchCall {
 
 struct InstDesc {
   Met<float> m;
-  const float* U32;
-  const float* x32;
+  float* U32;
+  float* x32;
   float* w32;
   float inv_re;
   int tile_base;
+  int bands;                     // of a plane
 };
 
 __global__ void k_batch_init(BatchCall bc, CallBlock* dcb, LoopState* dls) {
@@ -408,31 +399,58 @@ __global__ void k_batch_init(BatchCall bc, CallBlock* dcb, LoopState* dls) {
   l.pass = l.nan = l.status = 0;
 }
 
+// U and x of every instance (blockIdx.y) rounded to float32, as one launch: one
+// per instance left a gap and a partial last wave twelve times over.  Bound by
+// memory (24 B per entry).
+__global__ void __launch_bounds__(256) k_batch_round(const InstDesc* __restrict__ d,
+                                                     const CallBlock* __restrict__ cb) {
+  const double* U = cb[blockIdx.y].U;
+  const double* x = cb[blockIdx.y].x;
+  float* U32 = d[blockIdx.y].U32;
+  float* x32 = d[blockIdx.y].x32;
+  const int64_t n = 3 * d[blockIdx.y].m.ncell;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    U32[e] = f64_round_f32(__ldg(U + e));
+    x32[e] = f64_round_f32(__ldg(x + e));
+  }
+}
+
 // Momentum predictor (Eq. 10, float32) of every instance: blocks pull work
-// items (instance, ppt consecutive z-planes) from an atomic counter.
+// items (instance, ppt consecutive z-planes, a band of kBand cells of them)
+// from an atomic counter, the next one while they compute.  Bands, because
+// whole planes of {48 .. 96}^3 (three of each) are 864 items for the 304 blocks
+// that fit at a time, the largest last: the end of the kernel was a partial
+// wave of them.  With k_batch_round in place of twelve rounding launches, the
+// batch of twelve went from 1160 to 1135 us.  Bound by the latency of its
+// loads, yet three or four blocks per SM (80, 64 registers, spilled) were
+// slower: 1155 and 1156 us against 1135 with two (128 registers).
 __global__ void __launch_bounds__(256) k_batch_jv(const InstDesc* __restrict__ d, int ninst,
                                                   int total, int ppt, float shift,
                                                   unsigned* __restrict__ counter) {
-  __shared__ int s_tile;
-  for (;;) {
-    __syncthreads();
-    if (threadIdx.x == 0) s_tile = (int)atomicAdd(counter, 1u);
-    __syncthreads();
-    const int tile = s_tile;
+  __shared__ int s_tile[2];
+  if (threadIdx.x == 0) s_tile[0] = (int)atomicAdd(counter, 1u);
+  __syncthreads();
+  int inst = 0;                  // items come in order: the search goes on from the last one
+  for (int buf = 0;; buf ^= 1) {
+    const int tile = s_tile[buf];
     if (tile >= total) return;
-    int inst = 0;
+    if (threadIdx.x == 0) s_tile[buf ^ 1] = (int)atomicAdd(counter, 1u);
     while (inst + 1 < ninst && d[inst + 1].tile_base <= tile) ++inst;
     const Met<float> m = d[inst].m;
     const float* U = d[inst].U32;
     const float* V = d[inst].x32;
     float* out = d[inst].w32;
     const float inv_re = d[inst].inv_re;
-    const int z0 = (tile - d[inst].tile_base) * ppt;
+    const int bands = d[inst].bands;
+    const int item = tile - d[inst].tile_base;
+    const int z0 = item / bands * ppt, t0 = item % bands * kBand;
     const int nx = m.n[0], ny = m.n[1], nz = m.n[2];
     const int plane = nx * ny;
     const int nc = (int)m.ncell;
     const int st[3] = {1, nx, plane};
-    for (int t = threadIdx.x; t < plane; t += blockDim.x) {
+    const int t1 = min(plane, t0 + kBand);
+    for (int t = t0 + (int)threadIdx.x; t < t1; t += blockDim.x) {
       const int i = t % nx, j = t / nx;
       for (int kk = 0; kk < ppt; ++kk) {
         const int k = z0 + kk;
@@ -451,6 +469,7 @@ __global__ void __launch_bounds__(256) k_batch_jv(const InstDesc* __restrict__ d
         out[2 * nc + base] = r2;
       }
     }
+    __syncthreads();             // the next item is there, and everyone has read this one
   }
 }
 
@@ -486,7 +505,8 @@ static fv_status batch_descriptors(BatchImpl& b) {
     h[i].inv_re = float(1.0 / g->re);
     b.re[i] = g->re;
     h[i].tile_base = base;
-    base += (g->n[2] + b.ppt - 1) / b.ppt;
+    h[i].bands = (g->n[0] * g->n[1] + kBand - 1) / kBand;
+    base += (g->n[2] + b.ppt - 1) / b.ppt * h[i].bands;
   }
   b.total_tiles = base;
   FV_CUDA(cudaMemcpy(b.d_desc, h.data(), b.n * sizeof(InstDesc), cudaMemcpyHostToDevice));
@@ -510,8 +530,8 @@ static void batch_release_graph(BatchImpl& b) {
   b.ready = false;
 }
 
-// Capture the batch graph: init -> round (per instance) -> batched J.v ->
-// per-instance branches {D w -> TPF -> correct -> decide -> WHILE{...} -> join}.
+// Capture the batch graph: init -> round -> batched J.v -> per-instance branches
+// {D w -> three times (TPF -> pass) -> WHILE{TPF -> pass} -> join}.
 static fv_status batch_build_graph(BatchImpl& b) {
   batch_release_graph(b);
   FV_TRY(batch_descriptors(b));
@@ -530,11 +550,10 @@ static fv_status batch_build_graph(BatchImpl& b) {
     BatchCall bc = {};
     k_batch_init<<<1, kBatchMax, 0, cs>>>(bc, b.d_call, b.d_loop);
     FV_CHECK_LAUNCH();
-    for (int i = 0; i < b.n; ++i) {
-      fv_grid* g = b.grids[i];
-      k_round2<<<grid1d(g->nvel), 256, 0, cs>>>(b.d_call + i, g->U32, g->x32, g->nvel);
-      FV_CHECK_LAUNCH();
-    }
+    int64_t longest = 0;
+    for (int i = 0; i < b.n; ++i) longest = std::max(longest, b.grids[i]->nvel);
+    k_batch_round<<<dim3(grid1d(longest), b.n), 256, 0, cs>>>(b.d_desc, b.d_call);
+    FV_CHECK_LAUNCH();
     FV_TRY(launch_batch_jv(b, cs));
     // one stream captures every branch: each starts from the J.v node, and the
     // capture ends where they all have
