@@ -17,7 +17,7 @@ def test_batch_bands(planes):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     import paper_1704_08521_gb300 as fv
-    shapes = [(6, 5, 4), (7, 32, 32), (5, 25, 41), (8, 47, 51), (9, 3, 7)]      # nz, ny, nx
+    shapes = [(6, 5, 4), (7, 32, 32), (5, 25, 41), (8, 47, 51), (9, 4, 7)]      # nz, ny, nx
     grids, U, X, O = [], [], [], []
     for i, (nz, ny, nx) in enumerate(shapes):
         g = fv.Grid(nx, ny, nz, "cosine", alpha=0.3, re=400.0 + 100 * i)
