@@ -87,7 +87,7 @@ static fv_status capture_passes(fv_grid* g, int prec, cudaStream_t cs, cudaStrea
   FV_TRY(s2);
   FV_CUDA(e2);
   FV_CUDA(cudaStreamUpdateCaptureDependencies(cs, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies));
-  return launch_join(g, prec, cb, ls);
+  return launch_join(g, cb, ls);
 }
 
 // The two streams that graphs are captured on, kept by each host thread for
@@ -321,7 +321,7 @@ fv_status bench_kernel(fv_grid* g, int kind, int reps, double* ms) {
       case FV_K_MOMENTUM: return launch_jv_f32(g, nullptr, g->vel_buf[1], g->w32, 0.0);
       case FV_K_DIVERGENCE: return launch_div_f32(g, g->w32, g->r32);
       case FV_K_CORRECT:
-        // the second pass: the predictor and two corrections
+        // the second pass, the first that reads a float-float v
         return launch_pass(g, FV_MIXED, 1, (const CallBlock*)gc->d_call, gc->d_loop, nullptr, false);
       case FV_K_TPF_X: return tpf_one_transform_f32(g, 0);
       case FV_K_TPF_XINV: return tpf_one_transform_f32(g, 1);

@@ -353,7 +353,7 @@ void drop_capture_streams();
 // count it, take the stop decision and (h) set the WHILE condition
 fv_status launch_pass(const fv_grid* g, int prec, int idx, const CallBlock* cb, LoopState* ls,
                       const cudaGraphConditionalHandle* h, bool decide);
-fv_status launch_join(const fv_grid* g, int prec, const CallBlock* cb, LoopState* ls);
+fv_status launch_join(const fv_grid* g, const CallBlock* cb, LoopState* ls);
 
 // tensor-product pressure solve: phi = (D G)^+ r ; phi is float or double
 fv_status tpf_solve(const fv_grid* g, const double* r, void* phi, int prec);

@@ -3,16 +3,18 @@
 // keeps its rounding.
 //
 // A pass takes the new correction phi_m, forms the corrected velocity
-// v = w - omega G (phi_1 + ... + phi_m) and its divergence r = D v, the
-// right-hand side of the next solve.  v is not stored between the first three
-// passes (three is the usual number): the predictor w and the float32
-// corrections phi_1 .. phi_3 hold it exactly, so pass m reads w (12 B per cell
-// in float32, 24 B in float-float) and 4 m B of corrections and writes 4 B,
-// instead of reading and writing the float-float v and p (72 B).  The result
-// is formed once, by k_join, from the same terms in the same order.  Passes
-// beyond the third (slow inner solves, under-relaxation) store v: the fourth
-// folds w and all four corrections into a float-float buffer, later ones read
-// it and write the other.
+// v - omega G phi_m and its divergence r = D v, the right-hand side of the next
+// solve, in the order and with every rounding of the host-driven loop
+// (k_correct_ff): both give the same bits.  v goes from one float-float buffer
+// to the other, so that the next pass removes what this one's roundings left;
+// p is summed by k_join, if it is asked for, from the first three corrections
+// (three is the usual number), which are kept apart, or by the passes beyond
+// the third.  A version that kept only the predictor and the corrections and
+// formed v from them in every pass read less, but its float-float roundings were
+// not seen by the following solve, and with the lower parts of the sums added in
+// plain float32 |D v| came out 2 to 100 times larger.  With full sums it was no
+// faster either: 100^3 mixed 225 us an evaluation against 217, 256^3 float-float
+// 3990 against 3640.
 //
 // Every face belongs to two cells: a thread computes the three low faces of
 // its cell and gets the high ones from its x and y neighbours through shared
@@ -26,14 +28,11 @@
 // The last block to finish reduces the block maxima, takes the loop's decision
 // and sets the condition of the graph's WHILE node: no separate kernel.
 //
-// Bound by instruction issue (float-float arithmetic: about 290 instructions
-// per cell in the third float-float pass), not by memory.  Measured (cold
-// cache): the three passes at 100^3 mixed 15, 17 and 20 us against 23-27 us
-// each for the kernel that stored v and p; at 256^3 float-float 171, 240 and
-// 242 us against 355 us.  One cell per thread took 390 instructions and 18 us
-// for the second mixed pass at 100^3 (14 us with two); fetching the low
-// neighbours a plane ahead as well cost registers and 20 % of the float-float
-// time.
+// Bound by instruction issue (float-float arithmetic), not by memory (40 to 52 B
+// per cell).  An evaluation with these passes takes 217 us at 100^3 mixed and
+// 3640 us at 256^3 float-float, against 260 and 4216 us with one cell per thread
+// and a kernel of its own for the decision; fetching the low neighbours a plane
+// ahead as well cost registers and 20 % of the float-float time.
 #include "fv_ff.cuh"
 #include "fv_internal.cuh"
 #include "fv_tc5.cuh"
@@ -62,71 +61,29 @@ __device__ __forceinline__ float block_max(float v, float* red) {
 __device__ __forceinline__ ff base_of(float w) { return {w, 0.f}; }
 __device__ __forceinline__ ff base_of(float2 w) { return of2(w); }
 
-// v at a face: base - omega sum_s (a_s - b_s) / dc, the corrections a (this
-// cell) and b (low neighbour) in order.
-// Mixed form: each gradient in float32, as the form's contract has it.
-template <int NS>
-__device__ __forceinline__ ff face_mixed(ff v, const float (&a)[NS], const float (&b)[NS], float idc,
-                                         float omega) {
-#pragma unroll
-  for (int s = 0; s < NS; ++s) {
-    const float g = (a[s] - b[s]) * idc;
-    v = ff_add_f(v, -omega * g);
-  }
-  return v;
+// v at a face after one correction, a at this cell and b at its low neighbour:
+// v - omega (a - b) / dc.  Mixed form: the gradient in float32, as the form's
+// contract has it.
+__device__ __forceinline__ ff face_mixed(ff v, float a, float b, float idc, float omega) {
+  const float g = (a - b) * idc;
+  return ff_add_f(v, -omega * g);
 }
 
-// Float-float form: the differences of float32 values are exact sums of two
-// floats; they are added (|phi| falls by ~1e-6 per pass, so one TwoSum per
-// step keeps ~2^-48 of the first), then one product with omega / dc and one
-// subtraction: with the full TwoSum of both parts where v is returned, stored
-// or decides the last correction (ACC), else with the lower parts added in
-// float32.
-template <int NS, bool ACC>
-__device__ __forceinline__ ff face_ff(ff v, const float (&a)[NS], const float (&b)[NS], float2 idc) {
-  ff d = two_sum(a[0], -b[0]);
-#pragma unroll
-  for (int s = 1; s < NS; ++s) {
-    const ff t = two_sum(a[s], -b[s]);
-    const ff u = two_sum(d.hi, t.hi);
-    d = {u.hi, u.lo + (d.lo + t.lo)};
-  }
-  ff g;
-  g.hi = d.hi * idc.x;
-  g.lo = fma_f(d.hi, idc.x, -g.hi);
-  g.lo = fma_f(d.hi, idc.y, g.lo);
-  g.lo = fma_f(d.lo, idc.x, g.lo);
-  if (ACC) return ff_sub(v, fast_two_sum(g.hi, g.lo));
-  const ff u = two_sum(v.hi, -g.hi);
-  return {u.hi, u.lo + (v.lo - g.lo)};     // |lo| may exceed half an ulp of hi
+// Float-float form: the difference of two float32 values is an exact sum of two
+// floats; product and subtraction in float-float.
+__device__ __forceinline__ ff face_ff(ff v, float a, float b, float2 idc, float omega) {
+  ff g = ff_mul(two_sum(a, -b), of2(idc));
+  if (omega != 1.f) g = ff_mul_f(g, omega);
+  return ff_sub(v, g);
 }
 
-// one direction of the divergence: (hi - lo) / dx as an unevaluated sum
-template <bool ACC>
-__device__ __forceinline__ ff div_term(ff h, ff l, float2 idx) {
-  if (ACC) return ff_mul(ff_sub(h, l), of2(idx));
-  const ff d = two_sum(h.hi, -l.hi);
-  const float e = d.lo + (h.lo - l.lo);
-  ff p;
-  p.hi = d.hi * idx.x;
-  p.lo = fma_f(d.hi, idx.x, -p.hi);
-  p.lo = fma_f(d.hi, idx.y, p.lo);
-  p.lo = fma_f(e, idx.x, p.lo);
-  return p;
-}
-
-// the three directions added and rounded to float32
-template <bool ACC>
-__device__ __forceinline__ float div_sum(ff x, ff y, ff z) {
-  if (ACC) return ff_add(ff_add(x, y), z).hi;
-  const ff u = two_sum(x.hi, y.hi), w = two_sum(u.hi, z.hi);
-  return w.hi + (w.lo + u.lo + (x.lo + y.lo + z.lo));
-}
+// one direction of the divergence
+__device__ __forceinline__ ff div_term(ff h, ff l, float2 idx) { return ff_mul(ff_sub(h, l), of2(idx)); }
 
 struct PassArgs {
   MetFF m;
   const float* w32;            // mixed: the predictor
-  float2* vff[2];              // float-float: the predictor in vff[1]; folded states
+  float2* vff[2];              // v after n passes is in vff[(n + 1) & 1], so is the float-float predictor (n = 0)
   const float* phi[4];
   float2* p;
   float* r;
@@ -136,13 +93,9 @@ struct PassArgs {
   const unsigned* fault;
   cudaGraphConditionalHandle h;
   int set_handle, decide;
+  int idx;                     // which of the first three passes, 3: any later one
   int tx, ty, kz;
 };
-
-// omega / dc of the float-float form
-__device__ __forceinline__ float2 scaled(float2 idc, float omega) {
-  return omega == 1.f ? idc : to2(ff_mul_f(of2(idc), omega));
-}
 
 // two adjacent values: one access where VEC (p aligned), else p[0], p[second]
 template <bool VEC>
@@ -169,25 +122,21 @@ __device__ __forceinline__ void load2(const float2* p, int second, float2 (&v)[2
 }
 
 // values of one plane at this thread's two cells
-template <int NS, typename TB>
+template <typename TB>
 struct Plane {
-  float f[NS][2];
-  TB b[3][2];
+  float f[2];                  // the correction
+  TB b[3][2];                  // v
 };
 
-// One pass over the tile: base stored as TB, NS corrections (the last one
-// new); FOLD: v goes to vout and p to m.p; VEC: nx is even, pairs are aligned.
-// Updates this thread's maxima of |phi| (new) and |D v|.  Loads are not
-// predicated: indices are clamped to the grid, and what a wall or a thread
-// beyond the grid loads that way is not used.
-template <bool FF, int NS, typename TB, bool FOLD, bool VEC>
+// One pass over the tile: v stored as TB -> vout with the correction phi, and
+// p_terms corrections, the latest ones, to p (four: the first sum); VEC: nx is
+// even, pairs are aligned.  Updates this thread's maxima of |phi| and |D v|.
+// Loads are not predicated: indices are clamped to the grid, and what a wall or
+// a thread beyond the grid loads that way is not used.
+template <bool FF, typename TB, bool VEC>
 __device__ __forceinline__ void pass_body(const PassArgs& A, const TB* __restrict__ base,
-                                          const float* const (&phi)[NS], float2* __restrict__ vout,
-                                          bool p_first, float& aphi, float& adiv, float2* sh) {
-  // The right-hand side of the usual last solve (the second pass's, or any after
-  // the third) limits how divergence-free the float-float result is: it is
-  // summed in full; the first one's rounding is removed by the next pass.
-  constexpr bool ACC = FF && (NS == 2 || FOLD);
+                                          const float* __restrict__ phi, float2* __restrict__ vout,
+                                          int p_terms, float& aphi, float& adiv, float2* sh) {
   const MetFF& m = A.m;
   const int nx = m.n[0], ny = m.n[1], nz = m.n[2], nc = (int)m.ncell, nxy = nx * ny;
   const int LX = A.tx / 2 + 1;
@@ -200,10 +149,9 @@ __device__ __forceinline__ void pass_body(const PassArgs& A, const TB* __restric
   const float omega = A.cb->omega;
   const int col = in ? j * nx + i : 0;
   const int dx = in && i > 0 ? 1 : 0, dy = in && j > 0 ? nx : 0, d1 = in1 ? 1 : 0;
-  auto load = [&](int k, Plane<NS, TB>& P) {
+  auto load = [&](int k, Plane<TB>& P) {
     const int e = min(k, nz - 1) * nxy + col;
-#pragma unroll
-    for (int s = 0; s < NS; ++s) load2<VEC>(phi[s] + e, d1, P.f[s]);
+    load2<VEC>(phi + e, d1, P.f);
     load2<VEC>(base + 2 * nc + e, d1, P.b[2]);
     if (k < k1) {                             // plane k1: only its low z-faces (the chunk's top)
       load2<VEC>(base + e, d1, P.b[0]);
@@ -216,56 +164,47 @@ __device__ __forceinline__ void pass_body(const PassArgs& A, const TB* __restric
 #pragma unroll
     for (int q = 0; q < 2; ++q)
       if (i + q < nx) {
-        if (FF) cxf[q] = scaled(m.idcf[0][i + q], omega);
+        if (FF) cxf[q] = m.idcf[0][i + q];
         else cx[q] = m.idc[0][i + q];
         dxi[q] = m.idx[0][i + q];
       }
-    if (FF) cyf = scaled(m.idcf[1][j], omega);
+    if (FF) cyf = m.idcf[1][j];
     else cy = m.idc[1][j];
     dyi = m.idx[1][j];
   }
-  auto face = [&](ff b, const float (&a)[NS], const float (&c)[NS], float idc, float2 idcf) -> ff {
-    if constexpr (FF) return face_ff<NS, ACC>(b, a, c, idcf);
-    else return face_mixed<NS>(b, a, c, idc, omega);
+  auto face = [&](TB b, float a, float c, float idc, float2 idcf) -> ff {
+    if constexpr (FF) return face_ff(base_of(b), a, c, idcf, omega);
+    else return face_mixed(base_of(b), a, c, idc, omega);
   };
-  float fz[NS][2];             // the corrections of the plane below
-#pragma unroll
-  for (int s = 0; s < NS; ++s) load2<VEC>(phi[s] + max(k0 - 1, 0) * nxy + col, d1, fz[s]);
+  float fz[2];                 // the correction of the plane below
+  load2<VEC>(phi + max(k0 - 1, 0) * nxy + col, d1, fz);
   ff px[2] = {}, py[2] = {}, vzp[2] = {};    // of the plane whose z-face above is awaited
   const ff zero = {0.f, 0.f};
   // plane k (in cur; k + 1 is fetched into nxt)
-  auto step = [&](int k, Plane<NS, TB>& cur, Plane<NS, TB>& nxt) {
+  auto step = [&](int k, Plane<TB>& cur, Plane<TB>& nxt) {
     // the low neighbours of this plane: fetched one plane ago as other threads'
     // own cells, so near; the next plane itself: far, a plane ahead
-    float fx[NS], fy[NS][2];
+    float fx, fy[2];
     {
       const int e = min(k, nz - 1) * nxy + col;
-#pragma unroll
-      for (int s = 0; s < NS; ++s) {
-        fx[s] = __ldg(phi[s] + (e - dx));
-        load2<VEC>(phi[s] + (e - dy), d1, fy[s]);
-      }
+      fx = __ldg(phi + (e - dx));
+      load2<VEC>(phi + (e - dy), d1, fy);
     }
     if (k < k1) load(k + 1, nxt);
-    float a0[NS], a1[NS], c0[NS], c1[NS];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) { a0[s] = cur.f[s][0]; a1[s] = cur.f[s][1]; }
     // low z-faces of plane k, which close plane k - 1
     ff vz[2] = {zero, zero};
     if (k > 0 && k < nz) {
-#pragma unroll
-      for (int s = 0; s < NS; ++s) { c0[s] = fz[s][0]; c1[s] = fz[s][1]; }
       const float zc = FF ? 0.f : m.idc[2][k];
-      const float2 zcf = FF ? scaled(m.idcf[2][k], omega) : make_float2(0.f, 0.f);
-      vz[0] = face(base_of(cur.b[2][0]), a0, c0, zc, zcf);
-      vz[1] = face(base_of(cur.b[2][1]), a1, c1, zc, zcf);
+      const float2 zcf = FF ? m.idcf[2][k] : make_float2(0.f, 0.f);
+      vz[0] = face(cur.b[2][0], cur.f[0], fz[0], zc, zcf);
+      vz[1] = face(cur.b[2][1], cur.f[1], fz[1], zc, zcf);
     }
     if (k > k0 && own) {
       const float2 dz = m.idx[2][k - 1];
       float d[2];
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        d[q] = div_sum<ACC>(px[q], py[q], div_term<ACC>(vz[q], vzp[q], dz));
+        d[q] = ff_add(ff_add(px[q], py[q]), div_term(vz[q], vzp[q], dz)).hi;
         if (VEC || q == 0 || in1) {
           float a2 = fabsf(d[q]);
           if (!(a2 <= 3e38f)) a2 = __int_as_float(0x7f800000);
@@ -282,15 +221,11 @@ __device__ __forceinline__ void pass_body(const PassArgs& A, const TB* __restric
     }
     if (k == k1) return;
     ff vx[2], vy[2];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) c0[s] = fx[s];
-    vx[0] = face(base_of(cur.b[0][0]), a0, c0, cx[0], cxf[0]);
+    vx[0] = face(cur.b[0][0], cur.f[0], fx, cx[0], cxf[0]);
     if (dx == 0) vx[0] = zero;
-    vx[1] = face(base_of(cur.b[0][1]), a1, a0, cx[1], cxf[1]);
-#pragma unroll
-    for (int s = 0; s < NS; ++s) { c0[s] = fy[s][0]; c1[s] = fy[s][1]; }
-    vy[0] = face(base_of(cur.b[1][0]), a0, c0, cy, cyf);
-    vy[1] = face(base_of(cur.b[1][1]), a1, c1, cy, cyf);
+    vx[1] = face(cur.b[0][1], cur.f[1], cur.f[0], cx[1], cxf[1]);
+    vy[0] = face(cur.b[1][0], cur.f[0], fy[0], cy, cyf);
+    vy[1] = face(cur.b[1][1], cur.f[1], fy[1], cy, cyf);
     if (dy == 0) vy[0] = vy[1] = zero;
     float2* sx = sh + (k & 1) * 3 * kPassThreads;
     float4* sy = reinterpret_cast<float4*>(sx + kPassThreads);
@@ -300,38 +235,40 @@ __device__ __forceinline__ void pass_body(const PassArgs& A, const TB* __restric
     if (own) {
       const ff x2 = i + 2 < nx ? of2(sx[tid + 1]) : zero;
       const float4 y2 = j + 1 < ny ? sy[tid + LX] : make_float4(0.f, 0.f, 0.f, 0.f);
-      px[0] = div_term<ACC>(VEC || in1 ? vx[1] : zero, vx[0], dxi[0]);
-      px[1] = div_term<ACC>(x2, vx[1], dxi[1]);
-      py[0] = div_term<ACC>({y2.x, y2.y}, vy[0], dyi);
-      py[1] = div_term<ACC>({y2.z, y2.w}, vy[1], dyi);
+      px[0] = div_term(VEC || in1 ? vx[1] : zero, vx[0], dxi[0]);
+      px[1] = div_term(x2, vx[1], dxi[1]);
+      py[0] = div_term({y2.x, y2.y}, vy[0], dyi);
+      py[1] = div_term({y2.z, y2.w}, vy[1], dyi);
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        float u = fabsf(cur.f[NS - 1][q]);           // (beyond an odd row: the first cell again)
+        float u = fabsf(cur.f[q]);           // (beyond an odd row: the first cell again)
         if (!(u <= 3e38f)) u = __int_as_float(0x7f800000);
         aphi = fmaxf(aphi, u);
       }
-      if (FOLD) {
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          if (q == 1 && !in1) break;
-          const int e = k * nxy + col + q;
-          const ff o[3] = {vx[q], vy[q], vz[q]};
-#pragma unroll
-          for (int c = 0; c < 3; ++c)
-            vout[c * nc + e] = to2(o[c]);
-          ff w = p_first ? ff{omega * cur.f[0][q], 0.f} : ff_add_f(of2(A.p[e]), omega * cur.f[0][q]);
-#pragma unroll
-          for (int s = 1; s < NS; ++s) w = ff_add_f(w, omega * cur.f[s][q]);
-          A.p[e] = to2(w);
+      for (int c = 0; c < 3; ++c) {
+        const ff(&o)[2] = c == 0 ? vx : c == 1 ? vy : vz;
+        float2* d = vout + c * nc + k * nxy + col;
+        if (VEC) {
+          *reinterpret_cast<float4*>(d) = make_float4(o[0].hi, o[0].lo, o[1].hi, o[1].lo);
+        } else {
+          d[0] = to2(o[0]);
+          if (in1) d[1] = to2(o[1]);
         }
+      }
+      for (int q = 0; q < (p_terms ? in1 ? 2 : 1 : 0); ++q) {
+        const int e = k * nxy + col + q;
+        ff w = p_terms == 1 ? of2(A.p[e]) : ff{0.f, 0.f};
+        for (int s = 4 - p_terms; s < 4; ++s) w = ff_add_f(w, omega * __ldg(A.phi[s] + e));
+        A.p[e] = to2(w);
       }
     }
 #pragma unroll
     for (int q = 0; q < 2; ++q) vzp[q] = vz[q];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) { fz[s][0] = cur.f[s][0]; fz[s][1] = cur.f[s][1]; }
+    fz[0] = cur.f[0];
+    fz[1] = cur.f[1];
   };
-  Plane<NS, TB> P0, P1;
+  Plane<TB> P0, P1;
   load(k0, P0);
   for (int k = k0; k <= k1; k += 2) {
     step(k, P0, P1);
@@ -361,9 +298,9 @@ __device__ void decide(const PassArgs& A, float a, float d) {
   if (A.set_handle) cudaGraphSetConditional(A.h, go ? 1u : 0u);
 }
 
-// IDX 0, 1, 2: the first three passes (a loop that ended earlier leaves them
-// at once); 3: any later one.
-template <bool FF, int IDX, bool VEC>
+// A loop that ended before the pass leaves it at once.  FIRST: the first pass of
+// the mixed form, whose predictor is float32.
+template <bool FF, bool FIRST, bool VEC>
 __global__ void __launch_bounds__(kPassThreads, 2) k_pass(PassArgs A) {
   __shared__ __align__(16) float2 sh[6 * kPassThreads];
   __shared__ float red[32];
@@ -371,25 +308,12 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_pass(PassArgs A) {
   tc5::pdl_trigger();   // the pressure transform that follows may start its set-up
   if (A.decide && A.ls->status != 0) return;   // ended before this pass
   float aphi = 0.f, adiv = 0.f;
-  if constexpr (IDX < 3) {
-    const float* phi[IDX + 1];
-#pragma unroll
-    for (int s = 0; s <= IDX; ++s) phi[s] = A.phi[s];
-    if constexpr (FF) pass_body<true, IDX + 1, float2, false, VEC>(A, A.vff[1], phi, nullptr, true, aphi, adiv, sh);
-    else pass_body<false, IDX + 1, float, false, VEC>(A, A.w32, phi, nullptr, true, aphi, adiv, sh);
-  } else {
-    const int done = A.ls->pass;               // the result of fold f is in vff[f & 1], f = pass - 3
-    if (done == 3) {
-      const float* phi[4] = {A.phi[0], A.phi[1], A.phi[2], A.phi[3]};
-      if constexpr (FF) pass_body<true, 4, float2, true, VEC>(A, A.vff[1], phi, A.vff[0], true, aphi, adiv, sh);
-      else pass_body<false, 4, float, true, VEC>(A, A.w32, phi, A.vff[0], true, aphi, adiv, sh);
-    } else {
-      const float* phi[1] = {A.phi[3]};
-      const bool odd = (done & 1) != 0;
-      pass_body<FF, 1, float2, true, VEC>(A, odd ? A.vff[1] : A.vff[0], phi, odd ? A.vff[0] : A.vff[1], false, aphi,
-                                     adiv, sh);
-    }
-  }
+  const int done = A.idx < 3 ? A.idx : A.ls->pass;
+  const float2* vin = A.vff[(done + 1) & 1];
+  float2* vout = A.vff[done & 1];
+  const int p_terms = A.idx < 3 ? 0 : done == 3 ? 4 : 1;
+  if constexpr (FIRST) pass_body<FF, float, VEC>(A, A.w32, A.phi[0], vout, p_terms, aphi, adiv, sh);
+  else pass_body<FF, float2, VEC>(A, vin, A.phi[A.idx], vout, p_terms, aphi, adiv, sh);
   aphi = block_max(aphi, red);
   adiv = block_max(adiv, red);
   if (!A.decide) return;
@@ -418,8 +342,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_pass(PassArgs A) {
 }
 
 struct JoinArgs {
-  MetFF m;
-  const float* w32;
+  int n[3];
   const float2* vff[2];
   const float* phi[3];
   const float2* p;
@@ -428,80 +351,47 @@ struct JoinArgs {
   int kz;                  // planes per thread
 };
 
-// out = v - sigma x, p_out = p (float64): v and p from the terms that hold them
-template <bool FF, int NS>
-__device__ __forceinline__ void join_body(const JoinArgs& A) {
-  const MetFF& m = A.m;
+// out = v - sigma x, p_out = p (float64): the last v; p from the corrections, or
+// from where the fourth and later passes have summed them
+__global__ void __launch_bounds__(kCellThreads) k_join(JoinArgs A) {
+  const int pass = A.ls->pass;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && A.ls->status > A.ls->worst)
+    A.ls->worst = A.ls->status;
   const double* x = A.cb->x;
   double* out = A.cb->out;
   double* pout = A.cb->p;
   const float sigma = A.cb->sigma, omega = A.cb->omega;
-  const int nx = m.n[0], ny = m.n[1], nz = m.n[2], nc = (int)m.ncell, nxy = nx * ny;
+  const int nxy = A.n[0] * A.n[1], nz = A.n[2], nc = nxy * nz;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nxy) return;
-  const int i = t % nx, j = t / nx;
-  const int pos2[2] = {i, j}, st[3] = {1, nx, nxy};
-  const int pass = A.ls->pass;
-  const float2* v = A.vff[pass & 1];          // NS == 0: the last fold
+  const float2* v = pass & 1 ? A.vff[0] : A.vff[1];
 #pragma unroll 1
   for (int k = blockIdx.y * A.kz; k < min(nz, (int)(blockIdx.y + 1) * A.kz); ++k) {
     const int e = k * nxy + t;
-    float f[NS > 0 ? NS : 1];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) f[s] = __ldg(A.phi[s] + e);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const int q = c < 2 ? pos2[c] : k;
-      ff a = {0.f, 0.f};
-      if (q > 0) {
-        if constexpr (NS == 0) {
-          a = of2(v[c * nc + e]);
-        } else {
-          float g[NS];
-#pragma unroll
-          for (int s = 0; s < NS; ++s) g[s] = __ldg(A.phi[s] + e - st[c]);
-          if constexpr (FF) {
-            a = face_ff<NS, true>(of2(__ldg(A.vff[1] + c * nc + e)), f, g, scaled(m.idcf[c][q], omega));
-          } else {
-            a = face_mixed<NS>({__ldg(A.w32 + c * nc + e), 0.f}, f, g, m.idc[c][q], omega);
-          }
-        }
-      }
+      ff a = of2(__ldg(v + c * nc + e));
       if (sigma != 0.f) a = ff_sub(a, ff_mul_f(f64_split(__ldg(x + c * nc + e)), sigma));
       out[c * nc + e] = ff_join(a.hi, a.lo);
     }
     if (pout) {
-      ff q;
-      if constexpr (NS == 0) {
-        q = of2(A.p[e]);
-      } else {
-        q = {omega * f[0], 0.f};
+      ff q = {0.f, 0.f};
+      if (pass > 3) q = of2(A.p[e]);
 #pragma unroll
-        for (int s = 1; s < NS; ++s) q = ff_add_f(q, omega * f[s]);
-      }
+      for (int s = 0; s < 3; ++s)
+        if (s < pass && pass <= 3) q = ff_add_f(q, omega * __ldg(A.phi[s] + e));
       pout[e] = ff_join(q.hi, q.lo);
     }
   }
 }
 
-template <bool FF>
-__global__ void __launch_bounds__(kCellThreads) k_join(JoinArgs A) {
-  const int pass = A.ls->pass;
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && A.ls->status > A.ls->worst)
-    A.ls->worst = A.ls->status;
-  if (pass == 3) join_body<FF, 3>(A);
-  else if (pass == 2) join_body<FF, 2>(A);
-  else if (pass == 1) join_body<FF, 1>(A);
-  else join_body<FF, 0>(A);
-}
-
-template <bool FF, int IDX, bool VEC>
+template <bool FF, bool FIRST, bool VEC>
 fv_status run_pass_v(const PassArgs& A0, cudaStream_t s) {
   PassArgs A = A0;
   static int per_sm = 0;       // residency of the kernel, the same for every grid
   if (!per_sm) {
     int q = 0;
-    FV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, k_pass<FF, IDX, VEC>, kPassThreads, 0));
+    FV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, k_pass<FF, FIRST, VEC>, kPassThreads, 0));
     per_sm = q < 1 ? 1 : q;
   }
   // tiles of at most 64 cells along x that split it evenly; rows per tile and
@@ -530,14 +420,14 @@ fv_status run_pass_v(const PassArgs& A0, cudaStream_t s) {
   }
   const dim3 grid(ntx, nty, (n[2] + A.kz - 1) / A.kz);
   const int thr = (LX * (A.ty + 1) + 31) / 32 * 32;
-  k_pass<FF, IDX, VEC><<<grid, thr, 0, s>>>(A);
+  k_pass<FF, FIRST, VEC><<<grid, thr, 0, s>>>(A);
   FV_CHECK_LAUNCH();
   return FV_OK;
 }
 
-template <bool FF, int IDX>
+template <bool FF, bool FIRST>
 fv_status run_pass(const PassArgs& A, cudaStream_t s) {
-  return A.m.n[0] % 2 == 0 ? run_pass_v<FF, IDX, true>(A, s) : run_pass_v<FF, IDX, false>(A, s);
+  return A.m.n[0] % 2 == 0 ? run_pass_v<FF, FIRST, true>(A, s) : run_pass_v<FF, FIRST, false>(A, s);
 }
 
 }  // namespace
@@ -560,33 +450,26 @@ fv_status launch_pass(const fv_grid* g, int prec, int idx, const CallBlock* cb, 
   A.set_handle = h ? 1 : 0;
   A.decide = decide ? 1 : 0;
   LaunchScope ls_(g, FV_K_CORRECT);
-  if (prec == FV_FF) {
-    if (idx == 0) return run_pass<true, 0>(A, g->stream);
-    if (idx == 1) return run_pass<true, 1>(A, g->stream);
-    if (idx == 2) return run_pass<true, 2>(A, g->stream);
-    return run_pass<true, 3>(A, g->stream);
-  }
-  if (idx == 0) return run_pass<false, 0>(A, g->stream);
-  if (idx == 1) return run_pass<false, 1>(A, g->stream);
-  if (idx == 2) return run_pass<false, 2>(A, g->stream);
-  return run_pass<false, 3>(A, g->stream);
+  A.idx = idx;
+  if (prec == FV_FF) return run_pass<true, false>(A, g->stream);
+  if (idx == 0) return run_pass<false, true>(A, g->stream);
+  return run_pass<false, false>(A, g->stream);
 }
 
-fv_status launch_join(const fv_grid* g, int prec, const CallBlock* cb, LoopState* ls) {
+fv_status launch_join(const fv_grid* g, const CallBlock* cb, LoopState* ls) {
   JoinArgs A;
-  A.m = g->met_ff;
-  A.w32 = g->w32;
+  for (int d = 0; d < 3; ++d) {
+    A.n[d] = g->n[d];
+    A.phi[d] = g->phis[d];
+  }
   A.vff[0] = g->vff[0];
   A.vff[1] = g->vff[1];
-  for (int s = 0; s < 3; ++s) A.phi[s] = g->phis[s];
   A.p = g->pff;
   A.cb = cb;
   A.ls = ls;
   A.kz = cell_planes(g);
-  const int thr = cell_threads(g);
   LaunchScope ls_(g, FV_K_VECTOR);
-  if (prec == FV_FF) k_join<true><<<cell_grid_fit(g), thr, 0, g->stream>>>(A);
-  else k_join<false><<<cell_grid_fit(g), thr, 0, g->stream>>>(A);
+  k_join<<<cell_grid_fit(g), cell_threads(g), 0, g->stream>>>(A);
   FV_CHECK_LAUNCH();
   return FV_OK;
 }
