@@ -10,17 +10,29 @@
 // 2^-24 of the product.  Six BF16 products cost what three TF32 ones do, carry
 // two more bits and need 6 instead of 8 bytes of shared memory per element.
 //
+// The tensor core cuts off what a sum has beyond float32 (an FP32 FMA rounds), so
+// every addition to an accumulator takes up to an ulp of it away: 6 n / 16 of
+// them, all in one accumulator, made the solution 3e-6 .. 5e-6 of its largest
+// value wrong (sine map, 150^3), five times what the FP32 kernel's sums of n
+// terms did.  So h h, which carries the value, has an accumulator of its own
+// (n / 16 additions), cut in two halves of K where tensor memory has room for
+// three, and the five small products share another, whose cuts are 2^-8 of
+// that; the epilogue adds them.  Error of the first correction against float64,
+// relative to the FP32 kernels' (113 .. 520 cells, cosine and sine map): 0.15 ..
+// 0.7 in the mean square, 0.15 .. 1.2 in the largest.
+//
 // One block: 128 K-vectors of the field (the M side, one tensor-memory lane
-// each) and up to 256 rows of M (the N side, the columns).  K streams through
-// a ring of 16-entry chunks: the chunk of the pre-split matrix by a bulk copy,
-// the chunk of the field through registers (loaded two chunks ahead, split and
-// stored by eight warps).  A ninth warp issues the products, a tenth the
-// copies.  Two blocks per SM, so that one's epilogue overlaps the other's
-// products.  Measured: 16 us (y, z) and 27 us (x, whose 600-byte rows are not
-// 16-byte aligned) a transform at 150^3 against 44-55 us for the FP32 kernel it
-// replaces, 45 and 66 us at 256^3 (field read + write: 20 us at the measured
-// HBM rate; products: 22 us at the tensor rate, 512 blocks in 1.7 waves); a
-// float-float evaluation 1642 -> 1069 us and 7742 -> 4216 us.
+// each) and a chunk of the rows of M (the N side, the columns).  K streams
+// through a ring of 16-entry chunks: the chunk of the pre-split matrix by a bulk
+// copy, the chunk of the field through registers (loaded two turns ahead, split
+// and stored by two sets of eight warps in turn).  One more warp issues the
+// products, another the copies.  Chunks of up to 128 rows let two blocks share
+// an SM, so that one's epilogue overlaps the other's products; from 161 to 256
+// rows one chunk, one block per SM, since splitting the field twice costs more
+// (256^3 3860 us against 3980, 192^3 2255 against 2331; 150^3 1033 us with two
+// chunks of 80 rows against 1048 with one).  A float-float evaluation at 150^3 takes
+// 1033 us and at 256^3 3864 us, 1606 and 7730 with the FP32 kernels this replaces; with
+// all products in one accumulator it took 924 and 3631.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -34,17 +46,20 @@ namespace fv {
 
 namespace {
 
-constexpr int kXWorkers = 8;
+constexpr int kXGroups = 2;            // sets of eight warps that take the chunks in turn
+constexpr int kXWorkers = 8 * kXGroups;
 constexpr int kXThreads = 32 * (kXWorkers + 2);
-constexpr int kXRows = 256;            // rows of M per block at most
-constexpr int kXStages = 3;
+constexpr int kXStages = 4;
 constexpr int kXABytes = 3 * 128 * 16 * 2;
 constexpr int kXLimit = 1 << 22;       // polls of an mbarrier before the block gives up
 
 __host__ __device__ inline int up16(int n) { return (n + 15) & ~15; }
-// rows of M in chunk y of blockIdx.y (padded to a multiple of 16, all equal)
-__host__ __device__ inline int chunks_of(int n) { return (up16(n) + kXRows - 1) / kXRows; }
+// rows of M per block at most, chunks of them, rows of a chunk (a multiple of 16, all equal)
+__host__ __device__ inline int max_rows(int n) { return up16(n) > 160 && up16(n) <= 256 ? 256 : 128; }
+__host__ __device__ inline int chunks_of(int n) { return (up16(n) + max_rows(n) - 1) / max_rows(n); }
 __host__ __device__ inline int chunk_rows(int n) { return up16((n + chunks_of(n) - 1) / chunks_of(n)); }
+// accumulators of N columns: three where two blocks of an SM still fit its 512
+__host__ __device__ inline int accs(int N) { return 3 * N <= 256 ? 3 : 2; }
 inline size_t xf_smem(int n) { return (size_t)kXStages * (kXABytes + 96 * chunk_rows(n)); }
 
 struct XfArgs {
@@ -75,14 +90,16 @@ __global__ void __launch_bounds__(kXThreads, 2) k_xf(XfArgs A) {
   __shared__ uint32_t tslot;
   __shared__ int bad;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n = A.n, nk = (n + 15) >> 4, N = chunk_rows(n), p0 = blockIdx.y * N;
+  const int n = A.n, nk = (n + 15) >> 4, N = chunk_rows(n), nch = chunks_of(n);
+  const int chunk = (int)(blockIdx.x % (unsigned)nch), p0 = chunk * N;
+  const int nkh = accs(N) == 3 ? (nk + 1) / 2 : nk;   // chunks whose h h goes to the first accumulator
   const int bbytes = 96 * N, sbytes = kXABytes + bbytes;
-  const int64_t v0 = (int64_t)blockIdx.x * 128;
-  const unsigned char* mat = A.mat + (size_t)blockIdx.y * nk * bbytes;
+  const int64_t v0 = (int64_t)(blockIdx.x / (unsigned)nch) * 128;
+  const unsigned char* mat = A.mat + (size_t)chunk * nk * bbytes;
   if (tid == 0) {
     for (int s = 0; s < kXStages; ++s) {
       tc5::mbar_init(&full[s], 1);
-      tc5::mbar_init(&ready[s], kXWorkers);
+      tc5::mbar_init(&ready[s], 8);
       tc5::mbar_init(&empty[s], 1);
     }
     tc5::mbar_init(&done, 1);
@@ -111,8 +128,9 @@ __global__ void __launch_bounds__(kXThreads, 2) k_xf(XfArgs A) {
     // this thread's vector and its 8-entry run of every chunk.  LEFT: a warp
     // reads 32 consecutive vectors; RIGHT: 16 vectors x 2 runs (64 contiguous
     // bytes each).  Eight consecutive lanes fill a core matrix either way.
-    const int vl = RIGHT ? 16 * warp + (lane & 15) : 32 * (warp & 3) + lane;
-    const int run = RIGHT ? lane >> 4 : warp >> 2;
+    const int w8 = warp & 7, grp = warp >> 3;
+    const int vl = RIGHT ? 16 * w8 + (lane & 15) : 32 * (w8 & 3) + lane;
+    const int run = RIGHT ? lane >> 4 : w8 >> 2;
     const int64_t v = v0 + vl;
     const bool ok = v < A.nvec;
     const float* src = A.in;
@@ -133,8 +151,8 @@ __global__ void __launch_bounds__(kXThreads, 2) k_xf(XfArgs A) {
         for (int q = 0; q < 8; ++q) y[q] = (ok && k + q < n) ? __ldg(src + (k + q) * sk) : 0.f;
       }
     };
-    load(0, x[0]);
-    if (nk > 1) load(1, x[1]);
+    if (grp < nk) load(grp, x[0]);
+    if (grp + kXGroups < nk) load(grp + kXGroups, x[1]);
     bool live = true;
     auto step = [&](int c, float (&y)[8]) {
       uint32_t w[3][4];
@@ -145,7 +163,7 @@ __global__ void __launch_bounds__(kXThreads, 2) k_xf(XfArgs A) {
         w[1][q] = split2(a, b);
         w[2][q] = split2(a, b);
       }
-      if (c + 2 < nk) load(c + 2, y);
+      if (c + 2 * kXGroups < nk) load(c + 2 * kXGroups, y);
       const int st = c % kXStages, use = c / kXStages;
       // the products that read this stage before are done
       if (use > 0) live = tc5::mbar_wait(&empty[st], (uint32_t)(use - 1) & 1u, kXLimit) && live;
@@ -157,9 +175,9 @@ __global__ void __launch_bounds__(kXThreads, 2) k_xf(XfArgs A) {
       __syncwarp();
       if (lane == 0) tc5::mbar_arrive(&ready[st]);
     };
-    for (int c = 0; c < nk; c += 2) {
+    for (int c = grp; c < nk; c += 2 * kXGroups) {
       step(c, x[0]);
-      if (c + 1 < nk) step(c + 1, x[1]);
+      if (c + kXGroups < nk) step(c + kXGroups, x[1]);
     }
     if (!live) bad = 1;
   } else if (warp == kXWorkers && lane == 0) {
@@ -173,12 +191,14 @@ __global__ void __launch_bounds__(kXThreads, 2) k_xf(XfArgs A) {
       ok = tc5::mbar_wait(&ready[st], ph, kXLimit) && ok;
       tc5::fence_after_sync();
       const uint32_t a = base + st * sbytes, b = a + kXABytes;
+      const bool first = c == 0 || c == nkh;   // of a main accumulator
 #pragma unroll
       for (int s = 2; s >= 0; --s)             // small products first
 #pragma unroll
         for (int i = 0; i <= s; ++i)
-          tc5::mma_f16(tmem, tc5::sdesc(a + i * 4096, 128, 256), tc5::sdesc(b + (s - i) * 32 * N, 128, 256),
-                       idesc, c == 0 && s == 2 && i == 0 ? 0u : 1u);
+          tc5::mma_f16(tmem + (uint32_t)(s ? N : c < nkh ? 0 : 2 * N), tc5::sdesc(a + i * 4096, 128, 256),
+                       tc5::sdesc(b + (s - i) * 32 * N, 128, 256), idesc,
+                       (s == 0 ? first : s == 2 && i == 0 && c == 0) ? 0u : 1u);
       tc5::commit(&empty[st]);
     }
     tc5::commit(&done);
@@ -201,8 +221,8 @@ __global__ void __launch_bounds__(kXThreads, 2) k_xf(XfArgs A) {
     const int64_t v = v0 + 32 * (warp & 3) + lane;
     const bool ok = v < A.nvec;
     const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
-    const int half = (N / 8 + 1) / 2 * 8;
-    const int c_begin = warp < 4 ? 0 : half, c_end = warp < 4 ? half : N;
+    const int per = (N / 8 + kXWorkers / 4 - 1) / (kXWorkers / 4) * 8;
+    const int c_begin = min(N, (warp >> 2) * per), c_end = min(N, c_begin + per);
     float* o = A.out;
     if (ok) o += RIGHT ? v * n : (v / A.Q) * n * A.Q + v % A.Q;
     float lq = 0.f;
@@ -215,13 +235,21 @@ __global__ void __launch_bounds__(kXThreads, 2) k_xf(XfArgs A) {
     const bool vec4 = RIGHT && (n & 3) == 0 && ((uintptr_t)A.out & 15) == 0;
     const bool vec2 = RIGHT && (n & 1) == 0 && ((uintptr_t)A.out & 7) == 0;
     for (int c = c_begin; c < c_end; c += 8) {
-      float y[8];
+      float y[8], z[8];
       __syncwarp();   // tcgen05.ld is warp-collective
       tc5::ld8(trow + (uint32_t)c, y);
+      tc5::ld8(trow + (uint32_t)(N + c), z);
+      if (nkh < nk) {
+        float y2[8];
+        tc5::ld8(trow + (uint32_t)(2 * N + c), y2);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) y[q] += y2[q];
+      }
       const int p = p0 + c;
       if (!ok || p >= n) continue;
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
+        y[q] += z[q];
         if (SCALE) {
           const float l = p + q < n ? __ldg(A.lz + p + q) : 1.f;
           y[q] = (nullq && p + q == A.null_z) ? 0.f : y[q] / (l + lq);
@@ -306,7 +334,7 @@ fv_status build_xf(fv_grid* g) {
   FV_CUDA(cudaMemcpy(g->d_xf, h.data(), bytes, cudaMemcpyHostToDevice));
   for (int d = 0; d < 3; ++d)
     for (int q = 0; q < 2; ++q) g->xf[d][q] = (const unsigned char*)g->d_xf + off[d][q];
-  const int cap = (int)xf_smem(kXRows);
+  const int cap = (int)xf_smem(256);
   FV_CUDA(cudaFuncSetAttribute(k_xf<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   FV_CUDA(cudaFuncSetAttribute(k_xf<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   FV_CUDA(cudaFuncSetAttribute(k_xf<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
@@ -330,10 +358,10 @@ static fv_status xf_transform(const fv_grid* g, int axis, int inverse, bool scal
   A.nvec = g->ncell / A.n;
   A.Q = axis == 0 ? 1 : axis == 1 ? g->n[0] : (int64_t)g->n[0] * g->n[1];
   A.tcols = 32;
-  while ((int)A.tcols < chunk_rows(A.n)) A.tcols <<= 1;
+  while ((int)A.tcols < accs(chunk_rows(A.n)) * chunk_rows(A.n)) A.tcols <<= 1;
   A.fault = g->d_fault;
   A.skip = skip;
-  const dim3 grid((unsigned)((A.nvec + 127) / 128), (unsigned)chunks_of(A.n));
+  const dim3 grid((unsigned)((A.nvec + 127) / 128 * chunks_of(A.n)));
   const size_t smem = xf_smem(A.n);
   LaunchScope ls_(g, axis == 0 ? FV_K_TPF_X : FV_K_TPF_YZ);
   if (axis == 0) FV_CUDA(tc5::launch_pdl(k_xf<true, false>, grid, dim3(kXThreads), smem, g->stream, A));
