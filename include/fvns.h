@@ -46,9 +46,18 @@ typedef enum {
   FV_ECUDA = 3,    /* a CUDA call failed (message in fv_last_error) */
   FV_ENOCONV = 4,  /* an iteration cap was reached */
   FV_ENAN = 5,     /* a NaN/Inf appeared in a norm */
-  FV_ETIMEOUT = 6  /* a bounded device-side wait gave up (the tensor-core
-                      pressure transforms of FV_MIXED / FV_FF); the grid's
-                      sticky timeout word is cleared once reported */
+  FV_ETIMEOUT = 6  /* a bounded device-side wait gave up: in a tensor-core
+                      transform (FV_MIXED, FV_FF, and FV_FP64 along axes of at
+                      most 128 cells) or in the Gram-Schmidt step of a Krylov
+                      driver.  What the kernel had to write is NaN and the
+                      grid's timeout word is set; the word stays set until a
+                      call reports it, once.  Calls that report it: FV_MIXED
+                      and FV_FF evaluations that synchronise, batched ones, the
+                      Krylov drivers, and an FV_FP64 evaluation that meets a
+                      NaN.  Calls that only queue work (fv_pressure_solve,
+                      fv_plane_projection, async evaluations) return before it
+                      can be known: the next reporting call on the grid gives
+                      it, even if its own work went well */
 } fv_status;
 
 /* Grid stretching.  Section 3, Eq. 5: x -> x - 0.0975 sin(2 pi x) applied to
@@ -401,7 +410,8 @@ fv_status simple_krylov_solve_guess(const fv_grid* g, fv_unet* u, const double* 
  * axes and n along the normal one (e.g. (nz+1) x ny x (nx+1) for plane 0),
  * zero on the walls, with v_1 = rot(0, Psi, 0), v_2 = rot(Psi, 0, 0),
  * v_3 = rot(0, 0, Psi).  Wall entries of v are ignored.  v and vp may not
- * alias.  float64 throughout. */
+ * alias.  float64 throughout.  The work is queued and not waited for (see
+ * FV_ETIMEOUT). */
 fv_status fv_plane_projection(const fv_grid* g, const double* v, int plane, double* vp,
                               double* psi);
 
@@ -410,7 +420,8 @@ fv_status fv_plane_projection(const fv_grid* g, const double* v, int plane, doub
 fv_status fv_dot_w(const fv_grid* g, const double* a, const double* b, double* out /* host */);
 
 /* Section 3 step 1 alone: phi[n_cell] = zero-mean solution of D G phi = r
- * (Neumann) by the tensor-product factorisation; prec as above. */
+ * (Neumann) by the tensor-product factorisation; prec as above.  The work is
+ * queued and not waited for (see FV_ETIMEOUT). */
 fv_status fv_pressure_solve(const fv_grid* g, const double* r, double* phi, int prec);
 
 /* Section 3 step 1 by multigrid: phi[n_cell] (device, float64) = the
@@ -497,10 +508,9 @@ fv_status fv_profile_read(fv_grid* g, double* ms /* host, FV_NKIND */,
 int64_t fv_launch_count(void);
 /* Error-path testing without a device fault: set the grid's sticky device
  * timeout word exactly as a tensor-core pressure transform does when one of
- * its bounded mbarrier waits gives up, so that the next FV_MIXED / FV_FF
- * evaluation (or Krylov cycle) on the grid reports FV_ETIMEOUT.  Only
- * status == FV_ETIMEOUT is accepted (else FV_EINVAL).  Queued on the grid's
- * stream. */
+ * its bounded mbarrier waits gives up, so that the next call on the grid that
+ * reports it (see FV_ETIMEOUT) does.  Only status == FV_ETIMEOUT is accepted
+ * (else FV_EINVAL).  Queued on the grid's stream. */
 fv_status fv_debug_inject_status(fv_grid* g, int status);
 /* Time `reps` back-to-back launches of one FV_MIXED kernel class
  * (FV_K_MOMENTUM, FV_K_DIVERGENCE, FV_K_CORRECT, FV_K_TPF_X = one forward

@@ -259,7 +259,7 @@ fv_status mixed_krylov_graph(const fv_grid* gcst, const double* U, const double*
   if (phil) *phil = hls.phi_last;
   if (divl) *divl = hls.div_last;
   if (status) *status = hls.status;
-  if (hls.status == 4) FV_CUDA(cudaMemset(g->d_fault, 0, sizeof(unsigned)));   // reported once
+  if (hls.status == 4) FV_CUDA(cudaMemsetAsync(g->d_fault, 0, sizeof(unsigned), g->stream));   // reported once
   return FV_OK;
 }
 
@@ -277,7 +277,8 @@ fv_status status_error(int status) {
     case 2: set_error("SIMPLE loop reached max_pass"); return FV_ENOCONV;
     case 3: set_error("SIMPLE loop: NaN/Inf in the correction"); return FV_ENAN;
     case 4:
-      set_error("a bounded wait of a pressure transform or a Gram-Schmidt step gave up (device timeout)");
+      set_error("a bounded wait of a pressure transform or a Gram-Schmidt step gave up (device timeout), in this "
+                "call or in one queued before it on the grid");
       return FV_ETIMEOUT;
     default: return FV_OK;
   }
