@@ -512,6 +512,13 @@ int64_t fv_launch_count(void);
  * reports it (see FV_ETIMEOUT) does.  Only status == FV_ETIMEOUT is accepted
  * (else FV_EINVAL).  Queued on the grid's stream. */
 fv_status fv_debug_inject_status(fv_grid* g, int status);
+/* One Gram-Schmidt step of the Krylov drivers as they run it in float-float
+ * arithmetic: w[n_vel] against the j1 <= 128 W-orthonormal columns of V (device,
+ * n_vel apart), twice.  h (host) receives the j1 coefficients and the norm of
+ * what is left.  pairs = 0: V holds float64 and w becomes the new vector, as in
+ * newton_steady; 1: V holds float-float pairs and its column j1 becomes the new
+ * vector, as in arnoldi_leading.  Synchronises. */
+fv_status fv_debug_gram_schmidt(fv_grid* g, void* V, int pairs, int j1, double* w, double* h /* host */);
 /* Time `reps` back-to-back launches of one FV_MIXED kernel class
  * (FV_K_MOMENTUM, FV_K_DIVERGENCE, FV_K_CORRECT, FV_K_TPF_X = one forward
  * x-y slab transform, FV_K_TPF_XINV = one inverse x-y slab transform,

@@ -14,8 +14,9 @@
 //   partial products (w, v) | one block per v sums them | update, partial
 //   products again | sums | update, partial norm | norm, scaling.
 // A wait at a barrier is bounded; a block that gives up raises the grid's
-// fault flag, still arrives at the barriers that are left, and the step's
-// results are NaN.
+// timeout word and still arrives at the barriers that are left.  With the word
+// set the coefficients, the norm and the new vector are NaN (of a block that
+// gives up at the last barrier only: its slice).
 #include <algorithm>
 
 #include "fv_ff.cuh"
@@ -245,24 +246,24 @@ __global__ void __launch_bounds__(kGsThreads) k_cgs2(GsArgs A) {
   __shared__ double norm;
   if (warp == 0) {
     double s = gather(A, 0);
-    if (!ok) s = __longlong_as_double(0x7ff8000000000000ll);
+    if (!ok || *reinterpret_cast<const volatile unsigned*>(A.fault)) s = __longlong_as_double(0x7ff8000000000000ll);
     if (lane == 0) norm = s < 0.0 ? 0.0 : sqrt(s);
   }
   __syncthreads();
-  const double hn = norm, sc = hn > 0.0 || isnan(hn) ? 1.0 / hn : 0.0;
+  const double hn = norm, sc = hn == 0.0 ? 0.0 : 1.0 / hn;
   if (blockIdx.x == 0) {
     if (!A.norm_only)
       for (int v = tid; v < A.j1; v += kGsThreads)
-        A.hcol[(int64_t)v * A.ldh] = __ldcg(A.h + v) + __ldcg(A.h + kGsMaxVec + v);
+        A.hcol[(int64_t)v * A.ldh] = isnan(hn) ? hn : __ldcg(A.h + v) + __ldcg(A.h + kGsMaxVec + v);
     if (tid == 0) {
       A.hcol[(int64_t)A.j1 * A.ldh] = hn;
       if (A.scale) *A.scale = sc;
     }
   }
-  const double m = A.scale_w && hn > 0.0 ? sc : 1.0;
+  const double m = isnan(hn) || (A.scale_w && hn != 0.0) ? sc : 1.0;
   for (int e = tid; e < cnt; e += kGsThreads) {
     const double x = ff_join(ws[e].x, ws[e].y);
-    A.w[e0 + e] = A.scale_w ? m * x : x;
+    A.w[e0 + e] = m * x;
     if (A.colf) {
       const ff s = f64_split_trunc(sc * x);
       A.colf[e0 + e] = make_float2(s.hi, s.lo);
@@ -273,11 +274,12 @@ __global__ void __launch_bounds__(kGsThreads) k_cgs2(GsArgs A) {
 }  // namespace
 
 // Blocks and entries per block of a step on this grid; false beyond
-// kGsMaxSlice.  Leading eigenvalue with m = 40, this kernel against the
-// separate ones: 40^3 387 / 446 ms, 48^3 602 / 646, 52^3 784 / 826 (2776 entries
-// per block), 56^3 1471 / 1391 (3468), 64^3 2032 / 1711: a basis beyond L2 is
-// better streamed by three blocks per SM with asynchronous copies.  Newton at
-// 16^3: 449 ms with the separate kernels, 344 with this one.
+// kGsMaxSlice.  Leading eigenvalues with m = 40, microseconds per new vector, this
+// kernel against the separate ones (runs of the same input repeat to 0.1 %):
+// 16^3 127 / 158, 32^3 163 / 191, 40^3 197 / 228, 48^3 252 / 276, 52^3 316 / 324
+// (2776 entries per block), 56^3 376 / 350 (3468), 64^3 525 / 441: a basis beyond
+// L2 is better streamed by three blocks per SM with asynchronous copies.  Newton
+// at 16^3: 449 ms with the separate kernels, 344 with this one.
 static bool gs_shape(const fv_grid* g, int* blocks, int* slice) {
   static const int sms = [] {
     int dev = 0, v = 0;

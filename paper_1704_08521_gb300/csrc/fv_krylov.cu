@@ -1226,6 +1226,20 @@ static fv_status check_grid(const fv_grid* g, const char* who) {
 
 extern "C" {
 
+fv_status fv_debug_gram_schmidt(fv_grid* g, void* V, int pairs, int j1, double* w, double* h) {
+  if (!g || !V || !w || !h || j1 < 1 || j1 > 128) {
+    set_error("fv_debug_gram_schmidt: NULL argument or j1 outside [1, 128]");
+    return FV_EINVAL;
+  }
+  FV_TRY(ensure_krylov(g, 1));
+  if (!pairs) return cgs2(g, (const double*)V, j1, w, h, h + j1, true);
+  double* dh = g->kry_small + 4 * kMaxVec;             // behind what the step itself uses
+  FV_TRY(cgs2_dev(g, (float2*)V, nullptr, j1, w, dh, 1, dh + kMaxVec, false));
+  FV_CUDA(cudaMemcpyAsync(h, dh, (j1 + 1) * sizeof(double), cudaMemcpyDeviceToHost, g->stream));
+  FV_CUDA(cudaStreamSynchronize(g->stream));
+  return FV_OK;
+}
+
 fv_status ns_residual(const fv_grid* g, const double* U, const double* P, double* F_mom,
                       double* F_div) {
   FV_TRY(check_grid(g, "ns_residual"));
