@@ -451,7 +451,9 @@ typedef struct {
 
 typedef struct {
   int iterations;  /* conjugate-gradient iterations (one V-cycle each)         */
-  int levels;      /* grids of the hierarchy, the finest included              */
+  int levels;      /* grids that the coarsening to 4 cells has, the finest
+                      included (those below the exactly solved one are not
+                      visited)                                              */
   double rel_res;  /* ||b - A phi||_2 / ||b||_2 at the end                     */
 } fv_mg_stats;
 

@@ -17,7 +17,7 @@
 //
 // Hierarchy: full coarsening of every axis with more than two cells (coarse
 // cell I = fine cells 2I and 2I+1; an odd count leaves a last coarse cell of
-// one fine cell), until no axis has more than four cells.  Coarse operators
+// one fine cell), until no axis has more than 32 cells.  Coarse operators
 // are rediscretised from the coarse cells' widths and centre distances (the
 // same a_f formula).  Prolongation: tensor product of 1-D linear
 // interpolation between coarse cell centres in the stretched coordinate,
@@ -29,10 +29,10 @@
 // every line of one colour (lines coloured like a checkerboard of their two
 // transverse indices, so neighbour lines differ in colour) exactly, in place
 // (k_line).  Pre-smoothing x, y, z (colours 0, 1) and post-smoothing in the
-// exact reverse order, so the V-cycle is a symmetric preconditioner.  The first
-// level with at most 32 cells per axis is solved exactly by the separable
-// eigenbases of its operator (A = sum over axes of K_d (x) W_others, K_d E_d =
-// W_d E_d Lambda_d), null mode dropped, in place of the levels below it.
+// exact reverse order, so the V-cycle is a symmetric preconditioner.  The last
+// level is solved exactly by the separable eigenbases of its operator (A = sum
+// over axes of K_d (x) W_others, K_d E_d = W_d E_d Lambda_d), null mode dropped,
+// in place of the levels that coarsening to four cells would still have.
 //
 // The whole iteration, its stop test included, is one CUDA graph whose WHILE
 // node runs the conjugate-gradient steps on the device; the host waits once.
@@ -51,7 +51,7 @@ namespace fv {
 namespace {
 
 constexpr int kMgMaxLevels = 16;
-constexpr int kCoarseMax = 4;       // the hierarchy ends with at most this many cells per axis
+constexpr int kCoarseMax = 4;       // coarsening would end with at most this many cells per axis
 constexpr int kRedThreads = 256;
 constexpr int kRedBlocks = 608;     // 4 x 152: fixed, so the reductions are deterministic
 
@@ -770,8 +770,8 @@ struct MgLevelHost {
 }  // namespace
 
 struct MgState {
-  int nlev = 0;
-  int exact = 0;              // the level that k_exact solves
+  int levels = 0;             // grids that the coarsening has
+  int exact = 0;              // the one that k_exact solves, the last that is built
   MgLevelHost lev[kMgMaxLevels];
   Fine64 fine;
   CoarseDev coarse;
@@ -808,10 +808,13 @@ fv_status build_mg(fv_grid* g) {
   MgState* M = new MgState();
   g->mg = M;
   const int n0[3] = {g->n[0], g->n[1], g->n[2]};
-  M->nlev = count_levels(n0);
+  M->levels = count_levels(n0);
   for (int d = 0; d < 3; ++d) M->lev[0].ax[d] = axis_from_faces(g->h_x[d]);
-  for (int l = 1; l < M->nlev; ++l)
-    for (int d = 0; d < 3; ++d) M->lev[l].ax[d] = coarsen(M->lev[l - 1].ax[d]);
+  // down to the exactly solved level; those below it are never visited
+  auto longest = [&](const MgLevelHost& H) { return std::max(H.ax[0].n, std::max(H.ax[1].n, H.ax[2].n)); };
+  for (M->exact = 0; longest(M->lev[M->exact]) > kExactMax; ++M->exact)
+    for (int d = 0; d < 3; ++d) M->lev[M->exact + 1].ax[d] = coarsen(M->lev[M->exact].ax[d]);
+  const int lc = M->exact, nlev = lc + 1;
   // table layout: per level and axis w (n), t (n + 1), pw1 (n), rw (4 n_coarse) as
   // floats; pc0 (n), rf (4 n_coarse) as ints; level-0 w, t as doubles; the coarse
   // eigenbases and eigenvalues as floats
@@ -819,7 +822,7 @@ fv_status build_mg(fv_grid* g) {
   std::vector<int> ti;
   std::vector<double> td;
   struct Off { size_t w, t, pw1, rw, pc0, rf; } off[kMgMaxLevels][3];
-  for (int l = 0; l < M->nlev; ++l) {
+  for (int l = 0; l < nlev; ++l) {
     for (int d = 0; d < 3; ++d) {
       const Axis1D& a = M->lev[l].ax[d];
       Off& o = off[l][d];
@@ -827,7 +830,7 @@ fv_status build_mg(fv_grid* g) {
       for (double v : a.w) tf.push_back((float)v);
       o.t = tf.size();
       for (double v : a.t) tf.push_back((float)v);
-      if (l + 1 < M->nlev) {
+      if (l < lc) {
         std::vector<int> c0, rf;
         std::vector<double> w1, rw;
         const Axis1D& c = M->lev[l + 1].ax[d];
@@ -857,11 +860,6 @@ fv_status build_mg(fv_grid* g) {
   }
   // the exactly solved level: W-orthonormal eigenvectors of K_d E = W_d E Lambda
   size_t cE[3], cL[3];
-  M->exact = 0;
-  while (std::max(M->lev[M->exact].ax[0].n, std::max(M->lev[M->exact].ax[1].n, M->lev[M->exact].ax[2].n)) >
-         kExactMax)
-    ++M->exact;
-  const int lc = M->exact;
   for (int d = 0; d < 3; ++d) {
     const Axis1D& a = M->lev[lc].ax[d];
     const int n = a.n;
@@ -897,16 +895,17 @@ fv_status build_mg(fv_grid* g) {
   const float* F = (const float*)base;
   const int* I = (const int*)(base + oi);
   const double* Dd = (const double*)(base + od);
-  // level arrays: x, b, res and the pivots of three directions per level
-  size_t cells = 0;
-  for (int l = 0; l < M->nlev; ++l) {
+  // level arrays: x and b, where lines are swept also res and the pivots of three
+  // directions
+  size_t floats = 0;
+  for (int l = 0; l < nlev; ++l) {
     int64_t nc = 1;
     for (int d = 0; d < 3; ++d) nc *= M->lev[l].ax[d].n;
-    cells += (size_t)(nc + 63) / 64 * 64;
+    floats += (size_t)(nc + 63) / 64 * 64 * (l < lc ? 6 : 2);
   }
-  FV_CUDA(cudaMalloc(&M->d_work, cells * 6 * sizeof(float)));
+  FV_CUDA(cudaMalloc(&M->d_work, floats * sizeof(float)));
   float* wp = (float*)M->d_work;
-  for (int l = 0; l < M->nlev; ++l) {
+  for (int l = 0; l < nlev; ++l) {
     MgLevelHost& H = M->lev[l];
     LevDev& v = H.dev;
     int64_t nc = 1;
@@ -915,7 +914,7 @@ fv_status build_mg(fv_grid* g) {
       nc *= v.n[d];
       v.w[d] = F + off[l][d].w;
       v.t[d] = F + off[l][d].t;
-      const bool has = l + 1 < M->nlev;
+      const bool has = l < lc;
       v.pw1[d] = has ? F + off[l][d].pw1 : nullptr;
       v.rw[d] = has ? F + off[l][d].rw : nullptr;
       v.pc0[d] = has ? I + off[l][d].pc0 : nullptr;
@@ -925,6 +924,7 @@ fv_status build_mg(fv_grid* g) {
     const size_t stride = (size_t)(nc + 63) / 64 * 64;
     H.x = wp; wp += stride;
     H.b = wp; wp += stride;
+    if (l == lc) continue;
     H.res = wp; wp += stride;
     for (int d = 0; d < 3; ++d) {
       H.ip[d] = wp;
@@ -957,7 +957,7 @@ fv_status build_mg(fv_grid* g) {
   M->zo = (float*)(cg + 3 * nb + tail);
   FV_CUDA(cudaMemset(M->red.part, 0, tail));
   FV_CUDA(cudaMallocHost((void**)&M->h, sizeof(*M->h)));
-  for (int l = 0; l < M->exact; ++l) {
+  for (int l = 0; l < lc; ++l) {
     const MgLevelHost& H = M->lev[l];
     const LevDev& v = H.dev;
     auto blocks = [](int lines) { return (lines + 127) / 128; };
@@ -1207,7 +1207,7 @@ fv_status mg_solve(fv_grid* g, const double* r, double* phi, const double* guess
   FV_TRY(fetch());
   const double bnorm = std::sqrt(hs[S_BB]);
   fv_mg_stats sv = {};
-  sv.levels = M->nlev;
+  sv.levels = M->levels;
   sv.iterations = (int)hs[S_IT];
   sv.rel_res = bnorm > 0.0 ? rnorm() / bnorm : 0.0;
   if (stats) *stats = sv;
