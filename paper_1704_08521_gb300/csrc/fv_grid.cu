@@ -389,10 +389,16 @@ static fv_status build(fv_grid* g) {
     g->met_fn.ncell = g->ncell;
     for (int d = 0; d < 3; ++d) g->met_ff.idcf[d] = (const float2*)g->met_fn.idc[d];
   }
-  FV_CUDA(cudaMemset(g->d_fault, 0, 256));
-  FV_TRY(fill_face_weights(g));
   FV_CUDA(cudaMallocHost((void**)&g->h_scal, kScalars * sizeof(double)));
+  FV_CUDA(cudaMemset(g->d_fault, 0, 256));
   FV_CUDA(cudaMemset(g->d_scal, 0, kScalars * sizeof(double)));
+  // copies and sets above went through the legacy stream, the kernels below run
+  // on the grid's, and the first call may be on yet another one
+  // (fv_grid_set_stream): each waits for what is before it
+  FV_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+  FV_TRY(fill_face_weights(g));
+  FV_TRY(fill_oz_factors(g));
+  FV_CUDA(cudaStreamSynchronize(g->stream));
   return FV_OK;
 }
 

@@ -371,6 +371,7 @@ fv_status transform_axis_f64(const fv_grid* g, int axis, int inverse, const doub
 // grid), whether `axis` has them, one transform, its results times factors
 // (y or z axis; vectors are at most 2^30 / n)
 fv_status build_oz(fv_grid* g);
+fv_status fill_oz_factors(fv_grid* g);
 bool oz_ok(const fv_grid* g, int axis);
 struct OzScale {
   const double* inv = nullptr;   // factors, or none

@@ -444,17 +444,20 @@ fv_status build_oz(fv_grid* g) {
       g->oz.rexp[d][q] = (const int*)((const char*)g->d_oz + off[d][q] + one - 512);
     }
   }
-  if (all) {
-    g->oz.inv = (double*)((char*)g->d_oz + bytes);
-    k_inv_lam<<<(unsigned)std::min<int64_t>((g->ncell + 255) / 256, 152 * 16), 256, 0, g->stream>>>(
-        g->tpf_d, g->oz.inv, g->ncell);
-    FV_CHECK_LAUNCH();
-  }
+  if (all) g->oz.inv = (double*)((char*)g->d_oz + bytes);
   const int cap = (int)std::max(oz_smem(112), oz_smem(kOzMax));
   FV_CUDA(cudaFuncSetAttribute(k_oz<true, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   FV_CUDA(cudaFuncSetAttribute(k_oz<false, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   FV_CUDA(cudaFuncSetAttribute(k_oz<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   FV_CUDA(cudaFuncSetAttribute(k_oz<false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+  return FV_OK;
+}
+
+fv_status fill_oz_factors(fv_grid* g) {
+  if (!g->oz.inv) return FV_OK;
+  k_inv_lam<<<(unsigned)std::min<int64_t>((g->ncell + 255) / 256, 152 * 16), 256, 0, g->stream>>>(
+      g->tpf_d, g->oz.inv, g->ncell);
+  FV_CHECK_LAUNCH();
   return FV_OK;
 }
 
