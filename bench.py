@@ -126,7 +126,7 @@ def algorithmic(kind, n, prec):
     else:
         f = 4
         table = {"momentum": 36,                 # read U, v (3 x 4 B each), write w (3 x 4 B)
-                 "correct": 12 + 2 * 4 + 4,       # second pass: read w (3 x 4 B), two corrections, write r
+                 "correct": 24 + 4 + 24 + 4,      # second pass: read v (3 x 8 B) and phi, write v and r
                  "divergence": 16}               # read w (3 x 4 B), write r
     if kind in ("tpf_x", "tpf_xinv", "tpf_yz"):
         # fused tensor-core kernels (n <= 112) apply two 1-D transforms per
@@ -387,13 +387,14 @@ def run_ours(args):
     # writes w in float32; each pass moves the float64 state and the float32
     # pressure right-hand side and correction), over the time per solve; beside
     # it the bytes this implementation moves by design (float64 x read by J.v,
-    # D w, per pass m three transform launches and a pass over w and m
-    # corrections, join of v and p to float64)
+    # D w, per pass three transform launches and a pass from one float-float v
+    # to the other, the first one from float32, p beyond the third; join of v and,
+    # from at most three corrections, p to float64)
     solve_roof = None
     if mixed:
         bpc = 36 + 80 * passes
-        k = min(passes, 3)   # passes beyond the third store the float-float state (72 B)
-        impl = 48 + 16 + sum(3 * 8 + 16 + 4 * m for m in range(1, k + 1)) + (passes - k) * (3 * 8 + 72) + 12 + 4 * k + 32
+        k = min(passes, 3)
+        impl = 48 + 16 + passes * (3 * 8 + 56) - 12 + (passes - k) * 16 + 24 + 4 * k + 32
         bytes_solve = bpc * n ** 3
         ach = bytes_solve * value / ws / 1e9
         pk_hbm = pk.get("hbm_gbs", 6800.0)

@@ -22,7 +22,12 @@
 // times smaller than the largest entries of row and vector, so a version that
 // cut at 2^-54 of their product (36 products, groups 5 .. 7 joined) was up to
 // four times less accurate than float64 sums; this one is no less accurate
-// (tests/test_gpu_oz.py against extended precision).
+// (tests/test_gpu_oz.py against extended precision).  What a vector holds more than
+// 2^-60 below its largest entry is lost, where float64 keeps every entry relative
+// to itself; in a solve this shows nowhere: right-hand sides of single cells, wall
+// layers and entries over 18 orders of magnitude came out 3 to 7 times more accurate
+// than with the float64 kernels, in the largest error, the mean square and
+// component by component (median and 99 %).
 //
 // One block: N K-vectors of the field, all n <= 128 rows of M.  The field is
 // split once into its digits (N x K x 8 BF16, the B operands, resident); the

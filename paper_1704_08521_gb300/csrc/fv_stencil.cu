@@ -225,8 +225,8 @@ fv_status launch_momentum_jac(const fv_grid* g, const double* U, const double* v
 // float32 J.v of the mixed form: U from Ud (float64, rounded into g->U32
 // first, which drops a registered base flow) or, when Ud is null, from the
 // grid's registered base flow g->U32; x float64 rounded as its planes are
-// staged; float32 result.  call: graph launches read x from the evaluation's
-// device call block (whose U the graph has already rounded into g->U32).
+// staged; float32 result.  dcb, ls (evaluation graphs): where the kernel stores
+// the call's arguments and resets the loop state.
 fv_status launch_jv_f32(const fv_grid* g, const double* Ud, const double* x, float* out,
                         double shift, CallBlock* dcb, LoopState* ls) {
   if (Ud) {

@@ -159,9 +159,10 @@ __device__ __forceinline__ void stage_halo(bf16* xs, const ConvIn& in, int c0, i
 //   index; the [co][ci] rows are read transposed by ldmatrix.trans, so no
 //   flipped copy is made.  mask (optional): Y is zeroed where mask <= 0 (the
 //   ReLU of the layer that produced this input).
-// mma.sync rather than tcgen05: the sums must come out in the order (tap,
-// channel chunk) whatever the tiling, because every stored BF16 value (and
-// ReLU decision) downstream flips with the last bit of a float32 sum.
+// mma.sync rather than tcgen05: a choice, not a bound.  Taps and channel chunks
+// could be issued to a tensor-memory accumulator in this order as well; its sums
+// would round differently inside a step of 16 channels, and with the last bit of a
+// float32 sum stored BF16 values and ReLU decisions downstream flip.
 // Bound by launch latency at the coarse levels (8^3..16^3 cells) and by shared
 // memory at level 0 (3 KB of fragments per 16 KFLOP).  Measured 33 us for
 // 16 -> 16 at 64^3 and 10 us for 64 -> 64 at 8^3; the version that read its
