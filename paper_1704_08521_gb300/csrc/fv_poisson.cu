@@ -957,8 +957,9 @@ fv_status tpf_solve(const fv_grid* g, const double* r, void* phi, int prec) {
 // float-float result does not depend on how the inner solve rounds (the loop
 // removes it); a mixed one would move by ~5e-8 of v, the float32 rounding of its
 // first correction, well within the 2e-5 that the form promises.  That is the only
-// obstacle: at 150^3 a mixed evaluation takes 1229 us and a float-float one 1033,
-// so beyond this size the float-float form is both the exact and the faster one.
+// obstacle: a mixed evaluation takes 474 us at 113^3, 612 at 128^3 and 1223 at 150^3, a
+// float-float one 502, 568 and 1038, so from about 125 cells on the float-float form
+// is both the exact and the faster one.
 fv_status tpf_solve_f32(const fv_grid* g, const float* r, float* phi, int prec, const int* skip) {
   if (fused_ok(g)) return tpf_fused_f32(g, r, phi, skip);
   if (prec == FV_FF && xf_ok(g)) return xf_solve(g, r, phi, skip);
